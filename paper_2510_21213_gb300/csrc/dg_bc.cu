@@ -49,15 +49,89 @@ template cudaError_t launch_weighted_lex<float>(const LevelOp&, const LevelOp*, 
                                                 int, cudaStream_t);
 
 // ---------------------------------------------------------------------------
-// Strided batched GEMM: C[m,n] = alpha sum_k A[m,k] B[k,n] + beta C[m,n]
+// FP64 strided batched GEMM: C[m,n] = alpha sum_k A[m,k] B[k,n] + beta C[m,n]
 // with arbitrary element strides and a two-level batch index.
-// 64 x 64 output tile, K step 16, 256 threads with 4 x 4 outputs each.
+//
+// Bound by the FP64 pipe (2 FMA per clock and SM: a warp's FMA occupies a
+// quarter of an SM for 64 clocks), so shared-memory traffic and instruction
+// issue do not matter; what does is that no FMA is spent on padding and that
+// enough blocks are in flight. 32 x 32 output tile, K step 32, 8 warps; a warp
+// owns 4 rows and a lane one column of them, so rows outside M cost nothing and
+// columns are padded to 32 only (a 64 x 64 tile spent 10x the FMAs at 20 nodes
+// an axis). Long contractions (K = N_G L in the last step of the boundary data,
+// with few output tiles) are split into ranges of about 256 terms
+// (k_gemm_splitk_reduce<double> adds them in order).
 // ---------------------------------------------------------------------------
-// (FP64 instances; FP32 runs on the tensor cores in k_gemm_tc below.)
-// FP32 instances keep a compensated running sum across K tiles: each 16-term
-// tile is accumulated in registers and then added to (sum, carry) with
-// Knuth's TwoSum, so the error does not grow with K (K reaches N_G L ~ 10^4 in
-// the boundary-data contractions).
+constexpr int G64_T = 32;    // output tile and K step
+constexpr int G64_ROWS = 4;  // rows per warp
+
+__global__ void __launch_bounds__(256) k_gemm64(GemmArgs g, int batch_base, int nsplit, int kc, int nbc) {
+  __shared__ double sA[G64_T][G64_T + 1];
+  __shared__ double sB[G64_T][G64_T + 1];
+  const int bz = batch_base + (int)blockIdx.z / nsplit;
+  const int split = (int)blockIdx.z % nsplit;
+  const int kbeg = split * kc, kend = min(g.K, kbeg + kc);
+  const int b1 = bz / g.nb2, b2 = bz % g.nb2;
+  const double* A = (const double*)g.A + b1 * g.sA1 + b2 * g.sA2;
+  const double* B = (const double*)g.B + b1 * g.sB1 + b2 * g.sB2;
+  double* C = (double*)g.C + b1 * g.sC1 + b2 * g.sC2;
+  const int m0 = blockIdx.y * G64_T, n0 = blockIdx.x * G64_T;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const bool a_k_fast = g.sAk == 1;
+  const bool b_n_fast = g.sBn == 1;
+  const int r0 = warp * G64_ROWS;
+  const bool rows_in = m0 + r0 < g.M;
+  double acc[G64_ROWS];
+#pragma unroll
+  for (int i = 0; i < G64_ROWS; ++i) acc[i] = 0.0;
+  for (int k0 = kbeg; k0 < kend; k0 += G64_T) {
+#pragma unroll
+    for (int p = 0; p < G64_ROWS; ++p) {
+      const int slow = warp + 8 * p;  // the index that is slow in memory; lanes run along the fast one
+      const int ka = a_k_fast ? lane : slow, ma = a_k_fast ? slow : lane;
+      const int kb = b_n_fast ? slow : lane, nb = b_n_fast ? lane : slow;
+      sA[ka][ma] = (m0 + ma < g.M && k0 + ka < kend)
+                       ? A[(long long)(m0 + ma) * g.sAm + (long long)(k0 + ka) * g.sAk] : 0.0;
+      sB[kb][nb] = (n0 + nb < g.N && k0 + kb < kend)
+                       ? B[(long long)(k0 + kb) * g.sBk + (long long)(n0 + nb) * g.sBn] : 0.0;
+    }
+    __syncthreads();
+    if (rows_in) {
+      const int kn = min(G64_T, kend - k0);
+      if (kn == G64_T) {
+#pragma unroll 8
+        for (int kk = 0; kk < G64_T; ++kk) {
+          const double b = sB[kk][lane];
+#pragma unroll
+          for (int i = 0; i < G64_ROWS; ++i) acc[i] += sA[kk][r0 + i] * b;
+        }
+      } else {
+        for (int kk = 0; kk < kn; ++kk) {
+          const double b = sB[kk][lane];
+#pragma unroll
+          for (int i = 0; i < G64_ROWS; ++i) acc[i] += sA[kk][r0 + i] * b;
+        }
+      }
+    }
+    __syncthreads();
+  }
+  const int n = n0 + lane;
+  if (n >= g.N) return;
+#pragma unroll
+  for (int i = 0; i < G64_ROWS; ++i) {
+    const int m = m0 + r0 + i;
+    if (m >= g.M) break;
+    if (nsplit > 1) {
+      ((double*)g.work)[(((long long)split * nbc + (bz - batch_base)) * g.M + m) * g.N + n] = acc[i];
+      continue;
+    }
+    double* cp = C + (long long)m * g.sCm + (long long)n * g.sCn;
+    *cp = g.beta != 0.0 ? g.alpha * acc[i] + g.beta * (*cp) : g.alpha * acc[i];
+  }
+}
+
+// s + c is the running sum and its carry (Knuth's TwoSum): the error of a sum
+// does not grow with its length
 template <typename T>
 __device__ __forceinline__ void two_sum_add(T& s, T& c, T a) {
   const T t = s + a;
@@ -66,97 +140,12 @@ __device__ __forceinline__ void two_sum_add(T& s, T& c, T a) {
   s = t;
 }
 
-template <typename T>
-__global__ void __launch_bounds__(256) k_gemm(GemmArgs g, int batch_base) {
-  constexpr bool COMP = sizeof(T) == 4;
-  __shared__ T sA[16][64 + 1];
-  __shared__ T sB[16][64 + 1];
-  const int bz = batch_base + blockIdx.z;
-  const int b1 = bz / g.nb2, b2 = bz % g.nb2;
-  const T* A = (const T*)g.A + b1 * g.sA1 + b2 * g.sA2;
-  const T* B = (const T*)g.B + b1 * g.sB1 + b2 * g.sB2;
-  T* C = (T*)g.C + b1 * g.sC1 + b2 * g.sC2;
-  const int m0 = blockIdx.y * 64, n0 = blockIdx.x * 64;
-  const int tid = threadIdx.x, tx = tid % 16, ty = tid / 16;
-  const bool a_k_fast = g.sAk == 1;
-  const bool b_n_fast = g.sBn == 1;
-  T acc[4][4], sum[4][4], car[4][4];
-#pragma unroll
-  for (int i = 0; i < 4; ++i)
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      acc[i][j] = (T)0;
-      sum[i][j] = (T)0;
-      car[i][j] = (T)0;
-    }
-  for (int k0 = 0; k0 < g.K; k0 += 16) {
-    for (int t = tid; t < 64 * 16; t += 256) {
-      int kk, mm;
-      if (a_k_fast) {
-        kk = t % 16;
-        mm = t / 16;
-      } else {
-        mm = t % 64;
-        kk = t / 64;
-      }
-      const int m = m0 + mm, k = k0 + kk;
-      sA[kk][mm] = (m < g.M && k < g.K) ? A[(long long)m * g.sAm + (long long)k * g.sAk] : (T)0;
-      int nn, kb;
-      if (b_n_fast) {
-        nn = t % 64;
-        kb = t / 64;
-      } else {
-        kb = t % 16;
-        nn = t / 16;
-      }
-      const int n = n0 + nn, kx = k0 + kb;
-      sB[kb][nn] = (n < g.N && kx < g.K) ? B[(long long)kx * g.sBk + (long long)n * g.sBn] : (T)0;
-    }
-    __syncthreads();
-#pragma unroll
-    for (int kk = 0; kk < 16; ++kk) {
-      T a[4], b[4];
-#pragma unroll
-      for (int i = 0; i < 4; ++i) a[i] = sA[kk][ty + 16 * i];
-#pragma unroll
-      for (int j = 0; j < 4; ++j) b[j] = sB[kk][tx + 16 * j];
-#pragma unroll
-      for (int i = 0; i < 4; ++i)
-#pragma unroll
-        for (int j = 0; j < 4; ++j) acc[i][j] += a[i] * b[j];
-    }
-    if (COMP) {
-#pragma unroll
-      for (int i = 0; i < 4; ++i)
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-          two_sum_add(sum[i][j], car[i][j], acc[i][j]);
-          acc[i][j] = (T)0;
-        }
-    }
-    __syncthreads();
-  }
-  const T alpha = (T)g.alpha, beta = (T)g.beta;
-#pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    const int m = m0 + ty + 16 * i;
-    if (m >= g.M) continue;
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      const int n = n0 + tx + 16 * j;
-      if (n >= g.N) continue;
-      const T v = COMP ? sum[i][j] + car[i][j] : acc[i][j];
-      T* cp = C + (long long)m * g.sCm + (long long)n * g.sCn;
-      *cp = g.beta != 0.0 ? alpha * v + beta * (*cp) : alpha * v;
-    }
-  }
-}
-
 // ---------------------------------------------------------------------------
 // FP32 strided batched GEMM on the tensor cores: mma.sync m16n8k8 TF32 with
 // the 3xTF32 split (a = a_hi + a_lo, both TF32; a b ~ a_hi b_hi + a_hi b_lo +
-// a_lo b_hi, error ~ 2^-22 of |a b|) and the same compensated accumulation
-// across 16-term K tiles as k_gemm. 64 x 64 output tile, 4 warps of 32 x 32.
+// a_lo b_hi, error ~ 2^-22 of |a b|) and compensated accumulation
+// across K: each 16-term tile is accumulated in registers and then added to
+// (sum, carry) with TwoSum (K reaches N_G L ~ 10^4). 64 x 64 output tile, 4 warps of 32 x 32.
 // ---------------------------------------------------------------------------
 __device__ __forceinline__ unsigned to_tf32(float x) {
   unsigned r;
@@ -300,55 +289,57 @@ __global__ void __launch_bounds__(128) k_gemm_tc(GemmArgs g, int batch_base, int
 
 // C = alpha sum_split work[split] (+ beta C) for batches batch_base ..
 // batch_base + nbc - 1, splits added in order with TwoSum
+template <typename T>
 __global__ void k_gemm_splitk_reduce(GemmArgs g, int nsplit, int batch_base, int nbc) {
   const long long mn = (long long)g.M * g.N, total = (long long)nbc * mn;
-  const float* w = (const float*)g.work;
+  const T* w = (const T*)g.work;
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < total;
        i += (long long)gridDim.x * blockDim.x) {
-    float sum = 0.f, car = 0.f;
+    T sum = 0, car = 0;
     for (int sp = 0; sp < nsplit; ++sp) two_sum_add(sum, car, w[(long long)sp * total + i]);
     const long long bz = batch_base + i / mn, r = i % mn;
     const int m = (int)(r / g.N), n = (int)(r - (long long)m * g.N);
     const int b1 = (int)(bz / g.nb2), b2 = (int)(bz % g.nb2);
-    float* cp = (float*)g.C + b1 * g.sC1 + b2 * g.sC2 + (long long)m * g.sCm + (long long)n * g.sCn;
-    const float v = sum + car;
-    *cp = g.beta != 0.0 ? (float)g.alpha * v + (float)g.beta * (*cp) : (float)g.alpha * v;
+    T* cp = (T*)g.C + b1 * g.sC1 + b2 * g.sC2 + (long long)m * g.sCm + (long long)n * g.sCn;
+    const T v = sum + car;
+    *cp = g.beta != 0.0 ? (T)g.alpha * v + (T)g.beta * (*cp) : (T)g.alpha * v;
   }
 }
 
 template <typename T>
 cudaError_t launch_gemm(const GemmArgs& g, cudaStream_t s) {
   if (g.M <= 0 || g.N <= 0 || g.nb1 * (long long)g.nb2 <= 0) return cudaSuccess;
+  constexpr bool F32 = sizeof(T) == 4;
   const long long nb = (long long)g.nb1 * g.nb2;
-  const dim3 grid((g.N + 63) / 64, (g.M + 63) / 64, 1);
+  constexpr int TILE = F32 ? 64 : G64_T;
+  const dim3 grid((g.N + TILE - 1) / TILE, (g.M + TILE - 1) / TILE, 1);
   if (grid.y > 65535) return cudaErrorInvalidValue;
-  if constexpr (sizeof(T) == 4) {
-    // a long K is split over blocks into fixed 512-term ranges (from K alone,
-    // so a batch's sums do not depend on how many batches share the call);
-    // batches go through in chunks that fit the workspace
-    int nsplit = 1;
-    if (g.work && g.K >= 1024) nsplit = std::min(32, (g.K + 511) / 512);
-    const int kc = nsplit > 1 ? ((g.K + nsplit - 1) / nsplit + 15) / 16 * 16 : g.K;
-    if (nsplit > 1) nsplit = (g.K + kc - 1) / kc;  // no empty split
-    long long per = 65535 / nsplit;
-    if (nsplit > 1) per = std::min<long long>(per, g.work_elems / ((long long)nsplit * g.M * g.N));
-    if (per < 1) return cudaErrorInvalidValue;  // workspace too small for one batch
-    for (long long base = 0; base < nb; base += per) {
-      const long long cnt = nb - base < per ? nb - base : per;
+  // a long K is split over blocks into fixed ranges (512 terms in FP32, 256 in
+  // FP64; from K alone, so a batch's sums do not depend on how many batches
+  // share the call); batches go through in chunks that fit the workspace
+  constexpr int RANGE = F32 ? 512 : 256;
+  int nsplit = 1;
+  if (g.work && g.K >= 2 * RANGE) nsplit = std::min(32, (g.K + RANGE - 1) / RANGE);
+  // FP64 output larger than the workspace holds (over 500 nodes an axis): enough tiles without a split
+  if (!F32 && nsplit > 1 && g.work_elems < (long long)nsplit * g.M * g.N) nsplit = 1;
+  const int kc = nsplit > 1 ? ((g.K + nsplit - 1) / nsplit + 15) / 16 * 16 : g.K;
+  if (nsplit > 1) nsplit = (g.K + kc - 1) / kc;  // no empty split
+  long long per = 65535 / nsplit;
+  if (nsplit > 1) per = std::min<long long>(per, g.work_elems / ((long long)nsplit * g.M * g.N));
+  if (per < 1) return cudaErrorInvalidValue;  // workspace too small for one batch
+  for (long long base = 0; base < nb; base += per) {
+    const long long cnt = nb - base < per ? nb - base : per;
+    const dim3 gr(grid.x, grid.y, (unsigned)(cnt * nsplit));
+    count_launch();
+    if constexpr (F32)
+      k_gemm_tc<<<gr, 128, 0, s>>>(g, (int)base, nsplit, kc, (int)cnt);
+    else
+      k_gemm64<<<gr, 256, 0, s>>>(g, (int)base, nsplit, kc, (int)cnt);
+    if (nsplit > 1) {
       count_launch();
-      k_gemm_tc<<<dim3(grid.x, grid.y, (unsigned)(cnt * nsplit)), 128, 0, s>>>(g, (int)base, nsplit, kc, (int)cnt);
-      if (nsplit > 1) {
-        count_launch();
-        const long long total = cnt * g.M * g.N;
-        k_gemm_splitk_reduce<<<(unsigned)std::min<long long>((total + 255) / 256, 152LL * 16), 256, 0, s>>>(
-            g, nsplit, (int)base, (int)cnt);
-      }
-    }
-  } else {
-    for (long long base = 0; base < nb; base += 65535) {
-      const long long cnt = nb - base < 65535 ? nb - base : 65535;
-      count_launch();
-      k_gemm<T><<<dim3(grid.x, grid.y, (unsigned)cnt), 256, 0, s>>>(g, (int)base);
+      const long long total = cnt * g.M * g.N;
+      k_gemm_splitk_reduce<T><<<(unsigned)std::min<long long>((total + 255) / 256, 152LL * 16), 256, 0, s>>>(
+          g, nsplit, (int)base, (int)cnt);
     }
   }
   return cudaGetLastError();

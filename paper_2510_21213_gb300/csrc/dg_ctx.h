@@ -187,7 +187,7 @@ struct dg_ctx {
   int NG = 0, NG32 = 0;
   dg::BcAxisTables bct[3], bct32[3];
   dg::DevBuf flex32, T1_32, T2_32, g32;
-  dg::DevBuf gemm_ws;              // split-K partials of the FP32 boundary-data GEMMs
+  dg::DevBuf gemm_ws;              // split-K partials of the boundary-data GEMMs
   // workspaces
   dg::PrecWork<double> w64;
   dg::PrecWork<float> w32;

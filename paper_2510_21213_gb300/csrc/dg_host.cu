@@ -119,7 +119,7 @@ static int ensure_bc_work(dg_ctx* h, int nsrc, int NG, BcAxisTables* bct, DevBuf
   const size_t tb = sizeof(T) * 2 * (size_t)NG * maxface * nsrc;
   DG_CK(T1.ensure(tb));
   DG_CK(T2.ensure(tb));
-  if (sizeof(T) == 4) DG_CK(h->gemm_ws.ensure(sizeof(float) * (16LL << 20)));  // 64 MB of split-K partials
+  DG_CK(h->gemm_ws.ensure(64LL << 20));  // split-K partials
   return DG_OK;
 }
 
@@ -738,10 +738,8 @@ static int boundary_gausssum(dg_ctx* h, const double* f, int nsrc, T* g, BcAxisT
     c.sC2 = L1 * L2;
     c.alpha = 1.0;
     c.beta = 0.0;
-    if (sizeof(T) == 4) {  // K = N_G L over few output tiles: split K (FP32 path)
-      c.work = h->gemm_ws.p;
-      c.work_elems = (long long)(h->gemm_ws.bytes / sizeof(float));
-    }
+    c.work = h->gemm_ws.p;  // K = N_G L over few output tiles: split K
+    c.work_elems = (long long)(h->gemm_ws.bytes / sizeof(T));
     DG_CK(launch_gemm<T>(c, s));
     face_off += 2 * L1 * L2;
   }
