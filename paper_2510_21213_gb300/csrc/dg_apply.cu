@@ -1,331 +1,532 @@
 // Matrix-free SIPDG operator (Sec. 3.4 eq. sip_bilinear with the penalty of
 // Sec. 3.5 and Nitsche boundary faces) on the element-blocked layout.
 //
-// One work item = one element of one right-hand side. For element e the
-// kernel needs its own (p+1)^3 values and, for each of its six faces, the
-// neighbour's trace and reference normal derivative on that face (2 (p+1)^2
-// numbers per face): the off-diagonal blocks of the 1-D operator are rank 2.
-// Output node (a, b, c):
+// For an element the operator needs its own (p+1)^3 values and, for each of its
+// six faces, the neighbour's trace and reference normal derivative there (the
+// off-diagonal blocks of the 1-D operator are rank 2). Output node (a, b, c):
 //   (Au) = My_b Mz_c [sum_i Kx[a,i] u_ibc + cL.x(-x traces) + cR.x(+x traces)]
 //        + Mx_a Mz_c [ ... y ... ] + Mx_a My_b [ ... z ... ]
-// with Kx the element's diagonal block (volume term plus its own face terms,
-// Nitsche terms on boundary faces).
+//
+// Arithmetic of one line (N1 = p + 1 values along the direction). The GL nodes
+// are symmetric about the element's middle, so the interior element's 1-D block
+// K and the pair of couplings are invariant under reversing the line. With
+// e_i = v_i + v_(N1-1-i) and o_i = v_i - v_(N1-1-i) the line splits into an even
+// and an odd half of size N1/2: K costs N1^2/2 multiply-adds instead of N1^2,
+// the couplings to both neighbours 2 N1 instead of 4 N1. A boundary face is a
+// face whose neighbour has the traces
+//   value = -t,  derivative = d -+ sigma h t   (- left, + right)
+// with t, d the element's own trace and derivative there: inserted into the
+// interior coupling they turn it into the Nitsche terms, so every element of an
+// axis has the same tables and no element type is distinguished. 41 operations
+// a node instead of 52 (p = 7).
+//
+// Work split. A brick of 2 x 2 x 2 elements of one source (or a single element)
+// per slot; in the pass along a direction a thread owns the lines of the two
+// elements that are neighbours along it, so the traces across their common face
+// stay in registers, and a brick reads 24 outer neighbours instead of the 48 of
+// eight single elements. All global reads (own elements and the outer
+// neighbours' lines, reduced to traces at once) happen before the first
+// barrier. The tables are kernel parameters: every product takes its constant
+// from the constant bank, so shared memory carries only the field.
+//
+// Measured (GB300; before: one element per slot, dense blocks and tables in
+// shared memory): FP32 16^3, p = 7, 42 fields 0.720 -> 0.279 ms (2.5 TB/s of the
+// 0.70 GB in and out), 8^3, p = 6, 56 fields 0.100 -> 0.042 ms; bound by
+// shared-memory wavefronts, then by the neighbours' reads. FP64, at the rate of
+// its pipe before and after: 7.86 -> 7.25 ms and 0.955 -> 0.824 ms; at p = 3 and
+// 1, where folding saves nothing, 0.83 -> 0.86 ms and 0.089 -> 0.111 ms (16^3, 42
+// fields; 3 % and 0.4 % of an FP64 build).
 #include "dg_internal.h"
 
 namespace dg {
 
+#ifndef DG_APPLY_TIE32
+#define DG_APPLY_TIE32 128
+#endif
+#ifndef DG_APPLY_TIE64
+#define DG_APPLY_TIE64 64
+#endif
+#ifndef DG_APPLY_WANT32
+#define DG_APPLY_WANT32 768
+#endif
+#ifndef DG_APPLY_WANT64
+#define DG_APPLY_WANT64 640
+#endif
+#ifndef DG_APPLY_MIN_BLOCKS
+#define DG_APPLY_MIN_BLOCKS 304  // blocks that fill the chip (two per SM)
+#endif
 
-// Launch layout: EPB elements per block; in the three 1-D passes each thread
-// owns LPT lines of one element (line values in registers, the 1-D block rows
-// streamed from shared memory and reused across the lines). Loads of the
-// element, the neighbour traces and the final store are spread over all
-// threads of the block and coalesced.
-// Tuning constants (compile-time; the defaults were chosen by timing on a GB300)
-#ifndef DG_APPLY_LPT32
-#define DG_APPLY_LPT32 2      // lines per thread, FP32
-#endif
-#ifndef DG_APPLY_THREADS
-#define DG_APPLY_THREADS 256  // threads per block (at least)
-#endif
-#ifndef DG_APPLY_SMEM
-#define DG_APPLY_SMEM 38912   // shared-memory budget of the element slots (bytes)
-#endif
-#ifndef DG_SMEM_CARVEOUT
-#define DG_SMEM_CARVEOUT -1  // shared-memory carveout (percent) asked for the operator and patch kernels; -1: default
-#endif
-#ifndef DG_APPLY_MINB32
-#define DG_APPLY_MINB32 4     // resident blocks per SM asked of ptxas, FP32
-#endif
-// Element values in shared memory: node (a, b, c) at a + PB b + PB N1 c. With
-// an even N1 the rows are padded by one (PB = N1 + 1), so that the x-pass's
-// threads, which own consecutive x-lines, fall on different banks.
-template <int N1>
-struct ApplyPad {
-  static constexpr int PB = N1 % 2 == 0 ? N1 + 1 : N1;
-  static constexpr int PNPE = PB * N1 * N1;
-  // shared-memory index of the element-local node loc = a + N1 b + N1^2 c
-  __device__ static __forceinline__ int idx(int loc) { return loc + (PB - N1) * (loc / N1); }
+// 1-D tables of one level, folded into even and odd halves (host-built, passed
+// by value). HE = ceil(N1/2) even and HO = floor(N1/2) odd rows.
+//
+// N1 = 2 is not folded (two sums and differences per line cost what the halves
+// save): there Ke, Ko hold K[0][0], K[0][1], and likewise the couplings their
+// entries 0 and 1.
+template <typename T, int N1>
+struct ApplyTab {
+  static constexpr int HO = N1 / 2, HE = N1 - HO;
+  T Ke[3][HE][HE], Ko[3][HO][HO];                          // K on the even and the odd part
+  T cve[3][HE], cde[3][HE], cvo[3][HO], cdo[3][HO];        // couplings (neighbour value / derivative)
+  T tl[N1], dl[N1];                                        // trace and derivative at a line's left end
+  T gam[3];                                                // sigma h
+  T mm[3][N1 * N1];                                        // products of the two other axes' masses, by line
+  int n[3], nb[3];                                         // elements and bricks per axis
+  long long Nq, items;                                     // nodes of a source; bricks of all sources
 };
 
 template <typename T, int N1>
-struct ApplyCfg {
-  static constexpr int NPE = N1 * N1 * N1;
-  static constexpr int NF = N1 * N1;
-  static constexpr int PNPE = ApplyPad<N1>::PNPE;
-  static constexpr int LPT = sizeof(T) == 4 ? DG_APPLY_LPT32 : 1;
-  static constexpr int TPE = (NF + LPT - 1) / LPT;
-  static constexpr int PER_ELEM = (2 * PNPE + 12 * NF + 3) * (int)sizeof(T);
-  static constexpr int EPB_T = DG_APPLY_THREADS / TPE < 1 ? 1 : DG_APPLY_THREADS / TPE;
-  static constexpr int EPB_S = DG_APPLY_SMEM / PER_ELEM < 1 ? 1 : DG_APPLY_SMEM / PER_ELEM;
-  static constexpr int EPB = EPB_T < EPB_S ? EPB_T : EPB_S;
-  // the load and trace phases use every thread of the block; the line passes
-  // use the first EPB * TPE
-  static constexpr int THREADS = EPB * TPE < DG_APPLY_THREADS ? DG_APPLY_THREADS : EPB * TPE;
-  // resident blocks per SM asked of ptxas (p = 8 keeps 3: at 4 its registers spill)
-  static constexpr int MINB = sizeof(T) == 4 ? (N1 >= 9 ? 3 : DG_APPLY_MINB32) : 2;
-};
-
-// one direction of the operator for LPT lines of one element:
-// sacc[line] (+)= m1 * m2 * (K_ty v + cLv tv- + cLd td- + cRv tv+ + cRd td+)
-template <typename T, int N1, int LPT, int TPE, int DIR, bool ACCUM>
-__device__ __forceinline__ void ap_pass(const T* __restrict__ su, T* __restrict__ sacc, const T* __restrict__ K,
-                                        const T* __restrict__ cc, const T* __restrict__ tr,
-                                        const T* __restrict__ mA, const T* __restrict__ mB, int lt) {
-  constexpr int NF = N1 * N1;
-  constexpr int PB = ApplyPad<N1>::PB;
-  constexpr int stride = DIR == 0 ? 1 : (DIR == 1 ? PB : PB * N1);
-  T v[LPT][N1];
-  int base[LPT], tt[LPT];
-  bool ok[LPT];
-  T scale[LPT], tvm[LPT], tdm[LPT], tvp[LPT], tdp[LPT];
-#pragma unroll
-  for (int s = 0; s < LPT; ++s) {
-    const int l = lt + TPE * s;
-    ok[s] = l < NF;
-    const int l1 = ok[s] ? l % N1 : 0, l2 = ok[s] ? l / N1 : 0;
-    // line (l1, l2) = (b, c) for x, (a, c) for y, (a, b) for z
-    base[s] = DIR == 0 ? PB * l1 + PB * N1 * l2 : (DIR == 1 ? l1 + PB * N1 * l2 : l1 + PB * l2);
-    tt[s] = l1 + N1 * l2;
-    scale[s] = mA[l1] * mB[l2];
-    tvm[s] = tr[(0 * 2 + 0) * NF + tt[s]];
-    tdm[s] = tr[(0 * 2 + 1) * NF + tt[s]];
-    tvp[s] = tr[(1 * 2 + 0) * NF + tt[s]];
-    tdp[s] = tr[(1 * 2 + 1) * NF + tt[s]];
-#pragma unroll
-    for (int i = 0; i < N1; ++i) v[s][i] = su[base[s] + i * stride];
+static void fill_tab(ApplyTab<T, N1>& t, const LevelOp& op) {
+  constexpr int HO = N1 / 2, HE = N1 - HO;
+  for (int d = 0; d < 3; ++d) {
+    const AxisOp& A = op.ax[d];
+    // K[a][i], averaged with its mirror image (equal up to round-off)
+    auto K = [&](int a, int i) {
+      return 0.5 * (A.Kd[0][a * N1 + i] + A.Kd[0][(N1 - 1 - a) * N1 + (N1 - 1 - i)]);
+    };
+    for (int a = 0; a < HE; ++a)
+      for (int i = 0; i < HE; ++i)
+        t.Ke[d][a][i] = (T)(i < HO ? 0.5 * (K(a, i) + K(a, N1 - 1 - i)) : K(a, i));
+    for (int a = 0; a < HO; ++a)
+      for (int i = 0; i < HO; ++i) t.Ko[d][a][i] = (T)(0.5 * (K(a, i) - K(a, N1 - 1 - i)));
+    const AxisOp &B = op.ax[d == 0 ? 1 : 0], &C = op.ax[d == 2 ? 1 : 2];
+    for (int l = 0; l < N1 * N1; ++l) t.mm[d][l] = (T)(B.m[l % N1] * C.m[l / N1]);
+    for (int a = 0; a < HE; ++a) {
+      t.cve[d][a] = (T)(0.5 * (A.cLv[a] + A.cLv[N1 - 1 - a]));
+      t.cde[d][a] = (T)(0.5 * (A.cLd[a] + A.cLd[N1 - 1 - a]));
+    }
+    for (int a = 0; a < HO; ++a) {
+      t.cvo[d][a] = (T)(0.5 * (A.cLv[a] - A.cLv[N1 - 1 - a]));
+      t.cdo[d][a] = (T)(0.5 * (A.cLd[a] - A.cLd[N1 - 1 - a]));
+    }
+    t.gam[d] = (T)(A.sigma * A.h);
+    t.n[d] = op.n[d];
   }
-#pragma unroll 1
+  if (N1 == 2) {
+    for (int d = 0; d < 3; ++d) {
+      const AxisOp& A = op.ax[d];
+      t.Ke[d][0][0] = (T)A.Kd[0][0];
+      t.Ko[d][0][0] = (T)A.Kd[0][1];
+      t.cve[d][0] = (T)A.cLv[0];
+      t.cvo[d][0] = (T)A.cLv[1];
+      t.cde[d][0] = (T)A.cLd[0];
+      t.cdo[d][0] = (T)A.cLd[1];
+    }
+  }
   for (int a = 0; a < N1; ++a) {
-    T acc[LPT];
-    const T c0 = cc[0 * N1 + a], c1 = cc[1 * N1 + a], c2 = cc[2 * N1 + a], c3 = cc[3 * N1 + a];
-#pragma unroll
-    for (int s = 0; s < LPT; ++s) acc[s] = c0 * tvm[s] + c1 * tdm[s] + c2 * tvp[s] + c3 * tdp[s];
-#pragma unroll
-    for (int i = 0; i < N1; ++i) {
-      const T kv = K[a * N1 + i];
-#pragma unroll
-      for (int s = 0; s < LPT; ++s) acc[s] += kv * v[s][i];
-    }
-#pragma unroll
-    for (int s = 0; s < LPT; ++s)
-      if (ok[s]) {
-        T* dst = sacc + base[s] + a * stride;
-        if (ACCUM)
-          *dst += scale[s] * acc[s];
-        else
-          *dst = scale[s] * acc[s];
-      }
+    t.tl[a] = (T)op.tl[a];
+    t.dl[a] = (T)op.dl[a];
   }
+  t.Nq = op.Nq;
 }
 
-// Traces (value and reference normal derivative) of the neighbours across the
-// two faces of direction D of every slot: st[sl][2 D + side][0 / 1][tt].
-template <typename T, int N1, int EPB, int NT, int D>
-__device__ __forceinline__ void ap_traces(const T* __restrict__ u, const long long* sbase, const int (*snb)[6],
-                                          const T (*sTr)[N1], T* __restrict__ st, int tid) {
-  constexpr int NF = N1 * N1, NE = EPB * 2 * NF;
-  constexpr int SD = D == 0 ? 1 : (D == 1 ? N1 : NF);
-#pragma unroll 1
-  for (int t = tid; t < NE; t += NT) {
-    const int sl = t / (2 * NF), rem = t % (2 * NF), side = rem / NF, tt = rem % NF;
-    const long long b0 = sbase[sl];
-    const int nb = snb[sl][2 * D + side];
-    T val = 0, der = 0;
-    if (b0 >= 0 && nb != 0) {
-      const int t1 = tt % N1, t2 = tt / N1;
-      const int base = D == 0 ? N1 * t1 + NF * t2 : (D == 1 ? t1 + NF * t2 : t1 + N1 * t2);
-      const T* un = u + b0 + (long long)nb * (N1 * NF) + base;
-      T vals[N1];
-      // an x-line is N1 contiguous values: with N1 * sizeof(T) a multiple of 16
-      // bytes (and the field 16-byte aligned, as the library's are) it is read
-      // with 16-byte loads, so that a warp's load touches each sector once
-      constexpr bool VEC = D == 0 && (N1 * (int)sizeof(T)) % 16 == 0;
-      if (VEC && (reinterpret_cast<uintptr_t>(un) & 15) == 0) {
-        const uint4* p4 = reinterpret_cast<const uint4*>(un);
-#pragma unroll
-        for (int w = 0; w < (N1 * (int)sizeof(T)) / 16; ++w) {
-          const uint4 q = __ldg(p4 + w);
-          if constexpr (sizeof(T) == 4) {
-            vals[4 * w] = __uint_as_float(q.x);
-            vals[4 * w + 1] = __uint_as_float(q.y);
-            vals[4 * w + 2] = __uint_as_float(q.z);
-            vals[4 * w + 3] = __uint_as_float(q.w);
-          } else {
-            vals[2 * w] = __hiloint2double((int)q.y, (int)q.x);
-            vals[2 * w + 1] = __hiloint2double((int)q.w, (int)q.z);
-          }
-        }
-      } else {
-#pragma unroll
-        for (int i = 0; i < N1; ++i) vals[i] = un[i * SD];
-      }
-      // the -d neighbour meets us at its right end, the +d neighbour at its left end
-      const T* tv = side == 0 ? sTr[1] : sTr[0];
-      const T* td = side == 0 ? sTr[3] : sTr[2];
-#pragma unroll
-      for (int i = 0; i < N1; ++i) {
-        val += tv[i] * vals[i];
-        der += td[i] * vals[i];
-      }
-    }
-    T* dst = st + ((sl * 6 + 2 * D + side) * 2) * NF + tt;
-    dst[0] = val;
-    dst[NF] = der;
+// Bricks per block (at most 320 threads) that leave the fewest idle lanes in the last warp
+constexpr int best_bpb(int lines, int small) {
+  int best = 1;
+  for (int b = 2; b * lines <= 320; ++b) {
+    const int tb = (b * lines + 31) / 32 * 32, t0 = (best * lines + 31) / 32 * 32;
+    // more filled per thread, or as filled and still a small block
+    if (b * t0 > best * tb || (b * t0 == best * tb && tb <= small)) best = b;
   }
+  return best;
 }
 
-template <typename T, int N1, int MODE>
-__global__ void __launch_bounds__(ApplyCfg<T, N1>::THREADS, ApplyCfg<T, N1>::MINB)
-    k_apply(const LevelOp* __restrict__ op, const T* __restrict__ u, T* __restrict__ out,
-            const T* __restrict__ rin, const int* __restrict__ act, int nact) {
-  using C = ApplyCfg<T, N1>;
-  constexpr int NPE = C::NPE, NF = C::NF, EPB = C::EPB, NT = C::THREADS, TPE = C::TPE, LPT = C::LPT;
-  __shared__ T sK[3][4][NF];
-  __shared__ T sC[3][4][N1];
-  __shared__ T sM[3][N1];
-  __shared__ T sTr[4][N1];
-  __shared__ T su[EPB][C::PNPE];
-  __shared__ T sacc[EPB][C::PNPE];
-  __shared__ T st[EPB][6][2][NF];
-  __shared__ long long sbase[EPB];  // rhs * Nq + e * NPE of the slot, or -1
-  __shared__ int snb[EPB][6];       // neighbour element offset (elements) per face, 0 = none
-  __shared__ int sty[EPB][3];
+// Launch shape. BR: elements of a brick along each axis (2 or 1). FILL: several
+// bricks per block, so that warps are full; otherwise one, for problems too
+// small to give every SM a block.
+template <typename T, int N1, int BR, bool FILL>
+struct ApplyCfg {
+  static constexpr int NPE = N1 * N1 * N1, NF = N1 * N1;
+  static constexpr int EB = BR * BR * BR;        // elements of a brick
+  static constexpr int LINES = BR * BR * NF;     // threads of a brick: one (pair of) line(s) each
+  // node (a, b, c) of element e of the block at a + PB b + PZ c + ES e: the
+  // strides with the fewest shared-memory wavefronts of the three passes,
+  // counted over the warps of a block (1.4 to 1.9 per access; odd strides alone
+  // gave 1.9 to 2.5, and the FP32 kernel was bound by them at p = 7: 86 % of the
+  // data pipe)
+  static constexpr int PB = N1 == 8 ? 9 : N1;
+  static constexpr int PZ = N1 == 2 ? 4 : N1 == 3 ? 9 : N1 == 4 ? 19 : N1 == 5 ? 25 : N1 == 6 ? 41 : N1 == 7 ? 52
+                                                                                          : N1 == 8 ? 72 : 81;
+  static constexpr int ES = N1 == 2 ? 10 : N1 == 3 ? 41 : N1 == 4 ? 80 : N1 == 5 ? 153 : N1 == 6 ? 260
+                                                          : N1 == 7 ? 369 : N1 == 8 ? 575 : 736;
+  static_assert(PZ >= PB * (N1 - 1) + N1 && ES >= (PZ + PB + 1) * (N1 - 1) + 1, "element layout overlaps");
+  static constexpr int BPB = FILL ? best_bpb(LINES, sizeof(T) == 4 ? DG_APPLY_TIE32 : DG_APPLY_TIE64) : 1;
+  static constexpr int THREADS = (BPB * LINES + 31) / 32 * 32;
+  static constexpr size_t SMEM = sizeof(T) * 2 * (size_t)BPB * EB * ES;
+  // resident threads per SM asked of ptxas (register cap 65536 / that)
+  static constexpr int WANT = sizeof(T) == 4 ? DG_APPLY_WANT32 : DG_APPLY_WANT64;
+  static constexpr int MINB = WANT / THREADS < 1 ? 1 : WANT / THREADS;
+};
 
-  const int tid = threadIdx.x;
-  for (int i = tid; i < 3 * 4 * NF; i += NT) {
-    const int d = i / (4 * NF), r = i % (4 * NF);
-    sK[d][r / NF][r % NF] = (T)op->ax[d].Kd[r / NF][r % NF];
+// Every product and sum is written out with its rounding (mad, mul), so that the
+// instances of the kernel round alike: a source's result depends neither on the
+// work split nor, with it, on the number of sources in the call.
+__device__ __forceinline__ float mad(float a, float b, float c) { return __fmaf_rn(a, b, c); }
+__device__ __forceinline__ double mad(double a, double b, double c) { return __fma_rn(a, b, c); }
+__device__ __forceinline__ float mul(float a, float b) { return __fmul_rn(a, b); }
+__device__ __forceinline__ double mul(double a, double b) { return __dmul_rn(a, b); }
+
+// value and derivative at the left (RIGHT: right) end of a line
+template <typename T, int N1, bool RIGHT>
+__device__ __forceinline__ void end_trace(const ApplyTab<T, N1>& tab, const T* v, T& val, T& der) {
+  T a = mul(tab.tl[RIGHT ? N1 - 1 : 0], v[0]), b = mul(tab.dl[RIGHT ? N1 - 1 : 0], v[0]);
+#pragma unroll
+  for (int i = 1; i < N1; ++i) {
+    const int k = RIGHT ? N1 - 1 - i : i;
+    a = mad(tab.tl[k], v[i], a);
+    b = mad(tab.dl[k], v[i], b);
   }
-  for (int i = tid; i < 3 * N1; i += NT) {
-    const int d = i / N1, a = i % N1;
-    sC[d][0][a] = (T)op->ax[d].cLv[a];
-    sC[d][1][a] = (T)op->ax[d].cLd[a];
-    sC[d][2][a] = (T)op->ax[d].cRv[a];
-    sC[d][3][a] = (T)op->ax[d].cRd[a];
-    sM[d][a] = (T)op->ax[d].m[a];
-  }
-  for (int i = tid; i < N1; i += NT) {
-    sTr[0][i] = (T)op->tl[i];
-    sTr[1][i] = (T)op->tr[i];
-    sTr[2][i] = (T)op->dl[i];
-    sTr[3][i] = (T)op->dr[i];
-  }
-  const int nx = op->n[0], ny = op->n[1], nz = op->n[2];
-  const int E = op->E;
-  const long long Nq = op->Nq;
-  const int slot = tid / TPE, lt = tid % TPE;
-  const long long items = (long long)nact * E;
-  const long long groups = (items + EPB - 1) / EPB;
-  for (long long grp = blockIdx.x; grp < groups; grp += gridDim.x) {
-    __syncthreads();  // tables ready / previous group done with the shared buffers
-    for (int sl = tid; sl < EPB; sl += NT) {
-      const long long it = grp * EPB + sl;
-      if (it < items) {
-        const int k = (int)(it / E), e = (int)(it - (long long)k * E);
-        sbase[sl] = (long long)act[k] * Nq + (long long)e * NPE;
-        const int ex = e % nx, ey = (e / nx) % ny, ez = e / (nx * ny);
-        snb[sl][0] = ex > 0 ? -1 : 0;
-        snb[sl][1] = ex < nx - 1 ? 1 : 0;
-        snb[sl][2] = ey > 0 ? -nx : 0;
-        snb[sl][3] = ey < ny - 1 ? nx : 0;
-        snb[sl][4] = ez > 0 ? -nx * ny : 0;
-        snb[sl][5] = ez < nz - 1 ? nx * ny : 0;
-        sty[sl][0] = (ex == 0 ? 1 : 0) | (ex == nx - 1 ? 2 : 0);
-        sty[sl][1] = (ey == 0 ? 1 : 0) | (ey == ny - 1 ? 2 : 0);
-        sty[sl][2] = (ez == 0 ? 1 : 0) | (ez == nz - 1 ? 2 : 0);
-      } else {
-        sbase[sl] = -1;
-        for (int f = 0; f < 6; ++f) snb[sl][f] = 0;
-        sty[sl][0] = sty[sl][1] = sty[sl][2] = 0;
-      }
-    }
-    __syncthreads();
-    // own elements (coalesced over consecutive items)
-    for (int t = tid; t < EPB * NPE; t += NT) {
-      const int sl = t / NPE, loc = t - sl * NPE;
-      const long long b0 = sbase[sl];
-      su[sl][ApplyPad<N1>::idx(loc)] = b0 >= 0 ? u[b0 + loc] : (T)0;
-    }
-    // neighbour traces: face f = 2 d + side (side 0: -d neighbour, side 1: +d),
-    // one direction at a time so that the line stride is a constant
-    ap_traces<T, N1, EPB, NT, 0>(u, sbase, snb, sTr, &st[0][0][0][0], tid);
-    ap_traces<T, N1, EPB, NT, 1>(u, sbase, snb, sTr, &st[0][0][0][0], tid);
-    ap_traces<T, N1, EPB, NT, 2>(u, sbase, snb, sTr, &st[0][0][0][0], tid);
-    __syncthreads();
-    if (slot < EPB) {
-      ap_pass<T, N1, LPT, TPE, 0, false>(su[slot], sacc[slot], sK[0][sty[slot][0]], sC[0][0], &st[slot][0][0][0],
-                                         sM[1], sM[2], lt);
-    }
-    __syncthreads();
-    if (slot < EPB) {
-      ap_pass<T, N1, LPT, TPE, 1, true>(su[slot], sacc[slot], sK[1][sty[slot][1]], sC[1][0], &st[slot][2][0][0],
-                                        sM[0], sM[2], lt);
-    }
-    __syncthreads();
-    if (slot < EPB) {
-      ap_pass<T, N1, LPT, TPE, 2, true>(su[slot], sacc[slot], sK[2][sty[slot][2]], sC[2][0], &st[slot][4][0][0],
-                                        sM[0], sM[1], lt);
-    }
-    __syncthreads();
-    for (int t = tid; t < EPB * NPE; t += NT) {
-      const int sl = t / NPE, loc = t - sl * NPE;
-      const long long b0 = sbase[sl];
-      if (b0 >= 0) {
-        const long long gi = b0 + loc;
-        const T Au = sacc[sl][ApplyPad<N1>::idx(loc)];
-        if (MODE == 0) {
-          out[gi] = Au;
-        } else if (MODE == 1) {
-          out[gi] = rin[gi] - Au;
+  val = a;
+  der = RIGHT ? -b : b;
+}
+
+// line of N1 values at p with stride SD, reversed where rev is set; contiguous
+// lines that are a multiple of 16 bytes are read with 16-byte loads where the
+// field is aligned (vec)
+template <typename T, int N1, int SD>
+__device__ __forceinline__ void load_line(const T* __restrict__ p, bool rev, bool vec, T* v) {
+  constexpr int W = 16 / (int)sizeof(T);
+  if constexpr (SD == 1 && N1 % W == 0) {
+    if (vec) {
+      T q[N1];
+#pragma unroll
+      for (int w = 0; w < N1 / W; ++w) {
+        if constexpr (sizeof(T) == 4) {
+          const float4 t = __ldg(reinterpret_cast<const float4*>(p) + w);
+          q[4 * w] = t.x;
+          q[4 * w + 1] = t.y;
+          q[4 * w + 2] = t.z;
+          q[4 * w + 3] = t.w;
         } else {
-          out[gi] = out[gi] - Au;
+          const double2 t = __ldg(reinterpret_cast<const double2*>(p) + w);
+          q[2 * w] = t.x;
+          q[2 * w + 1] = t.y;
         }
+      }
+#pragma unroll
+      for (int i = 0; i < N1; ++i) v[i] = rev ? q[N1 - 1 - i] : q[i];
+      return;
+    }
+  }
+  const T* q = rev ? p + (N1 - 1) * SD : p;
+  const int st = rev ? -SD : SD;
+#pragma unroll
+  for (int i = 0; i < N1; ++i) v[i] = __ldg(q + i * st);
+}
+
+// one pass along direction D for this thread's line (pair): on entry v[s] holds
+// the line values, ov/od the traces beyond its two ends (0: left of the first, 1:
+// right of the last line). On exit v[s] holds the unscaled result.
+template <typename T, int N1, int BR, int D>
+__device__ __forceinline__ void line_op(const ApplyTab<T, N1>& tab, T (*v)[N1], const T* ov, const T* od,
+                                        bool second) {
+  constexpr int HO = N1 / 2, HE = N1 - HO;
+  T e[BR][HE], o[BR][HO == 0 ? 1 : HO];
+  T tv[BR], td[BR];  // the pair's traces on their common face
+#pragma unroll
+  for (int s = 0; s < BR; ++s) {
+    if (BR == 2) {
+      if (s == 0)
+        end_trace<T, N1, true>(tab, v[s], tv[s], td[s]);
+      else
+        end_trace<T, N1, false>(tab, v[s], tv[s], td[s]);
+    }
+    if constexpr (N1 > 2) {
+#pragma unroll
+      for (int i = 0; i < HO; ++i) {
+        e[s][i] = v[s][i] + v[s][N1 - 1 - i];
+        o[s][i] = v[s][i] - v[s][N1 - 1 - i];
+      }
+      if (HE > HO) e[s][HE - 1] = v[s][HO];
+    }
+  }
+#pragma unroll
+  for (int s = 0; s < BR; ++s) {
+    T nl, dl, nr, dr;  // the neighbours' traces, left and right
+    if (BR == 2) {
+      nl = s == 0 ? ov[0] : tv[0];
+      dl = s == 0 ? od[0] : td[0];
+      nr = s == 0 && second ? tv[BR - 1] : ov[1];
+      dr = s == 0 && second ? td[BR - 1] : od[1];
+    } else {
+      nl = ov[0];
+      dl = od[0];
+      nr = ov[1];
+      dr = od[1];
+    }
+    if constexpr (N1 == 2) {
+      const T v0 = v[s][0], v1 = v[s][1];
+      T x = mul(tab.cve[D][0], nl), y = mul(tab.cvo[D][0], nl);
+      x = mad(tab.cde[D][0], dl, x);
+      y = mad(tab.cdo[D][0], dl, y);
+      x = mad(tab.cvo[D][0], nr, x);
+      y = mad(tab.cve[D][0], nr, y);
+      x = mad(-tab.cdo[D][0], dr, x);
+      y = mad(-tab.cde[D][0], dr, y);
+      x = mad(tab.Ke[D][0][0], v0, x);
+      y = mad(tab.Ko[D][0][0], v0, y);
+      v[s][0] = mad(tab.Ko[D][0][0], v1, x);
+      v[s][1] = mad(tab.Ke[D][0][0], v1, y);
+      continue;
+    }
+    const T vp = nl + nr, vm = nl - nr, dm = dl - dr, dp = dl + dr;
+    T O[HO == 0 ? 1 : HO];
+#pragma unroll
+    for (int a = 0; a < HO; ++a) {
+      T acc = mad(tab.cdo[D][a], dp, mul(tab.cvo[D][a], vm));
+#pragma unroll
+      for (int i = 0; i < HO; ++i) acc = mad(tab.Ko[D][a][i], o[s][i], acc);
+      O[a] = acc;
+    }
+#pragma unroll
+    for (int a = 0; a < HE; ++a) {
+      T acc = mad(tab.cde[D][a], dm, mul(tab.cve[D][a], vp));
+#pragma unroll
+      for (int i = 0; i < HE; ++i) acc = mad(tab.Ke[D][a][i], e[s][i], acc);
+      if (a < HO) {
+        v[s][a] = acc + O[a];
+        v[s][N1 - 1 - a] = acc - O[a];
+      } else {
+        v[s][a] = acc;
       }
     }
   }
 }
 
-template <typename T, int N1>
-static cudaError_t apply_n1(const LevelOp& hop, const LevelOp* dop, int mode, const T* u, T* out, const T* rin,
-                            const int* act, int nact, cudaStream_t s) {
-  using C = ApplyCfg<T, N1>;
-  const long long items = (long long)nact * hop.E;
-  long long blocks = (items + C::EPB - 1) / C::EPB;
-  if (blocks == 0) return cudaSuccess;
-  // persistent-style grid: a few resident blocks per SM loop over element groups
-  const long long cap = 152LL * (2048 / C::THREADS) * 2;
-  if (blocks > cap) blocks = cap;
-#if DG_SMEM_CARVEOUT >= 0
-  static bool carve = false;  // ask for the largest shared-memory carveout (more resident blocks)
-  if (!carve) {
-    cudaFuncSetAttribute(k_apply<T, N1, 0>, cudaFuncAttributePreferredSharedMemoryCarveout, DG_SMEM_CARVEOUT);
-    cudaFuncSetAttribute(k_apply<T, N1, 1>, cudaFuncAttributePreferredSharedMemoryCarveout, DG_SMEM_CARVEOUT);
-    cudaFuncSetAttribute(k_apply<T, N1, 2>, cudaFuncAttributePreferredSharedMemoryCarveout, DG_SMEM_CARVEOUT);
-    carve = true;
+// traces beyond the ends of this thread's line (pair) along D: of the outer
+// neighbours where there are any (out0, out1), else those that the boundary
+// stands for, from the line's own values. Read reversed, the own line looks
+// like the neighbour's: value t and derivative -d at the common face. ue points
+// at the brick's first element, es is the element stride along D (elements).
+template <typename T, int N1, int BR, int D>
+__device__ __forceinline__ void outer_traces(const ApplyTab<T, N1>& tab, const T* __restrict__ ue, long long pair,
+                                             int l1, int l2, long long es, bool second, bool out0, bool out1,
+                                             bool vec, T* ov, T* od) {
+  constexpr int NF = N1 * N1, NPE = NF * N1;
+  constexpr int SD = D == 0 ? 1 : (D == 1 ? N1 : NF);
+  const int base = D == 0 ? N1 * l1 + NF * l2 : (D == 1 ? l1 + NF * l2 : l1 + N1 * l2);
+  const T* p = ue + pair * NPE + base;
+  const T gam = tab.gam[D];
+  T v[N1];
+  load_line<T, N1, SD>(out0 ? p - es * NPE : p, !out0, vec, v);
+  end_trace<T, N1, true>(tab, v, ov[0], od[0]);
+  if (!out0) {
+    od[0] = mad(-gam, ov[0], -od[0]);
+    ov[0] = -ov[0];
   }
-#endif
+  const int last = BR == 2 && second ? 1 : 0;
+  load_line<T, N1, SD>(p + (last + (out1 ? 1 : 0)) * es * NPE, !out1, vec, v);
+  end_trace<T, N1, false>(tab, v, ov[1], od[1]);
+  if (!out1) {
+    od[1] = mad(gam, ov[1], -od[1]);
+    ov[1] = -ov[1];
+  }
+}
+
+template <typename T, int N1, int BR, bool FILL>
+__global__ void __launch_bounds__(ApplyCfg<T, N1, BR, FILL>::THREADS, ApplyCfg<T, N1, BR, FILL>::MINB)
+    k_apply(const __grid_constant__ ApplyTab<T, N1> tab, const T* __restrict__ u, T* __restrict__ out,
+            const T* __restrict__ rin, const int* __restrict__ act, int mode, int vec_i) {
+  using C = ApplyCfg<T, N1, BR, FILL>;
+  constexpr int NPE = C::NPE, NF = C::NF, EB = C::EB, BPB = C::BPB, LINES = C::LINES;
+  constexpr int PB = C::PB, PZ = C::PZ, ES = C::ES;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  T* su = reinterpret_cast<T*>(smem_raw);
+  T* sacc = su + BPB * EB * ES;
+  __shared__ long long sbase[BPB];  // first value of the brick's first element, -1: no brick
+  __shared__ int sflag[BPB];        // bits d: second element along d; 3 + 2 d + side: outer neighbour
+  const int tid = threadIdx.x;
+  const bool vec = vec_i != 0;
+  const int nx = tab.n[0], ny = tab.n[1];
+  const long long est[3] = {1, nx, (long long)nx * ny};
+  if (tid < BPB) {
+    const long long it = (long long)blockIdx.x * BPB + tid;
+    long long base = -1;
+    int flag = 0;
+    if (it < tab.items) {
+      const unsigned nbr = (unsigned)(tab.nb[0] * tab.nb[1]) * (unsigned)tab.nb[2];
+      const unsigned k = (unsigned)(it / nbr), r = (unsigned)(it - (long long)k * nbr);
+      const unsigned bx = r % tab.nb[0], q = r / tab.nb[0], by = q % tab.nb[1], bz = q / tab.nb[1];
+      const int e[3] = {(int)bx * BR, (int)by * BR, (int)bz * BR};
+      base = (long long)act[k] * tab.Nq + (e[0] + est[1] * e[1] + est[2] * e[2]) * NPE;
+#pragma unroll
+      for (int d = 0; d < 3; ++d) {
+        const bool sec = BR == 2 && e[d] + 1 < tab.n[d];
+        if (sec) flag |= 1 << d;
+        if (e[d] > 0) flag |= 8 << (2 * d);
+        if (e[d] + (sec ? 2 : 1) < tab.n[d]) flag |= 16 << (2 * d);
+      }
+    }
+    sbase[tid] = base;
+    sflag[tid] = flag;
+  }
+  __syncthreads();
+  const int slot = tid / LINES, lt = tid - slot * LINES;
+  const int pr = lt / NF, l = lt - pr * NF, l1 = l % N1, l2 = l / N1;
+  const int p1 = pr & 1, p2 = pr >> 1;  // the pair's position along the lower and the higher other axis
+  const bool on = slot < BPB && sbase[slot < BPB ? slot : 0] >= 0;
+  const int flag = on ? sflag[slot] : 0;
+  const long long b0 = on ? sbase[slot] : 0;
+  const T* ue = u + b0;
+  // a pair is there if its position along both other axes is
+  bool have[3];
+  have[0] = on && (!p1 || (flag & 2)) && (!p2 || (flag & 4));
+  have[1] = on && (!p1 || (flag & 1)) && (!p2 || (flag & 4));
+  have[2] = on && (!p1 || (flag & 1)) && (!p2 || (flag & 2));
+  const long long pe[3] = {est[1] * p1 + est[2] * p2, est[0] * p1 + est[2] * p2, est[0] * p1 + est[1] * p2};
+  const int sb = (slot < BPB ? slot : 0) * EB * ES;
+  const int zat = sb + (p1 + 2 * p2) * ES + l1 + PB * l2;  // this thread's z line (pair): shared and global
+  const long long g0 = b0 + pe[2] * NPE + l;
+  T v[BR][N1];
+  // own elements, a z line (pair) per thread: coalesced, and no index arithmetic per value
+  if (have[2]) {
+#pragma unroll
+    for (int s = 0; s < BR; ++s)
+      if (s == 0 || (flag & 4)) {
+#pragma unroll
+        for (int i = 0; i < N1; ++i) v[s][i] = __ldg(u + g0 + s * est[2] * NPE + i * NF);
+#pragma unroll
+        for (int i = 0; i < N1; ++i) su[zat + 4 * s * ES + i * PZ] = v[s][i];
+      }
+  }
+  T ov[3][2], od[3][2];
+#define DG_OUT(d, s) ((flag & ((8 << (s)) << (2 * (d)))) != 0)
+  if (have[0])
+    outer_traces<T, N1, BR, 0>(tab, ue, pe[0], l1, l2, est[0], flag & 1, DG_OUT(0, 0), DG_OUT(0, 1), vec, ov[0], od[0]);
+  if (have[1])
+    outer_traces<T, N1, BR, 1>(tab, ue, pe[1], l1, l2, est[1], flag & 2, DG_OUT(1, 0), DG_OUT(1, 1), vec, ov[1], od[1]);
+  if (have[2])
+    outer_traces<T, N1, BR, 2>(tab, ue, pe[2], l1, l2, est[2], flag & 4, DG_OUT(2, 0), DG_OUT(2, 1), vec, ov[2], od[2]);
+  __syncthreads();
+  // x: line (b, c) = (l1, l2)
+  if (have[0]) {
+    const int at = sb + (2 * p1 + 4 * p2) * ES + PB * l1 + PZ * l2;
+    const bool sec = flag & 1;
+#pragma unroll
+    for (int s = 0; s < BR; ++s)
+#pragma unroll
+      for (int i = 0; i < N1; ++i) v[s][i] = s == 0 || sec ? su[at + s * ES + i] : (T)0;
+    line_op<T, N1, BR, 0>(tab, v, ov[0], od[0], sec);
+    const T sc = tab.mm[0][l];
+#pragma unroll
+    for (int s = 0; s < BR; ++s)
+      if (s == 0 || sec) {
+#pragma unroll
+        for (int i = 0; i < N1; ++i) sacc[at + s * ES + i] = mul(sc, v[s][i]);
+      }
+  }
+  __syncthreads();
+  // y: line (a, c)
+  if (have[1]) {
+    const int at = sb + (p1 + 4 * p2) * ES + l1 + PZ * l2;
+    const bool sec = flag & 2;
+#pragma unroll
+    for (int s = 0; s < BR; ++s)
+#pragma unroll
+      for (int i = 0; i < N1; ++i) v[s][i] = s == 0 || sec ? su[at + 2 * s * ES + i * PB] : (T)0;
+    line_op<T, N1, BR, 1>(tab, v, ov[1], od[1], sec);
+    const T sc = tab.mm[1][l];
+#pragma unroll
+    for (int s = 0; s < BR; ++s)
+      if (s == 0 || sec) {
+#pragma unroll
+        for (int i = 0; i < N1; ++i) {
+          T* p = sacc + at + 2 * s * ES + i * PB;
+          *p = mad(sc, v[s][i], *p);
+        }
+      }
+  }
+  __syncthreads();
+  // z: line (a, b), straight to the result
+  if (have[2]) {
+    const bool sec = flag & 4;
+    T r[BR][N1];
+    if (mode != 0) {
+      const T* rp = mode == 1 ? rin : out;
+#pragma unroll
+      for (int s = 0; s < BR; ++s)
+        if (s == 0 || sec) {
+#pragma unroll
+          for (int i = 0; i < N1; ++i) r[s][i] = rp[g0 + s * est[2] * NPE + i * NF];
+        }
+    }
+#pragma unroll
+    for (int s = 0; s < BR; ++s)
+#pragma unroll
+      for (int i = 0; i < N1; ++i) v[s][i] = s == 0 || sec ? su[zat + 4 * s * ES + i * PZ] : (T)0;
+    line_op<T, N1, BR, 2>(tab, v, ov[2], od[2], sec);
+    const T sc = tab.mm[2][l];
+#pragma unroll
+    for (int s = 0; s < BR; ++s)
+      if (s == 0 || sec) {
+#pragma unroll
+        for (int i = 0; i < N1; ++i) {
+          const T Au = mad(sc, v[s][i], sacc[zat + 4 * s * ES + i * PZ]);
+          out[g0 + s * est[2] * NPE + i * NF] = mode == 0 ? Au : r[s][i] - Au;
+        }
+      }
+  }
+#undef DG_OUT
+}
+
+template <typename T, int N1, int BR, bool FILL>
+static cudaError_t apply_br(const LevelOp& hop, int mode, const T* u, T* out, const T* rin, const int* act, int nact,
+                            cudaStream_t s) {
+  using C = ApplyCfg<T, N1, BR, FILL>;
+  ApplyTab<T, N1> tab;
+  fill_tab<T, N1>(tab, hop);
+  long long per = 1;
+  for (int d = 0; d < 3; ++d) {
+    tab.nb[d] = (hop.n[d] + BR - 1) / BR;
+    per *= tab.nb[d];
+  }
+  tab.items = per * nact;
+  const long long blocks = (tab.items + C::BPB - 1) / C::BPB;
+  if (blocks > 0x7fffffffLL) return cudaErrorInvalidValue;
+  // 16-byte reads of an element's values: the field and every element of it aligned
+  const int vec = ((uintptr_t)u & 15) == 0 && (C::NPE * sizeof(T)) % 16 == 0 && (hop.Nq * sizeof(T)) % 16 == 0;
+  auto kern = k_apply<T, N1, BR, FILL>;
+  if (C::SMEM > 48 * 1024) {
+    const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)C::SMEM);
+    if (e != cudaSuccess) return e;
+  }
   count_launch();
-  if (mode == 0)
-    k_apply<T, N1, 0><<<(unsigned)blocks, C::THREADS, 0, s>>>(dop, u, out, rin, act, nact);
-  else if (mode == 1)
-    k_apply<T, N1, 1><<<(unsigned)blocks, C::THREADS, 0, s>>>(dop, u, out, rin, act, nact);
-  else
-    k_apply<T, N1, 2><<<(unsigned)blocks, C::THREADS, 0, s>>>(dop, u, out, rin, act, nact);
+  kern<<<(unsigned)blocks, C::THREADS, C::SMEM, s>>>(tab, u, out, rin, act, mode, vec);
   return cudaGetLastError();
+}
+
+// Bricks of eight elements in FP32, where reading the neighbours is what bounds
+// the kernel; single elements in FP64 (bound by the FP64 pipe, to which a brick
+// saves nothing) and where bricks would leave SMs idle or, on odd meshes, hold
+// less than half of the elements that they have room for.
+template <typename T, int N1>
+static cudaError_t apply_n1(const LevelOp& hop, int mode, const T* u, T* out, const T* rin, const int* act, int nact,
+                            cudaStream_t s) {
+  if (nact == 0) return cudaSuccess;
+  const long long items = (long long)nact * hop.E;
+  if constexpr (sizeof(T) == 4) {
+    long long br = nact;
+    for (int d = 0; d < 3; ++d) br *= (hop.n[d] + 1) / 2;
+    if (br / ApplyCfg<T, N1, 2, true>::BPB >= DG_APPLY_MIN_BLOCKS && 8 * br <= 2 * items)
+      return apply_br<T, N1, 2, true>(hop, mode, u, out, rin, act, nact, s);
+  }
+  if (items / ApplyCfg<T, N1, 1, true>::BPB >= DG_APPLY_MIN_BLOCKS)
+    return apply_br<T, N1, 1, true>(hop, mode, u, out, rin, act, nact, s);
+  return apply_br<T, N1, 1, false>(hop, mode, u, out, rin, act, nact, s);
 }
 
 template <typename T>
 cudaError_t launch_apply(const LevelOp& hop, const LevelOp* dop, int mode, const T* u, T* out, const T* rin,
                          const int* act, int nact, cudaStream_t s) {
+  (void)dop;
   switch (hop.n1) {
-    case 2: return apply_n1<T, 2>(hop, dop, mode, u, out, rin, act, nact, s);
-    case 3: return apply_n1<T, 3>(hop, dop, mode, u, out, rin, act, nact, s);
-    case 4: return apply_n1<T, 4>(hop, dop, mode, u, out, rin, act, nact, s);
-    case 5: return apply_n1<T, 5>(hop, dop, mode, u, out, rin, act, nact, s);
-    case 6: return apply_n1<T, 6>(hop, dop, mode, u, out, rin, act, nact, s);
-    case 7: return apply_n1<T, 7>(hop, dop, mode, u, out, rin, act, nact, s);
-    case 8: return apply_n1<T, 8>(hop, dop, mode, u, out, rin, act, nact, s);
-    case 9: return apply_n1<T, 9>(hop, dop, mode, u, out, rin, act, nact, s);
+    case 2: return apply_n1<T, 2>(hop, mode, u, out, rin, act, nact, s);
+    case 3: return apply_n1<T, 3>(hop, mode, u, out, rin, act, nact, s);
+    case 4: return apply_n1<T, 4>(hop, mode, u, out, rin, act, nact, s);
+    case 5: return apply_n1<T, 5>(hop, mode, u, out, rin, act, nact, s);
+    case 6: return apply_n1<T, 6>(hop, mode, u, out, rin, act, nact, s);
+    case 7: return apply_n1<T, 7>(hop, mode, u, out, rin, act, nact, s);
+    case 8: return apply_n1<T, 8>(hop, mode, u, out, rin, act, nact, s);
+    case 9: return apply_n1<T, 9>(hop, mode, u, out, rin, act, nact, s);
     default: return cudaErrorInvalidValue;
   }
 }
