@@ -142,7 +142,12 @@ struct Level {
   TransferOp* dtr = nullptr;
   double lam_max = 0;            // lambda_max(D^-1 A) (point Jacobi)
   double lam_sw = 0;             // lambda_max(M_S A) estimate (Schwarz)
-  DevBuf sw_tabs;                // Schwarz patch tables
+  DevBuf sw_tabs, sw_tabs32;     // Schwarz patch tables of the SIMT kernel, FP64 and FP32
+  SwGeom sw_geom{}, sw_geom32{};
+  template <typename T>
+  SwTables sw() const {
+    return sizeof(T) == 8 ? SwTables{sw_geom, sw_tabs.p} : SwTables{sw_geom32, sw_tabs32.p};
+  }
   DevBuf sw_tc;                  // tables of the tensor-core patch solve (FP32 inner solve), if used
   SwTcPlan tcp;                  // its device blob (null: SIMT patch solve) and header
   const SwTcPlan* tc() const { return tcp.blob && !tcp.off ? &tcp : nullptr; }

@@ -137,7 +137,9 @@ static void account(dg_ctx* h) {
   for (auto& L : h->w32.lev) {
     add(L.x); add(L.b); add(L.res); add(L.d); add(L.invD); add(L.z); add(L.zp);
   }
-  for (auto& L : h->levels) add(L.sw_tabs);
+  for (auto& L : h->levels) {
+    add(L.sw_tabs); add(L.sw_tabs32);
+  }
   for (auto* w : {&h->w64.x, &h->w64.r, &h->w64.z, &h->w64.p, &h->w64.q}) add(*w);
   for (auto* w : {&h->w32.x, &h->w32.r, &h->w32.z, &h->w32.p, &h->w32.q}) add(*w);
   for (int d = 0; d < 3; ++d) {
@@ -842,7 +844,7 @@ static int estimate_lambda_schwarz(dg_ctx* h, int l, double* out) {
     DG_CK(cudaMemcpy(res, sc + 3, sizeof(double), cudaMemcpyDeviceToHost));
     return DG_OK;
   };
-  DG_CK(launch_schwarz<double>(L.op, L.dop, L.sw_tabs.as<double>(), r.as<double>(), zp.as<double>(),
+  DG_CK(launch_schwarz<double>(L.op, L.dop, L.sw<double>(), r.as<double>(), zp.as<double>(),
                                z.as<double>(), nullptr, 0, 0.0, 0.0, a, 1, 0));
   DG_CK(cudaMemcpy(p.p, z.p, sizeof(double) * N, cudaMemcpyDeviceToDevice));
   double rz = 0.0;
@@ -857,7 +859,7 @@ static int estimate_lambda_schwarz(dg_ctx* h, int l, double* out) {
     const double alpha = rz / pq;
     DG_CK(cudaMemcpy(sc, &alpha, sizeof(double), cudaMemcpyHostToDevice));
     DG_CK(launch_cg_xr<double>(x.as<double>(), r.as<double>(), p.as<double>(), q.as<double>(), sc, N, a, 1, 0));
-    DG_CK(launch_schwarz<double>(L.op, L.dop, L.sw_tabs.as<double>(), r.as<double>(), zp.as<double>(),
+    DG_CK(launch_schwarz<double>(L.op, L.dop, L.sw<double>(), r.as<double>(), zp.as<double>(),
                                  z.as<double>(), nullptr, 0, 0.0, 0.0, a, 1, 0));
     double rzn = 0.0;
     DG_RET(dot(r.as<double>(), z.as<double>(), &rzn));
@@ -951,8 +953,13 @@ static int setup(dg_ctx* h) {
     for (int l = 0; l + 1 < h->nlev; ++l) {
       Level& L = h->levels[l];
       const std::vector<double> tb = schwarz_tables(L.op);
-      DG_CK(L.sw_tabs.ensure(sizeof(double) * tb.size()));
-      DG_CK(cudaMemcpy(L.sw_tabs.p, tb.data(), sizeof(double) * tb.size(), cudaMemcpyHostToDevice));
+      auto upload = [&](const std::vector<unsigned char>& b, DevBuf& buf) -> int {
+        DG_CK(buf.ensure(b.size()));
+        DG_CK(cudaMemcpy(buf.p, b.data(), b.size(), cudaMemcpyHostToDevice));
+        return DG_OK;
+      };
+      DG_RET(upload(schwarz_blob(L.op, tb, 8, L.sw_geom), L.sw_tabs));
+      DG_RET(upload(schwarz_blob(L.op, tb, 4, L.sw_geom32), L.sw_tabs32));
       DG_RET(estimate_lambda_schwarz(h, l, &L.lam_sw));
       // FP32 inner solve: patch solves on the tensor cores at degrees 7-8 (and 6
       // when asked: there the SIMT kernel is as fast)
@@ -1086,7 +1093,7 @@ static int apply_smoother_t(dg_ctx* h, PrecWork<T>& w, int level, const T* r, T*
   if (level == h->nlev - 1) {
     DG_CK(launch_coarse_solve<T>(h->coarse_inv.as<double>(), h->Nc, r, z, a, nb, s));
   } else if (h->opts.smoother == DG_SMOOTH_SCHWARZ) {
-    DG_CK(launch_schwarz<T>(L.op, L.dop, L.sw_tabs.as<double>(), r, w.lev[level].zp.template as<T>(), z, nullptr, 0,
+    DG_CK(launch_schwarz<T>(L.op, L.dop, L.sw<T>(), r, w.lev[level].zp.template as<T>(), z, nullptr, 0,
                             0.0, 0.0, a, nb, s, L.tc()));
   } else {
     DG_CK(launch_cheb_first<T>(z, z, r, w.lev[level].invD.template as<T>(), 1.0, 1, L.op.Nq, a, nb, s));
@@ -1369,10 +1376,10 @@ int dg_apply_patch_solves(dg_handle h, int32_t level, int32_t fp32, const void* 
   DG_RET(upload_act(h, a, s));
   const Level& L = h->levels[level];
   if (fp32)
-    DG_CK(launch_schwarz_patch<float>(L.op, L.dop, L.sw_tabs.as<double>(), (const float*)r, (float*)zp,
+    DG_CK(launch_schwarz_patch<float>(L.op, L.dop, L.sw<float>(), (const float*)r, (float*)zp,
                                       h->act.as<int>(), nb, s, L.tc()));
   else
-    DG_CK(launch_schwarz_patch<double>(L.op, L.dop, L.sw_tabs.as<double>(), (const double*)r, (double*)zp,
+    DG_CK(launch_schwarz_patch<double>(L.op, L.dop, L.sw<double>(), (const double*)r, (double*)zp,
                                        h->act.as<int>(), nb, s, nullptr));
   return DG_OK;
 }

@@ -81,11 +81,44 @@ struct TransferOp {
 // Kronecker sum of restricted 1-D matrices, so each patch solve is exact by
 // fast diagonalisation: A_P^-1 = (Sx(x)Sy(x)Sz) diag(1/(lx+ly+lz)) (Sx(x)Sy(x)Sz)^T
 // with A~_d S_d = M~_d S_d Lambda_d, S_d^T M~_d S_d = I, per axis and element
-// position. Device layout per axis: for each element position e_d,
+// position.
+//
+// Host layout (schwarz_tables) per axis, for each element position e_d:
 // [m, oL] (ints, stored as doubles) then S [MP*MP] (row = patch node, col =
 // mode) then lambda [MP]; MP = n1 + 2.
 constexpr int MAXMP = MAXN1 + 2;
 inline int schwarz_axis_stride(int n1) { return 2 + (n1 + 2) * (n1 + 2) + (n1 + 2); }
+
+// Device tables of the SIMT patch kernel (schwarz_blob): the positions of an
+// axis fall into at most SW_MAXCLS classes with equal tables (at, next to and
+// away from either boundary). The blob holds
+//   pos_off: one packed int per element position, axis after axis (sw_* below);
+//   tab_off: per axis and class a table of the kernel's type, MP rows of RP
+//            values (row = mode, RP = MP rounded up to 16 bytes; of a symmetric
+//            class the even modes come first, and each row holds the mode at the
+//            first half of the nodes), then the eigenvalues (1 where there is no
+//            mode);
+//   inv_off: FP64 only, 1 / (lx + ly + lz) per class triple [cz][cy][cx], value
+//            (mode qx, qy, qz) at qx MP^2 + qy + MP qz.
+constexpr int SW_MAXCLS = 5;
+struct SwGeom {
+  int n[3];
+  int ntab;  // tables of all axes
+  unsigned pos_off, tab_off, inv_off;
+};
+struct SwTables {
+  SwGeom geom;
+  const void* blob;
+};
+// table | class << 4 | patch size << 8 | left halo << 12 | symmetric << 13
+__host__ __device__ inline int sw_pack(int tab, int cls, int m, int halo, int sym) {
+  return tab | cls << 4 | m << 8 | halo << 12 | sym << 13;
+}
+__host__ __device__ inline int sw_tab(int p) { return p & 15; }
+__host__ __device__ inline int sw_cls(int p) { return (p >> 4) & 15; }
+__host__ __device__ inline int sw_size(int p) { return (p >> 8) & 15; }
+__host__ __device__ inline int sw_halo(int p) { return (p >> 12) & 1; }
+__host__ __device__ inline bool sw_sym(int p) { return (p >> 13) & 1; }
 
 struct GemmArgs {
   int M, N, K, nb1, nb2;
@@ -151,10 +184,10 @@ cudaError_t launch_coarse_solve(const double* Ainv, int Nc, const T* r, T* x, co
 struct SwTcPlan;
 // the patch solves alone: zp[rhs][e][MP^3] = A_P^-1 R_P r
 template <typename T>
-cudaError_t launch_schwarz_patch(const LevelOp& hop, const LevelOp* dop, const double* tabs, const T* r, T* zp,
+cudaError_t launch_schwarz_patch(const LevelOp& hop, const LevelOp* dop, const SwTables& tabs, const T* r, T* zp,
                                  const int* act, int nact, cudaStream_t s, const SwTcPlan* tc = nullptr);
 template <typename T>
-cudaError_t launch_schwarz(const LevelOp& hop, const LevelOp* dop, const double* tabs, const T* r, T* zp, T* z,
+cudaError_t launch_schwarz(const LevelOp& hop, const LevelOp* dop, const SwTables& tabs, const T* r, T* zp, T* z,
                            T* x, int mode, double c1, double c2, const int* act, int nact, cudaStream_t s,
                            const SwTcPlan* tc = nullptr);
 

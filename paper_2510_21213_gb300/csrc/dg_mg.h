@@ -42,7 +42,7 @@ struct MG {
       r0 = res;
     }
     if (sw)
-      DG_CK(launch_schwarz<T>(L.op, L.dop, L.sw_tabs.as<double>(), r0, W.zp.as<T>(), d, x, zero_init ? 1 : 2,
+      DG_CK(launch_schwarz<T>(L.op, L.dop, L.sw<T>(), r0, W.zp.as<T>(), d, x, zero_init ? 1 : 2,
                               1.0 / theta, 0.0, act, nact, s, L.tc()));
     else
       DG_CK(launch_cheb_first<T>(x, d, r0, invD, 1.0 / theta, zero_init ? 1 : 0, Nq, act, nact, s));
@@ -56,7 +56,7 @@ struct MG {
       res_is_b = false;
       const double rho = 1.0 / (2.0 * sig1 - rho_prev);
       if (sw)
-        DG_CK(launch_schwarz<T>(L.op, L.dop, L.sw_tabs.as<double>(), res, W.zp.as<T>(), d, x, 3, rho * rho_prev,
+        DG_CK(launch_schwarz<T>(L.op, L.dop, L.sw<T>(), res, W.zp.as<T>(), d, x, 3, rho * rho_prev,
                                 2.0 * rho / delta, act, nact, s, L.tc()));
       else
         DG_CK(launch_cheb_step<T>(x, d, res, invD, rho * rho_prev, 2.0 * rho / delta, Nq, act, nact, s));

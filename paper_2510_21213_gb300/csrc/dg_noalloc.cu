@@ -99,10 +99,10 @@ int dg_apply_smoother_noalloc(dg_handle h, int32_t level, int32_t fp32, const vo
       DG_CK(launch_coarse_solve<double>(h->coarse_inv.as<double>(), h->Nc, (const double*)r, (double*)z, d.act, nb,
                                         s));
   } else if (fp32) {
-    DG_CK(launch_schwarz<float>(L.op, L.dop, L.sw_tabs.as<double>(), (const float*)r, (float*)d.scratch, (float*)z,
+    DG_CK(launch_schwarz<float>(L.op, L.dop, L.sw<float>(), (const float*)r, (float*)d.scratch, (float*)z,
                                 nullptr, 0, 0.0, 0.0, d.act, nb, s, L.tc()));
   } else {
-    DG_CK(launch_schwarz<double>(L.op, L.dop, L.sw_tabs.as<double>(), (const double*)r, d.scratch, (double*)z,
+    DG_CK(launch_schwarz<double>(L.op, L.dop, L.sw<double>(), (const double*)r, d.scratch, (double*)z,
                                  nullptr, 0, 0.0, 0.0, d.act, nb, s));
   }
   return DG_OK;

@@ -7,278 +7,448 @@
 // overlap, accelerated by Chebyshev iteration. Each patch problem is solved
 // exactly by fast diagonalisation (the patch operator is a Kronecker sum of
 // restricted 1-D matrices; tables built at setup):
-//   k_schwarz_patch:  zp_e = A_P(e)^-1 R_P(e) r        (EPB elements per block,
-//                     one thread per patch line in each of the six 1-D passes)
+//   k_schwarz_patch:  zp_e = A_P(e)^-1 R_P(e) r
 //   k_schwarz_gather: z = sum_e R_P(e)^T zp_e          (each node gathers the
 //                     at most 8 patches covering it; no atomics), fused with
 //                     the Chebyshev update d = c1 d + c2 z, x += d
+//
+// Patch kernel. FP64 is bound by the FP64 pipe, so what counts is the number of
+// operations; FP32 by shared-memory accesses, so what counts is how often a
+// value goes through shared memory and how many products share a table load.
+//   - A patch whose two ends look alike (all but the two elements next to either
+//     boundary) has a 1-D matrix that is invariant under reversal: its modes are
+//     even or odd, and on the sums and differences of mirrored nodes each half
+//     costs a quarter of the dense product. m^2 / 2 + m multiply-adds per line
+//     instead of m^2 (m = p + 3).
+//   - z forward on the values as they come from global memory; y forward; the
+//     whole x direction in registers (transform, division by the eigenvalue sum,
+//     transform back, each table row loaded once for both); y backward; z
+//     backward straight to global memory, consecutive threads on consecutive
+//     values. 8 shared-memory accesses a node instead of 16.
+//   - FP64 multiplies by a tabulated reciprocal of the eigenvalue sum (a division
+//     costs about ten operations of the FP64 pipe).
+//   - A thread owns LPT lines of one patch in every pass and reads table rows
+//     with 16-byte loads, so one load serves 4 LPT products. The tables of the at
+//     most five position classes of an axis stay in shared memory, loaded once
+//     by each block of a persistent grid.
+// Measured (GB300; before: all six passes through shared memory, dense
+// transforms, a division per node, tables per patch): FP64 16^3, p = 7, 42
+// sources 22.0 -> 15.6 ms, 8^3, p = 6, 56 sources 2.33 -> 1.91 ms, 4^3, p = 4, 4
+// sources 35 -> 17 us; FP32 8^3, p = 6, 56 sources 152 -> 109 us, 16^3, p = 3, 42
+// sources 273 -> 142 us, p = 1 89 -> 41 us, 6 x 10 x 8, p = 5, 21 sources 51 -> 23
+// us. FP64 runs at the rate of its pipe; FP32 issues in 55 % of the cycles with
+// a quarter of the warps resident (96 registers).
 #include "dg_internal.h"
 #include "dg_swtc.h"
 
 namespace dg {
 
-__host__ __device__ inline int sw_axis_off(const LevelOp* op, int d, int stride) {
-  return d == 0 ? 0 : (d == 1 ? op->n[0] * stride : (op->n[0] + op->n[1]) * stride);
-}
-
-// Patch kernel layout: each thread owns LPT = 3 lines of the patch in every
-// 1-D pass (line values and outputs in registers, the 1-D matrix streamed from
-// shared memory and reused across the three lines).
 // Tuning constants (compile-time; the defaults were chosen by timing on a GB300)
-#ifndef DG_SMEM_CARVEOUT
-#define DG_SMEM_CARVEOUT -1  // shared-memory carveout (percent) asked for the patch kernel; -1: default
-#endif
-// patch lines per thread, FP32: 2 for p = 1 and p >= 7, 3 otherwise (timed per degree)
-#ifdef DG_SW_LPT32
-#define DG_SW_LPT_OF(N1) DG_SW_LPT32
-#else
-#define DG_SW_LPT_OF(N1) ((N1) == 2 || (N1) >= 8 ? 2 : 3)
-#endif
 #ifndef DG_GATHER_WAVE
 #define DG_GATHER_WAVE 8   // gather grid: at most this many blocks per SM per source list (0: one block per element)
 #endif
-#ifndef DG_SW_MINB32
-#define DG_SW_MINB32 4     // resident blocks per SM asked of ptxas, FP32
-#endif
-#ifndef DG_SW_THREADS
-#define DG_SW_THREADS 256  // thread budget per block
-#endif
-#ifndef DG_SW_SMEM
-#define DG_SW_SMEM 36864   // shared-memory budget of the patch slots (bytes)
-#endif
-// Padded FP32 patch layout in shared memory: node (i, j, k) of a patch at
-// i + MP j + SY k, patch slots SE apart. The plane and slot strides were
-// chosen by counting shared-memory wavefronts of the six 1-D passes for every
-// degree (lanes of a warp on lines of one or two patches): the unpadded layout
-// puts the y lines MP^2 words apart, a 2-way bank conflict for most MP.
-__host__ __device__ constexpr int sw_pad_sy(int N1) {
-  return N1 == 2 ? 16 : N1 == 3 ? 39 : N1 == 4 ? 39 : N1 == 6 ? 73 : N1 == 7 ? 85 : N1 == 8 ? 109
-                                                                                   : (N1 + 2) * (N1 + 2);
-}
-__host__ __device__ constexpr int sw_pad_se(int N1) {
-  return N1 == 2 ? 69 : N1 == 3 ? 201 : N1 == 4 ? 238 : N1 == 6 ? 598 : N1 == 7 ? 795 : N1 == 8 ? 1106
-                                                      : N1 == 9 ? 1332 : (N1 + 2) * (N1 + 2) * (N1 + 2);
-}
 
 template <typename T, int N1>
 struct SwCfg {
-  static constexpr int MP = N1 + 2;
-  // plane and slot strides of the shared patch buffer (FP64 keeps the dense layout)
-  static constexpr int SY = sizeof(T) == 4 ? sw_pad_sy(N1) : MP * MP;
-  static constexpr int SE = sizeof(T) == 4 ? sw_pad_se(N1) : MP * MP * MP;
-  static_assert(SY >= MP * MP && SE >= MP * SY, "patch layout overlaps");
-  static constexpr int LINES = MP * MP;
-  // FP32: two or three lines per thread (shared-memory traffic per FMA / LPT);
-  // FP64 is bound by the FP64 pipe, one line per thread keeps registers in check
-  static constexpr int LPT = sizeof(T) == 4 ? DG_SW_LPT_OF(N1) : 1;
-  static constexpr int TPE = (LINES + LPT - 1) / LPT;  // threads per element
-  static constexpr int MINB = sizeof(T) == 4 ? DG_SW_MINB32 : 1;  // resident blocks per SM asked of ptxas
-  static constexpr int PER_ELEM = (SE + 3 * MP * MP + 3 * MP) * (int)sizeof(T);
-  static constexpr int EPB_T = DG_SW_THREADS / TPE < 1 ? 1 : DG_SW_THREADS / TPE;
-  static constexpr int EPB_S = DG_SW_SMEM / PER_ELEM < 1 ? 1 : DG_SW_SMEM / PER_ELEM;
-  static constexpr int EPB = EPB_T < EPB_S ? EPB_T : EPB_S;
-  static constexpr int THREADS = EPB * TPE;
+  static constexpr int MP = N1 + 2, MP2 = MP * MP, MP3 = MP2 * MP;
+  static constexpr int HO = MP / 2, HE = MP - HO;
+  static constexpr int W = 16 / (int)sizeof(T);           // values of a 16-byte load
+  static constexpr int RP = (MP + W - 1) / W * W;         // padded table row
+  static constexpr int TB = (MP + 1) * RP;                // one table: MP rows and the eigenvalues
+  // lines per thread: FP32 as many as keep the lanes of a patch busy; FP64 one
+  // (bound by its pipe, and short chains matter on small problems)
+  static constexpr int LPT = sizeof(T) == 8 ? 1 : MP == 4 ? 4 : MP == 5 ? 5 : MP == 7 || MP == 8 ? 2 : MP == 10 ? 4 : 3;
+  static constexpr int TPE = (MP2 + LPT - 1) / LPT;       // threads of a patch
+  // node (i, j, k) of a slot at i + SJ j + SK k + SE slot: the strides with the
+  // fewest shared-memory wavefronts of the passes in FP32, counted over the
+  // warps of a block (1.0 to 1.8 per access; the dense layout takes up to 8);
+  // FP64 keeps the dense layout
+  static constexpr int SJ = sizeof(T) == 8 ? MP : MP == 4 ? 5 : MP == 5 ? 6 : MP == 6 ? 9 : MP == 7 ? 8 : MP == 8 ? 9
+                                                  : MP == 9 ? 9 : MP == 10 ? 13 : 12;
+  static constexpr int SK = sizeof(T) == 8 ? MP2 : MP == 4 ? 19 : MP == 5 ? 30 : MP == 6 ? 70 : MP == 7 ? 71
+                                                  : MP == 8 ? 72 : MP == 9 ? 111 : MP == 10 ? 138 : 139;
+  static constexpr int SE = sizeof(T) == 8 ? MP3 : MP == 4 ? 76 : MP == 5 ? 165 : MP == 6 ? 428 : MP == 7 ? 505
+                                                  : MP == 8 ? 575 : MP == 9 ? 987 : MP == 10 ? 1369 : 1545;
+  static_assert(SK >= SJ * (MP - 1) + MP && SE >= (SK + SJ + 1) * (MP - 1) + 1, "patch layout overlaps");
+  // slots of a block: the fewest idle lanes in its last warp (as best_bpb of the operator)
+  static constexpr int slots(int small) {
+    int best = 1;
+    for (int b = 2; b * TPE <= 320; ++b) {
+      const int tb = (b * TPE + 31) / 32 * 32, t0 = (best * TPE + 31) / 32 * 32;
+      if (b * t0 > best * tb || (b * t0 == best * tb && tb <= small)) best = b;
+    }
+    return best;
+  }
 };
 
-// One 1-D pass over the lines l = lt + TPE s (s < LPT) of one patch, node
-// (i, j, k) at i + MP j + SY k. dir 0: x lines (j, k) stride 1; dir 1: y lines
-// (i, k) stride MP; dir 2: z lines (i, j) stride SY. Forward: v[q] <- sum_i S[i][q] v[i]; backward:
-// v[i] <- sum_q S[i][q] v[q].
-template <typename T, int MP, int SY, int TPE, int LPT, int DIR, bool BACKWARD>
-__device__ __forceinline__ void sw_pass3(T* __restrict__ buf, const T* __restrict__ S, int lt) {
-  constexpr int MP2 = MP * MP;
-  constexpr int stride = DIR == 0 ? 1 : (DIR == 1 ? MP : SY);
-  int base[LPT];
-  bool ok[LPT];
+template <typename T, int N1, bool FILL>
+struct SwShape {
+  using C = SwCfg<T, N1>;
+  static constexpr int EPB = FILL ? C::slots(sizeof(T) == 4 ? 128 : 64) : (C::TPE >= 32 ? 1 : 32 / C::TPE);
+  static constexpr int THREADS = (EPB * C::TPE + 31) / 32 * 32;
+  // resident threads per SM asked of ptxas
+  static constexpr int WANT = sizeof(T) == 4 && C::MP < 10 ? 640 : 512;
+  static constexpr int MINB = WANT / THREADS < 1 ? 1 : WANT / THREADS > 32 ? 32 : WANT / THREADS;
+  static constexpr size_t SMEM = sizeof(T) * ((size_t)SW_MAXCLS * 3 * C::TB + (size_t)EPB * C::SE);
+};
+
+// N values of a table row (16-byte aligned)
+template <typename T, int N>
+__device__ __forceinline__ void sw_row(const T* __restrict__ p, T* r) {
+  constexpr int W = 16 / (int)sizeof(T);
 #pragma unroll
-  for (int s = 0; s < LPT; ++s) {
-    const int l = lt + TPE * s;
-    ok[s] = l < MP2;
-    const int l1 = l % MP, l2 = l / MP;
-    base[s] = ok[s] ? (DIR == 0 ? l1 * MP + l2 * SY : (DIR == 1 ? l1 + SY * l2 : l1 + MP * l2)) : 0;
-  }
-  if (!BACKWARD) {
-    // o[q] = sum_i S[i][q] v[i]: inputs streamed row by row, outputs in registers
-    T o[LPT][MP];
+  for (int w = 0; w < (N + W - 1) / W; ++w) {
+    if constexpr (sizeof(T) == 4) {
+      const float4 q = reinterpret_cast<const float4*>(p)[w];
+      const float t[4] = {q.x, q.y, q.z, q.w};
 #pragma unroll
-    for (int s = 0; s < LPT; ++s)
-#pragma unroll
-      for (int q = 0; q < MP; ++q) o[s][q] = (T)0;
-#pragma unroll 1
-    for (int i = 0; i < MP; ++i) {
-      T vi[LPT];
-#pragma unroll
-      for (int s = 0; s < LPT; ++s) vi[s] = buf[base[s] + i * stride];
-#pragma unroll
-      for (int q = 0; q < MP; ++q) {
-        const T sv = S[i * MP + q];
-#pragma unroll
-        for (int s = 0; s < LPT; ++s) o[s][q] += sv * vi[s];
-      }
-    }
-#pragma unroll
-    for (int s = 0; s < LPT; ++s)
-      if (ok[s]) {
-#pragma unroll
-        for (int q = 0; q < MP; ++q) buf[base[s] + q * stride] = o[s][q];
-      }
-  } else {
-    // o[i] = sum_q S[i][q] v[q]: inputs in registers, IB outputs per line at
-    // a time (LPT * IB independent sums in q order), each written when done
-    constexpr int IB = MP % 3 == 0 ? 3 : 2;
-    T v[LPT][MP];
-#pragma unroll
-    for (int s = 0; s < LPT; ++s)
-#pragma unroll
-      for (int q = 0; q < MP; ++q) v[s][q] = buf[base[s] + q * stride];
-#pragma unroll 1
-    for (int i0 = 0; i0 < MP; i0 += IB) {
-      T acc[IB][LPT];
-#pragma unroll
-      for (int ib = 0; ib < IB; ++ib)
-#pragma unroll
-        for (int s = 0; s < LPT; ++s) acc[ib][s] = (T)0;
-      const int nb = MP - i0 < IB ? MP - i0 : IB;
-#pragma unroll
-      for (int q = 0; q < MP; ++q) {
-#pragma unroll
-        for (int ib = 0; ib < IB; ++ib) {
-          const T sv = ib < nb ? S[(i0 + ib) * MP + q] : (T)0;
-#pragma unroll
-          for (int s = 0; s < LPT; ++s) acc[ib][s] += sv * v[s][q];
-        }
-      }
-#pragma unroll
-      for (int ib = 0; ib < IB; ++ib)
-        if (ib < nb) {
-#pragma unroll
-          for (int s = 0; s < LPT; ++s)
-            if (ok[s]) buf[base[s] + (i0 + ib) * stride] = acc[ib][s];
-        }
+      for (int k = 0; k < 4; ++k)
+        if (4 * w + k < N) r[4 * w + k] = t[k];
+    } else {
+      const double2 q = reinterpret_cast<const double2*>(p)[w];
+      r[2 * w] = q.x;
+      if (2 * w + 1 < N) r[2 * w + 1] = q.y;
     }
   }
 }
 
-// Division by the patch eigenvalue sum: FP32 takes the fast approximate
-// quotient (within 2 ulp; the sums are positive and far from the range
-// limits), FP64 the exact one.
-__device__ __forceinline__ float sw_div(float a, float b) { return __fdividef(a, b); }
-__device__ __forceinline__ double sw_div(double a, double b) { return a / b; }
+// sums and differences of mirrored nodes in place: v[i] (i < HE) the even part,
+// v[HE + i] the odd part
+template <typename T, int MP>
+__device__ __forceinline__ void sw_fold(T* v) {
+  constexpr int HO = MP / 2, HE = MP - HO;
+  T o[HO];
+#pragma unroll
+  for (int i = 0; i < HO; ++i) {
+    o[i] = v[i] - v[MP - 1 - i];
+    v[i] = v[i] + v[MP - 1 - i];
+  }
+#pragma unroll
+  for (int i = 0; i < HO; ++i) v[HE + i] = o[i];
+}
+// the reverse: node values from the even and odd parts
+template <typename T, int MP>
+__device__ __forceinline__ void sw_unfold(T* v) {
+  constexpr int HO = MP / 2, HE = MP - HO;
+  T o[HO];
+#pragma unroll
+  for (int i = 0; i < HO; ++i) o[i] = v[HE + i];
+#pragma unroll
+  for (int i = 0; i < HO; ++i) {
+    v[MP - 1 - i] = v[i] - o[i];
+    v[i] = v[i] + o[i];
+  }
+}
 
-template <typename T, int N1>
-__global__ void __launch_bounds__(SwCfg<T, N1>::THREADS, SwCfg<T, N1>::MINB)
-    k_schwarz_patch(const LevelOp* __restrict__ op, const double* __restrict__ tabs, const T* __restrict__ r,
+// Transforms of LPT lines with the table tb (row q: mode q at the nodes, halved
+// rows where SYM: the first HE even, the rest odd). A half H of the modes works
+// on the values v[O .. O + N).
+// forward: put(s, q, sum_i S[i][q] v[s][i])
+template <typename T, int MP, int LPT, int N, int O, int Q0, int Q1, typename P>
+__device__ __forceinline__ void sw_fwd_half(const T* tb, int RP, const T (*v)[MP], P&& put) {
+#pragma unroll 2
+  for (int q = Q0; q < Q1; ++q) {
+    T r[N], a[LPT];
+    sw_row<T, N>(tb + q * RP, r);
+#pragma unroll
+    for (int s = 0; s < LPT; ++s) a[s] = r[0] * v[s][O];
+#pragma unroll
+    for (int i = 1; i < N; ++i)
+#pragma unroll
+      for (int s = 0; s < LPT; ++s) a[s] += r[i] * v[s][O + i];
+#pragma unroll
+    for (int s = 0; s < LPT; ++s) put(s, q, a[s]);
+  }
+}
+template <typename T, int MP, int LPT, typename P>
+__device__ __forceinline__ void sw_fwd(bool sym, const T* tb, int RP, T (*v)[MP], P&& put) {
+  constexpr int HO = MP / 2, HE = MP - HO;
+  if (sym) {
+#pragma unroll
+    for (int s = 0; s < LPT; ++s) sw_fold<T, MP>(v[s]);
+    sw_fwd_half<T, MP, LPT, HE, 0, 0, HE>(tb, RP, v, put);
+    sw_fwd_half<T, MP, LPT, HO, HE, HE, MP>(tb, RP, v, put);
+  } else {
+    sw_fwd_half<T, MP, LPT, MP, 0, 0, MP>(tb, RP, v, put);
+  }
+}
+// backward: v[s][i] = sum_q S[i][q] get(s, q)
+template <typename T, int MP, int LPT, int N, int O, int Q0, int Q1, typename G>
+__device__ __forceinline__ void sw_bwd_half(const T* tb, int RP, T (*v)[MP], G&& get) {
+#pragma unroll
+  for (int s = 0; s < LPT; ++s)
+#pragma unroll
+    for (int i = 0; i < N; ++i) v[s][O + i] = (T)0;
+#pragma unroll 2
+  for (int q = Q0; q < Q1; ++q) {
+    T r[N], c[LPT];
+#pragma unroll
+    for (int s = 0; s < LPT; ++s) c[s] = get(s, q);
+    sw_row<T, N>(tb + q * RP, r);
+#pragma unroll
+    for (int i = 0; i < N; ++i)
+#pragma unroll
+      for (int s = 0; s < LPT; ++s) v[s][O + i] += r[i] * c[s];
+  }
+}
+template <typename T, int MP, int LPT, typename G>
+__device__ __forceinline__ void sw_bwd(bool sym, const T* tb, int RP, T (*v)[MP], G&& get) {
+  constexpr int HO = MP / 2, HE = MP - HO;
+  if (sym) {
+    sw_bwd_half<T, MP, LPT, HE, 0, 0, HE>(tb, RP, v, get);
+    sw_bwd_half<T, MP, LPT, HO, HE, HE, MP>(tb, RP, v, get);
+#pragma unroll
+    for (int s = 0; s < LPT; ++s) sw_unfold<T, MP>(v[s]);
+  } else {
+    sw_bwd_half<T, MP, LPT, MP, 0, 0, MP>(tb, RP, v, get);
+  }
+}
+// both, with the scaling between: v[s] <- S diag(scale(s, q, .)) S^T v[s]
+template <typename T, int MP, int LPT, int N, int O, int Q0, int Q1, typename F>
+__device__ __forceinline__ void sw_mid_half(const T* tb, int RP, const T (*v)[MP], T (*w)[MP], F&& scale) {
+#pragma unroll
+  for (int s = 0; s < LPT; ++s)
+#pragma unroll
+    for (int i = 0; i < N; ++i) w[s][O + i] = (T)0;
+#pragma unroll 1
+  for (int q = Q0; q < Q1; ++q) {
+    T r[N], a[LPT];
+    sw_row<T, N>(tb + q * RP, r);
+#pragma unroll
+    for (int s = 0; s < LPT; ++s) a[s] = r[0] * v[s][O];
+#pragma unroll
+    for (int i = 1; i < N; ++i)
+#pragma unroll
+      for (int s = 0; s < LPT; ++s) a[s] += r[i] * v[s][O + i];
+#pragma unroll
+    for (int s = 0; s < LPT; ++s) a[s] = scale(s, q, a[s]);
+#pragma unroll
+    for (int i = 0; i < N; ++i)
+#pragma unroll
+      for (int s = 0; s < LPT; ++s) w[s][O + i] += r[i] * a[s];
+  }
+}
+template <typename T, int MP, int LPT, typename F>
+__device__ __forceinline__ void sw_mid(bool sym, const T* tb, int RP, T (*v)[MP], T (*w)[MP], F&& scale) {
+  constexpr int HO = MP / 2, HE = MP - HO;
+  if (sym) {
+#pragma unroll
+    for (int s = 0; s < LPT; ++s) sw_fold<T, MP>(v[s]);
+    sw_mid_half<T, MP, LPT, HE, 0, 0, HE>(tb, RP, v, w, scale);
+    sw_mid_half<T, MP, LPT, HO, HE, HE, MP>(tb, RP, v, w, scale);
+#pragma unroll
+    for (int s = 0; s < LPT; ++s) sw_unfold<T, MP>(w[s]);
+  } else {
+    sw_mid_half<T, MP, LPT, MP, 0, 0, MP>(tb, RP, v, w, scale);
+  }
+}
+
+template <typename T, int N1, bool FILL>
+__global__ void __launch_bounds__(SwShape<T, N1, FILL>::THREADS, SwShape<T, N1, FILL>::MINB)
+    k_schwarz_patch(const __grid_constant__ SwGeom g, const unsigned char* __restrict__ blob, const T* __restrict__ r,
                     T* __restrict__ zp, const int* __restrict__ act, int nact) {
   using C = SwCfg<T, N1>;
-  constexpr int MP = C::MP, MP2 = MP * MP, MP3 = MP * MP * MP, NPE = N1 * N1 * N1, STR = 2 + MP2 + MP;
-  constexpr int SY = C::SY, SE = C::SE;
-  constexpr int EPB = C::EPB, NT = C::THREADS, TPE = C::TPE, LPT = C::LPT;
-  __shared__ T sS[EPB][3][MP2];
-  __shared__ T sL[EPB][3][MP];
-  __shared__ T buf[EPB][SE];
-  __shared__ int sm[EPB][3], soL[EPB][3];
-  __shared__ int spos[EPB][4];  // element of each slot (-1: none) and its (x, y, z) position
-  __shared__ long long srhs[EPB];
-  const int nx = op->n[0], ny = op->n[1];
-  const int E = op->E;
-  const long long Nq = op->Nq;
-  // the runtime divisions (item -> source, element -> position) once per slot
-  if (threadIdx.x < EPB) {
-    const long long it = (long long)blockIdx.x * EPB + threadIdx.x;
-    const bool v = it < (long long)nact * E;
-    const int ee = v ? (int)(it % E) : 0;
-    spos[threadIdx.x][0] = v ? ee : -1;
-    spos[threadIdx.x][1] = ee % nx;
-    spos[threadIdx.x][2] = (ee / nx) % ny;
-    spos[threadIdx.x][3] = ee / (nx * ny);
-    srhs[threadIdx.x] = v ? act[it / E] : 0;
-  }
-  __syncthreads();
-  const int slot = threadIdx.x / TPE, lt = threadIdx.x % TPE;
-  const bool valid = spos[slot][0] >= 0;
-  const int e = valid ? spos[slot][0] : 0;
-  const long long rhs = srhs[slot];
-  const int pos[3] = {spos[slot][1], spos[slot][2], spos[slot][3]};
-  // patch tables of the EPB elements
-  for (int t = threadIdx.x; t < EPB * 3 * STR; t += NT) {
-    const int sl = t / (3 * STR), rem = t % (3 * STR);
-    const int d = rem / STR, k = rem % STR;
-    const int pd = spos[sl][1 + d];
-    const double* tb = tabs + sw_axis_off(op, d, STR) + (long long)pd * STR;
-    if (k < 2) {
-      if (k == 0)
-        sm[sl][d] = (int)tb[0];
-      else
-        soL[sl][d] = (int)tb[1];
-    } else if (k < 2 + MP2) {
-      sS[sl][d][k - 2] = (T)tb[k];
-    } else {
-      sL[sl][d][k - 2 - MP2] = (T)tb[k];
+  using H = SwShape<T, N1, FILL>;
+  constexpr int MP = C::MP, MP2 = C::MP2, MP3 = C::MP3, NF = N1 * N1, NPE = NF * N1;
+  constexpr int SJ = C::SJ, SK = C::SK, SE = C::SE, RP = C::RP, TB = C::TB, TPE = C::TPE, LPT = C::LPT;
+  constexpr int EPB = H::EPB, NT = H::THREADS;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  T* tabs = reinterpret_cast<T*>(smem_raw);
+  T* buf = tabs + SW_MAXCLS * 3 * TB;
+  __shared__ int spos[EPB][3];   // per axis: table | patch size | left halo | symmetric
+  __shared__ int selem[EPB];     // element, -1: none
+  __shared__ long long ssrc[EPB];
+  const int nx = g.n[0], ny = g.n[1];
+  const long long E = (long long)nx * ny * g.n[2], Nq = E * NPE, items = E * nact;
+  const int* pos = reinterpret_cast<const int*>(blob + g.pos_off);
+  const T* gt = reinterpret_cast<const T*>(blob + g.tab_off);
+  for (int t = threadIdx.x; t < g.ntab * TB / C::W; t += NT)
+    reinterpret_cast<uint4*>(tabs)[t] = reinterpret_cast<const uint4*>(gt)[t];
+  const int slot = threadIdx.x / TPE, lt = threadIdx.x - slot * TPE;
+  const int sl = slot < EPB ? slot : 0;
+  T* b = buf + sl * SE;
+  const long long groups = (items + EPB - 1) / EPB;
+  for (long long grp = blockIdx.x; grp < groups; grp += gridDim.x) {
+    if (threadIdx.x < EPB) {
+      const long long it = grp * EPB + threadIdx.x;
+      const bool v = it < items;
+      const int k = v ? (int)(it / E) : 0, e = v ? (int)(it - k * E) : 0;
+      const int ex = e % nx, q = e / nx, ey = q % ny, ez = q / ny;
+      selem[threadIdx.x] = v ? e : -1;
+      spos[threadIdx.x][0] = pos[ex];
+      spos[threadIdx.x][1] = pos[nx + ey];
+      spos[threadIdx.x][2] = pos[nx + ny + ez];
+      ssrc[threadIdx.x] = act[k];
     }
-  }
-  __syncthreads();
-  const int mx = sm[slot][0], my = sm[slot][1], mz = sm[slot][2];
-  const int oLx = soL[slot][0], oLy = soL[slot][1], oLz = soL[slot][2];
-  T* b = buf[slot];
-  // gather the patch residual (own element plus one node layer of each
-  // neighbour), one patch row (j, k) at a time: the row's element offsets are
-  // computed once, the row's MP entries are three segments (left neighbour,
-  // own element, right neighbour)
-  if (valid) {
-    const T* rr = r + rhs * Nq;
-    for (int row = lt; row < MP2; row += TPE) {
-      const int j = row % MP, k = row / MP;
-      T* brow = b + j * MP + k * SY;
-      if (j >= my || k >= mz) {
+    __syncthreads();  // slots (and, the first time, tables) ready; the previous group's reads of them are done
+    const int e = selem[sl];
+    const bool on = slot < EPB && e >= 0;
+    const int px = spos[sl][0], py = spos[sl][1], pz = spos[sl][2];
+    const long long src = ssrc[sl];
+    const T *tx = tabs + sw_tab(px) * TB, *ty = tabs + sw_tab(py) * TB, *tz = tabs + sw_tab(pz) * TB;
+    T v[LPT][MP];
+    if (on) {
+      // z forward, lines (i, j): the patch residual (own element plus one node
+      // layer of each neighbour), zero outside the domain
+      const int oLx = sw_halo(px), oLy = sw_halo(py), oLz = sw_halo(pz);
+      const int mx = sw_size(px), my = sw_size(py), mz = sw_size(pz);
+      const T* rr = r + src * Nq;
+      const int pe = nx * ny;  // elements of a z layer
 #pragma unroll
-        for (int i = 0; i < MP; ++i) brow[i] = (T)0;
-        continue;
+      for (int s = 0; s < LPT; ++s) {
+        const int l = lt + TPE * s, i = l % MP, j = l / MP;
+        const bool in = l < MP2 && i < mx && j < my;
+        int a = i - oLx, bb = j - oLy, ee = e;
+        if (a < 0) {
+          a = N1 - 1;
+          ee -= 1;
+        } else if (a >= N1) {
+          a = 0;
+          ee += 1;
+        }
+        if (bb < 0) {
+          bb = N1 - 1;
+          ee -= nx;
+        } else if (bb >= N1) {
+          bb = 0;
+          ee += nx;
+        }
+        const int at = a + N1 * bb;
+#pragma unroll
+        for (int k = 0; k < MP; ++k) {
+          int c = k - oLz, ek = ee;
+          if (k == 0 && c < 0) {
+            c = N1 - 1;
+            ek -= pe;
+          } else if (k >= N1 && c >= N1) {
+            c = 0;
+            ek += pe;
+          }
+          v[s][k] = in && k < mz ? __ldg(rr + (long long)ek * NPE + at + NF * c) : (T)0;
+        }
       }
-      const int Y = pos[1] * N1 - oLy + j, Z = pos[2] * N1 - oLz + k;
-      const int ey = Y / N1, ez = Z / N1;
-      const long long rowe = (long long)nx * (ey + (long long)ny * ez);  // element index without x
-      const int lyz = N1 * ((Y - ey * N1) + N1 * (Z - ez * N1));
-      const T* own = rr + (rowe + pos[0]) * NPE + lyz;
-      int i = 0;
-      if (oLx) brow[i++] = rr[(rowe + pos[0] - 1) * NPE + lyz + (N1 - 1)];
-#pragma unroll
-      for (int a = 0; a < N1; ++a) brow[i + a] = own[a];
-      i += N1;
-      if (i < mx) brow[i++] = rr[(rowe + pos[0] + 1) * NPE + lyz];
-      for (; i < MP; ++i) brow[i] = (T)0;
+      sw_fwd<T, MP, LPT>(sw_sym(pz), tz, RP, v, [&](int s, int q, T a) {
+        const int l = lt + TPE * s;
+        if (MP2 % LPT == 0 || l < MP2) b[l % MP + SJ * (l / MP) + SK * q] = a;
+      });
     }
-  } else {
-    for (int t = lt; t < SE; t += TPE) b[t] = (T)0;
-  }
-  __syncthreads();
-  sw_pass3<T, MP, SY, TPE, LPT, 0, false>(b, sS[slot][0], lt);
-  __syncthreads();
-  sw_pass3<T, MP, SY, TPE, LPT, 1, false>(b, sS[slot][1], lt);
-  __syncthreads();
-  sw_pass3<T, MP, SY, TPE, LPT, 2, false>(b, sS[slot][2], lt);
-  // scale by 1 / (lx + ly + lz) along this thread's z lines (i, j)
+    __syncthreads();
+    if (on) {
+      // y forward, lines (i, k)
+      int at[LPT];
 #pragma unroll
-  for (int s = 0; s < LPT; ++s) {
-    const int l = lt + TPE * s;
-    if (l < MP2) {
-      const int l1 = l % MP, l2 = l / MP;
+      for (int s = 0; s < LPT; ++s) {
+        const int l = lt + TPE * s;
+        at[s] = MP2 % LPT == 0 || l < MP2 ? l % MP + SK * (l / MP) : 0;
 #pragma unroll
-      for (int k = 0; k < MP; ++k) {
-        const int t = l + SY * k;
-        const bool in = l1 < mx && l2 < my && k < mz;
-        b[t] = in ? sw_div(b[t], sL[slot][0][l1] + sL[slot][1][l2] + sL[slot][2][k]) : (T)0;
+        for (int j = 0; j < MP; ++j) v[s][j] = b[at[s] + SJ * j];
+      }
+      sw_fwd<T, MP, LPT>(sw_sym(py), ty, RP, v, [&](int s, int q, T a) {
+        if (MP2 % LPT == 0 || lt + TPE * s < MP2) b[at[s] + SJ * q] = a;
+      });
+    }
+    __syncthreads();
+    if (on) {
+      // x, lines (j, k)
+      T w[LPT][MP];
+      const T* lx = tx + MP * RP;
+      T lyz[LPT];
+      const T* inv[LPT];
+#pragma unroll
+      for (int s = 0; s < LPT; ++s) {
+        const int l = lt + TPE * s, ll = MP2 % LPT == 0 || l < MP2 ? l : 0, j = ll % MP, k = ll / MP;
+        const int at = SJ * j + SK * k;
+#pragma unroll
+        for (int i = 0; i < MP; ++i) v[s][i] = b[at + i];
+        if constexpr (sizeof(T) == 8) {
+          inv[s] = reinterpret_cast<const T*>(blob + g.inv_off) +
+                   (((long long)sw_cls(pz) * SW_MAXCLS + sw_cls(py)) * SW_MAXCLS + sw_cls(px)) * MP3 + ll;
+          lyz[s] = (T)0;
+        } else {
+          inv[s] = nullptr;
+          lyz[s] = ty[MP * RP + j] + tz[MP * RP + k];
+        }
+      }
+      sw_mid<T, MP, LPT>(sw_sym(px), tx, RP, v, w, [&](int s, int q, T a) -> T {
+        if constexpr (sizeof(T) == 8)
+          return a * __ldg(inv[s] + q * MP2);
+        else
+          return __fdividef(a, lx[q] + lyz[s]);  // within 2 ulp; the sums are positive and far from the range limits
+      });
+#pragma unroll
+      for (int s = 0; s < LPT; ++s) {
+        const int l = lt + TPE * s, at = SJ * (l % MP) + SK * (l / MP);
+        if (MP2 % LPT == 0 || l < MP2) {
+#pragma unroll
+          for (int i = 0; i < MP; ++i) b[at + i] = w[s][i];
+        }
       }
     }
+    __syncthreads();
+    if (on) {
+      // y backward, lines (i, k)
+      int at[LPT];
+#pragma unroll
+      for (int s = 0; s < LPT; ++s) {
+        const int l = lt + TPE * s;
+        at[s] = MP2 % LPT == 0 || l < MP2 ? l % MP + SK * (l / MP) : 0;
+      }
+      sw_bwd<T, MP, LPT>(sw_sym(py), ty, RP, v, [&](int s, int q) -> T { return b[at[s] + SJ * q]; });
+#pragma unroll
+      for (int s = 0; s < LPT; ++s)
+        if (MP2 % LPT == 0 || lt + TPE * s < MP2) {
+#pragma unroll
+          for (int j = 0; j < MP; ++j) b[at[s] + SJ * j] = v[s][j];
+        }
+    }
+    __syncthreads();
+    if (on) {
+      // z backward, lines (i, j), to the patch buffer: node (i, j, k) at i + MP j + MP^2 k
+      sw_bwd<T, MP, LPT>(sw_sym(pz), tz, RP, v, [&](int s, int q) -> T {
+        const int l = lt + TPE * s, ll = MP2 % LPT == 0 || l < MP2 ? l : 0;
+        return b[ll % MP + SJ * (ll / MP) + SK * q];
+      });
+      T* out = zp + (src * E + e) * MP3;
+#pragma unroll
+      for (int s = 0; s < LPT; ++s) {
+        const int l = lt + TPE * s;
+        if (MP2 % LPT == 0 || l < MP2) {
+#pragma unroll
+          for (int k = 0; k < MP; ++k) out[l + MP2 * k] = v[s][k];
+        }
+      }
+    }
+    __syncthreads();  // everybody is done with the slots and the buffer
   }
-  sw_pass3<T, MP, SY, TPE, LPT, 2, true>(b, sS[slot][2], lt);
-  __syncthreads();
-  sw_pass3<T, MP, SY, TPE, LPT, 1, true>(b, sS[slot][1], lt);
-  __syncthreads();
-  sw_pass3<T, MP, SY, TPE, LPT, 0, true>(b, sS[slot][0], lt);
-  __syncthreads();
-  if (!valid) return;
-  T* out = zp + (rhs * E + e) * (long long)MP3;
-  for (int t = lt; t < MP3; t += TPE) out[t] = b[t % MP2 + SY * (t / MP2)];
+}
+
+template <typename T, int N1, bool FILL>
+static cudaError_t patch_shape(const SwTables& tb, const T* r, T* zp, const int* act, int nact, cudaStream_t s) {
+  using H = SwShape<T, N1, FILL>;
+  const SwGeom& g = tb.geom;
+  const long long items = (long long)g.n[0] * g.n[1] * g.n[2] * nact;
+  const long long groups = (items + H::EPB - 1) / H::EPB;
+  auto kern = k_schwarz_patch<T, N1, FILL>;
+  if (H::SMEM > 48 * 1024) {
+    const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)H::SMEM);
+    if (e != cudaSuccess) return e;
+  }
+  // persistent grid: the blocks that shared memory and the thread limit let an SM hold
+  constexpr int BY_SMEM = (int)(227 * 1024 / (H::SMEM + 1024)), BY_THREADS = 2048 / H::THREADS;
+  const long long cap = 152LL * (BY_SMEM < BY_THREADS ? BY_SMEM : BY_THREADS);
+  count_launch();
+  kern<<<(unsigned)(groups < cap ? groups : cap), H::THREADS, H::SMEM, s>>>(g, (const unsigned char*)tb.blob, r, zp, act,
+                                                                         nact);
+  return cudaGetLastError();
+}
+
+// Several patches per block, so that warps are full, once there are two such
+// blocks per SM; below that as many blocks as possible.
+template <typename T, int N1>
+static cudaError_t patch_n1(const SwTables& tb, const T* r, T* zp, const int* act, int nact, cudaStream_t s) {
+  const long long items = (long long)tb.geom.n[0] * tb.geom.n[1] * tb.geom.n[2] * nact;
+  if (items / SwShape<T, N1, true>::EPB >= 2 * 152) return patch_shape<T, N1, true>(tb, r, zp, act, nact, s);
+  return patch_shape<T, N1, false>(tb, r, zp, act, nact, s);
 }
 
 // Gather block shape: GE elements of NPE nodes per block (several small
@@ -391,27 +561,10 @@ __global__ void __launch_bounds__(GatherCfg<N1>::THREADS)
   }
 }
 
+// z = M r from the patch solutions (the second kernel of the smoother)
 template <typename T, int N1>
-static cudaError_t schwarz_n1(const LevelOp& hop, const LevelOp* dop, const double* tabs, const T* r, T* zp, T* z,
-                              T* x, int mode, double c1, double c2, const int* act, int nact, cudaStream_t s,
-                              const SwTcPlan* tc) {
-  using C = SwCfg<T, N1>;
-  const long long items = (long long)nact * hop.E;
-#if DG_SMEM_CARVEOUT >= 0
-  static bool carve = false;
-  if (!carve) {
-    cudaFuncSetAttribute(k_schwarz_patch<T, N1>, cudaFuncAttributePreferredSharedMemoryCarveout, DG_SMEM_CARVEOUT);
-    carve = true;
-  }
-#endif
-  if (sizeof(T) == 4 && tc && tc->blob) {
-    const cudaError_t e = launch_schwarz_patch_tc(hop, dop, *tc, (const float*)r, (float*)zp, act, nact, s);
-    if (e != cudaSuccess) return e;
-  } else {
-    count_launch();
-    k_schwarz_patch<T, N1><<<(unsigned)((items + C::EPB - 1) / C::EPB), C::THREADS, 0, s>>>(dop, tabs, r, zp, act,
-                                                                                           nact);
-  }
+static cudaError_t gather_n1(const LevelOp& hop, const LevelOp* dop, const T* zp, T* z, T* x, int mode, double c1,
+                             double c2, const int* act, int nact, cudaStream_t s) {
   constexpr int GT = GatherCfg<N1>::THREADS;
   // the gather indexes one source's patch buffer with 32-bit offsets
   if ((long long)hop.E * (N1 + 2) * (N1 + 2) * (N1 + 2) >= (1LL << 31)) return cudaErrorInvalidValue;
@@ -432,63 +585,53 @@ static cudaError_t schwarz_n1(const LevelOp& hop, const LevelOp* dop, const doub
   return cudaGetLastError();
 }
 
-// the patch solves alone (the first kernel of schwarz_n1)
-template <typename T, int N1>
-static cudaError_t schwarz_patch_n1(const LevelOp& hop, const LevelOp* dop, const double* tabs, const T* r, T* zp,
-                                    const int* act, int nact, cudaStream_t s, const SwTcPlan* tc) {
-  using C = SwCfg<T, N1>;
-  if (sizeof(T) == 4 && tc && tc->blob)
-    return launch_schwarz_patch_tc(hop, dop, *tc, (const float*)r, (float*)zp, act, nact, s);
-  const long long items = (long long)nact * hop.E;
-  count_launch();
-  k_schwarz_patch<T, N1><<<(unsigned)((items + C::EPB - 1) / C::EPB), C::THREADS, 0, s>>>(dop, tabs, r, zp, act,
-                                                                                         nact);
-  return cudaGetLastError();
-}
-
 template <typename T>
-cudaError_t launch_schwarz_patch(const LevelOp& hop, const LevelOp* dop, const double* tabs, const T* r, T* zp,
+cudaError_t launch_schwarz_patch(const LevelOp& hop, const LevelOp* dop, const SwTables& tabs, const T* r, T* zp,
                                  const int* act, int nact, cudaStream_t s, const SwTcPlan* tc) {
   if (nact == 0) return cudaSuccess;
+  if (sizeof(T) == 4 && tc && tc->blob)
+    return launch_schwarz_patch_tc(hop, dop, *tc, (const float*)r, (float*)zp, act, nact, s);
   switch (hop.n1) {
-    case 2: return schwarz_patch_n1<T, 2>(hop, dop, tabs, r, zp, act, nact, s, tc);
-    case 3: return schwarz_patch_n1<T, 3>(hop, dop, tabs, r, zp, act, nact, s, tc);
-    case 4: return schwarz_patch_n1<T, 4>(hop, dop, tabs, r, zp, act, nact, s, tc);
-    case 5: return schwarz_patch_n1<T, 5>(hop, dop, tabs, r, zp, act, nact, s, tc);
-    case 6: return schwarz_patch_n1<T, 6>(hop, dop, tabs, r, zp, act, nact, s, tc);
-    case 7: return schwarz_patch_n1<T, 7>(hop, dop, tabs, r, zp, act, nact, s, tc);
-    case 8: return schwarz_patch_n1<T, 8>(hop, dop, tabs, r, zp, act, nact, s, tc);
-    case 9: return schwarz_patch_n1<T, 9>(hop, dop, tabs, r, zp, act, nact, s, tc);
+    case 2: return patch_n1<T, 2>(tabs, r, zp, act, nact, s);
+    case 3: return patch_n1<T, 3>(tabs, r, zp, act, nact, s);
+    case 4: return patch_n1<T, 4>(tabs, r, zp, act, nact, s);
+    case 5: return patch_n1<T, 5>(tabs, r, zp, act, nact, s);
+    case 6: return patch_n1<T, 6>(tabs, r, zp, act, nact, s);
+    case 7: return patch_n1<T, 7>(tabs, r, zp, act, nact, s);
+    case 8: return patch_n1<T, 8>(tabs, r, zp, act, nact, s);
+    case 9: return patch_n1<T, 9>(tabs, r, zp, act, nact, s);
     default: return cudaErrorInvalidValue;
   }
 }
 
 template <typename T>
-cudaError_t launch_schwarz(const LevelOp& hop, const LevelOp* dop, const double* tabs, const T* r, T* zp, T* z,
+cudaError_t launch_schwarz(const LevelOp& hop, const LevelOp* dop, const SwTables& tabs, const T* r, T* zp, T* z,
                            T* x, int mode, double c1, double c2, const int* act, int nact, cudaStream_t s,
                            const SwTcPlan* tc) {
   if (nact == 0) return cudaSuccess;
+  const cudaError_t e = launch_schwarz_patch<T>(hop, dop, tabs, r, zp, act, nact, s, tc);
+  if (e != cudaSuccess) return e;
   switch (hop.n1) {
-    case 2: return schwarz_n1<T, 2>(hop, dop, tabs, r, zp, z, x, mode, c1, c2, act, nact, s, tc);
-    case 3: return schwarz_n1<T, 3>(hop, dop, tabs, r, zp, z, x, mode, c1, c2, act, nact, s, tc);
-    case 4: return schwarz_n1<T, 4>(hop, dop, tabs, r, zp, z, x, mode, c1, c2, act, nact, s, tc);
-    case 5: return schwarz_n1<T, 5>(hop, dop, tabs, r, zp, z, x, mode, c1, c2, act, nact, s, tc);
-    case 6: return schwarz_n1<T, 6>(hop, dop, tabs, r, zp, z, x, mode, c1, c2, act, nact, s, tc);
-    case 7: return schwarz_n1<T, 7>(hop, dop, tabs, r, zp, z, x, mode, c1, c2, act, nact, s, tc);
-    case 8: return schwarz_n1<T, 8>(hop, dop, tabs, r, zp, z, x, mode, c1, c2, act, nact, s, tc);
-    case 9: return schwarz_n1<T, 9>(hop, dop, tabs, r, zp, z, x, mode, c1, c2, act, nact, s, tc);
+    case 2: return gather_n1<T, 2>(hop, dop, zp, z, x, mode, c1, c2, act, nact, s);
+    case 3: return gather_n1<T, 3>(hop, dop, zp, z, x, mode, c1, c2, act, nact, s);
+    case 4: return gather_n1<T, 4>(hop, dop, zp, z, x, mode, c1, c2, act, nact, s);
+    case 5: return gather_n1<T, 5>(hop, dop, zp, z, x, mode, c1, c2, act, nact, s);
+    case 6: return gather_n1<T, 6>(hop, dop, zp, z, x, mode, c1, c2, act, nact, s);
+    case 7: return gather_n1<T, 7>(hop, dop, zp, z, x, mode, c1, c2, act, nact, s);
+    case 8: return gather_n1<T, 8>(hop, dop, zp, z, x, mode, c1, c2, act, nact, s);
+    case 9: return gather_n1<T, 9>(hop, dop, zp, z, x, mode, c1, c2, act, nact, s);
     default: return cudaErrorInvalidValue;
   }
 }
 
-template cudaError_t launch_schwarz_patch<double>(const LevelOp&, const LevelOp*, const double*, const double*,
+template cudaError_t launch_schwarz_patch<double>(const LevelOp&, const LevelOp*, const SwTables&, const double*,
                                                   double*, const int*, int, cudaStream_t, const SwTcPlan*);
-template cudaError_t launch_schwarz_patch<float>(const LevelOp&, const LevelOp*, const double*, const float*, float*,
+template cudaError_t launch_schwarz_patch<float>(const LevelOp&, const LevelOp*, const SwTables&, const float*, float*,
                                                  const int*, int, cudaStream_t, const SwTcPlan*);
-template cudaError_t launch_schwarz<double>(const LevelOp&, const LevelOp*, const double*, const double*, double*,
+template cudaError_t launch_schwarz<double>(const LevelOp&, const LevelOp*, const SwTables&, const double*, double*,
                                             double*, double*, int, double, double, const int*, int, cudaStream_t,
                                             const SwTcPlan*);
-template cudaError_t launch_schwarz<float>(const LevelOp&, const LevelOp*, const double*, const float*, float*,
+template cudaError_t launch_schwarz<float>(const LevelOp&, const LevelOp*, const SwTables&, const float*, float*,
                                            float*, float*, int, double, double, const int*, int, cudaStream_t,
                                            const SwTcPlan*);
 

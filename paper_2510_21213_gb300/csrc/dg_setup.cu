@@ -269,6 +269,120 @@ std::vector<double> schwarz_tables(const LevelOp& L) {
   return out;
 }
 
+// Even and odd generalised eigenpairs of the patch of element e of axis d, whose
+// 1-D matrix is invariant under reversal: two problems of half the size, so the
+// modes are even or odd exactly (those of the whole matrix are only up to
+// round-off over the eigenvalue gap). rows[q * HE + i]: mode q at node i (i < HE
+// even, the first HO of the odd ones); lam[q].
+static void schwarz_halves(const LevelOp& L, int d, int e, std::vector<double>& rows, std::vector<double>& lam) {
+  const int n1 = L.n1, m = n1 + 2, HO = m / 2, HE = m - HO, Ld = L.n[d] * n1, lo = e * n1 - 1;
+  const std::vector<double> A = axis_matrix(L.ax[d], L);
+  std::vector<double> Mi(m), B((size_t)m * m);
+  for (int i = 0; i < m; ++i) Mi[i] = 1.0 / std::sqrt(L.ax[d].m[(lo + i) % n1]);
+  for (int i = 0; i < m; ++i)
+    for (int j = 0; j < m; ++j) B[(size_t)i * m + j] = A[(size_t)(lo + i) * Ld + (lo + j)] * Mi[i] * Mi[j];
+  auto b = [&](int i, int j) {  // averaged with its mirror image and transpose
+    return 0.25 * (B[(size_t)i * m + j] + B[(size_t)j * m + i] + B[(size_t)(m - 1 - i) * m + (m - 1 - j)] +
+                   B[(size_t)(m - 1 - j) * m + (m - 1 - i)]);
+  };
+  rows.assign((size_t)m * HE, 0.0);
+  lam.assign(m, 0.0);
+  const double r2 = std::sqrt(0.5);
+  for (int par = 0; par < 2; ++par) {
+    const int k = par == 0 ? HE : HO;
+    std::vector<double> S((size_t)k * k), ev, V;
+    for (int i = 0; i < k; ++i)
+      for (int j = 0; j < k; ++j) {
+        const bool mi = i >= HO, mj = j >= HO;  // the middle node (even part of an odd m)
+        double v = par == 0 ? b(i, j) + b(i, m - 1 - j) : b(i, j) - b(i, m - 1 - j);
+        if (mi && mj)
+          v = b(i, j);
+        else if (mi || mj)
+          v = b(i, j) / r2;
+        S[(size_t)i * k + j] = v;
+      }
+    sym_eig(S, k, ev, V);
+    for (int q = 0; q < k; ++q) {
+      const int row = par == 0 ? q : HE + q;
+      lam[row] = ev[q];
+      for (int i = 0; i < k; ++i) rows[(size_t)row * HE + i] = Mi[i] * V[(size_t)i * k + q] * (i >= HO ? 1.0 : r2);
+    }
+  }
+}
+
+template <typename T>
+static std::vector<unsigned char> schwarz_blob_t(const LevelOp& L, const std::vector<double>& tb, SwGeom& g) {
+  const int n1 = L.n1, MP = n1 + 2, HE = MP - MP / 2, STR = schwarz_axis_stride(n1);
+  const int W = 16 / (int)sizeof(T), RP = (MP + W - 1) / W * W, TB = (MP + 1) * RP;
+  std::vector<int> pos;
+  std::vector<T> tab;
+  std::vector<double> lams[3][SW_MAXCLS];
+  int ncls[3] = {0, 0, 0};
+  g = SwGeom{};
+  size_t off = 0;
+  for (int d = 0; d < 3; ++d) {
+    const int n = L.n[d];
+    g.n[d] = n;
+    std::vector<int> key;  // distances to the two ends, up to 2: equal keys, equal tables
+    for (int e = 0; e < n; ++e, off += STR) {
+      const int kl = std::min(e, 2), kr = std::min(n - 1 - e, 2), k = 3 * kl + kr;
+      const double* t = tb.data() + off;
+      const int m = (int)t[0], oL = (int)t[1];
+      const bool sym = kl == kr && m == MP;
+      int c = (int)(std::find(key.begin(), key.end(), k) - key.begin());
+      if (c == (int)key.size()) {
+        key.push_back(k);
+        std::vector<double> rows, lam(MP, 1.0);
+        std::vector<T> one(TB, (T)0);
+        if (sym) {
+          schwarz_halves(L, d, e, rows, lam);
+          for (int q = 0; q < MP; ++q)
+            for (int i = 0; i < HE; ++i) one[(size_t)q * RP + i] = (T)rows[(size_t)q * HE + i];
+        } else {
+          for (int q = 0; q < m; ++q) {
+            lam[q] = t[2 + MP * MP + q];
+            for (int i = 0; i < m; ++i) one[(size_t)q * RP + i] = (T)t[2 + i * MP + q];
+          }
+        }
+        for (int q = 0; q < MP; ++q) one[(size_t)MP * RP + q] = (T)lam[q];
+        lams[d][c] = lam;
+        tab.insert(tab.end(), one.begin(), one.end());
+        ++ncls[d];
+      }
+      int base = 0;
+      for (int dd = 0; dd < d; ++dd) base += ncls[dd];
+      pos.push_back(sw_pack(base + c, c, m, oL, sym ? 1 : 0));
+    }
+  }
+  g.ntab = ncls[0] + ncls[1] + ncls[2];
+  g.pos_off = 0;
+  g.tab_off = (unsigned)((pos.size() * sizeof(int) + 15) / 16 * 16);
+  g.inv_off = (unsigned)(g.tab_off + tab.size() * sizeof(T));
+  std::vector<T> inv;
+  if (sizeof(T) == 8) {
+    const size_t mp3 = (size_t)MP * MP * MP;
+    inv.assign((size_t)SW_MAXCLS * SW_MAXCLS * SW_MAXCLS * mp3, (T)0);
+    for (int cz = 0; cz < ncls[2]; ++cz)
+      for (int cy = 0; cy < ncls[1]; ++cy)
+        for (int cx = 0; cx < ncls[0]; ++cx) {
+          T* o = inv.data() + (((size_t)cz * SW_MAXCLS + cy) * SW_MAXCLS + cx) * mp3;
+          for (int q = 0; q < MP; ++q)
+            for (int k = 0; k < MP; ++k)
+              for (int j = 0; j < MP; ++j)
+                o[((size_t)q * MP + k) * MP + j] = (T)(1.0 / (lams[0][cx][q] + lams[1][cy][j] + lams[2][cz][k]));
+        }
+  }
+  std::vector<unsigned char> out(g.inv_off + inv.size() * sizeof(T), 0);
+  std::memcpy(out.data(), pos.data(), pos.size() * sizeof(int));
+  std::memcpy(out.data() + g.tab_off, tab.data(), tab.size() * sizeof(T));
+  if (!inv.empty()) std::memcpy(out.data() + g.inv_off, inv.data(), inv.size() * sizeof(T));
+  return out;
+}
+
+std::vector<unsigned char> schwarz_blob(const LevelOp& L, const std::vector<double>& tb, int size, SwGeom& g) {
+  return size == 8 ? schwarz_blob_t<double>(L, tb, g) : schwarz_blob_t<float>(L, tb, g);
+}
+
 // lambda_max(D^-1 A) of the 3-D Kronecker-sum operator: A <= mu_d diag(A_d) in
 // each direction implies x^T A x <= max_d mu_d x^T D x, with equality for the
 // product of the 1-D maximisers, so the bound is exact for isotropic meshes.

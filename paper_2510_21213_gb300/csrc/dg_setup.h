@@ -26,6 +26,8 @@ double sym_max_eig(std::vector<double> S, int n);
 double level_lambda_max(const LevelOp& L);
 void sym_eig(std::vector<double> S, int n, std::vector<double>& lam, std::vector<double>& V);
 std::vector<double> schwarz_tables(const LevelOp& L);
+// device tables of the SIMT patch kernel from schwarz_tables' (layout in dg_internal.h); size: 8 (FP64) or 4 (FP32)
+std::vector<unsigned char> schwarz_blob(const LevelOp& L, const std::vector<double>& tb, int size, SwGeom& g);
 void build_transfer(TransferOp& T, const LevelOp& fine, const LevelOp& coarse);
 bool spd_inverse(std::vector<double>& A, int n);
 std::vector<double> level_dense(const LevelOp& L);
