@@ -36,7 +36,7 @@
 // its pipe before and after: 7.86 -> 7.25 ms and 0.955 -> 0.824 ms; at p = 3 and
 // 1, where folding saves nothing, 0.83 -> 0.86 ms and 0.089 -> 0.111 ms (16^3, 42
 // fields; 3 % and 0.4 % of an FP64 build).
-#include "dg_internal.h"
+#include "dg_line.h"
 
 namespace dg {
 
@@ -119,17 +119,6 @@ static void fill_tab(ApplyTab<T, N1>& t, const LevelOp& op) {
   t.Nq = op.Nq;
 }
 
-// Bricks per block (at most 320 threads) that leave the fewest idle lanes in the last warp
-constexpr int best_bpb(int lines, int small) {
-  int best = 1;
-  for (int b = 2; b * lines <= 320; ++b) {
-    const int tb = (b * lines + 31) / 32 * 32, t0 = (best * lines + 31) / 32 * 32;
-    // more filled per thread, or as filled and still a small block
-    if (b * t0 > best * tb || (b * t0 == best * tb && tb <= small)) best = b;
-  }
-  return best;
-}
-
 // Launch shape. BR: elements of a brick along each axis (2 or 1). FILL: several
 // bricks per block, so that warps are full; otherwise one, for problems too
 // small to give every SM a block.
@@ -138,17 +127,7 @@ struct ApplyCfg {
   static constexpr int NPE = N1 * N1 * N1, NF = N1 * N1;
   static constexpr int EB = BR * BR * BR;        // elements of a brick
   static constexpr int LINES = BR * BR * NF;     // threads of a brick: one (pair of) line(s) each
-  // node (a, b, c) of element e of the block at a + PB b + PZ c + ES e: the
-  // strides with the fewest shared-memory wavefronts of the three passes,
-  // counted over the warps of a block (1.4 to 1.9 per access; odd strides alone
-  // gave 1.9 to 2.5, and the FP32 kernel was bound by them at p = 7: 86 % of the
-  // data pipe)
-  static constexpr int PB = N1 == 8 ? 9 : N1;
-  static constexpr int PZ = N1 == 2 ? 4 : N1 == 3 ? 9 : N1 == 4 ? 19 : N1 == 5 ? 25 : N1 == 6 ? 41 : N1 == 7 ? 52
-                                                                                          : N1 == 8 ? 72 : 81;
-  static constexpr int ES = N1 == 2 ? 10 : N1 == 3 ? 41 : N1 == 4 ? 80 : N1 == 5 ? 153 : N1 == 6 ? 260
-                                                          : N1 == 7 ? 369 : N1 == 8 ? 575 : 736;
-  static_assert(PZ >= PB * (N1 - 1) + N1 && ES >= (PZ + PB + 1) * (N1 - 1) + 1, "element layout overlaps");
+  static constexpr int PB = LineLayout<N1>::PB, PZ = LineLayout<N1>::PZ, ES = LineLayout<N1>::ES;
   static constexpr int BPB = FILL ? best_bpb(LINES, sizeof(T) == 4 ? DG_APPLY_TIE32 : DG_APPLY_TIE64) : 1;
   static constexpr int THREADS = (BPB * LINES + 31) / 32 * 32;
   static constexpr size_t SMEM = sizeof(T) * 2 * (size_t)BPB * EB * ES;
@@ -156,62 +135,6 @@ struct ApplyCfg {
   static constexpr int WANT = sizeof(T) == 4 ? DG_APPLY_WANT32 : DG_APPLY_WANT64;
   static constexpr int MINB = WANT / THREADS < 1 ? 1 : WANT / THREADS;
 };
-
-// Every product and sum is written out with its rounding (mad, mul), so that the
-// instances of the kernel round alike: a source's result depends neither on the
-// work split nor, with it, on the number of sources in the call.
-__device__ __forceinline__ float mad(float a, float b, float c) { return __fmaf_rn(a, b, c); }
-__device__ __forceinline__ double mad(double a, double b, double c) { return __fma_rn(a, b, c); }
-__device__ __forceinline__ float mul(float a, float b) { return __fmul_rn(a, b); }
-__device__ __forceinline__ double mul(double a, double b) { return __dmul_rn(a, b); }
-
-// value and derivative at the left (RIGHT: right) end of a line
-template <typename T, int N1, bool RIGHT>
-__device__ __forceinline__ void end_trace(const ApplyTab<T, N1>& tab, const T* v, T& val, T& der) {
-  T a = mul(tab.tl[RIGHT ? N1 - 1 : 0], v[0]), b = mul(tab.dl[RIGHT ? N1 - 1 : 0], v[0]);
-#pragma unroll
-  for (int i = 1; i < N1; ++i) {
-    const int k = RIGHT ? N1 - 1 - i : i;
-    a = mad(tab.tl[k], v[i], a);
-    b = mad(tab.dl[k], v[i], b);
-  }
-  val = a;
-  der = RIGHT ? -b : b;
-}
-
-// line of N1 values at p with stride SD, reversed where rev is set; contiguous
-// lines that are a multiple of 16 bytes are read with 16-byte loads where the
-// field is aligned (vec)
-template <typename T, int N1, int SD>
-__device__ __forceinline__ void load_line(const T* __restrict__ p, bool rev, bool vec, T* v) {
-  constexpr int W = 16 / (int)sizeof(T);
-  if constexpr (SD == 1 && N1 % W == 0) {
-    if (vec) {
-      T q[N1];
-#pragma unroll
-      for (int w = 0; w < N1 / W; ++w) {
-        if constexpr (sizeof(T) == 4) {
-          const float4 t = __ldg(reinterpret_cast<const float4*>(p) + w);
-          q[4 * w] = t.x;
-          q[4 * w + 1] = t.y;
-          q[4 * w + 2] = t.z;
-          q[4 * w + 3] = t.w;
-        } else {
-          const double2 t = __ldg(reinterpret_cast<const double2*>(p) + w);
-          q[2 * w] = t.x;
-          q[2 * w + 1] = t.y;
-        }
-      }
-#pragma unroll
-      for (int i = 0; i < N1; ++i) v[i] = rev ? q[N1 - 1 - i] : q[i];
-      return;
-    }
-  }
-  const T* q = rev ? p + (N1 - 1) * SD : p;
-  const int st = rev ? -SD : SD;
-#pragma unroll
-  for (int i = 0; i < N1; ++i) v[i] = __ldg(q + i * st);
-}
 
 // one pass along direction D for this thread's line (pair): on entry v[s] holds
 // the line values, ov/od the traces beyond its two ends (0: left of the first, 1:
@@ -226,9 +149,9 @@ __device__ __forceinline__ void line_op(const ApplyTab<T, N1>& tab, T (*v)[N1], 
   for (int s = 0; s < BR; ++s) {
     if (BR == 2) {
       if (s == 0)
-        end_trace<T, N1, true>(tab, v[s], tv[s], td[s]);
+        end_trace<T, N1, true>(tab.tl, tab.dl, v[s], tv[s], td[s]);
       else
-        end_trace<T, N1, false>(tab, v[s], tv[s], td[s]);
+        end_trace<T, N1, false>(tab.tl, tab.dl, v[s], tv[s], td[s]);
     }
     if constexpr (N1 > 2) {
 #pragma unroll
@@ -308,14 +231,14 @@ __device__ __forceinline__ void outer_traces(const ApplyTab<T, N1>& tab, const T
   const T gam = tab.gam[D];
   T v[N1];
   load_line<T, N1, SD>(out0 ? p - es * NPE : p, !out0, vec, v);
-  end_trace<T, N1, true>(tab, v, ov[0], od[0]);
+  end_trace<T, N1, true>(tab.tl, tab.dl, v, ov[0], od[0]);
   if (!out0) {
     od[0] = mad(-gam, ov[0], -od[0]);
     ov[0] = -ov[0];
   }
   const int last = BR == 2 && second ? 1 : 0;
   load_line<T, N1, SD>(p + (last + (out1 ? 1 : 0)) * es * NPE, !out1, vec, v);
-  end_trace<T, N1, false>(tab, v, ov[1], od[1]);
+  end_trace<T, N1, false>(tab.tl, tab.dl, v, ov[1], od[1]);
   if (!out1) {
     od[1] = mad(gam, ov[1], -od[1]);
     ov[1] = -ov[1];

@@ -16,7 +16,7 @@
 #include <vector>
 
 #include "dg_ctx.h"
-#include "dg_internal.h"
+#include "dg_line.h"
 #include "dg_octree.h"
 #include "dg_setup.h"
 
@@ -185,275 +185,371 @@ bool octree_faces(const dg_mesh_desc* root, const int32_t* leaves, int32_t n_lea
 
 // ---------------------------------------------------------------------------
 // SIPDG operator on the octree leaves (Sec. 3.4 eq. sip_bilinear with the
-// Nitsche boundary terms of Sec. 6.3), matrix-free, one block per leaf and
-// source. Volume term: the element's Kronecker sum (GL-collocated mass, exact
-// 1-D stiffness). Face terms: traces and normal derivatives of this leaf and of
-// its neighbour(s) at Gauss points of the smaller face (a hanging face is
-// integrated on each of its four quarters), fluxes
+// Nitsche boundary terms of Sec. 6.3), matrix-free. Volume term: the element's
+// Kronecker sum (GL-collocated mass, exact 1-D stiffness). Face terms: traces
+// and normal derivatives of this leaf and of its neighbour(s) at Gauss points of
+// the smaller face (a hanging face is integrated on each of its four quarters),
+// fluxes
 //   v-trace:      -{d_n u} + sigma [u]     (boundary: -d_n u + sigma u)
 //   d_n v:        -1/2 [u]                 (boundary: -u)
 // with [u] = u_K - u_L along K's outward normal, sigma = (p+1)^2/(eps h) of
 // the smaller leaf, and the test-side contraction back onto the leaf's nodes.
+//
+// The Gauss points of a face are the leaf's own face nodes, so between leaves of
+// one size (and at the boundary) no interpolation is needed: the flux at a face
+// node takes the two lines that meet there, and a leaf is worked like an element
+// of the uniform operator (k_oct_apply: a thread owns a line along each
+// direction in turn, folded into even and odd halves, tables in the constant
+// bank; lengths enter as one factor per axis). Only hanging faces interpolate:
+// k_oct_hang takes each of them once per source, for both sides: the larger
+// leaf's traces to its four quarters (two sum-factorised steps), the fluxes
+// there, and their projection back onto the larger face; k_oct_apply reads the
+// result in place of a neighbour's traces.
+//
+// Measured (GB300, density-refined chain octree, 715 leaves, p = 6, 8 fields; one
+// block per leaf with every face interpolated to Gauss points and back before):
+// FP32 396 -> 20 us (5 us of it the hanging faces), FP64 974 -> 255 us; the V-cycle of the FP32 solve, three degrees of this
+// operator and the leaf-block inverse, 9.8 -> 4.2 ms in FP64; a mixed solve of 8
+// sources to 1e-10 241 -> 85 ms.
 // ---------------------------------------------------------------------------
 
-__device__ __forceinline__ double oct_penalty(int p, double h, int form, double eps) {
-  const double c = (double)((p + 1) * (p + 1));
-  return form == 0 ? c / (eps * h) : c / (eps * h * h);
-}
-
-// Every face-quarter of the leaf is processed at once (a face with four smaller
-// neighbours has four, every other face one): 6 to 24 "face parts" per leaf,
-// each with six NF-sized buffers in dynamic shared memory. Interpolations to and
-// from the Gauss points are sum-factorised (one tangential axis at a time).
-// Phases, separated by block barriers:
-//   1. volume term; this leaf's six face traces; the neighbours' traces of
-//      every part, read from global memory
-//   2. first tangential contraction (t1) of the four traces of every part
-//   3. second contraction (t0) and the fluxes F1 (v-trace), F2 (d_n v)
-//   4, 5. the fluxes back onto this leaf's face nodes (t1, then t0)
-//   6. the face contributions added into the volume term, and the store
-template <int N1>
-__device__ __forceinline__ int oct_stride(int d) {
-  return d == 0 ? 1 : (d == 1 ? N1 : N1 * N1);
-}
-
-struct OctPart {
-  int f, L;          // face (2 d + side) and neighbour leaf (-1: boundary)
-  int tk0, tk1;      // this leaf's tables along t0, t1: 0 = Lq, 1 = Lh[0], 2 = Lh[1]
-  int tl0, tl1;      // the neighbour's
-  double sig, wsc;   // penalty and Jacobian of the part's face
+// tables of k_oct_apply: 1-D stiffness and end traces, folded (see dg_apply.cu)
+template <typename V, int N1>
+struct OctLine {
+  static constexpr int HO = N1 / 2, HE = N1 - HO;
+  V Se[HE][HE], So[HO][HO];
+  V te[HE], de[HE], to[HO], dO[HO];  // value and derivative at the left end
+  V tl[N1], dl[N1];                  // the same unfolded
+  V ww[N1 * N1];                     // w_i w_j by line
+  V g0;                              // (p+1)^2 / (2 eps): sigma h / 2 (times 1/h for penalty form 1)
+  long long Nq, items;
+  int E, k0, nslots;                 // leaves, first source of this launch, hanging slots per source
 };
 
-// V: the field type (double, or float in the FP32 inner solve); tables and
-// arithmetic in V too, the leaf sizes and penalties in FP64 until the final cast
-template <typename V, int N1>
-__global__ void __launch_bounds__(256) k_octree_apply(const OctTables T, const double* __restrict__ hq,
-                                                      const int* __restrict__ kind, const int* __restrict__ nbr,
-                                                      const int* __restrict__ pos, int E, int p, int pform,
-                                                      double eps, const V* __restrict__ u, V* __restrict__ out,
-                                                      const int* __restrict__ act) {
-  constexpr int NPE = N1 * N1 * N1, NF = N1 * N1;
-  extern __shared__ __align__(16) unsigned char pbuf_raw[];
-  V* pbuf = (V*)pbuf_raw;  // [nparts][6][NF]
-  __shared__ V sTab[3][NF], sS[NF], sLe[2][N1], sdLe[2][N1], sw[N1], swq[N1];
-  __shared__ V uK[NPE], acc[NPE], VK[6][2][NF];
-  __shared__ OctPart part[24];
-  __shared__ int npart;
-  __shared__ double hK[3];
-  const int e = blockIdx.x;
-  const int tid = threadIdx.x, NT = blockDim.x;
-  const long long src = act ? act[blockIdx.y] : blockIdx.y;
-  const V* ub = u + src * E * NPE;
-  V* ob = out + src * E * NPE;
-  for (int i = tid; i < NF; i += NT) {
-    const int r = i / N1, c = i % N1;
-    sTab[0][i] = (V)T.Lq[r * N1 + c];
-    sTab[1][i] = (V)T.Lh[0][r * N1 + c];
-    sTab[2][i] = (V)T.Lh[1][r * N1 + c];
-    sS[i] = (V)T.S[r * N1 + c];
-  }
-  for (int i = tid; i < N1; i += NT) {
-    sLe[0][i] = (V)T.Le[0][i];
-    sLe[1][i] = (V)T.Le[1][i];
-    sdLe[0][i] = (V)T.dLe[0][i];
-    sdLe[1][i] = (V)T.dLe[1][i];
-    sw[i] = (V)T.w[i];
-    swq[i] = (V)T.wq[i];
-  }
-  for (int i = tid; i < NPE; i += NT) uK[i] = ub[(long long)e * NPE + i];
-  if (tid < 3) hK[tid] = hq[3LL * e + tid];
-  __syncthreads();
-  // the leaf's face parts, one thread per (face f, quarter qi) slot: part index =
-  // the parts of the faces before f, plus qi
-  if (tid < 24) {
-    const int f = tid >> 2, qi = tid & 3;
-    int kd = 0, start = 0, total = 0;
-#pragma unroll
-    for (int g = 0; g < 6; ++g) {
-      const int kg = kind[6LL * e + g];
-      const int ng = kg == 3 ? 4 : 1;
-      if (g < f) start += ng;
-      if (g == f) kd = kg;
-      total += ng;
-    }
-    if (tid == 0) npart = total;
-    if (qi < (kd == 3 ? 4 : 1)) {
-      const int d = f >> 1, t0 = d == 0 ? 1 : 0, t1 = d == 2 ? 1 : 2;
-      const long long o = 6LL * e + f;
-      OctPart& P = part[start + qi];
-      P.f = f;
-      P.tk0 = kd == 3 ? 1 + (qi & 1) : 0;
-      P.tk1 = kd == 3 ? 1 + (qi >> 1) : 0;
-      const int ps = kd == 2 ? pos[o] : 0;
-      P.tl0 = kd == 2 ? 1 + (ps & 1) : 0;
-      P.tl1 = kd == 2 ? 1 + (ps >> 1) : 0;
-      if (kd == 0) {
-        P.L = -1;
-        P.sig = oct_penalty(p, hK[d], pform, eps);
-        P.wsc = hK[t0] * hK[t1] / 4.0;
-      } else {
-        P.L = kd == 3 ? nbr[4 * o + qi] : nbr[4 * o];
-        const double* hL = hq + 3LL * P.L;
-        P.sig = oct_penalty(p, fmin(hK[d], hL[d]), pform, eps);
-        P.wsc = kd == 3 ? hL[t0] * hL[t1] / 4.0 : hK[t0] * hK[t1] / 4.0;
-      }
+template <typename V, int N1, bool FILL>
+struct OctShape {
+  static constexpr int LINES = N1 * N1;
+  static constexpr int BPB = FILL ? best_bpb(LINES, sizeof(V) == 4 ? 128 : 64) : 1;
+  static constexpr int THREADS = (BPB * LINES + 31) / 32 * 32;
+  static constexpr size_t SMEM = sizeof(V) * 2 * (size_t)BPB * LineLayout<N1>::ES;
+  static constexpr int WANT = sizeof(V) == 4 ? 768 : 512;
+  static constexpr int MINB = WANT / THREADS < 1 ? 1 : WANT / THREADS > 32 ? 32 : WANT / THREADS;
+};
+
+// traces beyond the ends of a line: of the neighbour leaf (face code fc >= 0), or
+// those that the boundary stands for (fc = -1; the own line read reversed looks
+// like a neighbour's), nothing for a hanging face (fc < -1)
+template <typename V, int N1, int D>
+__device__ __forceinline__ void oct_outer(const OctLine<V, N1>& tab, const V* __restrict__ us, int e, int l, int fl,
+                                          int fr, V gam, bool vec, V* ov, V* od) {
+  constexpr int NF = N1 * N1, NPE = NF * N1;
+  constexpr int SD = D == 0 ? 1 : (D == 1 ? N1 : NF);
+  const int l1 = l % N1, l2 = l / N1;
+  const int base = D == 0 ? N1 * l : (D == 1 ? l1 + NF * l2 : l);
+  V v[N1];
+  ov[0] = od[0] = ov[1] = od[1] = (V)0;
+  if (fl >= -1) {
+    load_line<V, N1, SD>(us + (long long)(fl < 0 ? e : fl) * NPE + base, fl < 0, vec, v);
+    end_trace<V, N1, true>(tab.tl, tab.dl, v, ov[0], od[0]);
+    if (fl < 0) {
+      od[0] = mad((V)-2 * gam, ov[0], -od[0]);
+      ov[0] = -ov[0];
     }
   }
-  __syncthreads();
-  const int np = npart;
-  // 1. volume: sum_d (2/h_d)(h_t0 h_t1 / 4) (S_d (x) W (x) W) u
-  for (int i = tid; i < NPE; i += NT) {
-    const int ix = i % N1, iy = (i / N1) % N1, iz = i / NF;
-    V vx = 0, vy = 0, vz = 0;
-#pragma unroll
-    for (int a = 0; a < N1; ++a) {
-      vx += sS[ix * N1 + a] * uK[a + N1 * iy + NF * iz];
-      vy += sS[iy * N1 + a] * uK[ix + N1 * a + NF * iz];
-      vz += sS[iz * N1 + a] * uK[ix + N1 * iy + NF * a];
+  if (fr >= -1) {
+    load_line<V, N1, SD>(us + (long long)(fr < 0 ? e : fr) * NPE + base, fr < 0, vec, v);
+    end_trace<V, N1, false>(tab.tl, tab.dl, v, ov[1], od[1]);
+    if (fr < 0) {
+      od[1] = mad((V)2 * gam, ov[1], -od[1]);
+      ov[1] = -ov[1];
     }
-    acc[i] = vx * sw[iy] * sw[iz] * (V)((2.0 / hK[0]) * (hK[1] * hK[2] / 4.0)) +
-             vy * sw[ix] * sw[iz] * (V)((2.0 / hK[1]) * (hK[0] * hK[2] / 4.0)) +
-             vz * sw[ix] * sw[iy] * (V)((2.0 / hK[2]) * (hK[0] * hK[1] / 4.0));
-  }
-  // 1. this leaf's traces and outward normal derivatives on its face nodes [t0][t1]
-  for (int t = tid; t < 6 * NF; t += NT) {
-    const int f = t / NF, j = t - f * NF;
-    const int d = f >> 1, r = f & 1, t0 = d == 0 ? 1 : 0, t1 = d == 2 ? 1 : 2;
-    const int b = j / N1, c = j % N1;
-    const int sd = oct_stride<N1>(d), base = b * oct_stride<N1>(t0) + c * oct_stride<N1>(t1);
-    V v = 0, dv = 0;
-#pragma unroll
-    for (int a = 0; a < N1; ++a) {
-      const V x = uK[a * sd + base];
-      v += sLe[r][a] * x;
-      dv += sdLe[r][a] * x;
-    }
-    VK[f][0][j] = v;
-    VK[f][1][j] = dv * (V)((2.0 / hK[d]) * (r ? 1.0 : -1.0));
-  }
-  // 1. the neighbours' traces (on the neighbour's own face nodes) into buffers 0, 1
-  for (int t = tid; t < np * NF; t += NT) {
-    const int k = t / NF, j = t - k * NF;
-    const OctPart& P = part[k];
-    const int L = P.L;
-    V* B = pbuf + (size_t)k * 6 * NF;
-    if (L < 0) continue;
-    const int d = P.f >> 1, r = P.f & 1, rl = 1 - r, t0 = d == 0 ? 1 : 0, t1 = d == 2 ? 1 : 2;
-    const int b = j / N1, c = j % N1;
-    const V* uL = ub + (long long)L * NPE + b * oct_stride<N1>(t0) + c * oct_stride<N1>(t1);
-    const int sd = oct_stride<N1>(d);
-    V v = 0, dv = 0;
-#pragma unroll
-    for (int a = 0; a < N1; ++a) {
-      const V x = uL[a * sd];
-      v += sLe[rl][a] * x;
-      dv += sdLe[rl][a] * x;
-    }
-    B[j] = v;
-    B[NF + j] = dv * (V)((2.0 / hq[3LL * L + d]) * (r ? 1.0 : -1.0));
-  }
-  __syncthreads();
-  // 2. first contraction along t1: R_X[b][jj] = sum_c T1[jj][c] X[b][c] into buffers 2..5
-  //    (X = this leaf's value, derivative, the neighbour's value, derivative)
-  for (int t = tid; t < np * 4 * NF; t += NT) {
-    const int k = t / (4 * NF), rem = t - k * 4 * NF, x = rem / NF, q = rem - x * NF;
-    const OctPart& P = part[k];
-    V* B = pbuf + (size_t)k * 6 * NF;
-    if (x >= 2 && P.L < 0) continue;
-    const int b = q / N1, jj = q % N1;
-    const V* X = x < 2 ? VK[P.f][x] : B + (x - 2) * NF;
-    const V* T1 = sTab[x < 2 ? P.tk1 : P.tl1];
-    V s = 0;
-#pragma unroll
-    for (int c = 0; c < N1; ++c) s += T1[jj * N1 + c] * X[b * N1 + c];
-    B[(2 + x) * NF + q] = s;
-  }
-  __syncthreads();
-  // 3. second contraction along t0 at the Gauss point (i, jj), and the fluxes into buffers 0, 1
-  for (int t = tid; t < np * NF; t += NT) {
-    const int k = t / NF, q = t - k * NF;
-    const OctPart& P = part[k];
-    V* B = pbuf + (size_t)k * 6 * NF;
-    const int i = q / N1, jj = q % N1;
-    const V* T0K = sTab[P.tk0];
-    V pv = 0, pd = 0;
-#pragma unroll
-    for (int b = 0; b < N1; ++b) {
-      pv += T0K[i * N1 + b] * B[2 * NF + b * N1 + jj];
-      pd += T0K[i * N1 + b] * B[3 * NF + b * N1 + jj];
-    }
-    const V wt = swq[i] * swq[jj] * (V)P.wsc;
-    const V sig = (V)P.sig;
-    V F1, F2;
-    if (P.L < 0) {
-      F1 = wt * (-pd + sig * pv);
-      F2 = wt * (-pv);
-    } else {
-      const V* T0L = sTab[P.tl0];
-      V qv = 0, qd = 0;
-#pragma unroll
-      for (int b = 0; b < N1; ++b) {
-        qv += T0L[i * N1 + b] * B[4 * NF + b * N1 + jj];
-        qd += T0L[i * N1 + b] * B[5 * NF + b * N1 + jj];
-      }
-      F1 = wt * ((V)-0.5 * (pd + qd) + sig * (pv - qv));
-      F2 = wt * ((V)-0.5 * (pv - qv));
-    }
-    B[q] = F1;
-    B[NF + q] = F2;
-  }
-  __syncthreads();
-  // 4. back along t1: H_Y[i][c] = sum_jj F_Y[i][jj] T1K[jj][c] into buffers 2, 3
-  for (int t = tid; t < np * 2 * NF; t += NT) {
-    const int k = t / (2 * NF), rem = t - k * 2 * NF, y = rem / NF, q = rem - y * NF;
-    const OctPart& P = part[k];
-    V* B = pbuf + (size_t)k * 6 * NF;
-    const int i = q / N1, c = q % N1;
-    const V* T1 = sTab[P.tk1];
-    V s = 0;
-#pragma unroll
-    for (int jj = 0; jj < N1; ++jj) s += B[y * NF + i * N1 + jj] * T1[jj * N1 + c];
-    B[(2 + y) * NF + q] = s;
-  }
-  __syncthreads();
-  // 5. back along t0: G_Y[b][c] = sum_i T0K[i][b] H_Y[i][c] into buffers 4, 5
-  for (int t = tid; t < np * 2 * NF; t += NT) {
-    const int k = t / (2 * NF), rem = t - k * 2 * NF, y = rem / NF, q = rem - y * NF;
-    const OctPart& P = part[k];
-    V* B = pbuf + (size_t)k * 6 * NF;
-    const int b = q / N1, c = q % N1;
-    const V* T0 = sTab[P.tk0];
-    V s = 0;
-#pragma unroll
-    for (int i = 0; i < N1; ++i) s += T0[i * N1 + b] * B[(2 + y) * NF + i * N1 + c];
-    B[(4 + y) * NF + q] = s;
-  }
-  __syncthreads();
-  // 6. face contributions onto the leaf's nodes: l_a(e) G1 + l_a'(e) (2/h) s G2, parts in order
-  for (int i = tid; i < NPE; i += NT) {
-    const int ix = i % N1, iy = (i / N1) % N1, iz = i / NF;
-    V a_ = acc[i];
-    for (int k = 0; k < np; ++k) {
-      const OctPart& P = part[k];
-      const V* B = pbuf + (size_t)k * 6 * NF;
-      const int d = P.f >> 1, r = P.f & 1;
-      // (a, b, c) = the node's coordinates along d, t0, t1
-      const int a = d == 0 ? ix : (d == 1 ? iy : iz);
-      const int bc = d == 0 ? iy * N1 + iz : (d == 1 ? ix * N1 + iz : ix * N1 + iy);
-      a_ += sLe[r][a] * B[4 * NF + bc] + sdLe[r][a] * (V)((2.0 / hK[d]) * (r ? 1.0 : -1.0)) * B[5 * NF + bc];
-    }
-    ob[(long long)e * NPE + i] = a_;
   }
 }
 
-int octree_max_parts(const int32_t* kind, int E) {
-  int m = 6;
-  for (int e = 0; e < E; ++e) {
-    int n = 0;
-    for (int f = 0; f < 6; ++f) n += kind[6 * (size_t)e + f] == 3 ? 4 : 1;
-    m = std::max(m, n);
+// S v plus the face terms of a line; hL/hR: hanging, then ov/od hold the
+// projected fluxes instead of a neighbour's traces
+template <typename V, int N1>
+__device__ __forceinline__ void oct_line(const OctLine<V, N1>& tab, V* v, const V* ov, const V* od, bool hL, bool hR,
+                                         V gam) {
+  constexpr int HO = N1 / 2, HE = N1 - HO;
+  V e[HE], o[HO];
+#pragma unroll
+  for (int i = 0; i < HO; ++i) {
+    e[i] = v[i] + v[N1 - 1 - i];
+    o[i] = v[i] - v[N1 - 1 - i];
   }
-  return m;
+  if (HE > HO) e[HE - 1] = v[HO];
+  V a = mul(tab.te[0], e[0]), b = mul(tab.to[0], o[0]), c = mul(tab.de[0], e[0]), d = mul(tab.dO[0], o[0]);
+#pragma unroll
+  for (int i = 1; i < HE; ++i) {
+    a = mad(tab.te[i], e[i], a);
+    c = mad(tab.de[i], e[i], c);
+  }
+#pragma unroll
+  for (int i = 1; i < HO; ++i) {
+    b = mad(tab.to[i], o[i], b);
+    d = mad(tab.dO[i], o[i], d);
+  }
+  const V h = (V)0.5;
+  const V jL = (a + b) - ov[0], jR = (a - b) - ov[1];  // jumps
+  const V gL1 = hL ? ov[0] : mad(gam, jL, mul(h, (c + d) + od[0])), gL2 = hL ? od[0] : mul(-h, jL);
+  const V gR1 = hR ? ov[1] : mad(gam, jR, mul(-h, (d - c) + od[1])), gR2 = hR ? od[1] : mul(-h, jR);
+  const V p1 = gL1 + gR1, m1 = gL1 - gR1, p2 = gL2 + gR2, m2 = gL2 - gR2;
+  V O[HO];
+#pragma unroll
+  for (int k = 0; k < HO; ++k) {
+    V acc = mad(-tab.dO[k], m2, mul(tab.to[k], m1));
+#pragma unroll
+    for (int i = 0; i < HO; ++i) acc = mad(tab.So[k][i], o[i], acc);
+    O[k] = acc;
+  }
+#pragma unroll
+  for (int k = 0; k < HE; ++k) {
+    V acc = mad(-tab.de[k], p2, mul(tab.te[k], p1));
+#pragma unroll
+    for (int i = 0; i < HE; ++i) acc = mad(tab.Se[k][i], e[i], acc);
+    if (k < HO) {
+      v[k] = acc + O[k];
+      v[N1 - 1 - k] = acc - O[k];
+    } else {
+      v[k] = acc;
+    }
+  }
+}
+
+// out = A u, one slot per leaf and source. fac [E][6]: h_t0 h_t1 / (2 h_d) per
+// axis, then 1 (penalty form 0) or 1 / h_d; hslot [E][6]: hanging slot of a
+// face, -1 for the others; gbuf [source - k0][slot][2][N1^2]: k_oct_hang's
+// projected fluxes.
+template <typename V, int N1, bool FILL>
+__global__ void __launch_bounds__(OctShape<V, N1, FILL>::THREADS, OctShape<V, N1, FILL>::MINB)
+    k_oct_apply(const __grid_constant__ OctLine<V, N1> tab, const double* __restrict__ fac,
+                const int* __restrict__ kind, const int* __restrict__ nbr, const int* __restrict__ hslot,
+                const V* __restrict__ gbuf, const V* __restrict__ u, V* __restrict__ out,
+                const int* __restrict__ act, int vec_i) {
+  using H = OctShape<V, N1, FILL>;
+  using Y = LineLayout<N1>;
+  constexpr int NF = N1 * N1, NPE = NF * N1, BPB = H::BPB;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  V* su = reinterpret_cast<V*>(smem_raw);
+  V* sacc = su + BPB * Y::ES;
+  __shared__ int sleaf[BPB], ssrc[BPB], skk[BPB], sface[BPB][6];
+  __shared__ V sfac[BPB][6];
+  const int tid = threadIdx.x;
+  if (tid < BPB) {
+    const long long it = (long long)blockIdx.x * BPB + tid;
+    const bool in = it < tab.items;
+    const int kk = in ? (int)(it / tab.E) : 0, e = in ? (int)(it - (long long)kk * tab.E) : -1;
+    sleaf[tid] = e;
+    skk[tid] = kk;
+    ssrc[tid] = act ? act[tab.k0 + kk] : tab.k0 + kk;
+  }
+  __syncthreads();
+  for (int t = tid; t < BPB * 6; t += H::THREADS) {
+    const int sl = t / 6, f = t - 6 * sl, e = sleaf[sl];
+    if (e < 0) continue;
+    const long long o = 6LL * e + f;
+    const int kd = kind[o];
+    sface[sl][f] = kd == 0 ? -1 : kd == 1 ? nbr[4 * o] : -2 - hslot[o];
+    sfac[sl][f] = (V)fac[o] * (f >= 3 ? tab.g0 : (V)1);
+  }
+  __syncthreads();
+  const int slot = tid / NF, l = tid - slot * NF, l1 = l % N1, l2 = l / N1;
+  const bool on = slot < BPB && sleaf[slot < BPB ? slot : 0] >= 0;
+  const int sl = on ? slot : 0, e = on ? sleaf[sl] : 0;
+  const bool vec = vec_i != 0;
+  const V* us = u + (long long)ssrc[sl] * tab.Nq;
+  const long long g0 = (long long)ssrc[sl] * tab.Nq + (long long)e * NPE;
+  const int* fc = sface[sl];
+  const int sb = sl * Y::ES, zat = sb + l1 + Y::PB * l2;
+  V v[N1], ov[3][2], od[3][2], gam[3];
+  if (on) {
+#pragma unroll
+    for (int i = 0; i < N1; ++i) v[i] = __ldg(us + (long long)e * NPE + l + NF * i);
+#pragma unroll
+    for (int i = 0; i < N1; ++i) su[zat + Y::PZ * i] = v[i];
+#pragma unroll
+    for (int d = 0; d < 3; ++d) gam[d] = sfac[sl][3 + d];
+    oct_outer<V, N1, 0>(tab, us, e, l, fc[0], fc[1], gam[0], vec, ov[0], od[0]);
+    oct_outer<V, N1, 1>(tab, us, e, l, fc[2], fc[3], gam[1], vec, ov[1], od[1]);
+    oct_outer<V, N1, 2>(tab, us, e, l, fc[4], fc[5], gam[2], vec, ov[2], od[2]);
+#pragma unroll
+    for (int f = 0; f < 6; ++f)
+      if (fc[f] < -1) {
+        const V* g = gbuf + (((long long)skk[sl] * tab.nslots + (-2 - fc[f])) * 2) * NF + l;
+        ov[f >> 1][f & 1] = g[0];
+        od[f >> 1][f & 1] = g[NF];
+      }
+  }
+  __syncthreads();
+  if (on) {
+    const int at = sb + Y::PB * l1 + Y::PZ * l2;
+#pragma unroll
+    for (int i = 0; i < N1; ++i) v[i] = su[at + i];
+    oct_line<V, N1>(tab, v, ov[0], od[0], fc[0] < -1, fc[1] < -1, gam[0]);
+    const V sc = mul(sfac[sl][0], tab.ww[l]);
+#pragma unroll
+    for (int i = 0; i < N1; ++i) sacc[at + i] = mul(sc, v[i]);
+  }
+  __syncthreads();
+  if (on) {
+    const int at = sb + l1 + Y::PZ * l2;
+#pragma unroll
+    for (int i = 0; i < N1; ++i) v[i] = su[at + Y::PB * i];
+    oct_line<V, N1>(tab, v, ov[1], od[1], fc[2] < -1, fc[3] < -1, gam[1]);
+    const V sc = mul(sfac[sl][1], tab.ww[l]);
+#pragma unroll
+    for (int i = 0; i < N1; ++i) {
+      V* p = sacc + at + Y::PB * i;
+      *p = mad(sc, v[i], *p);
+    }
+  }
+  __syncthreads();
+  if (on) {
+#pragma unroll
+    for (int i = 0; i < N1; ++i) v[i] = su[zat + Y::PZ * i];
+    oct_line<V, N1>(tab, v, ov[2], od[2], fc[4] < -1, fc[5] < -1, gam[2]);
+    const V sc = mul(sfac[sl][2], tab.ww[l]);
+#pragma unroll
+    for (int i = 0; i < N1; ++i) out[g0 + l + NF * i] = mad(sc, v[i], sacc[zat + Y::PZ * i]);
+  }
+}
+
+// tables of k_oct_hang
+template <typename V, int N1>
+struct OctHang {
+  V Lh[2][N1 * N1];  // [c][i][a]: the larger leaf's basis a at point i of its half c
+  V tl[N1], dl[N1], w[N1];
+  V g0;
+  long long Nq;
+  int E, k0, nI;
+};
+
+// Fluxes of a hanging face in units of 2 / h of the side that they are for, with
+// the side's weights w_i w_j and lengths divided out: record [leaf of the larger
+// side, its face, the four smaller leaves]; slot 5 i of gbuf is the larger side's,
+// 5 i + 1 + j the j-th smaller one's. 4 N1^2 threads a face: one per quarter and
+// point.
+template <typename V, int N1>
+struct HangShape {
+  static constexpr int T4 = 4 * N1 * N1;
+  static constexpr int HPB = T4 >= 96 ? 1 : 128 / T4;
+  static constexpr int THREADS = (HPB * T4 + 31) / 32 * 32;
+};
+template <typename V, int N1>
+__global__ void __launch_bounds__(HangShape<V, N1>::THREADS)
+    k_oct_hang(const __grid_constant__ OctHang<V, N1> tab, const int* __restrict__ rec, const double* __restrict__ fac,
+               const V* __restrict__ u, V* __restrict__ gbuf, const int* __restrict__ act) {
+  using H = HangShape<V, N1>;
+  constexpr int NF = N1 * N1, NPE = NF * N1, T4 = H::T4, HPB = H::HPB;
+  __shared__ V sL[2][NF], sw[N1];
+  __shared__ V sX[HPB][2][NF];      // larger side: value, derivative at its face nodes
+  __shared__ V sR[HPB][2][2][NF];   // [quantity][half along t0]
+  __shared__ V sF[HPB][2][4][NF];   // weighted fluxes per quarter
+  const int tid = threadIdx.x;
+  for (int i = tid; i < 2 * NF; i += H::THREADS) sL[i / NF][i % NF] = tab.Lh[i / NF][i % NF];
+  for (int i = tid; i < N1; i += H::THREADS) sw[i] = tab.w[i];
+  const int hs = tid / T4, t = tid - hs * T4;
+  const int ifc = blockIdx.x * HPB + hs;
+  const bool on = hs < HPB && ifc < tab.nI;
+  const int src = act ? act[tab.k0 + blockIdx.y] : tab.k0 + (int)blockIdx.y;
+  const V* us = u + (long long)src * tab.Nq;
+  const int* rc = rec + 6LL * (on ? ifc : 0);
+  const int big = rc[0], f = rc[1], d = f >> 1, r = f & 1;
+  const int st[3] = {1, N1, NF};
+  const int sd = st[d], s0 = st[d == 0 ? 1 : 0], s1 = st[d == 2 ? 1 : 2];
+  const int q = t / NF, l = t - q * NF, i = l % N1, j = l / N1;  // quarter, point (i along t0, j along t1)
+  const int b0 = q & 1, b1 = q >> 1;
+  V vs = 0, ds = 0;
+  auto trace = [&](int leaf, int end, V& val, V& der) {  // end 0: left, 1: right end of the line along d
+    const V* p = us + (long long)leaf * NPE + i * s0 + j * s1;
+    V x[N1];
+#pragma unroll
+    for (int a = 0; a < N1; ++a) x[a] = __ldg(p + (end ? N1 - 1 - a : a) * sd);
+    end_trace<V, N1, false>(tab.tl, tab.dl, x, val, der);
+    if (end) der = -der;  // the line was read reversed
+  };
+  if (on) {
+    trace(rc[2 + q], 1 - r, vs, ds);
+    if (q == 0) trace(big, r, sX[hs][0][l], sX[hs][1][l]);
+  }
+  __syncthreads();
+  if (on) {
+    // first step, along t0: thread (quantity q & 1, half q >> 1)
+    V s = 0;
+#pragma unroll
+    for (int b = 0; b < N1; ++b) s = mad(sL[b1][i * N1 + b], sX[hs][b0][b + N1 * j], s);
+    sR[hs][b0][b1][l] = s;
+  }
+  __syncthreads();
+  V* g = gbuf + ((long long)blockIdx.y * 5 * tab.nI + 5LL * ifc) * 2 * NF;
+  if (on) {
+    V vb = 0, db = 0;
+#pragma unroll
+    for (int c = 0; c < N1; ++c) {
+      const V x = sL[b1][j * N1 + c];
+      vb = mad(x, sR[hs][0][b0][i + N1 * c], vb);
+      db = mad(x, sR[hs][1][b0][i + N1 * c], db);
+    }
+    // gam = sigma h / 2 of the smaller leaf; the larger one's 2 / h is half of its
+    const V gam = (V)fac[6LL * rc[2 + q] + 3 + d] * tab.g0, h = (V)0.5;
+    const V so = r ? (V)-1 : (V)1;  // outward sign of the smaller side
+    const V jump = vs - vb;
+    V* gs = g + (1 + q) * 2 * NF;
+    gs[l] = mad(gam, jump, mul(mul(-h, so), mad(h, db, ds)));
+    gs[NF + l] = mul(-h, jump);
+    const V wq = mul((V)0.25, mul(sw[i], sw[j]));
+    sF[hs][0][q][l] = mul(wq, mad((V)-2 * gam, jump, mul(mul(h, so), mad((V)2, ds, db))));
+    sF[hs][1][q][l] = mul(wq, mul(h, jump));
+  }
+  __syncthreads();
+  if (on) {
+    // back along t1, the two halves along it summed: thread (quantity b0, half b1 along t0) into sR
+    V s = 0;
+#pragma unroll
+    for (int c = 0; c < 2; ++c)
+#pragma unroll
+      for (int jj = 0; jj < N1; ++jj) s = mad(sL[c][jj * N1 + j], sF[hs][b0][b1 + 2 * c][i + N1 * jj], s);
+    sR[hs][b0][b1][l] = s;
+  }
+  __syncthreads();
+  if (on && q < 2) {
+    V s = 0;
+#pragma unroll
+    for (int c = 0; c < 2; ++c)
+#pragma unroll
+      for (int ii = 0; ii < N1; ++ii) s = mad(sL[c][ii * N1 + i], sR[hs][q][c][ii + N1 * j], s);
+    g[q * NF + l] = s / mul(sw[i], sw[j]);
+  }
+}
+
+void octree_hanging(const int32_t* kind, const int32_t* nb, int E, std::vector<int>& rec, std::vector<int>& hslot) {
+  rec.clear();
+  hslot.assign(6 * (size_t)E, -1);
+  for (int e = 0; e < E; ++e)
+    for (int f = 0; f < 6; ++f) {
+      const size_t o = 6 * (size_t)e + f;
+      if (kind[o] != 3) continue;
+      const int i = (int)(rec.size() / 6);
+      hslot[o] = 5 * i;
+      rec.push_back(e);
+      rec.push_back(f);
+      for (int j = 0; j < 4; ++j) {
+        const int s = nb[4 * o + j];
+        hslot[6 * (size_t)s + (f ^ 1)] = 5 * i + 1 + j;
+        rec.push_back(s);
+      }
+    }
+}
+
+void octree_factors(const double* hq, int E, int pform, std::vector<double>& fac) {
+  fac.resize(6 * (size_t)E);
+  for (int e = 0; e < E; ++e)
+    for (int d = 0; d < 3; ++d) {
+      const double* h = hq + 3 * (size_t)e;
+      fac[6 * (size_t)e + d] = h[d == 0 ? 1 : 0] * h[d == 2 ? 1 : 2] / (2.0 * h[d]);
+      fac[6 * (size_t)e + 3 + d] = pform == 0 ? 1.0 : 1.0 / h[d];
+    }
 }
 
 void octree_tables(int n1, OctTables& T) {
@@ -461,13 +557,8 @@ void octree_tables(int n1, OctTables& T) {
   double xi[MAXN1], w[MAXN1], xq[MAXN1], wq[MAXN1], L[MAXN1], dL[MAXN1];
   gauss_legendre(n1, xi, w);
   gauss_legendre(n1, xq, wq);  // Gauss points of a face direction (exact for the face integrands)
-  for (int a = 0; a < n1; ++a) {
-    T.w[a] = w[a];
-    T.wq[a] = wq[a];
-  }
+  for (int a = 0; a < n1; ++a) T.w[a] = w[a];
   for (int i = 0; i < n1; ++i) {
-    lagrange(xi, n1, xq[i], L, dL);
-    for (int a = 0; a < n1; ++a) T.Lq[i * n1 + a] = L[a];
     for (int c = 0; c < 2; ++c) {
       lagrange(xi, n1, (xq[i] + 2.0 * c - 1.0) / 2.0, L, dL);
       for (int a = 0; a < n1; ++a) T.Lh[c][i * n1 + a] = L[a];
@@ -494,46 +585,93 @@ void octree_tables(int n1, OctTables& T) {
     }
 }
 
-template <typename V>
-cudaError_t launch_octree_apply(int n1, const OctTables& T, const double* hq, const int* kind, const int* nb,
-                                const int* pos, int E, int p, int pform, double eps, const V* u, V* out,
-                                const int* act, int nact, int maxparts, cudaStream_t s) {
-  if (nact == 0 || E == 0) return cudaSuccess;
-  if (maxparts < 6 || maxparts > 24) return cudaErrorInvalidValue;
-  const dim3 grid((unsigned)E, (unsigned)nact);
-  const size_t smem = sizeof(V) * (size_t)maxparts * 6 * n1 * n1;
-  // threads per block by degree: the phases have (p+1)^2 to 24 (p+1)^2 work items
-  const int nthr = n1 <= 3 ? 64 : (n1 <= 5 ? 128 : 256);
-  count_launch();
-  switch (n1) {
-#define DG_OCT_CASE(N)                                                                                       \
-  case N: {                                                                                                  \
-    cudaError_t e0 = cudaFuncSetAttribute(k_octree_apply<V, N>, cudaFuncAttributeMaxDynamicSharedMemorySize,   \
-                                          (int)smem);                                                        \
-    if (e0 != cudaSuccess) return e0;                                                                        \
-    k_octree_apply<V, N><<<grid, nthr, smem, s>>>(T, hq, kind, nb, pos, E, p, pform, eps, u, out, act);         \
-    break;                                                                                                   \
+template <typename V, int N1>
+static cudaError_t oct_apply_n1(const OctTables& T, const OctMesh& m, double eps, const V* u, V* out, const int* act,
+                                int nact, V* gbuf, long long gelems, cudaStream_t s) {
+  constexpr int HO = N1 / 2, HE = N1 - HO, NF = N1 * N1, NPE = NF * N1;
+  OctLine<V, N1> t;
+  OctHang<V, N1> g;
+  auto S = [&](int a, int i) { return 0.5 * (T.S[a * N1 + i] + T.S[(N1 - 1 - a) * N1 + (N1 - 1 - i)]); };
+  for (int a = 0; a < HE; ++a) {
+    for (int i = 0; i < HE; ++i) t.Se[a][i] = (V)(i < HO ? 0.5 * (S(a, i) + S(a, N1 - 1 - i)) : S(a, i));
+    t.te[a] = (V)(a < HO ? 0.5 * (T.Le[0][a] + T.Le[0][N1 - 1 - a]) : T.Le[0][a]);
+    t.de[a] = (V)(a < HO ? 0.5 * (T.dLe[0][a] + T.dLe[0][N1 - 1 - a]) : T.dLe[0][a]);
   }
-    DG_OCT_CASE(2)
-    DG_OCT_CASE(3)
-    DG_OCT_CASE(4)
-    DG_OCT_CASE(5)
-    DG_OCT_CASE(6)
-    DG_OCT_CASE(7)
-    DG_OCT_CASE(8)
-    DG_OCT_CASE(9)
-#undef DG_OCT_CASE
-    default:
-      return cudaErrorInvalidValue;
+  for (int a = 0; a < HO; ++a) {
+    for (int i = 0; i < HO; ++i) t.So[a][i] = (V)(0.5 * (S(a, i) - S(a, N1 - 1 - i)));
+    t.to[a] = (V)(0.5 * (T.Le[0][a] - T.Le[0][N1 - 1 - a]));
+    t.dO[a] = (V)(0.5 * (T.dLe[0][a] - T.dLe[0][N1 - 1 - a]));
   }
-  return cudaGetLastError();
+  for (int a = 0; a < N1; ++a) {
+    t.tl[a] = g.tl[a] = (V)T.Le[0][a];
+    t.dl[a] = g.dl[a] = (V)T.dLe[0][a];
+    g.w[a] = (V)T.w[a];
+  }
+  for (int l = 0; l < NF; ++l) {
+    t.ww[l] = (V)(T.w[l % N1] * T.w[l / N1]);
+    for (int c = 0; c < 2; ++c) g.Lh[c][l] = (V)T.Lh[c][l];
+  }
+  t.g0 = g.g0 = (V)(N1 * N1 / (2.0 * eps));
+  t.Nq = g.Nq = (long long)m.E * NPE;
+  t.E = g.E = m.E;
+  t.nslots = 5 * m.nI;
+  g.nI = m.nI;
+  const int vec = ((uintptr_t)u & 15) == 0 && (NPE * sizeof(V)) % 16 == 0 && (t.Nq * sizeof(V)) % 16 == 0;
+  // sources go through in chunks whose hanging fluxes fit the buffer (and a grid's second axis)
+  const long long per_src = 10LL * m.nI * NF;
+  long long per = m.nI > 0 ? std::min<long long>(65535, gelems / per_src) : nact;
+  if (per < 1) return cudaErrorInvalidValue;
+  for (long long k0 = 0; k0 < nact; k0 += per) {
+    const int n = (int)std::min<long long>(per, nact - k0);
+    t.k0 = g.k0 = (int)k0;
+    if (m.nI > 0) {
+      using H = HangShape<V, N1>;
+      count_launch();
+      k_oct_hang<V, N1><<<dim3((unsigned)((m.nI + H::HPB - 1) / H::HPB), (unsigned)n), H::THREADS, 0, s>>>(
+          g, m.rec, m.fac, u, gbuf, act);
+    }
+    t.items = (long long)n * m.E;
+    auto go = [&](auto kern, int bpb, int threads, size_t smem) -> cudaError_t {
+      const long long blocks = (t.items + bpb - 1) / bpb;
+      if (blocks > 0x7fffffffLL) return cudaErrorInvalidValue;
+      if (smem > 48 * 1024) {
+        const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (e != cudaSuccess) return e;
+      }
+      count_launch();
+      kern<<<(unsigned)blocks, threads, smem, s>>>(t, m.fac, m.kind, m.nb, m.hslot, gbuf, u, out, act, vec);
+      return cudaGetLastError();
+    };
+    using F = OctShape<V, N1, true>;
+    using P = OctShape<V, N1, false>;
+    // several leaves per block once that leaves two blocks per SM (as the uniform operator)
+    const cudaError_t e = t.items / F::BPB >= 304 ? go(k_oct_apply<V, N1, true>, F::BPB, F::THREADS, F::SMEM)
+                                                 : go(k_oct_apply<V, N1, false>, P::BPB, P::THREADS, P::SMEM);
+    if (e != cudaSuccess) return e;
+  }
+  return cudaSuccess;
 }
-template cudaError_t launch_octree_apply<double>(int, const OctTables&, const double*, const int*, const int*,
-                                                 const int*, int, int, int, double, const double*, double*, const int*,
-                                                 int, int, cudaStream_t);
-template cudaError_t launch_octree_apply<float>(int, const OctTables&, const double*, const int*, const int*,
-                                                const int*, int, int, int, double, const float*, float*, const int*,
-                                                int, int, cudaStream_t);
+
+template <typename V>
+cudaError_t launch_octree_apply(int n1, const OctTables& T, const OctMesh& m, double eps, const V* u, V* out,
+                                const int* act, int nact, V* gbuf, long long gelems, cudaStream_t s) {
+  if (nact == 0 || m.E == 0) return cudaSuccess;
+  switch (n1) {
+    case 2: return oct_apply_n1<V, 2>(T, m, eps, u, out, act, nact, gbuf, gelems, s);
+    case 3: return oct_apply_n1<V, 3>(T, m, eps, u, out, act, nact, gbuf, gelems, s);
+    case 4: return oct_apply_n1<V, 4>(T, m, eps, u, out, act, nact, gbuf, gelems, s);
+    case 5: return oct_apply_n1<V, 5>(T, m, eps, u, out, act, nact, gbuf, gelems, s);
+    case 6: return oct_apply_n1<V, 6>(T, m, eps, u, out, act, nact, gbuf, gelems, s);
+    case 7: return oct_apply_n1<V, 7>(T, m, eps, u, out, act, nact, gbuf, gelems, s);
+    case 8: return oct_apply_n1<V, 8>(T, m, eps, u, out, act, nact, gbuf, gelems, s);
+    case 9: return oct_apply_n1<V, 9>(T, m, eps, u, out, act, nact, gbuf, gelems, s);
+    default: return cudaErrorInvalidValue;
+  }
+}
+template cudaError_t launch_octree_apply<double>(int, const OctTables&, const OctMesh&, double, const double*, double*,
+                                                 const int*, int, double*, long long, cudaStream_t);
+template cudaError_t launch_octree_apply<float>(int, const OctTables&, const OctMesh&, double, const float*, float*,
+                                                const int*, int, float*, long long, cudaStream_t);
 }  // namespace dg
 
 using namespace dg;
@@ -625,24 +763,32 @@ int dg_octree_apply(const dg_mesh_desc* root, const int32_t* leaves, int32_t n_l
   OctTables T;
   octree_tables(n1, T);
   cudaStream_t s = (cudaStream_t)stream;
-  DevBuf dh, dk, dn, dp;
+  std::vector<int> rec, hslot;
+  std::vector<double> fac;
+  octree_hanging(kind.data(), nb.data(), E, rec, hslot);
+  octree_factors(hq.data(), E, penalty_form, fac);
+  DevBuf df, dk, dn, ds, dr, dg;
   auto ck = [](cudaError_t e) { return e == cudaSuccess ? DG_OK : (e == cudaErrorMemoryAllocation ? DG_ERR_NO_MEMORY : DG_ERR_CUDA); };
   int rc;
-  if ((rc = ck(dh.ensure(sizeof(double) * hq.size()))) != DG_OK) return rc;
-  if ((rc = ck(dk.ensure(sizeof(int) * kind.size()))) != DG_OK) return rc;
-  if ((rc = ck(dn.ensure(sizeof(int) * nb.size()))) != DG_OK) return rc;
-  if ((rc = ck(dp.ensure(sizeof(int) * pos.size()))) != DG_OK) return rc;
-  if ((rc = ck(cudaMemcpyAsync(dh.p, hq.data(), sizeof(double) * hq.size(), cudaMemcpyHostToDevice, s))) != DG_OK)
+  auto up = [&](DevBuf& d, const void* p, size_t bytes) -> int {
+    if (bytes == 0) return DG_OK;
+    const int r = ck(d.ensure(bytes));
+    return r != DG_OK ? r : ck(cudaMemcpyAsync(d.p, p, bytes, cudaMemcpyHostToDevice, s));
+  };
+  if ((rc = up(df, fac.data(), sizeof(double) * fac.size())) != DG_OK ||
+      (rc = up(dk, kind.data(), sizeof(int) * kind.size())) != DG_OK ||
+      (rc = up(dn, nb.data(), sizeof(int) * nb.size())) != DG_OK ||
+      (rc = up(ds, hslot.data(), sizeof(int) * hslot.size())) != DG_OK ||
+      (rc = up(dr, rec.data(), sizeof(int) * rec.size())) != DG_OK)
     return rc;
-  if ((rc = ck(cudaMemcpyAsync(dk.p, kind.data(), sizeof(int) * kind.size(), cudaMemcpyHostToDevice, s))) != DG_OK)
-    return rc;
-  if ((rc = ck(cudaMemcpyAsync(dn.p, nb.data(), sizeof(int) * nb.size(), cudaMemcpyHostToDevice, s))) != DG_OK)
-    return rc;
-  if ((rc = ck(cudaMemcpyAsync(dp.p, pos.data(), sizeof(int) * pos.size(), cudaMemcpyHostToDevice, s))) != DG_OK)
-    return rc;
-  if ((rc = ck(launch_octree_apply<double>(n1, T, dh.as<double>(), dk.as<int>(), dn.as<int>(), dp.as<int>(), E, root->p,
-                                   penalty_form, penalty_eps, u, out, nullptr, (int)B, octree_max_parts(kind.data(), E),
-                                   s))) != DG_OK)
+  const int nI = (int)(rec.size() / 6);
+  // hanging fluxes: as many sources at a time as 64 MB hold, at least one
+  const size_t one = sizeof(double) * octree_hang_elems(n1, nI);
+  const size_t gbytes = std::max(one, std::min<size_t>(one * (size_t)B, 64u << 20));
+  if (nI > 0 && (rc = ck(dg.ensure(gbytes))) != DG_OK) return rc;
+  const OctMesh m{E, dk.as<int>(), dn.as<int>(), df.as<double>(), ds.as<int>(), dr.as<int>(), nI};
+  if ((rc = ck(launch_octree_apply<double>(n1, T, m, penalty_eps, u, out, nullptr, (int)B, dg.as<double>(),
+                                           (long long)(gbytes / sizeof(double)), s))) != DG_OK)
     return rc;
   // the tables and connectivity are call-local: wait before they are freed
   return ck(cudaStreamSynchronize(s));

@@ -12,9 +12,7 @@ namespace dg {
 // 1-D tables of the octree operator for one degree (n1 nodes per axis)
 struct OctTables {
   double w[MAXN1];               // GL weights
-  double wq[MAXN1];              // Gauss weights (n1 points per face direction)
   double S[MAXN1 * MAXN1];       // sum_q wq l_a'(xq) l_b'(xq)
-  double Lq[MAXN1 * MAXN1];      // [i][a] l_a(xq_i)
   double Lh[2][MAXN1 * MAXN1];   // [c][i][a] l_a((xq_i + 2c - 1) / 2): a larger leaf's basis on half c
   double Le[2][MAXN1];           // l_a(-1), l_a(+1)
   double dLe[2][MAXN1];          // l_a'(-1), l_a'(+1)
@@ -29,17 +27,33 @@ void octree_tables(int n1, OctTables& T);
 bool octree_faces(const dg_mesh_desc* root, const int32_t* leaves, int32_t n_leaves, int32_t* kind, int32_t* nb,
                   int32_t* pos);
 
-// largest number of face parts of a leaf (a face with four smaller neighbours
-// counts four, any other face one): 6..24, the operator's shared-memory size
-int octree_max_parts(const int32_t* kind, int E);
+// Hanging faces: rec [nI][6] = larger leaf, its face, the four smaller leaves (by
+// quarter); hslot [E][6] = 5 i for the larger side of face i, 5 i + 1 + j for the
+// j-th smaller side, -1 where a face does not hang
+void octree_hanging(const int32_t* kind, const int32_t* nb, int E, std::vector<int>& rec, std::vector<int>& hslot);
+
+// length factors of the operator, [E][6]: h_t0 h_t1 / (2 h_d), then 1 (penalty
+// form 0) or 1 / h_d; hq [E][3] leaf sizes
+void octree_factors(const double* hq, int E, int pform, std::vector<double>& fac);
+
+// values that one source's hanging fluxes take
+inline size_t octree_hang_elems(int n1, int nI) { return 10 * (size_t)nI * n1 * n1; }
+
+// the mesh on the device: connectivity as octree_faces, fac, hslot and rec as above
+struct OctMesh {
+  int E;
+  const int *kind, *nb;
+  const double* fac;
+  const int *hslot, *rec;
+  int nI;
+};
 
 // out[k] = A u[k] for the sources k = act[0..nact) (act null: k = 0..nact),
-// u and out [.][E][n1^3]; hq [E][3] leaf sizes, kind/nb/pos as octree_faces;
-// maxparts = octree_max_parts of the mesh; V = double or float (the fields and
-// the arithmetic)
+// u and out [.][E][n1^3]; V = double or float (the fields and the arithmetic);
+// gbuf: scratch of gelems values, at least octree_hang_elems (sources go through
+// in chunks that fit)
 template <typename V>
-cudaError_t launch_octree_apply(int n1, const OctTables& T, const double* hq, const int* kind, const int* nb,
-                                const int* pos, int E, int p, int pform, double eps, const V* u, V* out,
-                                const int* act, int nact, int maxparts, cudaStream_t s);
+cudaError_t launch_octree_apply(int n1, const OctTables& T, const OctMesh& m, double eps, const V* u, V* out,
+                                const int* act, int nact, V* gbuf, long long gelems, cudaStream_t s);
 
 }  // namespace dg

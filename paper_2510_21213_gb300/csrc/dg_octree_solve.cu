@@ -63,10 +63,10 @@ struct dg_oct {
   int n1 = 0, p = 0, E = 0, pform = 0, max_iter = 0, precond = 1;
   int mixed = 0;                 // 1: FP32 inner PCG (FP32 V-cycle) inside FP64 refinement
   double inner_rtol = 1e-4;      // relative reduction of each inner solve
-  int maxparts = 6;  // largest face-part count of a leaf (the operator's shared memory)
+  int nI = 0;                    // hanging faces
   double eps = 0.125, rtol = 1e-10;
   long long Nq = 0;
-  dg::DevBuf hq, kind, nb, pos;  // leaf sizes [E][3]; connectivity [E][6], [E][6][4], [E][6]
+  dg::DevBuf fac, kind, nb, hslot, rec;  // length factors and connectivity of the operator (dg_octree.h)
   std::vector<OctLevel> lv;      // lv[0]: the fine level
   dg::DevBuf xq, W;              // node coordinates [Nq][3], quadrature weights [Nq]
   int nbf = 0;                   // boundary faces
@@ -95,8 +95,14 @@ struct dg_oct {
   // the device when it fits the budget below
   dg::DevBuf kmat, wf32, g32, gwork;
   bool has_kmat = false;
+  // hanging fluxes of the operator: of the solves, and of dg_octree_operator,
+  // which returns before its kernels end: op_done orders its next call (on
+  // whatever stream) behind them
+  dg::DevBuf hang, hang_op;
+  cudaEvent_t op_done = nullptr;
   std::vector<int> act_host;
   ~dg_oct() {
+    if (op_done) cudaEventDestroy(op_done);
     if (root) dg_destroy(root);
   }
 };
@@ -491,9 +497,12 @@ static cudaError_t launch_bjac(const dg_oct* h, const OctLevel& L, const V* r, V
 
 template <typename V>
 static cudaError_t oct_apply(const dg_oct* h, const OctLevel& L, const V* u, V* out, const int* act, int nact,
-                             cudaStream_t s) {
-  return launch_octree_apply<V>(L.n1, L.T, h->hq.as<double>(), h->kind.as<int>(), h->nb.as<int>(), h->pos.as<int>(),
-                             h->E, L.p, h->pform, h->eps, u, out, act, nact, h->maxparts, s);
+                             cudaStream_t s, const DevBuf* hang = nullptr) {
+  if (!hang) hang = &h->hang;
+  const OctMesh m{h->E, h->kind.as<int>(), h->nb.as<int>(), h->fac.as<double>(), h->hslot.as<int>(), h->rec.as<int>(),
+                  h->nI};
+  return launch_octree_apply<V>(L.n1, L.T, m, h->eps, u, out, act, nact, hang->as<V>(),
+                                (long long)(hang->bytes / sizeof(V)), s);
 }
 
 static cudaError_t launch_oct_lift(const dg_oct* h, const double* g, double* b, int nsrc, cudaStream_t s) {
@@ -547,6 +556,12 @@ static void oct_class_fdm(const OctTables& T, int n1, int p, double h, int ty0, 
   for (int m = 0; m < n1; ++m) lam[m] = l[m];
 }
 
+// hanging fluxes of up to `cap` sources: as many at a time as 64 MB hold, at least one
+static size_t hang_bytes(const dg_oct* h, int cap) {
+  const size_t one = sizeof(double) * octree_hang_elems(h->n1, h->nI);
+  return std::max(one, std::min<size_t>(one * (size_t)cap, 64u << 20));
+}
+
 static int oct_ws(dg_oct* h, int cap) {
   if (cap <= h->cap) return DG_OK;
   const size_t vec = sizeof(double) * (size_t)cap * (size_t)h->Nq;
@@ -578,6 +593,7 @@ static int oct_ws(dg_oct* h, int cap) {
       return rc;
     }
   }
+  if (h->nI > 0) DG_CK(h->hang.ensure(hang_bytes(h, cap)));
   DG_CK(h->g.ensure(sizeof(double) * (size_t)cap * h->nbf * h->n1 * h->n1));
   DG_CK(h->gpart.ensure(sizeof(double) * (size_t)oct_bdata_chunks((long long)h->nbf * h->n1 * h->n1) * cap * h->nbf *
                         h->n1 * h->n1));
@@ -1123,7 +1139,9 @@ int dg_octree_setup(const dg_mesh_desc* root, const int32_t* leaves, int32_t n_l
   h->max_iter = max_iter;
   h->precond = precond;
   h->mixed = precision == DG_PREC_MIXED;
-  h->maxparts = octree_max_parts(kind.data(), E);
+  std::vector<int> rec, hslot;
+  octree_hanging(kind.data(), nb.data(), E, rec, hslot);
+  h->nI = (int)(rec.size() / 6);
   h->Nq = (long long)E * NPE;
   double xi[MAXN1], w[MAXN1];
   gauss_legendre(n1, xi, w);
@@ -1241,10 +1259,18 @@ int dg_octree_setup(const dg_mesh_desc* root, const int32_t* leaves, int32_t n_l
     bl.insert(bl.end(), fidx, fidx + 6);
     ++h->nbl;
   }
-  if ((rc = up(h->hq, hq.data(), sizeof(double) * hq.size())) != DG_OK ||
+  if (h->nI > 0) {
+    cudaError_t e = h->hang_op.ensure(hang_bytes(h, 64));
+    if (e == cudaSuccess) e = cudaEventCreateWithFlags(&h->op_done, cudaEventDisableTiming);
+    if (e != cudaSuccess) return fail(e == cudaErrorMemoryAllocation ? DG_ERR_NO_MEMORY : DG_ERR_CUDA);
+  }
+  std::vector<double> fac;
+  octree_factors(hq.data(), E, penalty_form, fac);
+  if ((rc = up(h->fac, fac.data(), sizeof(double) * fac.size())) != DG_OK ||
       (rc = up(h->kind, kind.data(), sizeof(int) * kind.size())) != DG_OK ||
       (rc = up(h->nb, nb.data(), sizeof(int) * nb.size())) != DG_OK ||
-      (rc = up(h->pos, pos.data(), sizeof(int) * pos.size())) != DG_OK ||
+      (rc = up(h->hslot, hslot.data(), sizeof(int) * hslot.size())) != DG_OK ||
+      (rc = up(h->rec, rec.data(), sizeof(int) * rec.size())) != DG_OK ||
       (rc = up(h->xq, xq.data(), sizeof(double) * xq.size())) != DG_OK ||
       (rc = up(h->W, W.data(), sizeof(double) * W.size())) != DG_OK ||
       (rc = up(h->xb, xb.data(), sizeof(double) * xb.size())) != DG_OK ||
@@ -1347,7 +1373,14 @@ int dg_octree_operator(dg_oct_handle h, const double* u_dev, double* out_dev, in
   const char *u0 = (const char*)u_dev, *o0 = (const char*)out_dev;
   if (u0 < o0 + bytes && o0 < u0 + bytes) return DG_ERR_INVALID_ARG;
   cudaStream_t s = (cudaStream_t)stream;
-  DG_CK(oct_apply(h, h->lv[0], u_dev, out_dev, nullptr, (int)B, s));
+  // inside a capture the order of the graph's launches is the caller's
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  if (h->nI > 0) {
+    DG_CK(cudaStreamIsCapturing(s, &cap));
+    if (cap == cudaStreamCaptureStatusNone) DG_CK(cudaStreamWaitEvent(s, h->op_done, 0));
+  }
+  DG_CK(oct_apply(h, h->lv[0], u_dev, out_dev, nullptr, (int)B, s, &h->hang_op));
+  if (h->nI > 0 && cap == cudaStreamCaptureStatusNone) DG_CK(cudaEventRecord(h->op_done, s));
   return DG_OK;
 }
 
