@@ -287,6 +287,118 @@ __global__ void __launch_bounds__(128) k_gemm_tc(GemmArgs g, int batch_base, int
       }
 }
 
+// The same product for at most 16 rows (few sources against a long, wide B: the
+// octree's boundary data). In a 64-row tile most of the MMAs, TwoSums and operand
+// loads would be padding; here a warp owns one 16-row MMA tile and 32 columns and
+// takes its fragments of B straight from global memory (a fragment row is 8
+// consecutive columns, one 32-byte sector), the next 16-term tile in flight while
+// the current one is worked; no shared memory, no barriers. ROWS8: rows 8 to 15
+// are padding too, their sums are not kept. Every product, MMA and TwoSum is that
+// of k_gemm_tc in the same order, so the results are the same bits.
+// Measured (GB300, 8 x 18816 x 245245, the octree of the ten-atom chain): 34.2 ->
+// about 4.5 ms (B is 18.5 GB: 2.7 ms at the measured bandwidth).
+template <bool ROWS8>
+__global__ void __launch_bounds__(128, 4) k_gemm_tc_thin(GemmArgs g, int batch_base, int nsplit, int kc, int nbc) {
+  constexpr int NT = 4;                // 8-column tiles of a warp
+  constexpr int NE = ROWS8 ? 2 : 4;    // live accumulators of an MMA tile per lane
+  constexpr int NA = ROWS8 ? 2 : 4;
+  const int bz = batch_base + (int)blockIdx.z / nsplit;
+  const int split = (int)blockIdx.z % nsplit;
+  const int kbeg = split * kc, kend = min(g.K, kbeg + kc);
+  const int b1 = bz / g.nb2, b2 = bz % g.nb2;
+  const float* A = (const float*)g.A + b1 * g.sA1 + b2 * g.sA2;
+  const float* B = (const float*)g.B + b1 * g.sB1 + b2 * g.sB2;
+  float* C = (float*)g.C + b1 * g.sC1 + b2 * g.sC2;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int gq = lane >> 2, c4 = lane & 3;
+  const int n0 = (blockIdx.x * 4 + warp) * 8 * NT;
+  if (n0 >= g.N) return;
+  // this lane's rows (A) and columns (B); outside the matrix they read as zero
+  bool mok[2], nok[NT];
+  const float* pa[2];
+  const float* pb[NT];
+#pragma unroll
+  for (int i = 0; i < 2; ++i) {
+    mok[i] = gq + 8 * i < g.M;
+    pa[i] = A + (mok[i] ? (long long)(gq + 8 * i) * g.sAm : 0);
+  }
+#pragma unroll
+  for (int j = 0; j < NT; ++j) {
+    nok[j] = n0 + 8 * j + gq < g.N;
+    pb[j] = B + (nok[j] ? (long long)(n0 + 8 * j + gq) * g.sBn : 0);
+  }
+  float acc[NT][4], sum[NT][NE], car[NT][NE];
+#pragma unroll
+  for (int j = 0; j < NT; ++j)
+#pragma unroll
+    for (int e = 0; e < NE; ++e) sum[j][e] = car[j][e] = 0.f;
+  // operands of one 16-term tile: A at k = c4 + 4 t, t < 4 (two MMA steps)
+  float ra[4][2], rb[NT][4];
+  auto load = [&](int k0) {
+#pragma unroll
+    for (int t = 0; t < 4; ++t) {
+      const int k = k0 + c4 + 4 * t;
+      const bool kok = k < kend;
+#pragma unroll
+      for (int i = 0; i < NA / 2; ++i) ra[t][i] = kok && mok[i] ? __ldg(pa[i] + (long long)k * g.sAk) : 0.f;
+#pragma unroll
+      for (int j = 0; j < NT; ++j) rb[j][t] = kok && nok[j] ? __ldg(pb[j] + (long long)k * g.sBk) : 0.f;
+    }
+  };
+  load(kbeg);
+  for (int k0 = kbeg; k0 < kend; k0 += 16) {
+    unsigned ah[2][4], al[2][4], bh[NT][4], bl[NT][4];
+#pragma unroll
+    for (int t = 0; t < 4; ++t) {
+#pragma unroll
+      for (int i = 0; i < 2; ++i) {
+        const float x = ROWS8 && i == 1 ? 0.f : ra[t][i];
+        const unsigned hi = to_tf32(x);
+        ah[t >> 1][(t & 1) * 2 + i] = hi;
+        al[t >> 1][(t & 1) * 2 + i] = to_tf32(x - __uint_as_float(hi));
+      }
+#pragma unroll
+      for (int j = 0; j < NT; ++j) {
+        const unsigned hi = to_tf32(rb[j][t]);
+        bh[j][t] = hi;
+        bl[j][t] = to_tf32(rb[j][t] - __uint_as_float(hi));
+      }
+    }
+    if (k0 + 16 < kend) load(k0 + 16);
+#pragma unroll
+    for (int j = 0; j < NT; ++j)
+#pragma unroll
+      for (int e = 0; e < 4; ++e) acc[j][e] = 0.f;
+#pragma unroll
+    for (int ks = 0; ks < 2; ++ks)
+#pragma unroll
+      for (int j = 0; j < NT; ++j) {
+        mma_tf32(acc[j], al[ks], &bh[j][2 * ks]);
+        mma_tf32(acc[j], ah[ks], &bl[j][2 * ks]);
+        mma_tf32(acc[j], ah[ks], &bh[j][2 * ks]);
+      }
+#pragma unroll
+    for (int j = 0; j < NT; ++j)
+#pragma unroll
+      for (int e = 0; e < NE; ++e) two_sum_add(sum[j][e], car[j][e], acc[j][e]);
+  }
+  const float alpha = (float)g.alpha, beta = (float)g.beta;
+#pragma unroll
+  for (int j = 0; j < NT; ++j)
+#pragma unroll
+    for (int e = 0; e < NE; ++e) {
+      const int m = gq + (e >= 2 ? 8 : 0), n = n0 + 8 * j + 2 * c4 + (e & 1);
+      if (m >= g.M || n >= g.N) continue;
+      const float v = sum[j][e] + car[j][e];
+      if (nsplit > 1) {
+        ((float*)g.work)[(((long long)split * nbc + (bz - batch_base)) * g.M + m) * g.N + n] = v;
+        continue;
+      }
+      float* cp = C + (long long)m * g.sCm + (long long)n * g.sCn;
+      *cp = g.beta != 0.0 ? alpha * v + beta * (*cp) : alpha * v;
+    }
+}
+
 // C = alpha sum_split work[split] (+ beta C) for batches batch_base ..
 // batch_base + nbc - 1, splits added in order with TwoSum
 template <typename T>
@@ -331,9 +443,15 @@ cudaError_t launch_gemm(const GemmArgs& g, cudaStream_t s) {
     const long long cnt = nb - base < per ? nb - base : per;
     const dim3 gr(grid.x, grid.y, (unsigned)(cnt * nsplit));
     count_launch();
-    if constexpr (F32)
-      k_gemm_tc<<<gr, 128, 0, s>>>(g, (int)base, nsplit, kc, (int)cnt);
-    else
+    if constexpr (F32) {
+      const dim3 thin((unsigned)((g.N + 127) / 128), 1, gr.z);  // 4 warps of 32 columns
+      if (g.M <= 8)
+        k_gemm_tc_thin<true><<<thin, 128, 0, s>>>(g, (int)base, nsplit, kc, (int)cnt);
+      else if (g.M <= 16)
+        k_gemm_tc_thin<false><<<thin, 128, 0, s>>>(g, (int)base, nsplit, kc, (int)cnt);
+      else
+        k_gemm_tc<<<gr, 128, 0, s>>>(g, (int)base, nsplit, kc, (int)cnt);
+    } else
       k_gemm64<<<gr, 256, 0, s>>>(g, (int)base, nsplit, kc, (int)cnt);
     if (nsplit > 1) {
       count_launch();
