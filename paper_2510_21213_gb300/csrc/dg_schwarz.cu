@@ -34,19 +34,16 @@
 // Measured (GB300; before: all six passes through shared memory, dense
 // transforms, a division per node, tables per patch): FP64 16^3, p = 7, 42
 // sources 22.0 -> 15.6 ms, 8^3, p = 6, 56 sources 2.33 -> 1.91 ms, 4^3, p = 4, 4
-// sources 35 -> 17 us; FP32 8^3, p = 6, 56 sources 152 -> 109 us, 16^3, p = 3, 42
-// sources 273 -> 142 us, p = 1 89 -> 41 us, 6 x 10 x 8, p = 5, 21 sources 51 -> 23
+// sources 35 -> 17 us; FP32 8^3, p = 6, 56 sources 152 -> 101 us, 16^3, p = 3, 42
+// sources 273 -> 139 us, p = 1 89 -> 39 us, 6 x 10 x 8, p = 5, 21 sources 51 -> 22
 // us. FP64 runs at the rate of its pipe; FP32 issues in 55 % of the cycles with
 // a quarter of the warps resident (96 registers).
-#include "dg_internal.h"
+#include "dg_fdm.h"
 #include "dg_swtc.h"
 
 namespace dg {
 
-// Tuning constants (compile-time; the defaults were chosen by timing on a GB300)
-#ifndef DG_GATHER_WAVE
-#define DG_GATHER_WAVE 8   // gather grid: at most this many blocks per SM per source list (0: one block per element)
-#endif
+constexpr int GATHER_WAVE = 8;  // gather grid: at most this many blocks per SM per source list (16: the same to 1 %)
 
 template <typename T, int N1>
 struct SwCfg {
@@ -86,162 +83,12 @@ struct SwShape {
   using C = SwCfg<T, N1>;
   static constexpr int EPB = FILL ? C::slots(sizeof(T) == 4 ? 128 : 64) : (C::TPE >= 32 ? 1 : 32 / C::TPE);
   static constexpr int THREADS = (EPB * C::TPE + 31) / 32 * 32;
-  // resident threads per SM asked of ptxas
+  // resident threads per SM asked of ptxas (p = 6, 8^3, 56 sources: 101 us at 640, 104 at 768, 147 at 1024; two or
+  // one line per thread instead of three 105 to 117)
   static constexpr int WANT = sizeof(T) == 4 && C::MP < 10 ? 640 : 512;
   static constexpr int MINB = WANT / THREADS < 1 ? 1 : WANT / THREADS > 32 ? 32 : WANT / THREADS;
   static constexpr size_t SMEM = sizeof(T) * ((size_t)SW_MAXCLS * 3 * C::TB + (size_t)EPB * C::SE);
 };
-
-// N values of a table row (16-byte aligned)
-template <typename T, int N>
-__device__ __forceinline__ void sw_row(const T* __restrict__ p, T* r) {
-  constexpr int W = 16 / (int)sizeof(T);
-#pragma unroll
-  for (int w = 0; w < (N + W - 1) / W; ++w) {
-    if constexpr (sizeof(T) == 4) {
-      const float4 q = reinterpret_cast<const float4*>(p)[w];
-      const float t[4] = {q.x, q.y, q.z, q.w};
-#pragma unroll
-      for (int k = 0; k < 4; ++k)
-        if (4 * w + k < N) r[4 * w + k] = t[k];
-    } else {
-      const double2 q = reinterpret_cast<const double2*>(p)[w];
-      r[2 * w] = q.x;
-      if (2 * w + 1 < N) r[2 * w + 1] = q.y;
-    }
-  }
-}
-
-// sums and differences of mirrored nodes in place: v[i] (i < HE) the even part,
-// v[HE + i] the odd part
-template <typename T, int MP>
-__device__ __forceinline__ void sw_fold(T* v) {
-  constexpr int HO = MP / 2, HE = MP - HO;
-  T o[HO];
-#pragma unroll
-  for (int i = 0; i < HO; ++i) {
-    o[i] = v[i] - v[MP - 1 - i];
-    v[i] = v[i] + v[MP - 1 - i];
-  }
-#pragma unroll
-  for (int i = 0; i < HO; ++i) v[HE + i] = o[i];
-}
-// the reverse: node values from the even and odd parts
-template <typename T, int MP>
-__device__ __forceinline__ void sw_unfold(T* v) {
-  constexpr int HO = MP / 2, HE = MP - HO;
-  T o[HO];
-#pragma unroll
-  for (int i = 0; i < HO; ++i) o[i] = v[HE + i];
-#pragma unroll
-  for (int i = 0; i < HO; ++i) {
-    v[MP - 1 - i] = v[i] - o[i];
-    v[i] = v[i] + o[i];
-  }
-}
-
-// Transforms of LPT lines with the table tb (row q: mode q at the nodes, halved
-// rows where SYM: the first HE even, the rest odd). A half H of the modes works
-// on the values v[O .. O + N).
-// forward: put(s, q, sum_i S[i][q] v[s][i])
-template <typename T, int MP, int LPT, int N, int O, int Q0, int Q1, typename P>
-__device__ __forceinline__ void sw_fwd_half(const T* tb, int RP, const T (*v)[MP], P&& put) {
-#pragma unroll 2
-  for (int q = Q0; q < Q1; ++q) {
-    T r[N], a[LPT];
-    sw_row<T, N>(tb + q * RP, r);
-#pragma unroll
-    for (int s = 0; s < LPT; ++s) a[s] = r[0] * v[s][O];
-#pragma unroll
-    for (int i = 1; i < N; ++i)
-#pragma unroll
-      for (int s = 0; s < LPT; ++s) a[s] += r[i] * v[s][O + i];
-#pragma unroll
-    for (int s = 0; s < LPT; ++s) put(s, q, a[s]);
-  }
-}
-template <typename T, int MP, int LPT, typename P>
-__device__ __forceinline__ void sw_fwd(bool sym, const T* tb, int RP, T (*v)[MP], P&& put) {
-  constexpr int HO = MP / 2, HE = MP - HO;
-  if (sym) {
-#pragma unroll
-    for (int s = 0; s < LPT; ++s) sw_fold<T, MP>(v[s]);
-    sw_fwd_half<T, MP, LPT, HE, 0, 0, HE>(tb, RP, v, put);
-    sw_fwd_half<T, MP, LPT, HO, HE, HE, MP>(tb, RP, v, put);
-  } else {
-    sw_fwd_half<T, MP, LPT, MP, 0, 0, MP>(tb, RP, v, put);
-  }
-}
-// backward: v[s][i] = sum_q S[i][q] get(s, q)
-template <typename T, int MP, int LPT, int N, int O, int Q0, int Q1, typename G>
-__device__ __forceinline__ void sw_bwd_half(const T* tb, int RP, T (*v)[MP], G&& get) {
-#pragma unroll
-  for (int s = 0; s < LPT; ++s)
-#pragma unroll
-    for (int i = 0; i < N; ++i) v[s][O + i] = (T)0;
-#pragma unroll 2
-  for (int q = Q0; q < Q1; ++q) {
-    T r[N], c[LPT];
-#pragma unroll
-    for (int s = 0; s < LPT; ++s) c[s] = get(s, q);
-    sw_row<T, N>(tb + q * RP, r);
-#pragma unroll
-    for (int i = 0; i < N; ++i)
-#pragma unroll
-      for (int s = 0; s < LPT; ++s) v[s][O + i] += r[i] * c[s];
-  }
-}
-template <typename T, int MP, int LPT, typename G>
-__device__ __forceinline__ void sw_bwd(bool sym, const T* tb, int RP, T (*v)[MP], G&& get) {
-  constexpr int HO = MP / 2, HE = MP - HO;
-  if (sym) {
-    sw_bwd_half<T, MP, LPT, HE, 0, 0, HE>(tb, RP, v, get);
-    sw_bwd_half<T, MP, LPT, HO, HE, HE, MP>(tb, RP, v, get);
-#pragma unroll
-    for (int s = 0; s < LPT; ++s) sw_unfold<T, MP>(v[s]);
-  } else {
-    sw_bwd_half<T, MP, LPT, MP, 0, 0, MP>(tb, RP, v, get);
-  }
-}
-// both, with the scaling between: v[s] <- S diag(scale(s, q, .)) S^T v[s]
-template <typename T, int MP, int LPT, int N, int O, int Q0, int Q1, typename F>
-__device__ __forceinline__ void sw_mid_half(const T* tb, int RP, const T (*v)[MP], T (*w)[MP], F&& scale) {
-#pragma unroll
-  for (int s = 0; s < LPT; ++s)
-#pragma unroll
-    for (int i = 0; i < N; ++i) w[s][O + i] = (T)0;
-#pragma unroll 1
-  for (int q = Q0; q < Q1; ++q) {
-    T r[N], a[LPT];
-    sw_row<T, N>(tb + q * RP, r);
-#pragma unroll
-    for (int s = 0; s < LPT; ++s) a[s] = r[0] * v[s][O];
-#pragma unroll
-    for (int i = 1; i < N; ++i)
-#pragma unroll
-      for (int s = 0; s < LPT; ++s) a[s] += r[i] * v[s][O + i];
-#pragma unroll
-    for (int s = 0; s < LPT; ++s) a[s] = scale(s, q, a[s]);
-#pragma unroll
-    for (int i = 0; i < N; ++i)
-#pragma unroll
-      for (int s = 0; s < LPT; ++s) w[s][O + i] += r[i] * a[s];
-  }
-}
-template <typename T, int MP, int LPT, typename F>
-__device__ __forceinline__ void sw_mid(bool sym, const T* tb, int RP, T (*v)[MP], T (*w)[MP], F&& scale) {
-  constexpr int HO = MP / 2, HE = MP - HO;
-  if (sym) {
-#pragma unroll
-    for (int s = 0; s < LPT; ++s) sw_fold<T, MP>(v[s]);
-    sw_mid_half<T, MP, LPT, HE, 0, 0, HE>(tb, RP, v, w, scale);
-    sw_mid_half<T, MP, LPT, HO, HE, HE, MP>(tb, RP, v, w, scale);
-#pragma unroll
-    for (int s = 0; s < LPT; ++s) sw_unfold<T, MP>(w[s]);
-  } else {
-    sw_mid_half<T, MP, LPT, MP, 0, 0, MP>(tb, RP, v, w, scale);
-  }
-}
 
 template <typename T, int N1, bool FILL>
 __global__ void __launch_bounds__(SwShape<T, N1, FILL>::THREADS, SwShape<T, N1, FILL>::MINB)
@@ -293,7 +140,7 @@ __global__ void __launch_bounds__(SwShape<T, N1, FILL>::THREADS, SwShape<T, N1, 
       const int oLx = sw_halo(px), oLy = sw_halo(py), oLz = sw_halo(pz);
       const int mx = sw_size(px), my = sw_size(py), mz = sw_size(pz);
       const T* rr = r + src * Nq;
-      const int pe = nx * ny;  // elements of a z layer
+      const long long pe = (long long)nx * ny * NPE;  // values of a z layer of elements
 #pragma unroll
       for (int s = 0; s < LPT; ++s) {
         const int l = lt + TPE * s, i = l % MP, j = l / MP;
@@ -313,19 +160,13 @@ __global__ void __launch_bounds__(SwShape<T, N1, FILL>::THREADS, SwShape<T, N1, 
           bb = 0;
           ee += nx;
         }
-        const int at = a + N1 * bb;
+        const T* p = rr + (long long)ee * NPE + (a + N1 * bb);
+        const T *below = p - pe + (N1 - 1) * NF, *own = p - oLz * NF, *above = p + pe;
+        v[s][0] = in ? __ldg(oLz ? below : own) : (T)0;
 #pragma unroll
-        for (int k = 0; k < MP; ++k) {
-          int c = k - oLz, ek = ee;
-          if (k == 0 && c < 0) {
-            c = N1 - 1;
-            ek -= pe;
-          } else if (k >= N1 && c >= N1) {
-            c = 0;
-            ek += pe;
-          }
-          v[s][k] = in && k < mz ? __ldg(rr + (long long)ek * NPE + at + NF * c) : (T)0;
-        }
+        for (int k = 1; k < N1; ++k) v[s][k] = in ? __ldg(own + NF * k) : (T)0;
+        v[s][N1] = in && N1 < mz ? __ldg(oLz ? own + NF * N1 : above) : (T)0;
+        v[s][N1 + 1] = in && N1 + 1 < mz ? __ldg(above) : (T)0;
       }
       sw_fwd<T, MP, LPT>(sw_sym(pz), tz, RP, v, [&](int s, int q, T a) {
         const int l = lt + TPE * s;
@@ -466,21 +307,34 @@ struct GatherCfg {
 // mode 0: z = M r; 1: d = c1 M r, x = d; 2: d = c1 M r, x += d; 3: d = c1 d + c2 M r, x += d
 // (d is passed in z). GE elements per block and iteration (grid-stride), one thread per node,
 // GS sources per thread (the node's position, neighbour tests and offsets shared by them).
-#ifndef DG_GATHER_SOURCES
-#define DG_GATHER_SOURCES 4
-#endif
+// All loads of the group are issued before the first sum: the contributions of one
+// source at a time left too few bytes in flight. GS = 4 in FP32 (2 is 7 % slower
+// for the smoother at p = 7, 1 17 %), 2 in FP64 (registers; 4 is 1 % slower).
+// Measured (GB300, FP32, d and x not touched): 16^3, p = 7, 42 sources 0.516 ->
+// 0.262 ms for 1.04 GB, 8^3, p = 6, 56 sources 66 -> 36 us.
+template <typename T>
+constexpr int gather_sources() {
+  return sizeof(T) == 4 ? 4 : 2;
+}
 template <typename T, int N1, int MODE>
 __global__ void __launch_bounds__(GatherCfg<N1>::THREADS)
     k_schwarz_gather(const LevelOp* __restrict__ op, const T* __restrict__ zp, T* __restrict__ z, T* __restrict__ x,
                      T c1, T c2, const int* __restrict__ act, int nact) {
   constexpr int MP = N1 + 2, MP2 = MP * MP, MP3 = MP2 * MP, NPE = N1 * N1 * N1, GE = GatherCfg<N1>::GE;
-  constexpr int GS = DG_GATHER_SOURCES;
+  constexpr int GS = gather_sources<T>();
   const int nx = op->n[0], ny = op->n[1], nz = op->n[2];
   const int E = op->E;
   const long long Nq = op->Nq;
   // this block's sources (GS consecutive entries of the active list)
   const int k0 = blockIdx.y * GS;
   const int ns = min(GS, nact - k0);
+  long long zoff[GS], foff[GS];  // of each source in the patch buffer and in the fields
+#pragma unroll
+  for (int j = 0; j < GS; ++j) {
+    const long long rhs = act[k0 + min(j, ns - 1)];
+    zoff[j] = rhs * E * MP3;
+    foff[j] = rhs * Nq;
+  }
   const int slot = threadIdx.x / NPE, loc = threadIdx.x % NPE;
   const int a = loc % N1, bb = (loc / N1) % N1, c = loc / (N1 * N1);
   // element position, advanced by the grid stride without runtime divisions
@@ -520,35 +374,46 @@ __global__ void __launch_bounds__(GatherCfg<N1>::THREADS)
     const int oyz = (e + dy + dz) * MP3 + ix + MP * jy + MP2 * jz;
     const int oxyz = (e + dx + dy + dz) * MP3 + jx + MP * jy + MP2 * jz;
     const int gi = e * NPE + loc;
+    // every load of the group is issued before the first sum, contributions in a
+    // fixed order; sources past the end repeat the last one and are not stored
+    T acc[GS], v[7][GS], dv[GS], xv[GS];
+#pragma unroll
+    for (int j = 0; j < GS; ++j) {
+      const T* zs = zp + zoff[j];
+      acc[j] = zs[o0];
+      v[0][j] = dx ? zs[ox] : (T)0;
+      v[1][j] = dy ? zs[oy] : (T)0;
+      v[2][j] = dz ? zs[oz] : (T)0;
+      v[3][j] = dx && dy ? zs[oxy] : (T)0;
+      v[4][j] = dx && dz ? zs[oxz] : (T)0;
+      v[5][j] = dy && dz ? zs[oyz] : (T)0;
+      v[6][j] = dx && dy && dz ? zs[oxyz] : (T)0;
+      if (MODE == 3) dv[j] = z[foff[j] + gi];
+      if (MODE >= 2) xv[j] = x[foff[j] + gi];
+    }
+#pragma unroll
+    for (int c = 0; c < 7; ++c)
+#pragma unroll
+      for (int j = 0; j < GS; ++j) acc[j] += v[c][j];
 #pragma unroll
     for (int j = 0; j < GS; ++j) {
       if (j >= ns) break;
-      const long long rhs = act[k0 + j];
-      const T* zs = zp + rhs * E * (long long)MP3;
-      T* zg = z + rhs * Nq;
-      T* xg = x + rhs * Nq;
-      T acc = zs[o0];
-      if (dx) acc += zs[ox];
-      if (dy) acc += zs[oy];
-      if (dz) acc += zs[oz];
-      if (dx && dy) acc += zs[oxy];
-      if (dx && dz) acc += zs[oxz];
-      if (dy && dz) acc += zs[oyz];
-      if (dx && dy && dz) acc += zs[oxyz];
+      T* zg = z + foff[j] + gi;
+      T* xg = x + foff[j] + gi;
       if (MODE == 0) {
-        zg[gi] = acc;
+        *zg = acc[j];
       } else if (MODE == 1) {
-        const T v = c1 * acc;
-        zg[gi] = v;
-        xg[gi] = v;
+        const T w = c1 * acc[j];
+        *zg = w;
+        *xg = w;
       } else if (MODE == 2) {
-        const T v = c1 * acc;
-        zg[gi] = v;
-        xg[gi] += v;
+        const T w = c1 * acc[j];
+        *zg = w;
+        *xg = xv[j] + w;
       } else {
-        const T v = c1 * zg[gi] + c2 * acc;
-        zg[gi] = v;
-        xg[gi] += v;
+        const T w = c1 * dv[j] + c2 * acc[j];
+        *zg = w;
+        *xg = xv[j] + w;
       }
     }
     ex += sx;
@@ -569,12 +434,10 @@ static cudaError_t gather_n1(const LevelOp& hop, const LevelOp* dop, const T* zp
   // the gather indexes one source's patch buffer with 32-bit offsets
   if ((long long)hop.E * (N1 + 2) * (N1 + 2) * (N1 + 2) >= (1LL << 31)) return cudaErrorInvalidValue;
   long long gx = (hop.E + GatherCfg<N1>::GE - 1) / GatherCfg<N1>::GE;
-#if DG_GATHER_WAVE > 0
-  const long long ngroups = (nact + DG_GATHER_SOURCES - 1) / DG_GATHER_SOURCES;
-  const long long cap = 152LL * DG_GATHER_WAVE / (ngroups > 0 ? ngroups : 1) + 1;
+  const long long ngroups = (nact + gather_sources<T>() - 1) / gather_sources<T>();
+  const long long cap = 152LL * GATHER_WAVE / ngroups + 1;
   if (gx > cap) gx = cap;
-#endif
-  const dim3 grid((unsigned)gx, (unsigned)((nact + DG_GATHER_SOURCES - 1) / DG_GATHER_SOURCES));
+  const dim3 grid((unsigned)gx, (unsigned)ngroups);
   count_launch();
   switch (mode) {
     case 0: k_schwarz_gather<T, N1, 0><<<grid, GT, 0, s>>>(dop, zp, z, x, (T)c1, (T)c2, act, nact); break;
