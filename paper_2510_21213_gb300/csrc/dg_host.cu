@@ -1495,7 +1495,7 @@ static int exchange_build_range(dg_handle h, const double* psi, int32_t N, long 
   const int cap = std::max(1, std::min<int>(default_batch(h), (int)(src_end - src_begin)));
   DG_RET(prepare(h, cap));
   DG_CK(h->Wacc.ensure(sizeof(double) * N * Nq));
-  const int nch = kmat_chunks(Nq);
+  const int nch = kmat_chunks(Nq, N);
   DG_CK(h->kpart.ensure(sizeof(double) * (size_t)nch * N * N));
   DG_CK(h->Kdev.ensure(sizeof(double) * ((size_t)N * N + 4)));
   DG_CK(cudaMemsetAsync(h->Wacc.p, 0, sizeof(double) * N * Nq, s));

@@ -220,7 +220,7 @@ cudaError_t launch_exch_accum(const double* psi, const double* v, double* Wacc, 
 cudaError_t launch_kmat(const double* psi, const double* W, const double* Wacc, int N, long long Nq,
                         double* part, int nchunk, double* K, cudaStream_t s);
 
-int kmat_chunks(long long Nq);
+int kmat_chunks(long long Nq, int N);
 
 // per-element convolutional network of the learned initial guess (dg_nn.cu);
 // parameters FP32 [NN_NPARAM], W2 also as BF16 [27][co][ci] (W2t) and [27][ci][co] (W2o)

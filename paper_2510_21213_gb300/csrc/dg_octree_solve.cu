@@ -1438,7 +1438,7 @@ int dg_octree_exchange_build(dg_oct_handle h, const double* psi, int32_t N, doub
   const int cap = oct_cap(h, nsrc_total);
   DG_RET(oct_ws(h, cap));
   DG_CK(h->Wacc.ensure(sizeof(double) * (size_t)N * Nq));
-  const int nch = kmat_chunks(Nq);
+  const int nch = kmat_chunks(Nq, N);
   DG_CK(h->kpart.ensure(sizeof(double) * (size_t)nch * N * N));
   DG_CK(h->Kdev.ensure(sizeof(double) * (size_t)N * N));
   DG_CK(cudaMemsetAsync(h->Wacc.p, 0, sizeof(double) * (size_t)N * Nq, s));

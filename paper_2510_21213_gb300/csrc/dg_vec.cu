@@ -805,9 +805,13 @@ cudaError_t launch_exch_accum(const double* psi, const double* v, double* Wacc, 
 // ---------------------------------------------------------------------------
 static constexpr int KT = 32;   // output tile (KT x KT), 256 threads x 4 outputs
 static constexpr int KQ = 64;   // nodes per shared-memory stage
+static constexpr int KSMALL = 16;  // orbitals up to which a block holds all N^2 outputs
 
-int kmat_chunks(long long Nq) {
-  long long c = (Nq + 1023) / 1024;
+// node chunks: of 256 nodes, so that a small mesh's blocks reach many SMs, or of
+// 1024 where N^2 partial sums per chunk would take more memory than that is worth
+int kmat_chunks(long long Nq, int N) {
+  const int per = N <= 64 ? 256 : 1024;
+  long long c = (Nq + per - 1) / per;
   if (c > 2048) c = 2048;
   return (int)(c < 1 ? 1 : c);
 }
@@ -835,7 +839,8 @@ __global__ void k_kmat_partial(const double* __restrict__ psi, const double* __r
     for (int qq = 0; qq < KQ; ++qq) {
       const double bj = sb[qq][tx];
 #pragma unroll
-      for (int r = 0; r < 4; ++r) acc[r] += sa[qq][ty + 8 * r] * bj;
+      for (int r = 0; r < 4; ++r)
+        if (ti + ty + 8 * r < N) acc[r] += sa[qq][ty + 8 * r] * bj;  // uniform in a warp
     }
     __syncthreads();
   }
@@ -846,21 +851,63 @@ __global__ void k_kmat_partial(const double* __restrict__ psi, const double* __r
   }
 }
 
-__global__ void k_kmat_reduce(const double* __restrict__ part, int N, int nchunk, double* __restrict__ K) {
-  const int ij = blockIdx.x * blockDim.x + threadIdx.x;
-  if (ij >= N * N) return;
+// The same for N <= KSMALL: thread = one output (i, j) and one of 256 / N^2 slices
+// of a stage's nodes, so that no FMA is spent on the padding of a 32 x 32 tile
+// (10x at N = 10, 256x at N = 2); the slices are added in order at the end.
+// Measured (GB300): both kernels 4^3, p = 4, N = 2 276 -> 6 us, 8^3, p = 6, N = 10 542 -> 60 us.
+__global__ void __launch_bounds__(256) k_kmat_small(const double* __restrict__ psi, const double* __restrict__ W,
+                                                    const double* __restrict__ Wacc, int N, long long Nq,
+                                                    double* __restrict__ part) {
+  __shared__ double sa[KSMALL][KQ + 1], sb[KSMALL][KQ + 1], red[256];
+  const int nchunk = gridDim.x, np = N * N, slices = 256 / np;
+  const long long per = (Nq + nchunk - 1) / nchunk;
+  const long long q0 = (long long)blockIdx.x * per;
+  const long long q1 = q0 + per < Nq ? q0 + per : Nq;
+  const int g = threadIdx.x / np, ij = threadIdx.x - g * np, i = ij / N, j = ij - i * N;
   double acc = 0.0;
-  for (int c = 0; c < nchunk; ++c) acc += part[(long long)c * N * N + ij];
-  K[ij] = acc;
+  for (long long qs = q0; qs < q1; qs += KQ) {
+    for (int t = threadIdx.x; t < KQ * N; t += 256) {
+      const int qq = t % KQ, r = t / KQ;
+      const long long q = qs + qq;
+      sa[r][qq] = q < q1 ? psi[(long long)r * Nq + q] * W[q] : 0.0;
+      sb[r][qq] = q < q1 ? Wacc[(long long)r * Nq + q] : 0.0;
+    }
+    __syncthreads();
+    if (g < slices)
+      for (int qq = g; qq < KQ; qq += slices) acc += sa[i][qq] * sb[j][qq];
+    __syncthreads();
+  }
+  red[threadIdx.x] = acc;
+  __syncthreads();
+  if (threadIdx.x < np) {
+    double s = 0.0;
+    for (int k = 0; k < slices; ++k) s += red[k * np + threadIdx.x];
+    part[(long long)blockIdx.x * np + threadIdx.x] = s;
+  }
+}
+
+// one warp per output: lanes take every 32nd chunk, then a fixed tree
+__global__ void k_kmat_reduce(const double* __restrict__ part, int N, int nchunk, double* __restrict__ K) {
+  const long long ij = (long long)blockIdx.x * (blockDim.x / 32) + threadIdx.x / 32;
+  const int lane = threadIdx.x & 31;
+  if (ij >= (long long)N * N) return;
+  double acc = 0.0;
+  for (int c = lane; c < nchunk; c += 32) acc += part[(long long)c * N * N + ij];
+#pragma unroll
+  for (int d = 16; d > 0; d >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, d);
+  if (lane == 0) K[ij] = acc;
 }
 
 cudaError_t launch_kmat(const double* psi, const double* W, const double* Wacc, int N, long long Nq, double* part,
                         int nchunk, double* K, cudaStream_t s) {
   const int tiles = (N + KT - 1) / KT;
   count_launch();
-  k_kmat_partial<<<dim3(tiles, tiles, nchunk), 256, 0, s>>>(psi, W, Wacc, N, Nq, part);
+  if (N <= KSMALL)
+    k_kmat_small<<<nchunk, 256, 0, s>>>(psi, W, Wacc, N, Nq, part);
+  else
+    k_kmat_partial<<<dim3(tiles, tiles, nchunk), 256, 0, s>>>(psi, W, Wacc, N, Nq, part);
   count_launch();
-  k_kmat_reduce<<<(N * N + 255) / 256, 256, 0, s>>>(part, N, nchunk, K);
+  k_kmat_reduce<<<(unsigned)(((long long)N * N + 7) / 8), 256, 0, s>>>(part, N, nchunk, K);
   return cudaGetLastError();
 }
 
