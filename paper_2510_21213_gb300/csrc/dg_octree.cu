@@ -317,7 +317,7 @@ __device__ __forceinline__ void oct_line(const OctLine<V, N1>& tab, V* v, const 
   }
 }
 
-// out = A u, one slot per leaf and source. fac [E][6]: h_t0 h_t1 / (2 h_d) per
+// out = A u (rin null) or rin - A u, one slot per leaf and source. fac [E][6]: h_t0 h_t1 / (2 h_d) per
 // axis, then 1 (penalty form 0) or 1 / h_d; hslot [E][6]: hanging slot of a
 // face, -1 for the others; gbuf [source - k0][slot][2][N1^2]: k_oct_hang's
 // projected fluxes.
@@ -326,7 +326,7 @@ __global__ void __launch_bounds__(OctShape<V, N1, FILL>::THREADS, OctShape<V, N1
     k_oct_apply(const __grid_constant__ OctLine<V, N1> tab, const double* __restrict__ fac,
                 const int* __restrict__ kind, const int* __restrict__ nbr, const int* __restrict__ hslot,
                 const V* __restrict__ gbuf, const V* __restrict__ u, V* __restrict__ out,
-                const int* __restrict__ act, int vec_i) {
+                const V* __restrict__ rin, const int* __restrict__ act, int vec_i) {
   using H = OctShape<V, N1, FILL>;
   using Y = LineLayout<N1>;
   constexpr int NF = N1 * N1, NPE = NF * N1, BPB = H::BPB;
@@ -411,7 +411,10 @@ __global__ void __launch_bounds__(OctShape<V, N1, FILL>::THREADS, OctShape<V, N1
     oct_line<V, N1>(tab, v, ov[2], od[2], fc[4] < -1, fc[5] < -1, gam[2]);
     const V sc = mul(sfac[sl][2], tab.ww[l]);
 #pragma unroll
-    for (int i = 0; i < N1; ++i) out[g0 + l + NF * i] = mad(sc, v[i], sacc[zat + Y::PZ * i]);
+    for (int i = 0; i < N1; ++i) {
+      const V Au = mad(sc, v[i], sacc[zat + Y::PZ * i]);
+      out[g0 + l + NF * i] = rin ? rin[g0 + l + NF * i] - Au : Au;
+    }
   }
 }
 
@@ -586,8 +589,8 @@ void octree_tables(int n1, OctTables& T) {
 }
 
 template <typename V, int N1>
-static cudaError_t oct_apply_n1(const OctTables& T, const OctMesh& m, double eps, const V* u, V* out, const int* act,
-                                int nact, V* gbuf, long long gelems, cudaStream_t s) {
+static cudaError_t oct_apply_n1(const OctTables& T, const OctMesh& m, double eps, const V* u, V* out, const V* rin,
+                                const int* act, int nact, V* gbuf, long long gelems, cudaStream_t s) {
   constexpr int HO = N1 / 2, HE = N1 - HO, NF = N1 * N1, NPE = NF * N1;
   OctLine<V, N1> t;
   OctHang<V, N1> g;
@@ -639,7 +642,7 @@ static cudaError_t oct_apply_n1(const OctTables& T, const OctMesh& m, double eps
         if (e != cudaSuccess) return e;
       }
       count_launch();
-      kern<<<(unsigned)blocks, threads, smem, s>>>(t, m.fac, m.kind, m.nb, m.hslot, gbuf, u, out, act, vec);
+      kern<<<(unsigned)blocks, threads, smem, s>>>(t, m.fac, m.kind, m.nb, m.hslot, gbuf, u, out, rin, act, vec);
       return cudaGetLastError();
     };
     using F = OctShape<V, N1, true>;
@@ -654,24 +657,24 @@ static cudaError_t oct_apply_n1(const OctTables& T, const OctMesh& m, double eps
 
 template <typename V>
 cudaError_t launch_octree_apply(int n1, const OctTables& T, const OctMesh& m, double eps, const V* u, V* out,
-                                const int* act, int nact, V* gbuf, long long gelems, cudaStream_t s) {
+                                const V* rin, const int* act, int nact, V* gbuf, long long gelems, cudaStream_t s) {
   if (nact == 0 || m.E == 0) return cudaSuccess;
   switch (n1) {
-    case 2: return oct_apply_n1<V, 2>(T, m, eps, u, out, act, nact, gbuf, gelems, s);
-    case 3: return oct_apply_n1<V, 3>(T, m, eps, u, out, act, nact, gbuf, gelems, s);
-    case 4: return oct_apply_n1<V, 4>(T, m, eps, u, out, act, nact, gbuf, gelems, s);
-    case 5: return oct_apply_n1<V, 5>(T, m, eps, u, out, act, nact, gbuf, gelems, s);
-    case 6: return oct_apply_n1<V, 6>(T, m, eps, u, out, act, nact, gbuf, gelems, s);
-    case 7: return oct_apply_n1<V, 7>(T, m, eps, u, out, act, nact, gbuf, gelems, s);
-    case 8: return oct_apply_n1<V, 8>(T, m, eps, u, out, act, nact, gbuf, gelems, s);
-    case 9: return oct_apply_n1<V, 9>(T, m, eps, u, out, act, nact, gbuf, gelems, s);
+    case 2: return oct_apply_n1<V, 2>(T, m, eps, u, out, rin, act, nact, gbuf, gelems, s);
+    case 3: return oct_apply_n1<V, 3>(T, m, eps, u, out, rin, act, nact, gbuf, gelems, s);
+    case 4: return oct_apply_n1<V, 4>(T, m, eps, u, out, rin, act, nact, gbuf, gelems, s);
+    case 5: return oct_apply_n1<V, 5>(T, m, eps, u, out, rin, act, nact, gbuf, gelems, s);
+    case 6: return oct_apply_n1<V, 6>(T, m, eps, u, out, rin, act, nact, gbuf, gelems, s);
+    case 7: return oct_apply_n1<V, 7>(T, m, eps, u, out, rin, act, nact, gbuf, gelems, s);
+    case 8: return oct_apply_n1<V, 8>(T, m, eps, u, out, rin, act, nact, gbuf, gelems, s);
+    case 9: return oct_apply_n1<V, 9>(T, m, eps, u, out, rin, act, nact, gbuf, gelems, s);
     default: return cudaErrorInvalidValue;
   }
 }
 template cudaError_t launch_octree_apply<double>(int, const OctTables&, const OctMesh&, double, const double*, double*,
-                                                 const int*, int, double*, long long, cudaStream_t);
+                                                 const double*, const int*, int, double*, long long, cudaStream_t);
 template cudaError_t launch_octree_apply<float>(int, const OctTables&, const OctMesh&, double, const float*, float*,
-                                                const int*, int, float*, long long, cudaStream_t);
+                                                const float*, const int*, int, float*, long long, cudaStream_t);
 }  // namespace dg
 
 using namespace dg;
@@ -787,7 +790,7 @@ int dg_octree_apply(const dg_mesh_desc* root, const int32_t* leaves, int32_t n_l
   const size_t gbytes = std::max(one, std::min<size_t>(one * (size_t)B, 64u << 20));
   if (nI > 0 && (rc = ck(dg.ensure(gbytes))) != DG_OK) return rc;
   const OctMesh m{E, dk.as<int>(), dn.as<int>(), df.as<double>(), ds.as<int>(), dr.as<int>(), nI};
-  if ((rc = ck(launch_octree_apply<double>(n1, T, m, penalty_eps, u, out, nullptr, (int)B, dg.as<double>(),
+  if ((rc = ck(launch_octree_apply<double>(n1, T, m, penalty_eps, u, out, nullptr, nullptr, (int)B, dg.as<double>(),
                                            (long long)(gbytes / sizeof(double)), s))) != DG_OK)
     return rc;
   // the tables and connectivity are call-local: wait before they are freed

@@ -48,12 +48,12 @@ struct OctMesh {
   int nI;
 };
 
-// out[k] = A u[k] for the sources k = act[0..nact) (act null: k = 0..nact),
+// out[k] = A u[k] (rin null) or rin[k] - A u[k] for the sources k = act[0..nact) (act null: k = 0..nact),
 // u and out [.][E][n1^3]; V = double or float (the fields and the arithmetic);
 // gbuf: scratch of gelems values, at least octree_hang_elems (sources go through
 // in chunks that fit)
 template <typename V>
 cudaError_t launch_octree_apply(int n1, const OctTables& T, const OctMesh& m, double eps, const V* u, V* out,
-                                const int* act, int nact, V* gbuf, long long gelems, cudaStream_t s);
+                                const V* rin, const int* act, int nact, V* gbuf, long long gelems, cudaStream_t s);
 
 }  // namespace dg

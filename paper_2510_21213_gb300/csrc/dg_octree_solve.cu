@@ -39,6 +39,8 @@
 #include "dg_ctx.h"
 #include "dg_internal.h"
 #include "dg_mg.h"
+#include "dg_fdm.h"
+#include "dg_line.h"
 #include "dg_octree.h"
 #include "dg_setup.h"
 
@@ -50,11 +52,15 @@ struct OctLevel {
   long long Nq = 0;
   dg::OctTables T;
   dg::DevBuf cls;     // int [E][3]: 1-D class of each leaf axis
-  dg::DevBuf S, lam;  // per class: S [n1][n1] (row node, column mode), lambda [n1]
+  dg::DevBuf bj64, bj32;  // tables of the leaf-block inverse per class, FP64 and FP32
+  template <typename V>
+  const V* bj() const {
+    return (sizeof(V) == 8 ? bj64 : bj32).as<V>();
+  }
   int ncls = 0;
   double lam_max = 0;  // lambda_max(P^-1 A) estimate (power iteration at set-up)
   dg::DevBuf I;        // [n1][n1c]: the next coarser level's basis at this level's nodes
-  dg::DevBuf x, b, res, d, z, q;  // V-cycle workspace, [cap][Nq] each
+  dg::DevBuf x, b, res, d, z, q;  // V-cycle workspace, [cap][Nq] each (z, q: one field)
 };
 
 // Handle of the octree solver (opaque in the C ABI).
@@ -119,74 +125,100 @@ static inline dim3 ogrid(long long n, int nsrc) {
   return dim3((unsigned)gx, (unsigned)nsrc);
 }
 
-// z = P r on every leaf: the exact inverse of the leaf's diagonal block by
-// fast diagonalisation (one block per leaf and source)
-template <typename V, int N1>
-__global__ void __launch_bounds__(128) k_oct_bjac(const int* __restrict__ cls, const double* __restrict__ S,
-                                                  const double* __restrict__ lam, const V* __restrict__ r,
-                                                  V* __restrict__ z, long long Nq, const int* __restrict__ act) {
-  constexpr int NPE = N1 * N1 * N1, NF = N1 * N1;
-  __shared__ V sS[3][NF], sl[3][N1], u[NPE], t[NPE];
-  const int e = blockIdx.x;
-  const long long off = (long long)act[blockIdx.y] * Nq + (long long)e * NPE;
-  for (int i = threadIdx.x; i < 3 * NF; i += blockDim.x) {
-    const int d = i / NF;
-    sS[d][i % NF] = (V)S[(long long)cls[3 * e + d] * NF + i % NF];
-  }
-  for (int i = threadIdx.x; i < 3 * N1; i += blockDim.x) {
-    const int d = i / N1;
-    sl[d][i % N1] = (V)lam[(long long)cls[3 * e + d] * N1 + i % N1];
-  }
-  for (int i = threadIdx.x; i < NPE; i += blockDim.x) u[i] = r[off + i];
-  __syncthreads();
-  // forward: t = (S_x (x) S_y (x) S_z)^T u, one axis at a time (mode index replaces node index)
-  for (int i = threadIdx.x; i < NPE; i += blockDim.x) {
-    const int m = i % N1, rest = i - m;
-    V acc = 0;
+// y = P r on every leaf: the exact inverse of the leaf's diagonal block by fast
+// diagonalisation, fused with the Chebyshev update that it is for:
+//   mode 0: z = y; 1: z = c1 y, x = z; 2: z = c1 y, x += z; 3: z = c1 z + c2 y, x += z.
+// A thread owns a line of one leaf along each direction in turn: z forward on the
+// values as they come from global memory, y forward, x in registers (forward,
+// divided by the eigenvalue sum, back), y back, z back straight to the update, so
+// a value goes through shared memory 8 times instead of 14. Several leaves share a
+// block, each with its three tables (OctBjac<V, N1>::TB values per class: rows =
+// modes, then the eigenvalues; see oct_bjac_table).
+// Measured (GB300, 715 leaves, p = 6, 8 fields, FP32; one block per leaf, one output
+// per thread and pass, the update a kernel of its own before): 27 + 5 -> 21 us.
+template <typename V, int N1, bool FILL>
+struct OctBjac {
+  static constexpr int W = 16 / (int)sizeof(V);
+  static constexpr int RP = (N1 + W - 1) / W * W;
+  static constexpr int TB = (N1 + 1) * RP;
+  static constexpr int LINES = N1 * N1;
+  static constexpr int BPB = FILL ? best_bpb(LINES, sizeof(V) == 4 ? 128 : 64) : 1;
+  static constexpr int THREADS = (BPB * LINES + 31) / 32 * 32;
+  static constexpr size_t SMEM = sizeof(V) * (size_t)BPB * (3 * TB + (LineLayout<N1>::ES + W - 1) / W * W);
+};
+
+template <typename V, int N1, bool FILL>
+__global__ void __launch_bounds__(OctBjac<V, N1, FILL>::THREADS)
+    k_oct_bjac(const int* __restrict__ cls, const V* __restrict__ tab, const V* __restrict__ r, V* __restrict__ z,
+               V* __restrict__ x, V c1, V c2, int mode, int E, long long items, const int* __restrict__ act) {
+  using B = OctBjac<V, N1, FILL>;
+  using Y = LineLayout<N1>;
+  constexpr int NF = N1 * N1, NPE = NF * N1, BPB = B::BPB, RP = B::RP, TB = B::TB;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  V* tabs = reinterpret_cast<V*>(smem_raw);
+  V* buf = tabs + BPB * 3 * TB;
+  __shared__ long long soff[BPB];  // first value of the slot's leaf, -1: none
+  __shared__ int scls[BPB][3];
+  const int tid = threadIdx.x;
+  if (tid < BPB) {
+    const long long it = (long long)blockIdx.x * BPB + tid;
+    const bool in = it < items;
+    const int k = in ? (int)(it / E) : 0, e = in ? (int)(it - (long long)k * E) : 0;
+    soff[tid] = in ? ((long long)act[k] * E + e) * NPE : -1;
 #pragma unroll
-    for (int a = 0; a < N1; ++a) acc += sS[0][a * N1 + m] * u[rest + a];
-    t[i] = acc;
-  }
-  __syncthreads();
-  for (int i = threadIdx.x; i < NPE; i += blockDim.x) {
-    const int m = (i / N1) % N1, rest = i - m * N1;
-    V acc = 0;
-#pragma unroll
-    for (int b = 0; b < N1; ++b) acc += sS[1][b * N1 + m] * t[rest + b * N1];
-    u[i] = acc;
-  }
-  __syncthreads();
-  for (int i = threadIdx.x; i < NPE; i += blockDim.x) {
-    const int m = i / NF, rest = i - m * NF;
-    V acc = 0;
-#pragma unroll
-    for (int c = 0; c < N1; ++c) acc += sS[2][c * N1 + m] * u[rest + c * NF];
-    t[i] = acc / (sl[0][i % N1] + sl[1][(i / N1) % N1] + sl[2][m]);
-  }
-  __syncthreads();
-  // back: u = (S_x (x) S_y (x) S_z) t
-  for (int i = threadIdx.x; i < NPE; i += blockDim.x) {
-    const int c = i / NF, rest = i - c * NF;
-    V acc = 0;
-#pragma unroll
-    for (int m = 0; m < N1; ++m) acc += sS[2][c * N1 + m] * t[rest + m * NF];
-    u[i] = acc;
+    for (int d = 0; d < 3; ++d) scls[tid][d] = cls[3 * e + d];
   }
   __syncthreads();
-  for (int i = threadIdx.x; i < NPE; i += blockDim.x) {
-    const int b = (i / N1) % N1, rest = i - b * N1;
-    V acc = 0;
+  for (int t = tid; t < BPB * 3 * (TB / B::W); t += B::THREADS) {
+    const int sd = t / (TB / B::W), w = t - sd * (TB / B::W);
+    reinterpret_cast<uint4*>(tabs)[t] =
+        __ldg(reinterpret_cast<const uint4*>(tab + (long long)scls[sd / 3][sd % 3] * TB) + w);
+  }
+  const int slot = tid / NF, l = tid - slot * NF, l1 = l % N1, l2 = l / N1;
+  const bool on = slot < BPB && soff[slot < BPB ? slot : 0] >= 0;
+  const int sl = on ? slot : 0;
+  const long long off = on ? soff[sl] : 0;
+  const V *tx = tabs + sl * 3 * TB, *ty = tx + TB, *tz = ty + TB;
+  V* b = buf + sl * ((Y::ES + B::W - 1) / B::W * B::W);
+  const int at_x = Y::PB * l1 + Y::PZ * l2, at_y = l1 + Y::PZ * l2, at_z = l1 + Y::PB * l2;
+  V v[1][N1], w[1][N1];
+  if (on) {
 #pragma unroll
-    for (int m = 0; m < N1; ++m) acc += sS[1][b * N1 + m] * u[rest + m * N1];
-    t[i] = acc;
+    for (int c = 0; c < N1; ++c) v[0][c] = __ldg(r + off + l + NF * c);
   }
   __syncthreads();
-  for (int i = threadIdx.x; i < NPE; i += blockDim.x) {
-    const int a = i % N1, rest = i - a;
-    V acc = 0;
+  if (on)
+    sw_fwd_half<V, N1, 1, N1, 0, 0, N1>(tz, RP, v, [&](int, int q, V a) { b[at_z + Y::PZ * q] = a; });
+  __syncthreads();
+  if (on) {
 #pragma unroll
-    for (int m = 0; m < N1; ++m) acc += sS[0][a * N1 + m] * t[rest + m];
-    z[off + i] = acc;
+    for (int i = 0; i < N1; ++i) v[0][i] = b[at_y + Y::PB * i];
+    sw_fwd_half<V, N1, 1, N1, 0, 0, N1>(ty, RP, v, [&](int, int q, V a) { b[at_y + Y::PB * q] = a; });
+  }
+  __syncthreads();
+  if (on) {
+#pragma unroll
+    for (int i = 0; i < N1; ++i) v[0][i] = b[at_x + i];
+    const V lyz = ty[N1 * RP + l1] + tz[N1 * RP + l2];
+    sw_mid_half<V, N1, 1, N1, 0, 0, N1>(tx, RP, v, w, [&](int, int q, V a) -> V { return a / (tx[N1 * RP + q] + lyz); });
+#pragma unroll
+    for (int i = 0; i < N1; ++i) b[at_x + i] = w[0][i];
+  }
+  __syncthreads();
+  if (on) {
+    sw_bwd_half<V, N1, 1, N1, 0, 0, N1>(ty, RP, v, [&](int, int q) -> V { return b[at_y + Y::PB * q]; });
+#pragma unroll
+    for (int i = 0; i < N1; ++i) b[at_y + Y::PB * i] = v[0][i];
+  }
+  __syncthreads();
+  if (!on) return;
+  sw_bwd_half<V, N1, 1, N1, 0, 0, N1>(tz, RP, v, [&](int, int q) -> V { return b[at_z + Y::PZ * q]; });
+#pragma unroll
+  for (int c = 0; c < N1; ++c) {
+    const long long g = off + l + NF * c;
+    V y = mode == 0 ? v[0][c] : mode == 3 ? mad(c2, v[0][c], mul(c1, z[g])) : mul(c1, v[0][c]);
+    z[g] = y;
+    if (mode != 0) x[g] = mode == 1 ? y : x[g] + y;
   }
 }
 
@@ -474,34 +506,64 @@ __global__ void k_oct_restrict_root(const int* __restrict__ rptr, const int* __r
 
 namespace dg {
 
+// per class the table of k_oct_bjac in type V: row q = mode q at the nodes (padded
+// to 16 bytes), then the eigenvalues
 template <typename V>
-static cudaError_t launch_bjac(const dg_oct* h, const OctLevel& L, const V* r, V* z, const int* act, int nact,
-                               cudaStream_t s) {
-  if (nact == 0) return cudaSuccess;
-  const dim3 grid((unsigned)h->E, (unsigned)nact);
-  const int* c = L.cls.as<int>();
-  const double *S = L.S.as<double>(), *l = L.lam.as<double>();
+static std::vector<V> oct_bjac_table(int n1, int ncls, const std::vector<double>& S, const std::vector<double>& lam) {
+  const int W = 16 / (int)sizeof(V), RP = (n1 + W - 1) / W * W, TB = (n1 + 1) * RP;
+  std::vector<V> t((size_t)ncls * TB, (V)0);
+  for (int c = 0; c < ncls; ++c)
+    for (int q = 0; q < n1; ++q) {
+      for (int a = 0; a < n1; ++a) t[(size_t)c * TB + q * RP + a] = (V)S[((size_t)c * n1 + a) * n1 + q];
+      t[(size_t)c * TB + n1 * RP + q] = (V)lam[(size_t)c * n1 + q];
+    }
+  return t;
+}
+
+template <typename V, int N1, bool FILL>
+static cudaError_t bjac_shape(const dg_oct* h, const OctLevel& L, int mode, const V* r, V* z, V* x, double c1,
+                              double c2, const int* act, int nact, cudaStream_t s) {
+  using B = OctBjac<V, N1, FILL>;
+  const long long items = (long long)h->E * nact, blocks = (items + B::BPB - 1) / B::BPB;
+  if (blocks > 0x7fffffffLL) return cudaErrorInvalidValue;
+  auto kern = k_oct_bjac<V, N1, FILL>;
+  if (B::SMEM > 48 * 1024) {
+    const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)B::SMEM);
+    if (e != cudaSuccess) return e;
+  }
   count_launch();
+  kern<<<(unsigned)blocks, B::THREADS, B::SMEM, s>>>(L.cls.as<int>(), L.bj<V>(), r, z, x, (V)c1, (V)c2, mode, h->E, items,
+                                                    act);
+  return cudaGetLastError();
+}
+
+// mode, z, x, c1, c2 as k_oct_bjac
+template <typename V>
+static cudaError_t launch_bjac(const dg_oct* h, const OctLevel& L, int mode, const V* r, V* z, V* x, double c1,
+                               double c2, const int* act, int nact, cudaStream_t s) {
+  if (nact == 0) return cudaSuccess;
   switch (L.n1) {
-#define DG_BJ(N)                                                              \
-  case N:                                                                     \
-    k_oct_bjac<V, N><<<grid, 128, 0, s>>>(c, S, l, r, z, L.Nq, act);          \
-    break;
+#define DG_BJ(N)                                                                                       \
+  case N:                                                                                              \
+    /* several leaves per block once that leaves two blocks per SM */                                  \
+    return (long long)h->E * nact / OctBjac<V, N, true>::BPB >= 304                                    \
+               ? bjac_shape<V, N, true>(h, L, mode, r, z, x, c1, c2, act, nact, s)                     \
+               : bjac_shape<V, N, false>(h, L, mode, r, z, x, c1, c2, act, nact, s);
     DG_BJ(2) DG_BJ(3) DG_BJ(4) DG_BJ(5) DG_BJ(6) DG_BJ(7) DG_BJ(8) DG_BJ(9)
 #undef DG_BJ
     default:
       return cudaErrorInvalidValue;
   }
-  return cudaGetLastError();
 }
 
+// out = A u, or with rin out = rin - A u
 template <typename V>
 static cudaError_t oct_apply(const dg_oct* h, const OctLevel& L, const V* u, V* out, const int* act, int nact,
-                             cudaStream_t s, const DevBuf* hang = nullptr) {
+                             cudaStream_t s, const V* rin = nullptr, const DevBuf* hang = nullptr) {
   if (!hang) hang = &h->hang;
   const OctMesh m{h->E, h->kind.as<int>(), h->nb.as<int>(), h->fac.as<double>(), h->hslot.as<int>(), h->rec.as<int>(),
                   h->nI};
-  return launch_octree_apply<V>(L.n1, L.T, m, h->eps, u, out, act, nact, hang->as<V>(),
+  return launch_octree_apply<V>(L.n1, L.T, m, h->eps, u, out, rin, act, nact, hang->as<V>(),
                                 (long long)(hang->bytes / sizeof(V)), s);
 }
 
@@ -569,7 +631,8 @@ static int oct_ws(dg_oct* h, int cap) {
   for (size_t l = 0; l < h->lv.size(); ++l) {
     OctLevel& L = h->lv[l];
     const size_t lvec = sizeof(double) * (size_t)cap * (size_t)L.Nq;
-    for (DevBuf* v : {&L.res, &L.d, &L.z, &L.q}) DG_CK(v->ensure(lvec));
+    for (DevBuf* v : {&L.res, &L.d}) DG_CK(v->ensure(lvec));
+    for (DevBuf* v : {&L.z, &L.q}) DG_CK(v->ensure(sizeof(double) * (size_t)L.Nq));  // one field, for oct_lambda
     if (l > 0)
       for (DevBuf* v : {&L.x, &L.b}) DG_CK(v->ensure(lvec));
   }
@@ -689,33 +752,23 @@ template <typename V>
 static int oct_cheb(dg_oct* h, int l, const V* b, V* x, bool zero_init, bool want_res, const int* act, int n,
                     cudaStream_t s) {
   OctLevel& L = h->lv[l];
-  V *res = L.res.as<V>(), *d = L.d.as<V>(), *z = L.z.as<V>(), *q = L.q.as<V>();
+  V *res = L.res.as<V>(), *d = L.d.as<V>();
   const double bmax = 1.1 * L.lam_max, amin = bmax / h->cheb_range;
   const double theta = 0.5 * (bmax + amin), delta = 0.5 * (bmax - amin), sig1 = theta / delta;
-  const dim3 vg = ogrid(L.Nq, n);
-  auto resid = [&]() -> int {
-    DG_CK(oct_apply(h, L, x, q, act, n, s));
-    count_launch();
-    k_oct_sub<<<vg, OT, 0, s>>>(res, b, q, L.Nq, act);
-    DG_CK(cudaGetLastError());
-    return DG_OK;
-  };
   const V* r0 = b;
   if (!zero_init) {
-    DG_RET(resid());
+    DG_CK(oct_apply<V>(h, L, x, res, act, n, s, b));
     r0 = res;
   }
-  DG_CK(launch_bjac(h, L, r0, z, act, n, s));
-  DG_CK(launch_cheb_first<V>(x, d, z, nullptr, 1.0 / theta, zero_init ? 1 : 0, L.Nq, act, n, s));
+  DG_CK(launch_bjac<V>(h, L, zero_init ? 1 : 2, r0, d, x, 1.0 / theta, 0.0, act, n, s));
   double rho_prev = 1.0 / sig1;
   for (int j = 2; j <= h->cheb_k; ++j) {
-    DG_RET(resid());
+    DG_CK(oct_apply<V>(h, L, x, res, act, n, s, b));
     const double rho = 1.0 / (2.0 * sig1 - rho_prev);
-    DG_CK(launch_bjac(h, L, res, z, act, n, s));
-    DG_CK(launch_cheb_step<V>(x, d, z, nullptr, rho * rho_prev, 2.0 * rho / delta, L.Nq, act, n, s));
+    DG_CK(launch_bjac<V>(h, L, 3, res, d, x, rho * rho_prev, 2.0 * rho / delta, act, n, s));
     rho_prev = rho;
   }
-  if (want_res) DG_RET(resid());
+  if (want_res) DG_CK(oct_apply<V>(h, L, x, res, act, n, s, b));
   return DG_OK;
 }
 
@@ -770,7 +823,7 @@ static int oct_vcycle(dg_oct* h, int l, const V* b, V* x, const int* act, int n,
 template <typename V>
 static int oct_precond(dg_oct* h, const V* r, V* z, const int* act, int n, cudaStream_t s) {
   if (h->precond == 0) {
-    DG_CK(launch_bjac<V>(h, h->lv[0], r, z, act, n, s));
+    DG_CK(launch_bjac<V>(h, h->lv[0], 0, r, z, nullptr, 0.0, 0.0, act, n, s));
     return DG_OK;
   }
   return oct_vcycle<V>(h, 0, r, z, act, n, s);
@@ -797,7 +850,7 @@ static int oct_lambda(dg_oct* h, int l, cudaStream_t s) {
   DG_CK(cudaStreamSynchronize(s));
   for (int it = 0; it < 30; ++it) {
     DG_CK(oct_apply(h, L, x, q, act, 1, s));
-    DG_CK(launch_bjac(h, L, q, z, act, 1, s));
+    DG_CK(launch_bjac<double>(h, L, 0, q, z, nullptr, 0.0, 0.0, act, 1, s));
     DG_CK(launch_dot(z, z, (const double*)nullptr, nrm, h->part.as<double>(), L.Nq, act, 1, s));
     DG_CK(cudaMemcpyAsync(&nz, nrm, sizeof(double), cudaMemcpyDeviceToHost, s));
     DG_CK(cudaStreamSynchronize(s));
@@ -1207,9 +1260,11 @@ int dg_octree_setup(const dg_mesh_desc* root, const int32_t* leaves, int32_t n_l
         cls[3 * (size_t)e + d] = it->second;
       }
     L.ncls = (int)cmap.size();
+    const std::vector<double> t64 = oct_bjac_table<double>(L.n1, L.ncls, Sv, lv);
+    const std::vector<float> t32 = oct_bjac_table<float>(L.n1, L.ncls, Sv, lv);
     if ((rc = up(L.cls, cls.data(), sizeof(int) * cls.size())) != DG_OK ||
-        (rc = up(L.S, Sv.data(), sizeof(double) * Sv.size())) != DG_OK ||
-        (rc = up(L.lam, lv.data(), sizeof(double) * lv.size())) != DG_OK)
+        (rc = up(L.bj64, t64.data(), sizeof(double) * t64.size())) != DG_OK ||
+        (rc = up(L.bj32, t32.data(), sizeof(float) * t32.size())) != DG_OK)
       return fail(rc);
     if (precond == 0 || pl == 1) break;
     pl = std::max(1, pl / 2);
@@ -1379,7 +1434,7 @@ int dg_octree_operator(dg_oct_handle h, const double* u_dev, double* out_dev, in
     DG_CK(cudaStreamIsCapturing(s, &cap));
     if (cap == cudaStreamCaptureStatusNone) DG_CK(cudaStreamWaitEvent(s, h->op_done, 0));
   }
-  DG_CK(oct_apply(h, h->lv[0], u_dev, out_dev, nullptr, (int)B, s, &h->hang_op));
+  DG_CK(oct_apply<double>(h, h->lv[0], u_dev, out_dev, nullptr, (int)B, s, nullptr, &h->hang_op));
   if (h->nI > 0 && cap == cudaStreamCaptureStatusNone) DG_CK(cudaEventRecord(h->op_done, s));
   return DG_OK;
 }
