@@ -40,21 +40,6 @@
 
 namespace dg {
 
-#ifndef DG_APPLY_TIE32
-#define DG_APPLY_TIE32 128
-#endif
-#ifndef DG_APPLY_TIE64
-#define DG_APPLY_TIE64 64
-#endif
-#ifndef DG_APPLY_WANT32
-#define DG_APPLY_WANT32 768
-#endif
-#ifndef DG_APPLY_WANT64
-#define DG_APPLY_WANT64 640
-#endif
-#ifndef DG_APPLY_MIN_BLOCKS
-#define DG_APPLY_MIN_BLOCKS 304  // blocks that fill the chip (two per SM)
-#endif
 
 // 1-D tables of one level, folded into even and odd halves (host-built, passed
 // by value). HE = ceil(N1/2) even and HO = floor(N1/2) odd rows.
@@ -119,20 +104,18 @@ static void fill_tab(ApplyTab<T, N1>& t, const LevelOp& op) {
   t.Nq = op.Nq;
 }
 
-// Launch shape. BR: elements of a brick along each axis (2 or 1). FILL: several
-// bricks per block, so that warps are full; otherwise one, for problems too
-// small to give every SM a block.
-template <typename T, int N1, int BR, bool FILL>
+// Launch shape. BR: elements of a brick along each axis (2 or 1).
+template <typename T, int N1, int BR>
 struct ApplyCfg {
   static constexpr int NPE = N1 * N1 * N1, NF = N1 * N1;
   static constexpr int EB = BR * BR * BR;        // elements of a brick
   static constexpr int LINES = BR * BR * NF;     // threads of a brick: one (pair of) line(s) each
   static constexpr int PB = LineLayout<N1>::PB, PZ = LineLayout<N1>::PZ, ES = LineLayout<N1>::ES;
-  static constexpr int BPB = FILL ? best_bpb(LINES, sizeof(T) == 4 ? DG_APPLY_TIE32 : DG_APPLY_TIE64) : 1;
+  static constexpr int BPB = best_bpb(LINES, sizeof(T) == 4 ? 128 : 64);
   static constexpr int THREADS = (BPB * LINES + 31) / 32 * 32;
   static constexpr size_t SMEM = sizeof(T) * 2 * (size_t)BPB * EB * ES;
   // resident threads per SM asked of ptxas (register cap 65536 / that)
-  static constexpr int WANT = sizeof(T) == 4 ? DG_APPLY_WANT32 : DG_APPLY_WANT64;
+  static constexpr int WANT = sizeof(T) == 4 ? 768 : 640;
   static constexpr int MINB = WANT / THREADS < 1 ? 1 : WANT / THREADS;
 };
 
@@ -245,11 +228,11 @@ __device__ __forceinline__ void outer_traces(const ApplyTab<T, N1>& tab, const T
   }
 }
 
-template <typename T, int N1, int BR, bool FILL>
-__global__ void __launch_bounds__(ApplyCfg<T, N1, BR, FILL>::THREADS, ApplyCfg<T, N1, BR, FILL>::MINB)
+template <typename T, int N1, int BR>
+__global__ void __launch_bounds__(ApplyCfg<T, N1, BR>::THREADS, ApplyCfg<T, N1, BR>::MINB)
     k_apply(const __grid_constant__ ApplyTab<T, N1> tab, const T* __restrict__ u, T* __restrict__ out,
             const T* __restrict__ rin, const int* __restrict__ act, int mode, int vec_i) {
-  using C = ApplyCfg<T, N1, BR, FILL>;
+  using C = ApplyCfg<T, N1, BR>;
   constexpr int NPE = C::NPE, NF = C::NF, EB = C::EB, BPB = C::BPB, LINES = C::LINES;
   constexpr int PB = C::PB, PZ = C::PZ, ES = C::ES;
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -391,10 +374,92 @@ __global__ void __launch_bounds__(ApplyCfg<T, N1, BR, FILL>::THREADS, ApplyCfg<T
 #undef DG_OUT
 }
 
-template <typename T, int N1, int BR, bool FILL>
+// The operator where there are too few elements to fill the chip: one element per
+// block and a group of threads per direction, which work at the same time (a warp
+// issues an FP64 operation every 67 cycles whatever else it has to do, so the chain
+// that a thread runs is the kernel's time). The three results are scaled and added
+// in the order of k_apply: the same bits.
+// Measured (GB300, FP64, in a graph; the passes one after the other before): 4^3, p =
+// 4, 4 fields 10.3 -> 6.2 us, 5 x 7 x 3, p = 5, 3 fields 24.0 -> 15.7 us, 4^3, p = 8, 1
+// field 31.6 -> 14.3 us.
+template <int N1>
+struct ApplySmall {
+  static constexpr int GROUP = (N1 * N1 + 31) / 32 * 32;  // whole warps per direction
+  static constexpr int THREADS = 3 * GROUP;
+};
+
+template <typename T, int N1, int D>
+__device__ __forceinline__ void small_pass(const ApplyTab<T, N1>& tab, const T* su, T* res, int l1, int l2, const T* ov,
+                                           const T* od) {
+  using Y = LineLayout<N1>;
+  constexpr int ST = D == 0 ? 1 : (D == 1 ? Y::PB : Y::PZ);
+  const int at = D == 0 ? Y::PB * l1 + Y::PZ * l2 : (D == 1 ? l1 + Y::PZ * l2 : l1 + Y::PB * l2);
+  T v[1][N1];
+#pragma unroll
+  for (int i = 0; i < N1; ++i) v[0][i] = su[at + ST * i];
+  line_op<T, N1, 1, D>(tab, v, ov, od, false);
+#pragma unroll
+  for (int i = 0; i < N1; ++i) res[at + ST * i] = v[0][i];
+}
+
+template <typename T, int N1>
+__global__ void __launch_bounds__(ApplySmall<N1>::THREADS)
+    k_apply_small(const __grid_constant__ ApplyTab<T, N1> tab, const T* __restrict__ u, T* __restrict__ out,
+                  const T* __restrict__ rin, const int* __restrict__ act, int mode, int vec_i) {
+  using Y = LineLayout<N1>;
+  constexpr int NF = N1 * N1, NPE = NF * N1, GROUP = ApplySmall<N1>::GROUP, NT = ApplySmall<N1>::THREADS;
+  __shared__ T su[Y::ES], sr[3][Y::ES];
+  const int nx = tab.n[0], ny = tab.n[1], E = nx * ny * tab.n[2];
+  const int k = blockIdx.x / E, e = blockIdx.x - k * E;
+  const int ex = e % nx, eq = e / nx, ey = eq % ny, ez = eq / ny;
+  const long long g0 = (long long)act[k] * tab.Nq + (long long)e * NPE;
+  const T* ue = u + g0;
+  for (int t = threadIdx.x; t < NPE; t += NT) su[t % N1 + Y::PB * ((t / N1) % N1) + Y::PZ * (t / NF)] = __ldg(ue + t);
+  const int d = threadIdx.x / GROUP, l = threadIdx.x - d * GROUP, l1 = l % N1, l2 = l / N1;
+  const bool on = l < NF, vec = vec_i != 0;
+  T ov[2], od[2];
+  if (on) {
+    if (d == 0)
+      outer_traces<T, N1, 1, 0>(tab, ue, 0, l1, l2, 1, false, ex > 0, ex < nx - 1, vec, ov, od);
+    else if (d == 1)
+      outer_traces<T, N1, 1, 1>(tab, ue, 0, l1, l2, nx, false, ey > 0, ey < ny - 1, vec, ov, od);
+    else
+      outer_traces<T, N1, 1, 2>(tab, ue, 0, l1, l2, (long long)nx * ny, false, ez > 0, ez < tab.n[2] - 1, vec, ov, od);
+  }
+  __syncthreads();
+  if (on) {
+    if (d == 0)
+      small_pass<T, N1, 0>(tab, su, sr[0], l1, l2, ov, od);
+    else if (d == 1)
+      small_pass<T, N1, 1>(tab, su, sr[1], l1, l2, ov, od);
+    else
+      small_pass<T, N1, 2>(tab, su, sr[2], l1, l2, ov, od);
+  }
+  __syncthreads();
+  for (int t = threadIdx.x; t < NPE; t += NT) {
+    const int a = t % N1, b = (t / N1) % N1, c = t / NF, at = a + Y::PB * b + Y::PZ * c;
+    T Au = mul(tab.mm[0][b + N1 * c], sr[0][at]);
+    Au = mad(tab.mm[1][a + N1 * c], sr[1][at], Au);
+    Au = mad(tab.mm[2][a + N1 * b], sr[2][at], Au);
+    out[g0 + t] = mode == 0 ? Au : (mode == 1 ? rin : out)[g0 + t] - Au;
+  }
+}
+
+template <typename T, int N1>
+static cudaError_t apply_small(const LevelOp& hop, int mode, const T* u, T* out, const T* rin, const int* act, int nact,
+                               cudaStream_t s) {
+  ApplyTab<T, N1> tab;
+  fill_tab<T, N1>(tab, hop);
+  const int vec = ((uintptr_t)u & 15) == 0 && (N1 * N1 * N1 * sizeof(T)) % 16 == 0 && (hop.Nq * sizeof(T)) % 16 == 0;
+  count_launch();
+  k_apply_small<T, N1><<<(unsigned)(hop.E * nact), ApplySmall<N1>::THREADS, 0, s>>>(tab, u, out, rin, act, mode, vec);
+  return cudaGetLastError();
+}
+
+template <typename T, int N1, int BR>
 static cudaError_t apply_br(const LevelOp& hop, int mode, const T* u, T* out, const T* rin, const int* act, int nact,
                             cudaStream_t s) {
-  using C = ApplyCfg<T, N1, BR, FILL>;
+  using C = ApplyCfg<T, N1, BR>;
   ApplyTab<T, N1> tab;
   fill_tab<T, N1>(tab, hop);
   long long per = 1;
@@ -407,7 +472,7 @@ static cudaError_t apply_br(const LevelOp& hop, int mode, const T* u, T* out, co
   if (blocks > 0x7fffffffLL) return cudaErrorInvalidValue;
   // 16-byte reads of an element's values: the field and every element of it aligned
   const int vec = ((uintptr_t)u & 15) == 0 && (C::NPE * sizeof(T)) % 16 == 0 && (hop.Nq * sizeof(T)) % 16 == 0;
-  auto kern = k_apply<T, N1, BR, FILL>;
+  auto kern = k_apply<T, N1, BR>;
   if (C::SMEM > 48 * 1024) {
     const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)C::SMEM);
     if (e != cudaSuccess) return e;
@@ -417,24 +482,34 @@ static cudaError_t apply_br(const LevelOp& hop, int mode, const T* u, T* out, co
   return cudaGetLastError();
 }
 
-// Bricks of eight elements in FP32, where reading the neighbours is what bounds
-// the kernel; single elements in FP64 (bound by the FP64 pipe, to which a brick
-// saves nothing) and where bricks would leave SMs idle or, on odd meshes, hold
-// less than half of the elements that they have room for.
+// Few elements: one group of threads per direction, while its warps are at most 24 per
+// SM in FP64, and 13 in FP32 or where N1^2 divides 32 (p = 1, 3: the other kernel's
+// warps are full there). Measured around the line (us, small / single elements): FP64
+// p = 4 256 elements 6.2 / 10.3, 1024 15.3 / 17.1, 4096 51 / 47; p = 6 512 23.6 / 23.9,
+// 2048 76 / 67; p = 8 256 24.8 / 31.8; p = 2 1024 9.4 / 12.4; p = 3 512 7.7 / 7.7, 2048
+// 22 / 14; p = 1 512 4.7 / 5.1, 2048 12.1 / 5.1; FP32 p = 5 315 3.7 / 4.2, 1260 6.3 /
+// 5.1; p = 4 256 2.9 / 3.3, 1024 3.9 / 3.6; p = 8 64 4.0 / 4.4, 256 5.4 / 4.5.
+// Then bricks of eight elements in FP32, where reading the neighbours is what bounds
+// the kernel (single elements / bricks: p = 6 4096 elements 10.7 / 8.2 us, 512 4.1 /
+// 4.5; p = 5 2880 6.5 / 6.3, 960 4.3 / 4.9), with two blocks for every SM and, on odd
+// meshes, at least half of the elements that the bricks have room for; single
+// elements otherwise and in FP64 (bound by the FP64 pipe, to which a brick saves
+// nothing).
 template <typename T, int N1>
 static cudaError_t apply_n1(const LevelOp& hop, int mode, const T* u, T* out, const T* rin, const int* act, int nact,
                             cudaStream_t s) {
   if (nact == 0) return cudaSuccess;
   const long long items = (long long)nact * hop.E;
+  constexpr int warps = sizeof(T) == 8 && 32 % (N1 * N1) != 0 ? 24 : 13;
+  if (items * (ApplySmall<N1>::THREADS / 32) <= 152 * warps)
+    return apply_small<T, N1>(hop, mode, u, out, rin, act, nact, s);
   if constexpr (sizeof(T) == 4) {
     long long br = nact;
     for (int d = 0; d < 3; ++d) br *= (hop.n[d] + 1) / 2;
-    if (br / ApplyCfg<T, N1, 2, true>::BPB >= DG_APPLY_MIN_BLOCKS && 8 * br <= 2 * items)
-      return apply_br<T, N1, 2, true>(hop, mode, u, out, rin, act, nact, s);
+    if (br / ApplyCfg<T, N1, 2>::BPB >= 2 * 152 && 8 * br <= 2 * items)
+      return apply_br<T, N1, 2>(hop, mode, u, out, rin, act, nact, s);
   }
-  if (items / ApplyCfg<T, N1, 1, true>::BPB >= DG_APPLY_MIN_BLOCKS)
-    return apply_br<T, N1, 1, true>(hop, mode, u, out, rin, act, nact, s);
-  return apply_br<T, N1, 1, false>(hop, mode, u, out, rin, act, nact, s);
+  return apply_br<T, N1, 1>(hop, mode, u, out, rin, act, nact, s);
 }
 
 template <typename T>

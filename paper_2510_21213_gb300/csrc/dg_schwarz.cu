@@ -78,10 +78,10 @@ struct SwCfg {
   }
 };
 
-template <typename T, int N1, bool FILL>
+template <typename T, int N1>
 struct SwShape {
   using C = SwCfg<T, N1>;
-  static constexpr int EPB = FILL ? C::slots(sizeof(T) == 4 ? 128 : 64) : (C::TPE >= 32 ? 1 : 32 / C::TPE);
+  static constexpr int EPB = C::slots(sizeof(T) == 4 ? 128 : 64);
   static constexpr int THREADS = (EPB * C::TPE + 31) / 32 * 32;
   // resident threads per SM asked of ptxas (p = 6, 8^3, 56 sources: 101 us at 640, 104 at 768, 147 at 1024; two or
   // one line per thread instead of three 105 to 117)
@@ -90,12 +90,12 @@ struct SwShape {
   static constexpr size_t SMEM = sizeof(T) * ((size_t)SW_MAXCLS * 3 * C::TB + (size_t)EPB * C::SE);
 };
 
-template <typename T, int N1, bool FILL>
-__global__ void __launch_bounds__(SwShape<T, N1, FILL>::THREADS, SwShape<T, N1, FILL>::MINB)
+template <typename T, int N1>
+__global__ void __launch_bounds__(SwShape<T, N1>::THREADS, SwShape<T, N1>::MINB)
     k_schwarz_patch(const __grid_constant__ SwGeom g, const unsigned char* __restrict__ blob, const T* __restrict__ r,
                     T* __restrict__ zp, const int* __restrict__ act, int nact) {
   using C = SwCfg<T, N1>;
-  using H = SwShape<T, N1, FILL>;
+  using H = SwShape<T, N1>;
   constexpr int MP = C::MP, MP2 = C::MP2, MP3 = C::MP3, NF = N1 * N1, NPE = NF * N1;
   constexpr int SJ = C::SJ, SK = C::SK, SE = C::SE, RP = C::RP, TB = C::TB, TPE = C::TPE, LPT = C::LPT;
   constexpr int EPB = H::EPB, NT = H::THREADS;
@@ -263,13 +263,210 @@ __global__ void __launch_bounds__(SwShape<T, N1, FILL>::THREADS, SwShape<T, N1, 
   }
 }
 
-template <typename T, int N1, bool FILL>
-static cudaError_t patch_shape(const SwTables& tb, const T* r, T* zp, const int* act, int nact, cudaStream_t s) {
-  using H = SwShape<T, N1, FILL>;
+// The same patch solves where there are too few patches to fill the chip: one
+// patch per block and two lanes per line, so that the chain of operations that a
+// thread runs is half as long (a warp issues an FP64 operation every 67 cycles
+// whatever else it has to do, so at 4^3 elements and p = 4 that chain is the
+// kernel's time). Lane h = 0 takes the even modes (of a patch without symmetry the
+// first half of the modes, and of the nodes on the way back), h = 1 the rest; even
+// and odd parts of the nodes change hands by a shuffle. Each sum is that of
+// k_schwarz_patch, so the results are the same bits. Only the patch's own three
+// tables are staged, and the reciprocals are loaded up front.
+// Measured (GB300, FP64, inside a solve; one lane per line before): 4^3, 4 sources, p =
+// 4 14.1 -> 13.3 us, p = 2 8.9 -> 6.0.
+template <typename T, int N1>
+struct SwSmall {
+  using C = SwCfg<T, N1>;
+  static constexpr int THREADS = (2 * C::MP2 + 31) / 32 * 32;
+  static constexpr size_t SMEM = sizeof(T) * (3 * C::TB + (size_t)C::SE);
+};
+
+// modes h HE + t of the line v: put(t, sum_i S[i][q] v[i])
+template <typename T, int MP, int RP, typename P>
+__device__ __forceinline__ void sw_fwd2(bool sym, const T* tb, int h, const T* v, P&& put) {
+  constexpr int HO = MP / 2, HE = MP - HO;
+  const T* row = tb + h * HE * RP;
+  const int n = h ? HO : HE;
+  if (sym) {
+    T x[HE];
+#pragma unroll
+    for (int i = 0; i < HO; ++i) x[i] = h ? v[i] - v[MP - 1 - i] : v[i] + v[MP - 1 - i];
+    if (HE > HO) x[HE - 1] = h ? (T)0 : v[HO];  // the odd rows are zero there
+#pragma unroll
+    for (int t = 0; t < HE; ++t)
+      if (t < n) {
+        T a = row[t * RP] * x[0];
+#pragma unroll
+        for (int i = 1; i < HE; ++i) a += row[t * RP + i] * x[i];
+        put(t, a);
+      }
+  } else {
+#pragma unroll
+    for (int t = 0; t < HE; ++t)
+      if (t < n) {
+        T a = row[t * RP] * v[0];
+#pragma unroll
+        for (int i = 1; i < MP; ++i) a += row[t * RP + i] * v[i];
+        put(t, a);
+      }
+  }
+}
+// nodes from the modes at line + st q: put(node, value) for this lane's nodes (the
+// first HE with h = 0, the others with h = 1), after every lane has read its modes.
+// Every lane of the warp takes part.
+template <typename T, int MP, int RP, typename P>
+__device__ __forceinline__ void sw_bwd2(bool sym, const T* tb, int h, const T* line, int st, P&& put) {
+  constexpr int HO = MP / 2, HE = MP - HO;
+  T x[HE];
+#pragma unroll
+  for (int t = 0; t < HE; ++t) x[t] = (T)0;
+  if (sym) {
+    const int n = h ? HO : HE;
+#pragma unroll
+    for (int t = 0; t < HE; ++t)
+      if (t < n) {
+        const int q = h * HE + t;
+        const T c = line[st * q];
+#pragma unroll
+        for (int i = 0; i < HE; ++i) x[i] += tb[q * RP + i] * c;
+      }
+    __syncwarp();
+#pragma unroll
+    for (int i = 0; i < HO; ++i) {
+      const T y = __shfl_xor_sync(0xffffffffu, x[i], 1);
+      if (h == 0)
+        put(i, x[i] + y);
+      else
+        put(MP - 1 - i, y - x[i]);
+    }
+    if (HE > HO && h == 0) put(HO, x[HE - 1]);
+  } else {
+#pragma unroll
+    for (int q = 0; q < MP; ++q) {
+      const T c = line[st * q];
+#pragma unroll
+      for (int t = 0; t < HE; ++t)
+        if (t < HO || h == 0) x[t] += tb[q * RP + h * HE + t] * c;
+    }
+    __syncwarp();
+#pragma unroll
+    for (int t = 0; t < HE; ++t)
+      if (t < HO || h == 0) put(h * HE + t, x[t]);
+  }
+}
+
+template <typename T, int N1>
+__global__ void __launch_bounds__(SwSmall<T, N1>::THREADS)
+    k_schwarz_patch_small(const __grid_constant__ SwGeom g, const unsigned char* __restrict__ blob,
+                          const T* __restrict__ r, T* __restrict__ zp, const int* __restrict__ act) {
+  using C = SwCfg<T, N1>;
+  constexpr int MP = C::MP, MP2 = C::MP2, MP3 = C::MP3, NF = N1 * N1, NPE = NF * N1, HE = C::HE, HO = C::HO;
+  constexpr int SJ = C::SJ, SK = C::SK, RP = C::RP, TB = C::TB, NT = SwSmall<T, N1>::THREADS;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  T* tabs = reinterpret_cast<T*>(smem_raw);
+  T* b = tabs + 3 * TB;
+  const int nx = g.n[0], ny = g.n[1], E = nx * ny * g.n[2];
+  const int k = blockIdx.x / E, e = blockIdx.x - k * E;
+  const int ex = e % nx, eq = e / nx, ey = eq % ny, ez = eq / ny;
+  const int* pos = reinterpret_cast<const int*>(blob + g.pos_off);
+  const int px = __ldg(pos + ex), py = __ldg(pos + nx + ey), pz = __ldg(pos + nx + ny + ez);
+  const long long src = act[k], Nq = (long long)E * NPE;
+  const T* gt = reinterpret_cast<const T*>(blob + g.tab_off);
+  const int from[3] = {sw_tab(px), sw_tab(py), sw_tab(pz)};
+#pragma unroll
+  for (int d = 0; d < 3; ++d)
+    for (int t = threadIdx.x; t < TB / C::W; t += NT)
+      reinterpret_cast<uint4*>(tabs + d * TB)[t] = __ldg(reinterpret_cast<const uint4*>(gt + from[d] * TB) + t);
+  const T *tx = tabs, *ty = tabs + TB, *tz = tabs + 2 * TB;
+  const int h = threadIdx.x & 1, l0 = threadIdx.x >> 1;
+  const bool on = l0 < MP2;
+  const int l = on ? l0 : 0, l1 = l % MP, l2 = l / MP;
+  // z line (i, j) = (l1, l2) of the patch residual, zero outside the domain
+  T v[MP], inv[HE];
+  {
+    const int oLx = sw_halo(px), oLy = sw_halo(py), oLz = sw_halo(pz);
+    const int mz = sw_size(pz);
+    const bool in = on && l1 < sw_size(px) && l2 < sw_size(py);
+    int a = l1 - oLx, bb = l2 - oLy, ee = e;
+    if (a < 0) {
+      a = N1 - 1;
+      ee -= 1;
+    } else if (a >= N1) {
+      a = 0;
+      ee += 1;
+    }
+    if (bb < 0) {
+      bb = N1 - 1;
+      ee -= nx;
+    } else if (bb >= N1) {
+      bb = 0;
+      ee += nx;
+    }
+    const T* p = r + src * Nq + (long long)ee * NPE + (a + N1 * bb);
+    const long long pe = (long long)nx * ny * NPE;
+    const T *below = p - pe + (N1 - 1) * NF, *own = p - oLz * NF, *above = p + pe;
+    v[0] = in ? __ldg(oLz ? below : own) : (T)0;
+#pragma unroll
+    for (int c = 1; c < N1; ++c) v[c] = in ? __ldg(own + NF * c) : (T)0;
+    v[N1] = in && N1 < mz ? __ldg(oLz ? own + NF * N1 : above) : (T)0;
+    v[N1 + 1] = in && N1 + 1 < mz ? __ldg(above) : (T)0;
+  }
+  if constexpr (sizeof(T) == 8) {
+    const T* ip = reinterpret_cast<const T*>(blob + g.inv_off) +
+                  (((long long)sw_cls(pz) * SW_MAXCLS + sw_cls(py)) * SW_MAXCLS + sw_cls(px)) * MP3 + l;
+#pragma unroll
+    for (int t = 0; t < HE; ++t) inv[t] = t < HO || h == 0 ? __ldg(ip + (h * HE + t) * MP2) : (T)0;
+  }
+  __syncthreads();
+  const int az = l1 + SJ * l2, ay = l1 + SK * l2, ax = SJ * l1 + SK * l2;
+  sw_fwd2<T, MP, RP>(sw_sym(pz), tz, h, v, [&](int t, T a) {
+    if (on) b[az + SK * (h * HE + t)] = a;
+  });
+  __syncthreads();
+#pragma unroll
+  for (int j = 0; j < MP; ++j) v[j] = b[ay + SJ * j];
+  __syncwarp();
+  sw_fwd2<T, MP, RP>(sw_sym(py), ty, h, v, [&](int t, T a) {
+    if (on) b[ay + SJ * (h * HE + t)] = a;
+  });
+  __syncthreads();
+#pragma unroll
+  for (int i = 0; i < MP; ++i) v[i] = b[ax + i];
+  __syncwarp();
+  const T lyz = ty[MP * RP + l1] + tz[MP * RP + l2];
+  sw_fwd2<T, MP, RP>(sw_sym(px), tx, h, v, [&](int t, T a) {
+    if constexpr (sizeof(T) == 8)
+      a *= inv[t];
+    else
+      a = __fdividef(a, tx[MP * RP + h * HE + t] + lyz);
+    if (on) b[ax + h * HE + t] = a;
+  });
+  __syncwarp();
+  // back: the values of a line's other lane are read before any of its nodes is written
+  auto back = [&](bool sym, const T* tb, int at, int st, auto&& put) {
+    sw_bwd2<T, MP, RP>(sym, tb, h, b + at, st, put);
+  };
+  back(sw_sym(px), tx, ax, 1, [&](int i, T a) {
+    if (on) b[ax + i] = a;
+  });
+  __syncthreads();
+  back(sw_sym(py), ty, ay, SJ, [&](int j, T a) {
+    if (on) b[ay + SJ * j] = a;
+  });
+  __syncthreads();
+  T* out = zp + (src * E + e) * MP3 + l;
+  back(sw_sym(pz), tz, az, SK, [&](int kk, T a) {
+    if (on) out[MP2 * kk] = a;
+  });
+}
+
+template <typename T, int N1>
+static cudaError_t patch_fill(const SwTables& tb, const T* r, T* zp, const int* act, int nact, cudaStream_t s) {
+  using H = SwShape<T, N1>;
   const SwGeom& g = tb.geom;
   const long long items = (long long)g.n[0] * g.n[1] * g.n[2] * nact;
   const long long groups = (items + H::EPB - 1) / H::EPB;
-  auto kern = k_schwarz_patch<T, N1, FILL>;
+  auto kern = k_schwarz_patch<T, N1>;
   if (H::SMEM > 48 * 1024) {
     const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)H::SMEM);
     if (e != cudaSuccess) return e;
@@ -283,13 +480,23 @@ static cudaError_t patch_shape(const SwTables& tb, const T* r, T* zp, const int*
   return cudaGetLastError();
 }
 
-// Several patches per block, so that warps are full, once there are two such
-// blocks per SM; below that as many blocks as possible.
+// Few patches (the warps of k_schwarz_patch_small at most 24 per SM, at p = 8 8): one
+// patch per block and two lanes per line; otherwise several per block, so that warps
+// are full.
+// Measured around the line (us, small / several): FP64 p = 4 256 patches 13.3 / 22.4,
+// 1024 41.3 / 41.5, 4096 152 / 119; p = 6 512 54 / 68, 1024 103 / 100; p = 8 64 28.1 /
+// 29.7, 256 53.7 / 50.1; p = 1 512 4.2 / 6.6, 4096 14.6 / 14.1; FP32 p = 6 512 6.2 / 7.9, 1024 9.2 / 8.0; p = 4 256 3.2 / 4.4,
+// 1024 5.6 / 5.0; p = 2 1024 3.5 / 5.7.
 template <typename T, int N1>
 static cudaError_t patch_n1(const SwTables& tb, const T* r, T* zp, const int* act, int nact, cudaStream_t s) {
   const long long items = (long long)tb.geom.n[0] * tb.geom.n[1] * tb.geom.n[2] * nact;
-  if (items / SwShape<T, N1, true>::EPB >= 2 * 152) return patch_shape<T, N1, true>(tb, r, zp, act, nact, s);
-  return patch_shape<T, N1, false>(tb, r, zp, act, nact, s);
+  if (items * (SwSmall<T, N1>::THREADS / 32) > 152 * (N1 < 9 ? 24 : 8)) return patch_fill<T, N1>(tb, r, zp, act, nact, s);
+  using S = SwSmall<T, N1>;
+  static_assert(S::SMEM <= 48 * 1024, "one patch and its tables");
+  count_launch();
+  k_schwarz_patch_small<T, N1><<<(unsigned)items, S::THREADS, S::SMEM, s>>>(tb.geom, (const unsigned char*)tb.blob, r,
+                                                                           zp, act);
+  return cudaGetLastError();
 }
 
 // Gather block shape: GE elements of NPE nodes per block (several small
