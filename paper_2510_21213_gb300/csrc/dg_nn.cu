@@ -55,7 +55,8 @@ struct NNCfg {
   static constexpr int P3 = P * P * P;
   static constexpr int NPE = N1 * N1 * N1;
   static constexpr int MT = (NPE + 15) / 16;  // 16-node tiles
-  static constexpr int THREADS = 256;
+  // elements that the backward kernel works on at once, each with its own border
+  static constexpr int GROUP = N1 == 2 ? 12 : (N1 == 3 ? 8 : (N1 == 4 ? 4 : (N1 == 5 ? 2 : 1)));
 };
 
 template <int N1>
@@ -63,6 +64,13 @@ __device__ __forceinline__ int pad_index(int n) {
   constexpr int P = N1 + 2;
   const int x = n % N1, y = (n / N1) % N1, z = n / (N1 * N1);
   return (z + 1) * P * P + (y + 1) * P + (x + 1);
+}
+// the same for node n of a group of elements
+template <int N1>
+__device__ __forceinline__ int group_index(int n) {
+  using C = NNCfg<N1>;
+  if constexpr (C::GROUP == 1) return pad_index<N1>(n);
+  return n / C::NPE * C::P3 + pad_index<N1>(n % C::NPE);
 }
 template <int N1>
 __device__ __forceinline__ int tap_offset(int t) {
@@ -247,204 +255,366 @@ __global__ void __launch_bounds__(NN_FWD_THREADS, 1)
 
 // ---------------------------------------------------------------------------
 // backward: per-block partial gradients, reduced in a fixed order afterwards
+//
+// One block per SM, 16 warps. All four weight contractions are matrix products
+// on the tensor cores (mma.sync BF16, FP32 accumulate):
+//   dW2[t] (ci x co)  += a1[n + t]^T g_a2[n]           K = nodes
+//   g_a1[n]           = sum_t g_a2[n - t] W2[t]^T      K = channels
+//   dW3[t] (ci x co)  += a2[n]^T g3[n - t]             K = nodes
+//   dW1[t] (co x ci)  += g_a1[n]^T in[n + t]           K = nodes
+// The last two have an FP32 operand (g3, in) with two channels: each value is
+// split exactly into three BF16 numbers (24 bits), so the two channels fill six
+// of the eight columns of one MMA tile and the products are those of the FP32
+// values; an element's sums are added up and joined to a compensated running sum,
+// and the blocks' partials are added in FP64 (the error against float64 sums of
+// the same operands stays below that of the FP32 chains before).
+// In SIMT form these two took 885 k products per element at two shared-memory
+// loads each, most of the kernel's time. Shared-memory activations are swizzled
+// as in the forward kernel (unswizzled rows put an ldmatrix phase on four banks),
+// W2 stays in shared memory, and operand tiles are loaded once for all taps of a
+// warp. g_a2 (FP32 weights and inputs, K = 54) stays on the FP32 pipe, 16
+// channels of a node per thread.
+// Measured (GB300, 16384 elements, p = 7): 28.8 -> 7.2 ms; 2000 elements at p = 6
+// 6.7 -> 1.18 ms. Elements with few nodes go through in groups (p = 1: up to 12),
+// since one of them fills neither the warps nor an MMA row tile: 4000 elements at p =
+// 1 0.294 -> 0.141 ms (one at a time 0.476), 500 at p = 4 0.587 -> 0.155 ms (0.179).
 // ---------------------------------------------------------------------------
-template <int N1>
-__global__ void __launch_bounds__(256, 1)
-    k_nn_backward(const float* __restrict__ prm, const __nv_bfloat16* __restrict__ W2o, const float* __restrict__ in,
-                  const __nv_bfloat16* __restrict__ a1g, const __nv_bfloat16* __restrict__ a2g,
-                  const float* __restrict__ gout, float* __restrict__ part, long long ne) {
-  using C = NNCfg<N1>;
-  constexpr int P3 = C::P3, NPE = C::NPE, MT = C::MT;
-  extern __shared__ __align__(16) unsigned char smem[];
-  // sA1 holds a1 until the layer-2 weight gradient is done, then g_a1 (masked);
-  // the BF16 arrays come first: ldmatrix rows must be 16-byte aligned
-  __nv_bfloat16* sA1 = (__nv_bfloat16*)smem;                           // [P3][32]
-  __nv_bfloat16* sA2 = sA1 + P3 * NN_H;                                 // [P3][32] -> g_a2 (masked)
-  float* sIn = (float*)(sA2 + P3 * NN_H);                              // [P3][2]
-  float* sG3 = sIn + 2 * P3;                                           // [P3][2]
-  float* sW3 = sG3 + 2 * P3;                                           // [27][32][2]
-  float* dW1 = sW3 + 1728;                                             // [27][2][32]
-  float* dW3 = dW1 + 1728;                                             // [27][32][2]
-  float* db = dW3 + 1728;                                              // b1[32] b2[32] b3[2]
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  for (int i = tid; i < 4 * P3; i += 256) sIn[i] = 0.f;  // sIn and sG3
-  for (int i = tid; i < 2 * P3 * NN_H; i += 256) sA1[i] = __float2bfloat16(0.f);
-  for (int i = tid; i < 1728; i += 256) sW3[i] = prm[NN_OW3 + i];
-  for (int i = tid; i < 1728 * 2 + 66; i += 256) dW1[i] = 0.f;
-  // dW2 accumulators: warp owns taps warp, warp + 8, warp + 16, warp + 24 (< 27);
-  // per tap 32 (ci) x 32 (co) = 2 x 4 mma tiles
-  float accW[4][2][4][4];
+constexpr int NN_BWD_THREADS = 512;
+
+__device__ __forceinline__ void ldsm_x2_t(unsigned addr, unsigned& r0, unsigned& r1) {
+  asm volatile("ldmatrix.sync.aligned.m8n8.x2.trans.shared.b16 {%0,%1}, [%2];" : "=r"(r0), "=r"(r1) : "r"(addr));
+}
+
+// x = hi + mid + lo exactly (8 bits each, truncated); what is not finite stays in hi
+__device__ __forceinline__ void split3(float x, __nv_bfloat16* o) {
+  const unsigned b = __float_as_uint(x);
+  const bool fin = (b & 0x7f800000u) != 0x7f800000u;
+  const float hi = fin ? __uint_as_float(b & 0xffff0000u) : x;
+  const float r1 = fin ? x - hi : 0.f;
+  const float mid = __uint_as_float(__float_as_uint(r1) & 0xffff0000u);
+  o[0] = __float2bfloat16(hi);
+  o[1] = __float2bfloat16(mid);
+  o[2] = __float2bfloat16(r1 - mid);
+}
+
+// shared-memory index of entry (row, co) of the staged W2o
+__device__ __forceinline__ int swz_w2(int row, int co) {
+  return row * 32 + ((((co >> 3) ^ ((row >> 1) & 3)) << 3) | (co & 7));
+}
+
+// Adds one element's tile sums (rows g, g + 8; columns = three split parts of two
+// channels) to the running sum, compensated (TwoSum): lane c4 keeps row g + 8 (c4 >> 1), channel c4 & 1.
+__device__ __forceinline__ void join3(const float* d, int c4, float& run, float& car) {
+  float x[4];
 #pragma unroll
-  for (int a = 0; a < 4; ++a)
+  for (int h = 0; h < 2; ++h) {
+    const float p = d[2 * h] + d[2 * h + 1];
+    x[2 * h] = c4 == 0 ? p : (c4 == 1 ? d[2 * h] : 0.f);
+    x[2 * h + 1] = c4 == 2 ? p : (c4 == 1 ? d[2 * h + 1] : 0.f);
+  }
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    x[k] += __shfl_xor_sync(0xffffffffu, x[k], 1);
+    x[k] += __shfl_xor_sync(0xffffffffu, x[k], 2);
+  }
+  const float v = c4 == 0 ? x[0] : c4 == 1 ? x[1] : c4 == 2 ? x[2] : x[3];
+  const float t = run + v, b = t - run;
+  car += (run - (t - b)) + (v - b);
+  run = t;
+}
+
+// per-tap contraction over the nodes of the element with split columns:
+// acc[a] (32 rows x 8 columns) = sum_n act[n]^T col[n + sgn off(tap a)] for this
+// warp's taps, joined to run[a][m] every JOIN node tiles. The tensor core rounds
+// its accumulator toward zero: dW1 is 4.5e-7 off its float64 sums at 16384 elements
+// with one chain over the element (JOIN 32), 2.0e-7 with 16, 1.1e-7 with 8 (7.6
+// against 7.2 ms); the FP32 chains before were 4.4e-7 off. dW3: 0.4e-7, 2.9e-7.
+template <int N1, int JOIN>
+__device__ __forceinline__ void split_grad(const __nv_bfloat16* act, const __nv_bfloat16* col, int sgn, int np,
+                                           int warp, int lane, float (*run)[2], float (*car)[2]) {
+  constexpr int NW = NN_BWD_THREADS / 32;
+  const int MT = (np + 15) / 16;
+  const int j = lane >> 3, r = lane & 7, c4 = lane & 3;
+  float acc[2][2][4];
+#pragma unroll
+  for (int a = 0; a < 2; ++a)
 #pragma unroll
     for (int m = 0; m < 2; ++m)
+#pragma unroll
+      for (int c = 0; c < 4; ++c) acc[a][m][c] = 0.f;
+#pragma unroll 1
+  for (int kt = 0; kt < MT; ++kt) {
+    const int na = kt * 16 + r + 8 * (j >> 1), nb = kt * 16 + (lane & 15);
+    const int pA = na < np ? group_index<N1>(na) : 0;
+    const int pB = nb < np ? group_index<N1>(nb) : -1;
+    unsigned A[2][4];
+#pragma unroll
+    for (int m = 0; m < 2; ++m)
+      ldsm_x4_t(smem_u32(act + swz(pA, m * 16 + 8 * (j & 1))), A[m][0], A[m][1], A[m][2], A[m][3]);
+#pragma unroll
+    for (int a = 0; a < 2; ++a) {
+      const int t = warp + NW * a;
+      if (t >= 27) continue;
+      unsigned b0, b1;
+      ldsm_x2_t(smem_u32(col + (pB < 0 ? 0 : pB + sgn * tap_offset<N1>(t)) * 8), b0, b1);
+#pragma unroll
+      for (int m = 0; m < 2; ++m) mma16816(acc[a][m], A[m][0], A[m][1], A[m][2], A[m][3], b0, b1);
+    }
+    if (kt % JOIN == JOIN - 1 || kt == MT - 1) {
+#pragma unroll
+      for (int a = 0; a < 2; ++a)
+#pragma unroll
+        for (int m = 0; m < 2; ++m) {
+          join3(acc[a][m], c4, run[a][m], car[a][m]);
+#pragma unroll
+          for (int c = 0; c < 4; ++c) acc[a][m][c] = 0.f;
+        }
+    }
+  }
+}
+
+template <int N1>
+__global__ void __launch_bounds__(NN_BWD_THREADS, 1)
+    k_nn_backward(const float* __restrict__ prm, const __nv_bfloat16* __restrict__ W2o, const float* __restrict__ in,
+                  const __nv_bfloat16* __restrict__ a1g, const __nv_bfloat16* __restrict__ a2g,
+                  const float* __restrict__ gout, float* __restrict__ part, long long ne, int ng) {
+  using C = NNCfg<N1>;
+  constexpr int P3 = C::P3 * C::GROUP, NT = NN_BWD_THREADS, NW = NT / 32;
+  extern __shared__ __align__(16) unsigned char smem[];
+  // sA1 holds a1 until the layer-2 weight gradient is done, then g_a1 (masked)
+  __nv_bfloat16* sA1 = (__nv_bfloat16*)smem;                           // [P3][32] swizzled
+  __nv_bfloat16* sA2 = sA1 + P3 * NN_H;                                 // [P3][32] swizzled -> g_a2 (masked)
+  __nv_bfloat16* sGs = sA2 + P3 * NN_H;                                 // [P3][8] g3 split
+  __nv_bfloat16* sIs = sGs + P3 * 8;                                    // [P3][8] in split
+  __nv_bfloat16* sW2 = sIs + P3 * 8;                                    // [27 * 32 ci][32 co] swizzled
+  float* sW3 = (float*)(sW2 + 27 * 32 * 32);                           // [27][32][2]
+  float* sred = sW3 + 1728;                                            // [NW][32]
+  float* sG3 = sred + NW * 32;                                         // [P3][2]
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  for (int i = tid; i < P3 * (NN_H + 8); i += NT) ((unsigned*)sA1)[i] = 0u;  // sA1, sA2, sGs, sIs
+  for (int i = tid; i < 2 * P3; i += NT) sG3[i] = 0.f;
+  for (int i = tid; i < 1728; i += NT) sW3[i] = prm[NN_OW3 + i];
+  for (int i = tid; i < 27 * 32 * 4; i += NT)
+    *(uint4*)(sW2 + swz_w2(i >> 2, (i & 3) * 8)) = ((const uint4*)W2o)[i];
+  // dW2 accumulators: warp owns taps warp, warp + 16 (< 27); per tap 32 (ci) x 32 (co) = 2 x 4 mma tiles
+  float accW[2][2][4][4], run1[2][2], run3[2][2], car1[2][2], car3[2][2];
+#pragma unroll
+  for (int a = 0; a < 2; ++a)
+#pragma unroll
+    for (int m = 0; m < 2; ++m) {
+      run1[a][m] = run3[a][m] = car1[a][m] = car3[a][m] = 0.f;
 #pragma unroll
       for (int n = 0; n < 4; ++n)
 #pragma unroll
         for (int c = 0; c < 4; ++c) accW[a][m][n][c] = 0.f;
+    }
+  float db1 = 0.f, db2 = 0.f, db3 = 0.f;  // of thread (channel) < 32, < 32, < 2
   __syncthreads();
   const int j = lane >> 3, r = lane & 7, g = lane >> 2, c4 = lane & 3;
-  for (long long e = blockIdx.x; e < ne; e += gridDim.x) {
-    for (int i = tid; i < NPE; i += 256) {
-      const int p = pad_index<N1>(i);
-      sIn[2 * p] = in[(e * NPE + i) * 2];
-      sIn[2 * p + 1] = in[(e * NPE + i) * 2 + 1];
-      sG3[2 * p] = gout[(e * NPE + i) * 2];
-      sG3[2 * p + 1] = gout[(e * NPE + i) * 2 + 1];
+  // sum over the nodes of a masked gradient's channels: 16 partial sums per channel, joined by join_bias
+  auto bias_part = [&](const __nv_bfloat16* A, int np) {
+    float acc = 0.f;
+    for (int n = warp; n < np; n += NW) acc += __bfloat162float(A[swz(group_index<N1>(n), lane)]);
+    sred[warp * 32 + lane] = acc;
+  };
+  auto bias_join = [&](float& db) {
+    if (tid < 32) {
+      float acc = 0.f;
+#pragma unroll
+      for (int w = 0; w < NW; ++w) acc += sred[w * 32 + tid];
+      db += acc;
     }
-    for (int i = tid; i < NPE * 16; i += 256) {
-      const int n = i >> 4, c = i & 15;
-      const int p = pad_index<N1>(n);
-      ((__nv_bfloat162*)(sA1 + p * NN_H))[c] = ((const __nv_bfloat162*)(a1g + (e * NPE + n) * NN_H))[c];
-      ((__nv_bfloat162*)(sA2 + p * NN_H))[c] = ((const __nv_bfloat162*)(a2g + (e * NPE + n) * NN_H))[c];
+  };
+  for (long long e0 = (long long)blockIdx.x * ng; e0 < ne; e0 += (long long)gridDim.x * ng) {
+    const long long nb0 = e0 * C::NPE;  // first node of the pass; np nodes
+    const int np = (int)(ne - e0 < ng ? ne - e0 : ng) * C::NPE, MT = (np + 15) / 16;
+    for (int i = tid; i < np; i += NT) {
+      const int p = group_index<N1>(i);
+      const float2 x = ((const float2*)in)[nb0 + i], y = ((const float2*)gout)[nb0 + i];
+      sG3[2 * p] = y.x;
+      sG3[2 * p + 1] = y.y;
+      split3(x.x, sIs + 8 * p);
+      split3(x.y, sIs + 8 * p + 3);
+      split3(y.x, sGs + 8 * p);
+      split3(y.y, sGs + 8 * p + 3);
+    }
+    for (int i = tid; i < np * 4; i += NT) {
+      const int n = i >> 2, c = i & 3;
+      const int q = swz(group_index<N1>(n), 8 * c);
+      *(uint4*)(sA1 + q) = ((const uint4*)(a1g + (nb0 + n) * NN_H))[c];
+      *(uint4*)(sA2 + q) = ((const uint4*)(a2g + (nb0 + n) * NN_H))[c];
     }
     __syncthreads();
-    // layer 3 weights: dW3[t][ci][co] += sum_n g3[n][co] a2[n + t][ci]; db3
-    for (int w = tid; w < 1728 + 2; w += 256) {
-      if (w < 1728) {
-        const int t = w / 64, ci = (w / 2) % 32, co = w % 2;
-        const int off = tap_offset<N1>(t);
-        float acc = 0.f;
-        for (int n = 0; n < NPE; ++n) {
-          const int p = pad_index<N1>(n);
-          acc += sG3[2 * p + co] * __bfloat162float(sA2[(p + off) * NN_H + ci]);
-        }
-        dW3[w] += acc;
-      } else {
-        const int co = w - 1728;
-        float acc = 0.f;
-        for (int n = 0; n < NPE; ++n) acc += sG3[2 * pad_index<N1>(n) + co];
-        db[64 + co] += acc;
+    // layer 3 weights and bias
+    split_grad<N1, 32>(sA2, sGs, -1, np, warp, lane, run3, car3);
+    {
+      float x = 0.f, y = 0.f;
+      for (int i = tid; i < np; i += NT) {
+        const int p = group_index<N1>(i);
+        x += sG3[2 * p];
+        y += sG3[2 * p + 1];
+      }
+#pragma unroll
+      for (int d = 16; d > 0; d >>= 1) {
+        x += __shfl_xor_sync(0xffffffffu, x, d);
+        y += __shfl_xor_sync(0xffffffffu, y, d);
+      }
+      if (lane == 0) {
+        sred[warp * 32] = x;
+        sred[warp * 32 + 1] = y;
       }
     }
     __syncthreads();
-    // g_a2[n][ci] = (sum_t sum_co W3[t][ci][co] g3[n - t][co]) * (a2[n][ci] > 0), in place of a2
-    for (int w = tid; w < NPE * NN_H; w += 256) {
-      const int n = w >> 5, ci = w & 31;
-      const int p = pad_index<N1>(n);
+    if (tid < 2) {
       float acc = 0.f;
+#pragma unroll
+      for (int w = 0; w < NW; ++w) acc += sred[w * 32 + tid];
+      db3 += acc;
+    }
+    // g_a2[n][ci] = (sum_t sum_co W3[t][ci][co] g3[n - t][co]) * (a2[n][ci] > 0), in place of a2:
+    // thread = node and half of the channels (the same for a warp: weights are broadcast reads)
+    for (int w = warp; w < (np + 31) / 32 * 2; w += NW) {
+      const int n = (w >> 1) * 32 + lane, c0 = (w & 1) * 16;
+      const int p = n < np ? group_index<N1>(n) : group_index<N1>(0);
+      float acc[16];
+#pragma unroll
+      for (int c = 0; c < 16; ++c) acc[c] = 0.f;
 #pragma unroll 1
       for (int t = 0; t < 27; ++t) {
         const int q = p - tap_offset<N1>(t);
-        acc += sW3[t * 64 + ci * 2] * sG3[2 * q] + sW3[t * 64 + ci * 2 + 1] * sG3[2 * q + 1];
+        const float g0 = sG3[2 * q], g1 = sG3[2 * q + 1];
+        const float4* wt = (const float4*)(sW3 + t * 64 + c0 * 2);
+#pragma unroll
+        for (int c = 0; c < 8; ++c) {
+          const float4 v = wt[c];
+          acc[2 * c] += v.x * g0 + v.y * g1;
+          acc[2 * c + 1] += v.z * g0 + v.w * g1;
+        }
       }
-      const float a2v = __bfloat162float(sA2[p * NN_H + ci]);
-      sA2[p * NN_H + ci] = __float2bfloat16(a2v > 0.f ? acc : 0.f);
+      if (n < np) {
+#pragma unroll
+        for (int c = 0; c < 2; ++c) {
+          uint4* dst = (uint4*)(sA2 + swz(p, c0 + 8 * c));
+          uint4 raw = *dst;
+          __nv_bfloat162* hv = (__nv_bfloat162*)&raw;
+#pragma unroll
+          for (int k = 0; k < 4; ++k) {
+            const float2 v = __bfloat1622float2(hv[k]);
+            hv[k] = __floats2bfloat162_rn(v.x > 0.f ? acc[8 * c + 2 * k] : 0.f, v.y > 0.f ? acc[8 * c + 2 * k + 1] : 0.f);
+          }
+          *dst = raw;
+        }
+      }
     }
     __syncthreads();
-    for (int ci = tid; ci < NN_H; ci += 256) {
-      float acc = 0.f;
-      for (int n = 0; n < NPE; ++n) acc += __bfloat162float(sA2[pad_index<N1>(n) * NN_H + ci]);
-      db[32 + ci] += acc;
-    }
-    // layer 2 weights on the tensor cores: dW2[t] (ci x co) += sum_n a1[n + t][ci] g_a2[n][co]
-#pragma unroll
-    for (int a = 0; a < 4; ++a) {
-      const int t = warp + 8 * a;
-      if (t >= 27) continue;
-      const int off = tap_offset<N1>(t);
+    bias_part(sA2, np);
+    // layer 2 weights: dW2[t] (ci x co) += sum_n a1[n + t][ci] g_a2[n][co]
 #pragma unroll 1
-      for (int kt = 0; kt < MT; ++kt) {
-        // k = 16 nodes of tile kt; lane row address: node kt*16 + r + 8*(j>>1)
-        const int node = kt * 16 + r + 8 * (j >> 1);
-        const int pA = node < NPE ? pad_index<N1>(node) + off : 0;
-        const int pB = node < NPE ? pad_index<N1>(node) : 0;
+    for (int kt = 0; kt < MT; ++kt) {
+      // k = 16 nodes of tile kt; lane row address: node kt*16 + r + 8*(j>>1)
+      const int node = kt * 16 + r + 8 * (j >> 1);
+      const int p = node < np ? group_index<N1>(node) : -1;
+      unsigned b[2][4];
+#pragma unroll
+      for (int nh = 0; nh < 2; ++nh)
+        ldsm_x4_t(smem_u32(sA2 + swz(p < 0 ? 0 : p, nh * 16 + 8 * (j & 1))), b[nh][0], b[nh][1], b[nh][2], b[nh][3]);
+#pragma unroll
+      for (int a = 0; a < 2; ++a) {
+        const int t = warp + NW * a;
+        if (t >= 27) continue;
+        const int pA = p < 0 ? 0 : p + tap_offset<N1>(t);
 #pragma unroll
         for (int m = 0; m < 2; ++m) {
-          // A (m = ci, k = node): transposed 8x8 blocks of a1[node][ci]
           unsigned a0, a1r, a2r, a3;
-          ldsm_x4_t(smem_u32(sA1 + pA * NN_H + m * 16 + 8 * (j & 1)), a0, a1r, a2r, a3);
+          ldsm_x4_t(smem_u32(sA1 + swz(pA, m * 16 + 8 * (j & 1))), a0, a1r, a2r, a3);
 #pragma unroll
           for (int nh = 0; nh < 2; ++nh) {
-            // B (k = node, n = co): transposed blocks of g_a2[node][co], two n-tiles
-            unsigned b0, b1, b2, b3;
-            ldsm_x4_t(smem_u32(sA2 + pB * NN_H + nh * 16 + 8 * (j & 1)), b0, b1, b2, b3);
-            mma16816(accW[a][m][2 * nh], a0, a1r, a2r, a3, b0, b2);
-            mma16816(accW[a][m][2 * nh + 1], a0, a1r, a2r, a3, b1, b3);
+            mma16816(accW[a][m][2 * nh], a0, a1r, a2r, a3, b[nh][0], b[nh][2]);
+            mma16816(accW[a][m][2 * nh + 1], a0, a1r, a2r, a3, b[nh][1], b[nh][3]);
           }
         }
       }
     }
     __syncthreads();
-    // layer 2 input gradient on the tensor cores: g_a1[n][ci] = mask * sum_t sum_co g_a2[n - t][co] W2[t][ci][co],
-    // written over a1 (each lane reads the mask of exactly the entries it writes)
-    for (int mt = warp; mt < MT; mt += 8) {
-      float acc[4][4];
+    bias_join(db2);
+    // layer 2 input gradient: g_a1[n][ci] = mask * sum_t sum_co g_a2[n - t][co] W2[t][ci][co], written over a1
+    // (each lane reads the mask of exactly the entries it writes); two node tiles per warp share the W2 tiles
+    for (int mt0 = warp; mt0 < MT; mt0 += 2 * NW) {
+      float acc[2][4][4];
 #pragma unroll
-      for (int b = 0; b < 4; ++b)
+      for (int a = 0; a < 2; ++a)
 #pragma unroll
-        for (int c = 0; c < 4; ++c) acc[b][c] = 0.f;
-      const int node = mt * 16 + r + 8 * (j & 1);
-      const int prow = node < NPE ? pad_index<N1>(node) : -1;
+        for (int b = 0; b < 4; ++b)
+#pragma unroll
+          for (int c = 0; c < 4; ++c) acc[a][b][c] = 0.f;
+      int prow[2];
+#pragma unroll
+      for (int a = 0; a < 2; ++a) {
+        const int node = (mt0 + NW * a) * 16 + r + 8 * (j & 1);
+        prow[a] = node < np ? group_index<N1>(node) : -1;
+      }
 #pragma unroll 1
       for (int t = 0; t < 27; ++t) {
         const int off = tap_offset<N1>(t);
-        const int q = prow >= 0 ? prow - off : 0;
+        // W2 tiles: matrices j = (kh, 8-column half) of the 8 rows ci of column tile nt
+        unsigned w2[4][4];
 #pragma unroll
-        for (int kh = 0; kh < 2; ++kh) {
-          unsigned a0, a1r, a2r, a3;
-          ldsm_x4(smem_u32(sA2 + q * NN_H + kh * 16 + 8 * (j >> 1)), a0, a1r, a2r, a3);
+        for (int nt = 0; nt < 4; ++nt)
+          ldsm_x4(smem_u32(sW2 + swz_w2(t * 32 + nt * 8 + r, 8 * j)), w2[nt][0], w2[nt][1], w2[nt][2], w2[nt][3]);
 #pragma unroll
-          for (int nt = 0; nt < 4; ++nt) {
-            const __nv_bfloat16* wp = W2o + ((long long)t * 32 + nt * 8 + g) * 32 + kh * 16 + 2 * c4;
-            mma16816(acc[nt], a0, a1r, a2r, a3, *(const unsigned*)wp, *(const unsigned*)(wp + 8));
+        for (int a = 0; a < 2; ++a) {
+          if (mt0 + NW * a >= MT) continue;
+          const int q = prow[a] >= 0 ? prow[a] - off : 0;
+#pragma unroll
+          for (int kh = 0; kh < 2; ++kh) {
+            unsigned a0, a1r, a2r, a3;
+            ldsm_x4(smem_u32(sA2 + swz(q, kh * 16 + 8 * (j >> 1))), a0, a1r, a2r, a3);
+#pragma unroll
+            for (int nt = 0; nt < 4; ++nt) mma16816(acc[a][nt], a0, a1r, a2r, a3, w2[nt][2 * kh], w2[nt][2 * kh + 1]);
           }
         }
       }
 #pragma unroll
-      for (int h = 0; h < 2; ++h) {
-        const int nn = mt * 16 + g + 8 * h;
-        if (nn >= NPE) continue;
-        const int p = pad_index<N1>(nn);
+      for (int a = 0; a < 2; ++a)
 #pragma unroll
-        for (int nt = 0; nt < 4; ++nt) {
-          const int ci = nt * 8 + 2 * c4;
-          __nv_bfloat162* dst = (__nv_bfloat162*)(sA1 + p * NN_H + ci);
-          const float2 a1v = __bfloat1622float2(*dst);
-          *dst = __floats2bfloat162_rn(a1v.x > 0.f ? acc[nt][2 * h] : 0.f, a1v.y > 0.f ? acc[nt][2 * h + 1] : 0.f);
+        for (int h = 0; h < 2; ++h) {
+          const int nn = (mt0 + NW * a) * 16 + g + 8 * h;
+          if (nn >= np) continue;
+          const int p = group_index<N1>(nn);
+#pragma unroll
+          for (int nt = 0; nt < 4; ++nt) {
+            __nv_bfloat162* dst = (__nv_bfloat162*)(sA1 + swz(p, nt * 8 + 2 * c4));
+            const float2 a1v = __bfloat1622float2(*dst);
+            *dst = __floats2bfloat162_rn(a1v.x > 0.f ? acc[a][nt][2 * h] : 0.f,
+                                         a1v.y > 0.f ? acc[a][nt][2 * h + 1] : 0.f);
+          }
         }
-      }
     }
     __syncthreads();
-    // layer 1 weights and biases
-    for (int w = tid; w < 1728 + 32; w += 256) {
-      if (w < 1728) {
-        const int t = w / 64, ci = (w / 32) % 2, co = w % 32;
-        const int off = tap_offset<N1>(t);
-        float acc = 0.f;
-        for (int n = 0; n < NPE; ++n) {
-          const int p = pad_index<N1>(n);
-          acc += sIn[2 * (p + off) + ci] * __bfloat162float(sA1[p * NN_H + co]);
-        }
-        dW1[w] += acc;
-      } else {
-        const int co = w - 1728;
-        float acc = 0.f;
-        for (int n = 0; n < NPE; ++n) acc += __bfloat162float(sA1[pad_index<N1>(n) * NN_H + co]);
-        db[co] += acc;
-      }
-    }
+    // layer 1 weights and bias
+    split_grad<N1, 16>(sA1, sIs, 1, np, warp, lane, run1, car1);
+    bias_part(sA1, np);
     __syncthreads();
+    bias_join(db1);
     // a1 and a2 were overwritten by their gradients at interior nodes only;
     // the zero borders stay, the interiors are reloaded for the next element
   }
   // write this block's partial gradients in parameter order
   float* pb = part + (long long)blockIdx.x * NN_NPARAM;
-  for (int i = tid; i < 1728; i += 256) {
-    pb[NN_OW1 + i] = dW1[i];
-    pb[NN_OW3 + i] = dW3[i];
+  if (tid < 32) {
+    pb[NN_OB1 + tid] = db1;
+    pb[NN_OB2 + tid] = db2;
   }
-  for (int i = tid; i < 32; i += 256) {
-    pb[NN_OB1 + i] = db[i];
-    pb[NN_OB2 + i] = db[32 + i];
-  }
-  if (tid < 2) pb[NN_OB3 + tid] = db[64 + tid];
+  if (tid < 2) pb[NN_OB3 + tid] = db3;
 #pragma unroll
-  for (int a = 0; a < 4; ++a) {
-    const int t = warp + 8 * a;
+  for (int a = 0; a < 2; ++a) {
+    const int t = warp + NW * a;
     if (t >= 27) continue;
 #pragma unroll
-    for (int m = 0; m < 2; ++m)
+    for (int m = 0; m < 2; ++m) {
+      const int row = m * 16 + g + 8 * (c4 >> 1), ch = c4 & 1;
+      pb[NN_OW3 + t * 64 + row * 2 + ch] = run3[a][m] + car3[a][m];
+      pb[NN_OW1 + t * 64 + ch * 32 + row] = run1[a][m] + car1[a][m];
 #pragma unroll
       for (int n = 0; n < 4; ++n)
 #pragma unroll
@@ -453,15 +623,17 @@ __global__ void __launch_bounds__(256, 1)
           pb[NN_OW2 + (t * 32 + ci) * 32 + co] = accW[a][m][n][2 * h];
           pb[NN_OW2 + (t * 32 + ci) * 32 + co + 1] = accW[a][m][n][2 * h + 1];
         }
+    }
   }
 }
 
 __global__ void k_nn_reduce(const float* __restrict__ part, int nblk, float* __restrict__ grad) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= NN_NPARAM) return;
-  float acc = 0.f;
+  double acc = 0.0;
+#pragma unroll 16
   for (int b = 0; b < nblk; ++b) acc += part[(long long)b * NN_NPARAM + i];
-  grad[i] = acc;
+  grad[i] = (float)acc;
 }
 
 // BF16 copies of W2 in both layouts
@@ -492,10 +664,10 @@ static size_t fwd_smem(int n1) {
   return 2 * sizeof(__nv_bfloat16) * P3 * NN_H + sizeof(__nv_bfloat16) * 27 * 32 * NN_W2LD + sizeof(float) * 2 * P3 +
          sizeof(float) * (1760 + 1730 + 32);
 }
-static size_t bwd_smem(int n1) {
-  const int P3 = (n1 + 2) * (n1 + 2) * (n1 + 2), NPE = n1 * n1 * n1;
-  (void)NPE;
-  return sizeof(float) * 4 * P3 + 2 * sizeof(__nv_bfloat16) * P3 * NN_H + sizeof(float) * (1728 * 3 + 66);
+static size_t bwd_smem(int n1, int group) {
+  const int P3 = group * (n1 + 2) * (n1 + 2) * (n1 + 2);
+  return sizeof(__nv_bfloat16) * (2 * P3 * (NN_H + 8) + 27 * 32 * 32) +
+         sizeof(float) * (2 * P3 + 1728 + NN_BWD_THREADS);
 }
 
 static int sm_count() {
@@ -539,10 +711,10 @@ template <int N1>
 static int nn_bwd_blocks(long long ne) {
   static int bps = 0;
   if (!bps) {
-    const size_t sm = bwd_smem(N1);
+    const size_t sm = bwd_smem(N1, NNCfg<N1>::GROUP);
     if (cudaFuncSetAttribute(k_nn_backward<N1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm) != cudaSuccess)
       return 0;
-    bps = blocks_per_sm(k_nn_backward<N1>, sm);
+    bps = blocks_per_sm(k_nn_backward<N1>, sm, NN_BWD_THREADS);
   }
   const long long cap = (long long)sm_count() * bps;
   return (int)(ne < cap ? (ne < 1 ? 1 : ne) : cap);
@@ -552,8 +724,10 @@ template <int N1>
 static cudaError_t nn_bwd_n1(const float* prm, const __nv_bfloat16* W2o, const float* in, const __nv_bfloat16* a1,
                              const __nv_bfloat16* a2, const float* gout, float* part, int nblk, long long ne,
                              cudaStream_t s) {
+  const long long per = (ne + nblk - 1) / nblk;  // elements per block: no more at once than that
   count_launch();
-  k_nn_backward<N1><<<nblk, 256, bwd_smem(N1), s>>>(prm, W2o, in, a1, a2, gout, part, ne);
+  k_nn_backward<N1><<<nblk, NN_BWD_THREADS, bwd_smem(N1, NNCfg<N1>::GROUP), s>>>(
+      prm, W2o, in, a1, a2, gout, part, ne, (int)(per < NNCfg<N1>::GROUP ? (per < 1 ? 1 : per) : NNCfg<N1>::GROUP));
   return cudaGetLastError();
 }
 
