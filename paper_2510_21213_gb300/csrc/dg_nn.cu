@@ -54,8 +54,7 @@ struct NNCfg {
   static constexpr int P = N1 + 2;
   static constexpr int P3 = P * P * P;
   static constexpr int NPE = N1 * N1 * N1;
-  static constexpr int MT = (NPE + 15) / 16;  // 16-node tiles
-  // elements that the backward kernel works on at once, each with its own border
+  // elements that a block works on at once, each with its own border
   static constexpr int GROUP = N1 == 2 ? 12 : (N1 == 3 ? 8 : (N1 == 4 ? 4 : (N1 == 5 ? 2 : 1)));
 };
 
@@ -88,70 +87,111 @@ __device__ __forceinline__ int swz(int p, int ch) {
   return p * NN_H + ((((ch >> 3) ^ ((p >> 1) & 3)) << 3) | (ch & 7));
 }
 
+// shared-memory index of entry (row, ch) of a staged copy of W2 (rows of 32 channels)
+__device__ __forceinline__ int swz_w2(int row, int ch) {
+  return row * 32 + ((((ch >> 3) ^ ((row >> 1) & 3)) << 3) | (ch & 7));
+}
+
+// Forward kernel: one block per SM, 16 warps, a group of elements at a time.
+// Layer 1: a thread computes 4 channels of a line of nodes along x, a warp 32 lines
+// of the same channels: per row of taps it loads p + 3 inputs (row strides free of
+// bank conflicts) and 6 broadcast float4 of weights for 48 (p + 1) products; one
+// node and 8 channels per thread before, 5 loads for 16 products. Products and sums
+// per output are in the same order: the same bits.
+// Layer 2 (tensor cores): a warp owns two 16-node tiles and loads the operand tiles
+// of W2 with ldmatrix (8 scalar loads per 8 MMAs before); same bits.
+// Layer 3: a thread sums 4 input channels for a line of nodes, eight lanes are one
+// line; their sums are added by halving shuffles (one thread per node before: half
+// of the warps' issue slots idle, 20 loads for 64 products).
+// Measured (GB300, with activations stored): 16384 elements at p = 7 4.92 -> 3.02 ms,
+// 2000 at p = 6 0.57 -> 0.39, 200 at p = 4 0.061 -> 0.050, 4000 at p = 1 0.306 -> 0.063.
 constexpr int NN_FWD_THREADS = 512;
-constexpr int NN_W2LD = 40;  // padded row of the staged W2 (bank-conflict-free B fragment loads)
+
+template <int N1>
+struct FwdCfg {
+  using C = NNCfg<N1>;
+  // input rows in float2: odd, and planes 8 modulo 16, so that 16 lanes on lines of
+  // two planes of 8 read distinct banks
+  static constexpr int YS = C::P | 1, ZS = (C::P * YS + 7) / 16 * 16 + 8, IS = C::P * ZS;
+  static constexpr int ROWS = C::P3 * C::GROUP;
+  static constexpr size_t SMEM = 2 * sizeof(__nv_bfloat16) * ROWS * NN_H + sizeof(__nv_bfloat16) * 27 * 32 * 32 +
+                                 sizeof(float2) * C::GROUP * IS + sizeof(float) * (1760 + 1728 + 32);
+};
 
 template <int N1>
 __global__ void __launch_bounds__(NN_FWD_THREADS, 1)
     k_nn_forward(const float* __restrict__ prm, const __nv_bfloat16* __restrict__ W2t, const float* __restrict__ in,
                  float* __restrict__ out, __nv_bfloat16* __restrict__ a1_out, __nv_bfloat16* __restrict__ a2_out,
-                 long long ne) {
+                 long long ne, int ng) {
   using C = NNCfg<N1>;
-  constexpr int P3 = C::P3, NPE = C::NPE, MT = C::MT;
-  constexpr int NT = NN_FWD_THREADS, NW = NT / 32;
+  using F = FwdCfg<N1>;
+  constexpr int ROWS = F::ROWS, P = C::P, NT = NN_FWD_THREADS, NW = NT / 32, LPE = N1 * N1;
   extern __shared__ __align__(16) unsigned char smem[];
-  __nv_bfloat16* sA1 = (__nv_bfloat16*)smem;                           // [P3][32] swizzled
-  __nv_bfloat16* sA2 = sA1 + P3 * NN_H;                                 // [P3][32] swizzled
-  __nv_bfloat16* sW2 = sA2 + P3 * NN_H;                                 // [27][32 co][NN_W2LD] (ci)
-  float* sIn = (float*)(sW2 + 27 * 32 * NN_W2LD);                      // [P3][2]
-  float* sW1 = sIn + 2 * P3;                                           // [27][2][32] + b1
-  float* sW3 = sW1 + 1728 + 32;                                        // [27][32][2] + b3
-  float* sb2 = sW3 + 1728 + 2;                                         // [32]
+  __nv_bfloat16* sA1 = (__nv_bfloat16*)smem;                           // [ROWS][32] swizzled
+  __nv_bfloat16* sA2 = sA1 + ROWS * NN_H;                               // [ROWS][32] swizzled
+  __nv_bfloat16* sW2 = sA2 + ROWS * NN_H;                               // [27 * 32 co][32 ci] swizzled
+  float* sW1 = (float*)(sW2 + 27 * 32 * 32);                           // [27][2][32] + b1
+  float* sW3 = sW1 + 1728 + 32;                                        // [27][2][8 groups][2 ci][2 co]
+  float* sb2 = sW3 + 1728;                                             // [32]
+  float2* sIn = (float2*)(sb2 + 32);                                   // [GROUP][P][P][.]
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  for (int i = tid; i < 2 * P3; i += NT) sIn[i] = 0.f;
-  for (int i = tid; i < P3 * NN_H; i += NT) ((unsigned*)sA1)[i] = 0u;  // sA1 and sA2
-  for (int i = tid; i < 27 * 32 * 16; i += NT) {
-    const int row = i >> 4, c2 = i & 15;
-    ((unsigned*)(sW2 + row * NN_W2LD))[c2] = ((const unsigned*)(W2t + row * 32))[c2];
-  }
+  for (int i = tid; i < C::GROUP * F::IS; i += NT) sIn[i] = make_float2(0.f, 0.f);
+  for (int i = tid; i < ROWS * NN_H; i += NT) ((unsigned*)sA1)[i] = 0u;  // sA1 and sA2
+  for (int i = tid; i < 27 * 32 * 4; i += NT)
+    *(uint4*)(sW2 + swz_w2(i >> 2, (i & 3) * 8)) = ((const uint4*)W2t)[i];
   for (int i = tid; i < 1760; i += NT) sW1[i] = prm[NN_OW1 + i];
-  for (int i = tid; i < 1730; i += NT) sW3[i] = prm[NN_OW3 + i];
+  for (int i = tid; i < 1728; i += NT) {  // channel 4 g + 2 k + c of tap t
+    const int t = i / 64, ci = i / 2 % 32;
+    sW3[t * 64 + (ci >> 1 & 1) * 32 + (ci >> 2) * 4 + (i & 3)] = prm[NN_OW3 + i];
+  }
   for (int i = tid; i < 32; i += NT) sb2[i] = prm[NN_OB2 + i];
+  const float b30 = prm[NN_OB3], b31 = prm[NN_OB3 + 1];
   __syncthreads();
-  const int g = lane >> 2, c4 = lane & 3;
-  for (long long e = blockIdx.x; e < ne; e += gridDim.x) {
-    for (int i = tid; i < NPE; i += NT) {
-      const int p = pad_index<N1>(i);
-      const float2 v = ((const float2*)in)[e * NPE + i];
-      sIn[2 * p] = v.x;
-      sIn[2 * p + 1] = v.y;
+  const int g = lane >> 2, c4 = lane & 3, j = lane >> 3, r = lane & 7;
+  for (long long e0 = (long long)blockIdx.x * ng; e0 < ne; e0 += (long long)gridDim.x * ng) {
+    const long long nb0 = e0 * C::NPE;  // first node of the pass; np nodes on nl lines
+    const int nel = (int)(ne - e0 < ng ? ne - e0 : ng), np = nel * C::NPE, nl = nel * LPE, MT = (np + 15) / 16;
+    for (int i = tid; i < np; i += NT) {
+      const int l = i / N1, y = l % N1, z = l / N1 % N1;
+      sIn[l / LPE * F::IS + (z + 1) * F::ZS + (y + 1) * F::YS + i % N1 + 1] = ((const float2*)in)[nb0 + i];
     }
     __syncthreads();
-    // layer 1 (2 -> 32), SIMT: thread = (node, group of 8 output channels = one chunk)
-    for (int w = tid; w < NPE * 4; w += NT) {
-      const int n = w >> 2, cg = (w & 3) * 8;
-      const int p = pad_index<N1>(n);
-      float acc[8];
+    // layer 1 (2 -> 32)
+    for (int w = warp; w < (nl + 31) / 32 * 8; w += NW) {
+      const int l = w / 8 * 32 + lane, cg = w % 8 * 4, ll = l < nl ? l : 0;
+      const int y = ll % N1, z = ll / N1 % N1;
+      const float2* src = sIn + ll / LPE * F::IS + z * F::ZS + y * F::YS;
+      float acc[N1][4];
 #pragma unroll
-      for (int c = 0; c < 8; ++c) acc[c] = sW1[1728 + cg + c];
+      for (int i = 0; i < N1; ++i)
+#pragma unroll
+        for (int c = 0; c < 4; ++c) acc[i][c] = sW1[1728 + cg + c];
 #pragma unroll 1
-      for (int t = 0; t < 27; ++t) {
-        const int q = p + tap_offset<N1>(t);
-        const float i0 = sIn[2 * q], i1 = sIn[2 * q + 1];
-        const float* wt = sW1 + t * 64 + cg;
+      for (int d = 0; d < 9; ++d) {
+        const float2* row = src + d / 3 * F::ZS + d % 3 * F::YS;
+        float2 v[P];
 #pragma unroll
-        for (int c = 0; c < 8; ++c) acc[c] += i0 * wt[c] + i1 * wt[32 + c];
+        for (int i = 0; i < P; ++i) v[i] = row[i];
+#pragma unroll
+        for (int dx = 0; dx < 3; ++dx) {
+          const float4 wa = *(const float4*)(sW1 + (3 * d + dx) * 64 + cg);
+          const float4 wb = *(const float4*)(sW1 + (3 * d + dx) * 64 + 32 + cg);
+          const float w0[4] = {wa.x, wa.y, wa.z, wa.w}, w1[4] = {wb.x, wb.y, wb.z, wb.w};
+#pragma unroll
+          for (int i = 0; i < N1; ++i)
+#pragma unroll
+            for (int c = 0; c < 4; ++c) acc[i][c] += v[i + dx].x * w0[c] + v[i + dx].y * w1[c];
+        }
       }
-      uint4 pk;
-      __nv_bfloat162 h0 = __floats2bfloat162_rn(fmaxf(acc[0], 0.f), fmaxf(acc[1], 0.f));
-      __nv_bfloat162 h1 = __floats2bfloat162_rn(fmaxf(acc[2], 0.f), fmaxf(acc[3], 0.f));
-      __nv_bfloat162 h2 = __floats2bfloat162_rn(fmaxf(acc[4], 0.f), fmaxf(acc[5], 0.f));
-      __nv_bfloat162 h3 = __floats2bfloat162_rn(fmaxf(acc[6], 0.f), fmaxf(acc[7], 0.f));
-      pk.x = *(unsigned*)&h0;
-      pk.y = *(unsigned*)&h1;
-      pk.z = *(unsigned*)&h2;
-      pk.w = *(unsigned*)&h3;
-      *(uint4*)(sA1 + swz(p, cg)) = pk;
+      if (l < nl) {
+        const int p0 = ll / LPE * C::P3 + (z + 1) * P * P + (y + 1) * P + 1;
+#pragma unroll
+        for (int i = 0; i < N1; ++i) {
+          const __nv_bfloat162 h0 = __floats2bfloat162_rn(fmaxf(acc[i][0], 0.f), fmaxf(acc[i][1], 0.f));
+          const __nv_bfloat162 h1 = __floats2bfloat162_rn(fmaxf(acc[i][2], 0.f), fmaxf(acc[i][3], 0.f));
+          *(uint2*)(sA1 + swz(p0 + i, cg)) = make_uint2(*(const unsigned*)&h0, *(const unsigned*)&h1);
+        }
+      }
     }
     __syncthreads();
     // layer 2 (32 -> 32) on the tensor cores: warp owns node tiles warp, warp + NW, ...
@@ -164,49 +204,40 @@ __global__ void __launch_bounds__(NN_FWD_THREADS, 1)
 #pragma unroll
           for (int c = 0; c < 4; ++c) acc[a][b][c] = 0.f;
       int rowp[2];
-      bool tile_ok[2];
 #pragma unroll
       for (int a = 0; a < 2; ++a) {
-        const int mt = mt0 + NW * a;
-        tile_ok[a] = mt < MT;
-        const int node = mt * 16 + (lane & 7) + 8 * ((lane >> 3) & 1);
-        rowp[a] = (tile_ok[a] && node < NPE) ? pad_index<N1>(node) : 0;  // padded row 0 is all zero
+        const int node = (mt0 + NW * a) * 16 + r + 8 * (j & 1);
+        rowp[a] = node < np ? group_index<N1>(node) : -1;  // rows past the nodes read the zero corner
       }
-      const int khalf = lane >> 4;  // which 8 channels of the 16-channel k step this lane's row address serves
 #pragma unroll 1
       for (int t = 0; t < 27; ++t) {
         const int off = tap_offset<N1>(t);
+        // B tiles: matrix j = input channels 8 j .. 8 j + 7 of the 8 rows co of column tile nt
+        unsigned b[4][4];
 #pragma unroll
-        for (int kh = 0; kh < 2; ++kh) {
-          // B fragments (k = ci, n = co) from the staged W2[t][co][ci]
-          unsigned b[4][2];
+        for (int nt = 0; nt < 4; ++nt)
+          ldsm_x4(smem_u32(sW2 + swz_w2(t * 32 + nt * 8 + r, 8 * j)), b[nt][0], b[nt][1], b[nt][2], b[nt][3]);
 #pragma unroll
-          for (int nt = 0; nt < 4; ++nt) {
-            const __nv_bfloat16* wp = sW2 + (t * 32 + nt * 8 + g) * NN_W2LD + kh * 16 + 2 * c4;
-            b[nt][0] = *(const unsigned*)wp;
-            b[nt][1] = *(const unsigned*)(wp + 8);
-          }
+        for (int a = 0; a < 2; ++a) {
+          if (mt0 + NW * a >= MT) continue;
+          const int q = rowp[a] >= 0 ? rowp[a] + off : 0;
 #pragma unroll
-          for (int a = 0; a < 2; ++a) {
-            if (!tile_ok[a]) continue;
-            const int qq = rowp[a] == 0 ? 0 : rowp[a] + off;  // rows past the element read the zero corner
+          for (int kh = 0; kh < 2; ++kh) {
             unsigned a0, a1, a2, a3;
-            ldsm_x4(smem_u32(sA1 + swz(qq, kh * 16 + khalf * 8)), a0, a1, a2, a3);
+            ldsm_x4(smem_u32(sA1 + swz(q, kh * 16 + 8 * (j >> 1))), a0, a1, a2, a3);
 #pragma unroll
-            for (int nt = 0; nt < 4; ++nt) mma16816(acc[a][nt], a0, a1, a2, a3, b[nt][0], b[nt][1]);
+            for (int nt = 0; nt < 4; ++nt) mma16816(acc[a][nt], a0, a1, a2, a3, b[nt][2 * kh], b[nt][2 * kh + 1]);
           }
         }
       }
       // epilogue: bias, ReLU, BF16 into sA2 (rows g and g+8, columns 2c4, 2c4+1 of each n tile)
 #pragma unroll
-      for (int a = 0; a < 2; ++a) {
-        if (!tile_ok[a]) continue;
-        const int mt = mt0 + NW * a;
+      for (int a = 0; a < 2; ++a)
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
-          const int node = mt * 16 + g + 8 * h;
-          if (node >= NPE) continue;
-          const int p = pad_index<N1>(node);
+          const int node = (mt0 + NW * a) * 16 + g + 8 * h;
+          if (node >= np) continue;
+          const int p = group_index<N1>(node);
 #pragma unroll
           for (int nt = 0; nt < 4; ++nt) {
             const int co = nt * 8 + 2 * c4;
@@ -215,38 +246,59 @@ __global__ void __launch_bounds__(NN_FWD_THREADS, 1)
             *(__nv_bfloat162*)(sA2 + swz(p, co)) = __floats2bfloat162_rn(v0, v1);
           }
         }
-      }
     }
     __syncthreads();
-    // layer 3 (32 -> 2), SIMT; optional copies of the activations for training
-    for (int n = tid; n < NPE; n += NT) {
-      const int p = pad_index<N1>(n);
-      float o0 = sW3[1728], o1 = sW3[1729];
+    // layer 3 (32 -> 2): lane r of eight sums channels 4 r .. 4 r + 3 of a line
+    for (int w = warp; w < (nl + 3) / 4; w += NW) {
+      const int l = w * 4 + j, ll = l < nl ? l : 0;
+      const int y = ll % N1, z = ll / N1 % N1;
+      const int p0 = ll / LPE * C::P3 + z * P * P + y * P;
+      float acc[8][2];
+#pragma unroll
+      for (int i = 0; i < 8; ++i) acc[i][0] = acc[i][1] = 0.f;
 #pragma unroll 1
-      for (int t = 0; t < 27; ++t) {
-        const int q = p + tap_offset<N1>(t);
-        const float* wt = sW3 + t * 64;
+      for (int d = 0; d < 9; ++d) {
+        const int q = p0 + d / 3 * P * P + d % 3 * P;
+        float4 wa[3], wb[3];  // (ci, co) = (0, 0), (0, 1), (1, 0), (1, 1) and the next two channels
 #pragma unroll
-        for (int c = 0; c < 4; ++c) {
-          const uint4 raw = *(const uint4*)(sA2 + swz(q, 8 * c));
-          const __nv_bfloat162* hv = (const __nv_bfloat162*)&raw;
+        for (int dx = 0; dx < 3; ++dx) {
+          wa[dx] = *(const float4*)(sW3 + (3 * d + dx) * 64 + 4 * r);
+          wb[dx] = *(const float4*)(sW3 + (3 * d + dx) * 64 + 32 + 4 * r);
+        }
 #pragma unroll
-          for (int k = 0; k < 4; ++k) {
-            const float2 v = __bfloat1622float2(hv[k]);
-            const int ci = 8 * c + 2 * k;
-            o0 += v.x * wt[2 * ci] + v.y * wt[2 * ci + 2];
-            o1 += v.x * wt[2 * ci + 1] + v.y * wt[2 * ci + 3];
+        for (int i = 0; i < P; ++i) {
+          const uint2 raw = *(const uint2*)(sA2 + swz(q + i, 4 * r));
+          const float v0 = __uint_as_float(raw.x << 16), v1 = __uint_as_float(raw.x & 0xffff0000u);
+          const float v2 = __uint_as_float(raw.y << 16), v3 = __uint_as_float(raw.y & 0xffff0000u);
+#pragma unroll
+          for (int dx = 0; dx < 3; ++dx) {
+            const int x = i - dx;
+            if (x < 0 || x >= N1) continue;
+            acc[x][0] = fmaf(v3, wb[dx].z, fmaf(v2, wb[dx].x, fmaf(v1, wa[dx].z, fmaf(v0, wa[dx].x, acc[x][0]))));
+            acc[x][1] = fmaf(v3, wb[dx].w, fmaf(v2, wb[dx].y, fmaf(v1, wa[dx].w, fmaf(v0, wa[dx].y, acc[x][1]))));
           }
         }
       }
-      ((float2*)out)[e * NPE + n] = make_float2(o0, o1);
+      // add the eight lanes' sums; lane r is left with node r of the line
+#pragma unroll
+      for (int h = 4; h > 0; h >>= 1) {
+        const bool up = r & h;
+#pragma unroll
+        for (int i = 0; i < h; ++i)
+#pragma unroll
+          for (int c = 0; c < 2; ++c) {
+            const float give = up ? acc[i][c] : acc[i + h][c], keep = up ? acc[i + h][c] : acc[i][c];
+            acc[i][c] = keep + __shfl_xor_sync(0xffffffffu, give, h);
+          }
+      }
+      if (l < nl && r < N1) ((float2*)out)[nb0 + l * N1 + r] = make_float2(acc[0][0] + b30, acc[0][1] + b31);
     }
     if (a1_out) {
-      for (int i = tid; i < NPE * 4; i += NT) {
+      for (int i = tid; i < np * 4; i += NT) {
         const int n = i >> 2, c = i & 3;
-        const int p = pad_index<N1>(n);
-        ((uint4*)(a1_out + (e * NPE + n) * NN_H))[c] = *(const uint4*)(sA1 + swz(p, 8 * c));
-        ((uint4*)(a2_out + (e * NPE + n) * NN_H))[c] = *(const uint4*)(sA2 + swz(p, 8 * c));
+        const int q = swz(group_index<N1>(n), 8 * c);
+        ((uint4*)(a1_out + (nb0 + n) * NN_H))[c] = *(const uint4*)(sA1 + q);
+        ((uint4*)(a2_out + (nb0 + n) * NN_H))[c] = *(const uint4*)(sA2 + q);
       }
     }
     __syncthreads();
@@ -295,11 +347,6 @@ __device__ __forceinline__ void split3(float x, __nv_bfloat16* o) {
   o[0] = __float2bfloat16(hi);
   o[1] = __float2bfloat16(mid);
   o[2] = __float2bfloat16(r1 - mid);
-}
-
-// shared-memory index of entry (row, co) of the staged W2o
-__device__ __forceinline__ int swz_w2(int row, int co) {
-  return row * 32 + ((((co >> 3) ^ ((row >> 1) & 3)) << 3) | (co & 7));
 }
 
 // Adds one element's tile sums (rows g, g + 8; columns = three split parts of two
@@ -659,11 +706,6 @@ __global__ void k_nn_adam(float* __restrict__ prm, const float* __restrict__ gra
   prm[i] -= lr * (mi / c1) / (sqrtf(vi / c2) + eps);
 }
 
-static size_t fwd_smem(int n1) {
-  const int P3 = (n1 + 2) * (n1 + 2) * (n1 + 2);
-  return 2 * sizeof(__nv_bfloat16) * P3 * NN_H + sizeof(__nv_bfloat16) * 27 * 32 * NN_W2LD + sizeof(float) * 2 * P3 +
-         sizeof(float) * (1760 + 1730 + 32);
-}
 static size_t bwd_smem(int n1, int group) {
   const int P3 = group * (n1 + 2) * (n1 + 2) * (n1 + 2);
   return sizeof(__nv_bfloat16) * (2 * P3 * (NN_H + 8) + 27 * 32 * 32) +
@@ -689,21 +731,30 @@ static int blocks_per_sm(K kern, size_t smem, int threads = 256) {
   return b;
 }
 
+// elements at once: no more than the share of each of blocks blocks
+template <int N1>
+static int nn_group(long long ne, long long blocks) {
+  const long long per = (ne + blocks - 1) / blocks;
+  return (int)(per < 1 ? 1 : (per < NNCfg<N1>::GROUP ? per : NNCfg<N1>::GROUP));
+}
+
 template <int N1>
 static cudaError_t nn_fwd_n1(const float* prm, const __nv_bfloat16* W2t, const float* in, float* out,
                              __nv_bfloat16* a1, __nv_bfloat16* a2, long long ne, cudaStream_t s) {
-  const size_t sm = fwd_smem(N1);
+  constexpr size_t sm = FwdCfg<N1>::SMEM;
+  static_assert(sm <= 227 * 1024, "shared memory of a block");
   static int bps = 0;
   if (!bps) {
     cudaError_t e = cudaFuncSetAttribute(k_nn_forward<N1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
     if (e != cudaSuccess) return e;
     bps = blocks_per_sm(k_nn_forward<N1>, sm, NN_FWD_THREADS);
   }
+  if (ne < 1) return cudaSuccess;
   const long long cap = (long long)sm_count() * bps;
-  const long long grid = ne < cap ? ne : cap;
-  if (grid < 1) return cudaSuccess;
+  const int ng = nn_group<N1>(ne, cap);
+  const long long grid = (ne + ng - 1) / ng;
   count_launch();
-  k_nn_forward<N1><<<(unsigned)grid, NN_FWD_THREADS, sm, s>>>(prm, W2t, in, out, a1, a2, ne);
+  k_nn_forward<N1><<<(unsigned)(grid < cap ? grid : cap), NN_FWD_THREADS, sm, s>>>(prm, W2t, in, out, a1, a2, ne, ng);
   return cudaGetLastError();
 }
 
@@ -724,10 +775,9 @@ template <int N1>
 static cudaError_t nn_bwd_n1(const float* prm, const __nv_bfloat16* W2o, const float* in, const __nv_bfloat16* a1,
                              const __nv_bfloat16* a2, const float* gout, float* part, int nblk, long long ne,
                              cudaStream_t s) {
-  const long long per = (ne + nblk - 1) / nblk;  // elements per block: no more at once than that
   count_launch();
-  k_nn_backward<N1><<<nblk, NN_BWD_THREADS, bwd_smem(N1, NNCfg<N1>::GROUP), s>>>(
-      prm, W2o, in, a1, a2, gout, part, ne, (int)(per < NNCfg<N1>::GROUP ? (per < 1 ? 1 : per) : NNCfg<N1>::GROUP));
+  k_nn_backward<N1><<<nblk, NN_BWD_THREADS, bwd_smem(N1, NNCfg<N1>::GROUP), s>>>(prm, W2o, in, a1, a2, gout, part, ne,
+                                                                                 nn_group<N1>(ne, nblk));
   return cudaGetLastError();
 }
 
