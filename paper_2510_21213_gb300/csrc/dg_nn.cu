@@ -55,7 +55,7 @@ struct NNCfg {
   static constexpr int P3 = P * P * P;
   static constexpr int NPE = N1 * N1 * N1;
   // elements that a block works on at once, each with its own border
-  static constexpr int GROUP = N1 == 2 ? 12 : (N1 == 3 ? 8 : (N1 == 4 ? 4 : (N1 == 5 ? 2 : 1)));
+  static constexpr int GROUP = N1 == 2 ? 12 : (N1 == 3 ? 7 : (N1 == 4 ? 4 : (N1 == 5 ? 2 : 1)));
 };
 
 template <int N1>
@@ -93,8 +93,8 @@ __device__ __forceinline__ int swz_w2(int row, int ch) {
 }
 
 // Forward kernel: one block per SM, 16 warps, a group of elements at a time.
-// Layer 1: a thread computes 4 channels of a line of nodes along x, a warp 32 lines
-// of the same channels: per row of taps it loads p + 3 inputs (row strides free of
+// Layer 1: a thread computes 4 channels of a line of nodes along x, a warp (mostly)
+// lines of the same channels: per row of taps it loads p + 3 inputs (row strides free of
 // bank conflicts) and 6 broadcast float4 of weights for 48 (p + 1) products; one
 // node and 8 channels per thread before, 5 loads for 16 products. Products and sums
 // per output are in the same order: the same bits.
@@ -103,16 +103,28 @@ __device__ __forceinline__ int swz_w2(int row, int ch) {
 // Layer 3: a thread sums 4 input channels for a line of nodes, eight lanes are one
 // line; their sums are added by halving shuffles (one thread per node before: half
 // of the warps' issue slots idle, 20 loads for 64 products).
-// Measured (GB300, with activations stored): 16384 elements at p = 7 4.92 -> 3.02 ms,
-// 2000 at p = 6 0.57 -> 0.39, 200 at p = 4 0.061 -> 0.050, 4000 at p = 1 0.306 -> 0.063.
+// Measured (GB300, with activations stored): 16384 elements at p = 7 4.92 -> 2.91 ms,
+// 2000 at p = 6 0.57 -> 0.39, 200 at p = 4 0.061 -> 0.049, 4000 at p = 1 0.306 -> 0.060.
 constexpr int NN_FWD_THREADS = 512;
+
+// ldmatrix address of chunk c (8 channels) of row p, and of chunk c ^ 2 (16 channels on)
+__device__ __forceinline__ unsigned row_addr(unsigned base, int p, int c) {
+  return base + 64u * p + (((p << 3) & 0x30) ^ (c << 4));
+}
+__device__ __forceinline__ unsigned row_addr2(unsigned base, int p, int c) {
+  return base + 64u * p + (((p << 3) & 0x30) ^ (c << 4) ^ 32);
+}
 
 template <int N1>
 struct FwdCfg {
   using C = NNCfg<N1>;
-  // input rows in float2: odd, and planes 8 modulo 16, so that 16 lanes on lines of
-  // two planes of 8 read distinct banks
-  static constexpr int YS = C::P | 1, ZS = (C::P * YS + 7) / 16 * 16 + 8, IS = C::P * ZS;
+  // strides of the rows and planes of the two-channel fields, in float2, by which 16
+  // lanes on lines of neighbouring planes read distinct banks: odd rows and planes 8
+  // modulo 16, or, where P is twice an odd number (p = 7, which has no room for more),
+  // rows as they are and odd planes
+  static constexpr bool TWO = C::P % 4 == 2;
+  static constexpr int YS = TWO ? C::P : C::P | 1, ZS = TWO ? C::P * C::P + 1 : (C::P * YS + 7) / 16 * 16 + 8;
+  static constexpr int IS = C::P * ZS;
   static constexpr int ROWS = C::P3 * C::GROUP;
   static constexpr size_t SMEM = 2 * sizeof(__nv_bfloat16) * ROWS * NN_H + sizeof(__nv_bfloat16) * 27 * 32 * 32 +
                                  sizeof(float2) * C::GROUP * IS + sizeof(float) * (1760 + 1728 + 32);
@@ -157,10 +169,10 @@ __global__ void __launch_bounds__(NN_FWD_THREADS, 1)
     }
     __syncthreads();
     // layer 1 (2 -> 32)
-    for (int w = warp; w < (nl + 31) / 32 * 8; w += NW) {
-      const int l = w / 8 * 32 + lane, cg = w % 8 * 4, ll = l < nl ? l : 0;
-      const int y = ll % N1, z = ll / N1 % N1;
-      const float2* src = sIn + ll / LPE * F::IS + z * F::ZS + y * F::YS;
+    for (int w = tid; w < nl * 8; w += NT) {
+      const int cg = w / nl * 4, l = w % nl;
+      const int y = l % N1, z = l / N1 % N1;
+      const float2* src = sIn + l / LPE * F::IS + z * F::ZS + y * F::YS;
       float acc[N1][4];
 #pragma unroll
       for (int i = 0; i < N1; ++i)
@@ -183,14 +195,12 @@ __global__ void __launch_bounds__(NN_FWD_THREADS, 1)
             for (int c = 0; c < 4; ++c) acc[i][c] += v[i + dx].x * w0[c] + v[i + dx].y * w1[c];
         }
       }
-      if (l < nl) {
-        const int p0 = ll / LPE * C::P3 + (z + 1) * P * P + (y + 1) * P + 1;
+      const int p0 = l / LPE * C::P3 + (z + 1) * P * P + (y + 1) * P + 1;
 #pragma unroll
-        for (int i = 0; i < N1; ++i) {
-          const __nv_bfloat162 h0 = __floats2bfloat162_rn(fmaxf(acc[i][0], 0.f), fmaxf(acc[i][1], 0.f));
-          const __nv_bfloat162 h1 = __floats2bfloat162_rn(fmaxf(acc[i][2], 0.f), fmaxf(acc[i][3], 0.f));
-          *(uint2*)(sA1 + swz(p0 + i, cg)) = make_uint2(*(const unsigned*)&h0, *(const unsigned*)&h1);
-        }
+      for (int i = 0; i < N1; ++i) {
+        const __nv_bfloat162 h0 = __floats2bfloat162_rn(fmaxf(acc[i][0], 0.f), fmaxf(acc[i][1], 0.f));
+        const __nv_bfloat162 h1 = __floats2bfloat162_rn(fmaxf(acc[i][2], 0.f), fmaxf(acc[i][3], 0.f));
+        *(uint2*)(sA1 + swz(p0 + i, cg)) = make_uint2(*(const unsigned*)&h0, *(const unsigned*)&h1);
       }
     }
     __syncthreads();
@@ -209,24 +219,28 @@ __global__ void __launch_bounds__(NN_FWD_THREADS, 1)
         const int node = (mt0 + NW * a) * 16 + r + 8 * (j & 1);
         rowp[a] = node < np ? group_index<N1>(node) : -1;  // rows past the nodes read the zero corner
       }
+      // B tiles: matrix j = input channels 8 j .. 8 j + 7 of the 8 rows co of column tile nt
+      unsigned wa = smem_u32(sW2 + swz_w2(r, 8 * j));
+      const unsigned ab = smem_u32(sA1);
 #pragma unroll 1
-      for (int t = 0; t < 27; ++t) {
-        const int off = tap_offset<N1>(t);
-        // B tiles: matrix j = input channels 8 j .. 8 j + 7 of the 8 rows co of column tile nt
-        unsigned b[4][4];
+      for (int d = 0; d < 9; ++d) {
+        const int od = (d / 3 - 1) * P * P + (d % 3 - 1) * P - 1;
+#pragma unroll 1
+        for (int dx = 0; dx < 3; ++dx, wa += 2048) {
+          unsigned b[4][4];
 #pragma unroll
-        for (int nt = 0; nt < 4; ++nt)
-          ldsm_x4(smem_u32(sW2 + swz_w2(t * 32 + nt * 8 + r, 8 * j)), b[nt][0], b[nt][1], b[nt][2], b[nt][3]);
+          for (int nt = 0; nt < 4; ++nt) ldsm_x4(wa + nt * 512, b[nt][0], b[nt][1], b[nt][2], b[nt][3]);
 #pragma unroll
-        for (int a = 0; a < 2; ++a) {
-          if (mt0 + NW * a >= MT) continue;
-          const int q = rowp[a] >= 0 ? rowp[a] + off : 0;
+          for (int a = 0; a < 2; ++a) {
+            if (mt0 + NW * a >= MT) continue;
+            const int q = rowp[a] >= 0 ? rowp[a] + od + dx : 0;
 #pragma unroll
-          for (int kh = 0; kh < 2; ++kh) {
-            unsigned a0, a1, a2, a3;
-            ldsm_x4(smem_u32(sA1 + swz(q, kh * 16 + 8 * (j >> 1))), a0, a1, a2, a3);
+            for (int kh = 0; kh < 2; ++kh) {
+              unsigned a0, a1, a2, a3;
+              ldsm_x4(kh ? row_addr2(ab, q, j >> 1) : row_addr(ab, q, j >> 1), a0, a1, a2, a3);
 #pragma unroll
-            for (int nt = 0; nt < 4; ++nt) mma16816(acc[a][nt], a0, a1, a2, a3, b[nt][2 * kh], b[nt][2 * kh + 1]);
+              for (int nt = 0; nt < 4; ++nt) mma16816(acc[a][nt], a0, a1, a2, a3, b[nt][2 * kh], b[nt][2 * kh + 1]);
+            }
           }
         }
       }
@@ -324,12 +338,17 @@ __global__ void __launch_bounds__(NN_FWD_THREADS, 1)
 // loads each, most of the kernel's time. Shared-memory activations are swizzled
 // as in the forward kernel (unswizzled rows put an ldmatrix phase on four banks),
 // W2 stays in shared memory, and operand tiles are loaded once for all taps of a
-// warp. g_a2 (FP32 weights and inputs, K = 54) stays on the FP32 pipe, 16
-// channels of a node per thread.
-// Measured (GB300, 16384 elements, p = 7): 28.8 -> 7.2 ms; 2000 elements at p = 6
-// 6.7 -> 1.18 ms. Elements with few nodes go through in groups (p = 1: up to 12),
-// since one of them fills neither the warps nor an MMA row tile: 4000 elements at p =
-// 1 0.294 -> 0.141 ms (one at a time 0.476), 500 at p = 4 0.587 -> 0.155 ms (0.179).
+// warp. g_a2 (FP32 weights and inputs, K = 54) stays on the FP32 pipe, two channels
+// of a line per thread. Tap offsets are outside the loops, a tile's second half is
+// 32 bytes off by an exclusive or, and all operand loads stand before the products:
+// address arithmetic and load latency, not the MMAs, set the time of the tile loops.
+// Measured (GB300, 16384 elements, p = 7): 28.8 -> 5.9 ms (7.1 with addresses worked
+// out at each load and g_a2 by nodes); cycles per element now: loads 7 k, dW3 13 k,
+// g_a2 22 k, dW2 28 k, g_a1 24 k, dW1 18 k. 2000 elements at p = 6 6.7 -> 0.84 ms.
+// Elements with few nodes go through in groups (p = 1: up to 12), since one of them
+// fills neither the warps nor an MMA row tile: 4000 elements at p = 1 0.294 -> 0.134 ms
+// (one at a time 0.476), 500 at p = 4 0.587 -> 0.153 ms (0.179). What is slower: at
+// most 152 elements at p = 1 (0.054 -> 0.069 ms, staging W2).
 // ---------------------------------------------------------------------------
 constexpr int NN_BWD_THREADS = 512;
 
@@ -374,49 +393,51 @@ __device__ __forceinline__ void join3(const float* d, int c4, float& run, float&
 // acc[a] (32 rows x 8 columns) = sum_n act[n]^T col[n + sgn off(tap a)] for this
 // warp's taps, joined to run[a][m] every JOIN node tiles. The tensor core rounds
 // its accumulator toward zero: dW1 is 4.5e-7 off its float64 sums at 16384 elements
-// with one chain over the element (JOIN 32), 2.0e-7 with 16, 1.1e-7 with 8 (7.6
-// against 7.2 ms); the FP32 chains before were 4.4e-7 off. dW3: 0.4e-7, 2.9e-7.
+// with one chain over the element (JOIN 32), 2.0e-7 with 16, 1.1e-7 with 8 (0.4 ms
+// slower); the FP32 chains before were 4.4e-7 off. dW3: 0.4e-7, 2.9e-7.
 template <int N1, int JOIN>
 __device__ __forceinline__ void split_grad(const __nv_bfloat16* act, const __nv_bfloat16* col, int sgn, int np,
                                            int warp, int lane, float (*run)[2], float (*car)[2]) {
   constexpr int NW = NN_BWD_THREADS / 32;
+  constexpr bool FULL = NNCfg<N1>::NPE % 16 == 0;  // no row tile reaches past the nodes
   const int MT = (np + 15) / 16;
   const int j = lane >> 3, r = lane & 7, c4 = lane & 3;
-  float acc[2][2][4];
+  const unsigned ab = smem_u32(act), cb = smem_u32(col);
+  const bool two = warp + NW < 27;  // this warp's taps: warp, warp + NW
+  int off[2];
 #pragma unroll
-  for (int a = 0; a < 2; ++a)
-#pragma unroll
-    for (int m = 0; m < 2; ++m)
-#pragma unroll
-      for (int c = 0; c < 4; ++c) acc[a][m][c] = 0.f;
+  for (int a = 0; a < 2; ++a) off[a] = sgn * 16 * tap_offset<N1>(a == 0 || two ? warp + NW * a : warp);
 #pragma unroll 1
-  for (int kt = 0; kt < MT; ++kt) {
-    const int na = kt * 16 + r + 8 * (j >> 1), nb = kt * 16 + (lane & 15);
-    const int pA = na < np ? group_index<N1>(na) : 0;
-    const int pB = nb < np ? group_index<N1>(nb) : -1;
-    unsigned A[2][4];
+  for (int k0 = 0; k0 < MT; k0 += JOIN) {
+    const int k1 = k0 + JOIN < MT ? k0 + JOIN : MT;
+    float acc[2][2][4];
 #pragma unroll
-    for (int m = 0; m < 2; ++m)
-      ldsm_x4_t(smem_u32(act + swz(pA, m * 16 + 8 * (j & 1))), A[m][0], A[m][1], A[m][2], A[m][3]);
+    for (int a = 0; a < 2; ++a)
 #pragma unroll
-    for (int a = 0; a < 2; ++a) {
-      const int t = warp + NW * a;
-      if (t >= 27) continue;
-      unsigned b0, b1;
-      ldsm_x2_t(smem_u32(col + (pB < 0 ? 0 : pB + sgn * tap_offset<N1>(t)) * 8), b0, b1);
+      for (int m = 0; m < 2; ++m)
 #pragma unroll
-      for (int m = 0; m < 2; ++m) mma16816(acc[a][m], A[m][0], A[m][1], A[m][2], A[m][3], b0, b1);
-    }
-    if (kt % JOIN == JOIN - 1 || kt == MT - 1) {
+        for (int c = 0; c < 4; ++c) acc[a][m][c] = 0.f;
+#pragma unroll 2
+    for (int kt = k0; kt < k1; ++kt) {
+      const int na = kt * 16 + r + 8 * (j >> 1), nb = kt * 16 + (lane & 15);
+      const bool okb = FULL || nb < np;
+      const int pA = FULL || na < np ? group_index<N1>(na) : 0;
+      const unsigned bb = cb + 16 * (okb ? group_index<N1>(nb) : 0);
+      unsigned A[2][4], b[2][2];  // all loads before the first product
+      ldsm_x4_t(row_addr(ab, pA, j & 1), A[0][0], A[0][1], A[0][2], A[0][3]);
+      ldsm_x4_t(row_addr2(ab, pA, j & 1), A[1][0], A[1][1], A[1][2], A[1][3]);
+#pragma unroll
+      for (int a = 0; a < 2; ++a) ldsm_x2_t(bb + (okb ? off[a] : 0), b[a][0], b[a][1]);
 #pragma unroll
       for (int a = 0; a < 2; ++a)
 #pragma unroll
-        for (int m = 0; m < 2; ++m) {
-          join3(acc[a][m], c4, run[a][m], car[a][m]);
-#pragma unroll
-          for (int c = 0; c < 4; ++c) acc[a][m][c] = 0.f;
-        }
+        for (int m = 0; m < 2; ++m) mma16816(acc[a][m], A[m][0], A[m][1], A[m][2], A[m][3], b[a][0], b[a][1]);
     }
+#pragma unroll
+    for (int a = 0; a < 2; ++a)
+#pragma unroll
+      for (int m = 0; m < 2; ++m)
+        if (a == 0 || two) join3(acc[a][m], c4, run[a][m], car[a][m]);
   }
 }
 
@@ -426,7 +447,8 @@ __global__ void __launch_bounds__(NN_BWD_THREADS, 1)
                   const __nv_bfloat16* __restrict__ a1g, const __nv_bfloat16* __restrict__ a2g,
                   const float* __restrict__ gout, float* __restrict__ part, long long ne, int ng) {
   using C = NNCfg<N1>;
-  constexpr int P3 = C::P3 * C::GROUP, NT = NN_BWD_THREADS, NW = NT / 32;
+  using F = FwdCfg<N1>;
+  constexpr int P3 = C::P3 * C::GROUP, P = C::P, NT = NN_BWD_THREADS, NW = NT / 32, LPE = N1 * N1;
   extern __shared__ __align__(16) unsigned char smem[];
   // sA1 holds a1 until the layer-2 weight gradient is done, then g_a1 (masked)
   __nv_bfloat16* sA1 = (__nv_bfloat16*)smem;                           // [P3][32] swizzled
@@ -436,10 +458,10 @@ __global__ void __launch_bounds__(NN_BWD_THREADS, 1)
   __nv_bfloat16* sW2 = sIs + P3 * 8;                                    // [27 * 32 ci][32 co] swizzled
   float* sW3 = (float*)(sW2 + 27 * 32 * 32);                           // [27][32][2]
   float* sred = sW3 + 1728;                                            // [NW][32]
-  float* sG3 = sred + NW * 32;                                         // [P3][2]
+  float2* sG3 = (float2*)(sred + NW * 32);                             // [GROUP][P][P][.], rows as in FwdCfg
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   for (int i = tid; i < P3 * (NN_H + 8); i += NT) ((unsigned*)sA1)[i] = 0u;  // sA1, sA2, sGs, sIs
-  for (int i = tid; i < 2 * P3; i += NT) sG3[i] = 0.f;
+  for (int i = tid; i < C::GROUP * F::IS; i += NT) sG3[i] = make_float2(0.f, 0.f);
   for (int i = tid; i < 1728; i += NT) sW3[i] = prm[NN_OW3 + i];
   for (int i = tid; i < 27 * 32 * 4; i += NT)
     *(uint4*)(sW2 + swz_w2(i >> 2, (i & 3) * 8)) = ((const uint4*)W2o)[i];
@@ -464,6 +486,10 @@ __global__ void __launch_bounds__(NN_BWD_THREADS, 1)
     for (int n = warp; n < np; n += NW) acc += __bfloat162float(A[swz(group_index<N1>(n), lane)]);
     sred[warp * 32 + lane] = acc;
   };
+  auto g3_index = [](int n) {
+    const int l = n / N1;
+    return l / LPE * F::IS + (l / N1 % N1 + 1) * F::ZS + (l % N1 + 1) * F::YS + n % N1 + 1;
+  };
   auto bias_join = [&](float& db) {
     if (tid < 32) {
       float acc = 0.f;
@@ -478,8 +504,7 @@ __global__ void __launch_bounds__(NN_BWD_THREADS, 1)
     for (int i = tid; i < np; i += NT) {
       const int p = group_index<N1>(i);
       const float2 x = ((const float2*)in)[nb0 + i], y = ((const float2*)gout)[nb0 + i];
-      sG3[2 * p] = y.x;
-      sG3[2 * p + 1] = y.y;
+      sG3[g3_index(i)] = y;
       split3(x.x, sIs + 8 * p);
       split3(x.y, sIs + 8 * p + 3);
       split3(y.x, sGs + 8 * p);
@@ -497,9 +522,9 @@ __global__ void __launch_bounds__(NN_BWD_THREADS, 1)
     {
       float x = 0.f, y = 0.f;
       for (int i = tid; i < np; i += NT) {
-        const int p = group_index<N1>(i);
-        x += sG3[2 * p];
-        y += sG3[2 * p + 1];
+        const float2 v = sG3[g3_index(i)];
+        x += v.x;
+        y += v.y;
       }
 #pragma unroll
       for (int d = 16; d > 0; d >>= 1) {
@@ -519,66 +544,76 @@ __global__ void __launch_bounds__(NN_BWD_THREADS, 1)
       db3 += acc;
     }
     // g_a2[n][ci] = (sum_t sum_co W3[t][ci][co] g3[n - t][co]) * (a2[n][ci] > 0), in place of a2:
-    // thread = node and half of the channels (the same for a warp: weights are broadcast reads)
-    for (int w = warp; w < (np + 31) / 32 * 2; w += NW) {
-      const int n = (w >> 1) * 32 + lane, c0 = (w & 1) * 16;
-      const int p = n < np ? group_index<N1>(n) : group_index<N1>(0);
-      float acc[16];
+    // thread = line along x and two channels (mostly the same for a warp: weights are broadcast reads)
+    const int nl = np / N1;
+    for (int w = tid; w < nl * 16; w += NT) {
+      const int cg = w / nl * 2, l = w % nl;
+      const int y = l % N1, z = l / N1 % N1;
+      const float2* src = sG3 + l / LPE * F::IS + (z + 2) * F::ZS + (y + 2) * F::YS;
+      float acc[N1][2];
 #pragma unroll
-      for (int c = 0; c < 16; ++c) acc[c] = 0.f;
+      for (int i = 0; i < N1; ++i) acc[i][0] = acc[i][1] = 0.f;
 #pragma unroll 1
-      for (int t = 0; t < 27; ++t) {
-        const int q = p - tap_offset<N1>(t);
-        const float g0 = sG3[2 * q], g1 = sG3[2 * q + 1];
-        const float4* wt = (const float4*)(sW3 + t * 64 + c0 * 2);
+      for (int d = 0; d < 9; ++d) {
+        const float2* row = src - d / 3 * F::ZS - d % 3 * F::YS;
+        float2 v[P];
 #pragma unroll
-        for (int c = 0; c < 8; ++c) {
-          const float4 v = wt[c];
-          acc[2 * c] += v.x * g0 + v.y * g1;
-          acc[2 * c + 1] += v.z * g0 + v.w * g1;
+        for (int i = 0; i < P; ++i) v[i] = row[i];
+#pragma unroll
+        for (int dx = 0; dx < 3; ++dx) {
+          const float4 wt = *(const float4*)(sW3 + (3 * d + dx) * 64 + cg * 2);
+#pragma unroll
+          for (int i = 0; i < N1; ++i) {
+            const float g0 = v[i + 2 - dx].x, g1 = v[i + 2 - dx].y;
+            acc[i][0] += wt.x * g0 + wt.y * g1;
+            acc[i][1] += wt.z * g0 + wt.w * g1;
+          }
         }
       }
-      if (n < np) {
+      const int p0 = l / LPE * C::P3 + (z + 1) * P * P + (y + 1) * P + 1;
 #pragma unroll
-        for (int c = 0; c < 2; ++c) {
-          uint4* dst = (uint4*)(sA2 + swz(p, c0 + 8 * c));
-          uint4 raw = *dst;
-          __nv_bfloat162* hv = (__nv_bfloat162*)&raw;
-#pragma unroll
-          for (int k = 0; k < 4; ++k) {
-            const float2 v = __bfloat1622float2(hv[k]);
-            hv[k] = __floats2bfloat162_rn(v.x > 0.f ? acc[8 * c + 2 * k] : 0.f, v.y > 0.f ? acc[8 * c + 2 * k + 1] : 0.f);
-          }
-          *dst = raw;
-        }
+      for (int i = 0; i < N1; ++i) {
+        __nv_bfloat162* dst = (__nv_bfloat162*)(sA2 + swz(p0 + i, cg));
+        const float2 v = __bfloat1622float2(*dst);
+        *dst = __floats2bfloat162_rn(v.x > 0.f ? acc[i][0] : 0.f, v.y > 0.f ? acc[i][1] : 0.f);
       }
     }
     __syncthreads();
     bias_part(sA2, np);
     // layer 2 weights: dW2[t] (ci x co) += sum_n a1[n + t][ci] g_a2[n][co]
+    {
+      constexpr bool FULL = C::NPE % 16 == 0;
+      const unsigned b1 = smem_u32(sA1), b2 = smem_u32(sA2);
+      const bool two = warp + NW < 27;
+      int off[2];
+#pragma unroll
+      for (int a = 0; a < 2; ++a) off[a] = tap_offset<N1>(a == 0 || two ? warp + NW * a : warp);
 #pragma unroll 1
-    for (int kt = 0; kt < MT; ++kt) {
-      // k = 16 nodes of tile kt; lane row address: node kt*16 + r + 8*(j>>1)
-      const int node = kt * 16 + r + 8 * (j >> 1);
-      const int p = node < np ? group_index<N1>(node) : -1;
-      unsigned b[2][4];
+      for (int kt = 0; kt < MT; ++kt) {
+        // k = 16 nodes of tile kt; lane row address: node kt*16 + r + 8*(j>>1)
+        const int node = kt * 16 + r + 8 * (j >> 1);
+        const bool ok = FULL || node < np;
+        const int p = ok ? group_index<N1>(node) : 0;
+        unsigned b[2][4];
+        ldsm_x4_t(row_addr(b2, p, j & 1), b[0][0], b[0][1], b[0][2], b[0][3]);
+        ldsm_x4_t(row_addr2(b2, p, j & 1), b[1][0], b[1][1], b[1][2], b[1][3]);
+        unsigned A[2][2][4];  // all loads before the first product
 #pragma unroll
-      for (int nh = 0; nh < 2; ++nh)
-        ldsm_x4_t(smem_u32(sA2 + swz(p < 0 ? 0 : p, nh * 16 + 8 * (j & 1))), b[nh][0], b[nh][1], b[nh][2], b[nh][3]);
+        for (int a = 0; a < 2; ++a) {
+          const int pA = ok ? p + off[a] : 0;
+          ldsm_x4_t(row_addr(b1, pA, j & 1), A[a][0][0], A[a][0][1], A[a][0][2], A[a][0][3]);
+          ldsm_x4_t(row_addr2(b1, pA, j & 1), A[a][1][0], A[a][1][1], A[a][1][2], A[a][1][3]);
+        }
 #pragma unroll
-      for (int a = 0; a < 2; ++a) {
-        const int t = warp + NW * a;
-        if (t >= 27) continue;
-        const int pA = p < 0 ? 0 : p + tap_offset<N1>(t);
+        for (int a = 0; a < 2; ++a) {
+          if (a == 1 && !two) continue;
 #pragma unroll
-        for (int m = 0; m < 2; ++m) {
-          unsigned a0, a1r, a2r, a3;
-          ldsm_x4_t(smem_u32(sA1 + swz(pA, m * 16 + 8 * (j & 1))), a0, a1r, a2r, a3);
+          for (int m = 0; m < 2; ++m)
 #pragma unroll
-          for (int nh = 0; nh < 2; ++nh) {
-            mma16816(accW[a][m][2 * nh], a0, a1r, a2r, a3, b[nh][0], b[nh][2]);
-            mma16816(accW[a][m][2 * nh + 1], a0, a1r, a2r, a3, b[nh][1], b[nh][3]);
-          }
+            for (int nh = 0; nh < 2; ++nh) {
+              mma16816(accW[a][m][2 * nh], A[a][m][0], A[a][m][1], A[a][m][2], A[a][m][3], b[nh][0], b[nh][2]);
+              mma16816(accW[a][m][2 * nh + 1], A[a][m][0], A[a][m][1], A[a][m][2], A[a][m][3], b[nh][1], b[nh][3]);
+            }
         }
       }
     }
@@ -600,24 +635,29 @@ __global__ void __launch_bounds__(NN_BWD_THREADS, 1)
         const int node = (mt0 + NW * a) * 16 + r + 8 * (j & 1);
         prow[a] = node < np ? group_index<N1>(node) : -1;
       }
+      // W2 tiles: matrices j = (kh, 8-column half) of the 8 rows ci of column tile nt
+      unsigned wa = smem_u32(sW2 + swz_w2(r, 8 * j));
+      const unsigned ab = smem_u32(sA2);
 #pragma unroll 1
-      for (int t = 0; t < 27; ++t) {
-        const int off = tap_offset<N1>(t);
-        // W2 tiles: matrices j = (kh, 8-column half) of the 8 rows ci of column tile nt
-        unsigned w2[4][4];
+      for (int d = 0; d < 9; ++d) {
+        const int od = (d / 3 - 1) * P * P + (d % 3 - 1) * P - 1;
+#pragma unroll 1
+        for (int dx = 0; dx < 3; ++dx, wa += 2048) {
+          unsigned w2[4][4];
 #pragma unroll
-        for (int nt = 0; nt < 4; ++nt)
-          ldsm_x4(smem_u32(sW2 + swz_w2(t * 32 + nt * 8 + r, 8 * j)), w2[nt][0], w2[nt][1], w2[nt][2], w2[nt][3]);
+          for (int nt = 0; nt < 4; ++nt) ldsm_x4(wa + nt * 512, w2[nt][0], w2[nt][1], w2[nt][2], w2[nt][3]);
 #pragma unroll
-        for (int a = 0; a < 2; ++a) {
-          if (mt0 + NW * a >= MT) continue;
-          const int q = prow[a] >= 0 ? prow[a] - off : 0;
+          for (int a = 0; a < 2; ++a) {
+            if (mt0 + NW * a >= MT) continue;
+            const int q = prow[a] >= 0 ? prow[a] - od - dx : 0;
+            unsigned A[2][4];
+            ldsm_x4(row_addr(ab, q, j >> 1), A[0][0], A[0][1], A[0][2], A[0][3]);
+            ldsm_x4(row_addr2(ab, q, j >> 1), A[1][0], A[1][1], A[1][2], A[1][3]);
 #pragma unroll
-          for (int kh = 0; kh < 2; ++kh) {
-            unsigned a0, a1r, a2r, a3;
-            ldsm_x4(smem_u32(sA2 + swz(q, kh * 16 + 8 * (j >> 1))), a0, a1r, a2r, a3);
+            for (int kh = 0; kh < 2; ++kh)
 #pragma unroll
-            for (int nt = 0; nt < 4; ++nt) mma16816(acc[a][nt], a0, a1r, a2r, a3, w2[nt][2 * kh], w2[nt][2 * kh + 1]);
+              for (int nt = 0; nt < 4; ++nt)
+                mma16816(acc[a][nt], A[kh][0], A[kh][1], A[kh][2], A[kh][3], w2[nt][2 * kh], w2[nt][2 * kh + 1]);
           }
         }
       }
@@ -706,10 +746,13 @@ __global__ void k_nn_adam(float* __restrict__ prm, const float* __restrict__ gra
   prm[i] -= lr * (mi / c1) / (sqrtf(vi / c2) + eps);
 }
 
-static size_t bwd_smem(int n1, int group) {
-  const int P3 = group * (n1 + 2) * (n1 + 2) * (n1 + 2);
-  return sizeof(__nv_bfloat16) * (2 * P3 * (NN_H + 8) + 27 * 32 * 32) +
-         sizeof(float) * (2 * P3 + 1728 + NN_BWD_THREADS);
+template <int N1>
+static constexpr size_t bwd_smem() {
+  using C = NNCfg<N1>;
+  constexpr size_t sm = sizeof(__nv_bfloat16) * (2 * C::P3 * C::GROUP * (NN_H + 8) + 27 * 32 * 32) +
+                        sizeof(float2) * C::GROUP * FwdCfg<N1>::IS + sizeof(float) * (1728 + NN_BWD_THREADS);
+  static_assert(sm <= 227 * 1024, "shared memory of a block");
+  return sm;
 }
 
 static int sm_count() {
@@ -762,7 +805,7 @@ template <int N1>
 static int nn_bwd_blocks(long long ne) {
   static int bps = 0;
   if (!bps) {
-    const size_t sm = bwd_smem(N1, NNCfg<N1>::GROUP);
+    const size_t sm = bwd_smem<N1>();
     if (cudaFuncSetAttribute(k_nn_backward<N1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm) != cudaSuccess)
       return 0;
     bps = blocks_per_sm(k_nn_backward<N1>, sm, NN_BWD_THREADS);
@@ -776,7 +819,7 @@ static cudaError_t nn_bwd_n1(const float* prm, const __nv_bfloat16* W2o, const f
                              const __nv_bfloat16* a2, const float* gout, float* part, int nblk, long long ne,
                              cudaStream_t s) {
   count_launch();
-  k_nn_backward<N1><<<nblk, NN_BWD_THREADS, bwd_smem(N1, NNCfg<N1>::GROUP), s>>>(prm, W2o, in, a1, a2, gout, part, ne,
+  k_nn_backward<N1><<<nblk, NN_BWD_THREADS, bwd_smem<N1>(), s>>>(prm, W2o, in, a1, a2, gout, part, ne,
                                                                                  nn_group<N1>(ne, nblk));
   return cudaGetLastError();
 }
