@@ -501,7 +501,9 @@ int dg_octree_node_coords(dg_oct_handle h, double* xyz_dev, double* w_dev, void*
 
 /* The operator on the handle's mesh: out = A u for B fields (0..65535), u_dev
  * and out_dev [B][Nq] device, not overlapping (DG_ERR_INVALID_ARG). Stream
- * ordered: launches one kernel and returns without synchronising. */
+ * ordered: launches its one or two kernels (two where the mesh has hanging
+ * faces) and returns without synchronising; calls on several streams share the
+ * handle's flux scratch and run one after the other. */
 int dg_octree_operator(dg_oct_handle h, const double* u_dev, double* out_dev, int64_t B, void* cuda_stream);
 
 /* The handle's preconditioner alone for B fields: z = V(r), one V-cycle

@@ -208,9 +208,10 @@ bool octree_faces(const dg_mesh_desc* root, const int32_t* leaves, int32_t n_lea
 //
 // Measured (GB300, density-refined chain octree, 715 leaves, p = 6, 8 fields; one
 // block per leaf with every face interpolated to Gauss points and back before):
-// FP32 396 -> 20 us (5 us of it the hanging faces), FP64 974 -> 255 us; the V-cycle of the FP32 solve, three degrees of this
-// operator and the leaf-block inverse, 9.8 -> 4.2 ms in FP64; a mixed solve of 8
-// sources to 1e-10 241 -> 85 ms.
+// FP32 396 -> 20 us (5 us of it the hanging faces), FP64 974 -> 255 us; the V-cycle of
+// the FP64 solve, three degrees of this operator and the leaf-block inverse, 9.8 ->
+// 4.2 ms; a mixed solve of 8 sources to 1e-10 241 -> 85 ms by this alone (43 ms with
+// the fused leaf-block inverse and the 16-row boundary GEMM).
 // ---------------------------------------------------------------------------
 
 // tables of k_oct_apply: 1-D stiffness and end traces, folded (see dg_apply.cu)

@@ -32,6 +32,7 @@
 #include <cmath>
 #include <cstring>
 #include <map>
+#include <mutex>
 #include <string>
 #include <tuple>
 #include <vector>
@@ -106,6 +107,7 @@ struct dg_oct {
   // whatever stream) behind them
   dg::DevBuf hang, hang_op;
   cudaEvent_t op_done = nullptr;
+  std::mutex op_mutex;
   std::vector<int> act_host;
   ~dg_oct() {
     if (op_done) cudaEventDestroy(op_done);
@@ -559,12 +561,15 @@ static cudaError_t launch_bjac(const dg_oct* h, const OctLevel& L, int mode, con
 // out = A u, or with rin out = rin - A u
 template <typename V>
 static cudaError_t oct_apply(const dg_oct* h, const OctLevel& L, const V* u, V* out, const int* act, int nact,
-                             cudaStream_t s, const V* rin = nullptr, const DevBuf* hang = nullptr) {
-  if (!hang) hang = &h->hang;
+                             cudaStream_t s, const V* rin = nullptr, void* hang = nullptr, size_t bytes = 0) {
+  if (!hang) {
+    hang = h->hang.p;
+    bytes = h->hang.bytes;
+  }
   const OctMesh m{h->E, h->kind.as<int>(), h->nb.as<int>(), h->fac.as<double>(), h->hslot.as<int>(), h->rec.as<int>(),
                   h->nI};
-  return launch_octree_apply<V>(L.n1, L.T, m, h->eps, u, out, rin, act, nact, hang->as<V>(),
-                                (long long)(hang->bytes / sizeof(V)), s);
+  return launch_octree_apply<V>(L.n1, L.T, m, h->eps, u, out, rin, act, nact, (V*)hang,
+                                (long long)(bytes / sizeof(V)), s);
 }
 
 static cudaError_t launch_oct_lift(const dg_oct* h, const double* g, double* b, int nsrc, cudaStream_t s) {
@@ -1428,14 +1433,27 @@ int dg_octree_operator(dg_oct_handle h, const double* u_dev, double* out_dev, in
   const char *u0 = (const char*)u_dev, *o0 = (const char*)out_dev;
   if (u0 < o0 + bytes && o0 < u0 + bytes) return DG_ERR_INVALID_ARG;
   cudaStream_t s = (cudaStream_t)stream;
-  // inside a capture the order of the graph's launches is the caller's
-  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-  if (h->nI > 0) {
-    DG_CK(cudaStreamIsCapturing(s, &cap));
-    if (cap == cudaStreamCaptureStatusNone) DG_CK(cudaStreamWaitEvent(s, h->op_done, 0));
+  if (h->nI == 0) {
+    DG_CK(oct_apply<double>(h, h->lv[0], u_dev, out_dev, nullptr, (int)B, s));
+    return DG_OK;
   }
-  DG_CK(oct_apply<double>(h, h->lv[0], u_dev, out_dev, nullptr, (int)B, s, nullptr, &h->hang_op));
-  if (h->nI > 0 && cap == cudaStreamCaptureStatusNone) DG_CK(cudaEventRecord(h->op_done, s));
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  DG_CK(cudaStreamIsCapturing(s, &cap));
+  if (cap != cudaStreamCaptureStatusNone) {
+    // the graph allocates and frees its own scratch: its replays may overlap with
+    // anything else that runs on the handle
+    const size_t hb = hang_bytes(h, (int)std::min<int64_t>(B, 64));
+    void* p = nullptr;
+    DG_CK(cudaMallocAsync(&p, hb, s));
+    const cudaError_t e = oct_apply<double>(h, h->lv[0], u_dev, out_dev, nullptr, (int)B, s, nullptr, p, hb);
+    DG_CK(cudaFreeAsync(p, s));
+    DG_CK(e);
+    return DG_OK;
+  }
+  std::lock_guard<std::mutex> lock(h->op_mutex);  // wait, launches and record of one call belong together
+  DG_CK(cudaStreamWaitEvent(s, h->op_done, 0));
+  DG_CK(oct_apply<double>(h, h->lv[0], u_dev, out_dev, nullptr, (int)B, s, nullptr, h->hang_op.p, h->hang_op.bytes));
+  DG_CK(cudaEventRecord(h->op_done, s));
   return DG_OK;
 }
 
