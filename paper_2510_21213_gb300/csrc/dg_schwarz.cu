@@ -485,8 +485,8 @@ static cudaError_t patch_fill(const SwTables& tb, const T* r, T* zp, const int* 
 // are full.
 // Measured around the line (us, small / several): FP64 p = 4 256 patches 13.3 / 22.4,
 // 1024 41.3 / 41.5, 4096 152 / 119; p = 6 512 54 / 68, 1024 103 / 100; p = 8 64 28.1 /
-// 29.7, 256 53.7 / 50.1; p = 1 512 4.2 / 6.6, 4096 14.6 / 14.1; FP32 p = 6 512 6.2 / 7.9, 1024 9.2 / 8.0; p = 4 256 3.2 / 4.4,
-// 1024 5.6 / 5.0; p = 2 1024 3.5 / 5.7.
+// 29.7, 256 53.7 / 50.1; p = 1 512 4.2 / 6.6, 4096 14.6 / 14.1; FP32 p = 6 512 6.2 /
+// 7.9, 1024 9.2 / 8.0; p = 4 256 3.2 / 4.4, 1024 5.6 / 5.0; p = 2 1024 3.5 / 5.7.
 template <typename T, int N1>
 static cudaError_t patch_n1(const SwTables& tb, const T* r, T* zp, const int* act, int nact, cudaStream_t s) {
   const long long items = (long long)tb.geom.n[0] * tb.geom.n[1] * tb.geom.n[2] * nact;
