@@ -291,14 +291,16 @@ __global__ void __launch_bounds__(128) k_gemm_tc(GemmArgs g, int batch_base, int
 // octree's boundary data). In a 64-row tile most of the MMAs, TwoSums and operand
 // loads would be padding; here a warp owns one 16-row MMA tile and 32 columns and
 // takes its fragments of B straight from global memory (a fragment row is 8
-// consecutive columns, one 32-byte sector), the next 16-term tile in flight while
-// the current one is worked; no shared memory, no barriers. ROWS8: rows 8 to 15
+// consecutive columns, one 32-byte sector), the next two 16-term tiles in flight
+// while the current one is worked; no shared memory, no barriers. ROWS8: rows 8 to 15
 // are padding too, their sums are not kept. Every product, MMA and TwoSum is that
 // of k_gemm_tc in the same order, so the results are the same bits.
-// Measured (GB300, 8 x 18816 x 245245, the octree of the ten-atom chain): 34.2 ->
-// about 4.5 ms (B is 18.5 GB: 2.7 ms at the measured bandwidth).
+// Measured (GB300, 18816 x 245245, the octree of the ten-atom chain): 8 rows 34.2 ->
+// 4.17 ms (4.51 with one tile in flight), 16 rows 5.51 ms (6.94; three blocks per SM
+// there, with four the accumulators of rows 8 to 15 spill). B is 18.5 GB: 2.7 ms at
+// the measured bandwidth.
 template <bool ROWS8>
-__global__ void __launch_bounds__(128, 4) k_gemm_tc_thin(GemmArgs g, int batch_base, int nsplit, int kc, int nbc) {
+__global__ void __launch_bounds__(128, ROWS8 ? 4 : 3) k_gemm_tc_thin(GemmArgs g, int batch_base, int nsplit, int kc, int nbc) {
   constexpr int NT = 4;                // 8-column tiles of a warp
   constexpr int NE = ROWS8 ? 2 : 4;    // live accumulators of an MMA tile per lane
   constexpr int NA = ROWS8 ? 2 : 4;
@@ -313,74 +315,80 @@ __global__ void __launch_bounds__(128, 4) k_gemm_tc_thin(GemmArgs g, int batch_b
   const int gq = lane >> 2, c4 = lane & 3;
   const int n0 = (blockIdx.x * 4 + warp) * 8 * NT;
   if (n0 >= g.N) return;
-  // this lane's rows (A) and columns (B); outside the matrix they read as zero
+  // this lane's rows (A) and columns (B), from term kbeg + c4 on; outside the matrix they read as zero
   bool mok[2], nok[NT];
-  const float* pa[2];
-  const float* pb[NT];
 #pragma unroll
-  for (int i = 0; i < 2; ++i) {
-    mok[i] = gq + 8 * i < g.M;
-    pa[i] = A + (mok[i] ? (long long)(gq + 8 * i) * g.sAm : 0);
-  }
+  for (int i = 0; i < 2; ++i) mok[i] = gq + 8 * i < g.M;
 #pragma unroll
-  for (int j = 0; j < NT; ++j) {
-    nok[j] = n0 + 8 * j + gq < g.N;
-    pb[j] = B + (nok[j] ? (long long)(n0 + 8 * j + gq) * g.sBn : 0);
-  }
-  float acc[NT][4], sum[NT][NE], car[NT][NE];
+  for (int j = 0; j < NT; ++j) nok[j] = n0 + 8 * j + gq < g.N;
+  const float* pa = A + (long long)gq * g.sAm + (long long)(kbeg + c4) * g.sAk;
+  const float* pb = B + (long long)(n0 + gq) * g.sBn + (long long)(kbeg + c4) * g.sBk;
+  float sum[NT][NE], car[NT][NE];
 #pragma unroll
   for (int j = 0; j < NT; ++j)
 #pragma unroll
     for (int e = 0; e < NE; ++e) sum[j][e] = car[j][e] = 0.f;
-  // operands of one 16-term tile: A at k = c4 + 4 t, t < 4 (two MMA steps)
-  float ra[4][2], rb[NT][4];
-  auto load = [&](int k0) {
+  // operands of two 16-term tiles: A at k = c4 + 4 t, t < 4 (two MMA steps)
+  float ra[2][4][NA / 2], rb[2][NT][4];
+  auto load_a = [&](float (*r)[NA / 2], const float* p, int k0) {
 #pragma unroll
-    for (int t = 0; t < 4; ++t) {
-      const int k = k0 + c4 + 4 * t;
-      const bool kok = k < kend;
+    for (int t = 0; t < 4; ++t, p += 4 * (long long)g.sAk)
 #pragma unroll
-      for (int i = 0; i < NA / 2; ++i) ra[t][i] = kok && mok[i] ? __ldg(pa[i] + (long long)k * g.sAk) : 0.f;
-#pragma unroll
-      for (int j = 0; j < NT; ++j) rb[j][t] = kok && nok[j] ? __ldg(pb[j] + (long long)k * g.sBk) : 0.f;
-    }
+      for (int i = 0; i < NA / 2; ++i)
+        r[t][i] = k0 + c4 + 4 * t < kend && mok[i] ? __ldg(p + 8 * i * (long long)g.sAm) : 0.f;
   };
-  load(kbeg);
-  for (int k0 = kbeg; k0 < kend; k0 += 16) {
-    unsigned ah[2][4], al[2][4], bh[NT][4], bl[NT][4];
+  auto load_b = [&](float* r, const float* p, int j, int k0) {
+    p += 8 * j * (long long)g.sBn;
 #pragma unroll
-    for (int t = 0; t < 4; ++t) {
+    for (int t = 0; t < 4; ++t, p += 4 * (long long)g.sBk) r[t] = k0 + c4 + 4 * t < kend && nok[j] ? __ldg(p) : 0.f;
+  };
+  // one tile; its registers take the loads of the tile after next as they come free
+  auto tile = [&](float (*xa)[NA / 2], float (*xb)[4], int k0) {
+    unsigned ah[2][4], al[2][4];
+#pragma unroll
+    for (int t = 0; t < 4; ++t)
 #pragma unroll
       for (int i = 0; i < 2; ++i) {
-        const float x = ROWS8 && i == 1 ? 0.f : ra[t][i];
+        const float x = ROWS8 && i == 1 ? 0.f : xa[t][i];
         const unsigned hi = to_tf32(x);
         ah[t >> 1][(t & 1) * 2 + i] = hi;
         al[t >> 1][(t & 1) * 2 + i] = to_tf32(x - __uint_as_float(hi));
       }
+    load_a(xa, pa, k0 + 32);
+    pa += 16 * (long long)g.sAk;
 #pragma unroll
-      for (int j = 0; j < NT; ++j) {
-        const unsigned hi = to_tf32(rb[j][t]);
-        bh[j][t] = hi;
-        bl[j][t] = to_tf32(rb[j][t] - __uint_as_float(hi));
+    for (int j = 0; j < NT; ++j) {
+      unsigned bh[4], bl[4];
+#pragma unroll
+      for (int t = 0; t < 4; ++t) {
+        bh[t] = to_tf32(xb[j][t]);
+        bl[t] = to_tf32(xb[j][t] - __uint_as_float(bh[t]));
       }
+      load_b(xb[j], pb, j, k0 + 32);
+      float acc[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+      for (int ks = 0; ks < 2; ++ks) {
+        mma_tf32(acc, al[ks], bh + 2 * ks);
+        mma_tf32(acc, ah[ks], bl + 2 * ks);
+        mma_tf32(acc, ah[ks], bh + 2 * ks);
+      }
+#pragma unroll
+      for (int e = 0; e < NE; ++e) two_sum_add(sum[j][e], car[j][e], acc[e]);
     }
-    if (k0 + 16 < kend) load(k0 + 16);
+    pb += 16 * (long long)g.sBk;
+  };
 #pragma unroll
-    for (int j = 0; j < NT; ++j)
+  for (int b = 0; b < 2; ++b) {
+    load_a(ra[b], pa, kbeg + 16 * b);
 #pragma unroll
-      for (int e = 0; e < 4; ++e) acc[j][e] = 0.f;
-#pragma unroll
-    for (int ks = 0; ks < 2; ++ks)
-#pragma unroll
-      for (int j = 0; j < NT; ++j) {
-        mma_tf32(acc[j], al[ks], &bh[j][2 * ks]);
-        mma_tf32(acc[j], ah[ks], &bl[j][2 * ks]);
-        mma_tf32(acc[j], ah[ks], &bh[j][2 * ks]);
-      }
-#pragma unroll
-    for (int j = 0; j < NT; ++j)
-#pragma unroll
-      for (int e = 0; e < NE; ++e) two_sum_add(sum[j][e], car[j][e], acc[j][e]);
+    for (int j = 0; j < NT; ++j) load_b(rb[b][j], pb, j, kbeg + 16 * b);
+    pa += 16 * (long long)g.sAk;
+    pb += 16 * (long long)g.sBk;
+  }
+#pragma unroll 1
+  for (int k0 = kbeg; k0 < kend; k0 += 32) {
+    tile(ra[0], rb[0], k0);
+    if (k0 + 16 < kend) tile(ra[1], rb[1], k0 + 16);
   }
   const float alpha = (float)g.alpha, beta = (float)g.beta;
 #pragma unroll
