@@ -77,6 +77,12 @@ __device__ __forceinline__ int tap_offset(int t) {
   return (t / 9 - 1) * P * P + ((t / 3) % 3 - 1) * P + (t % 3 - 1);
 }
 
+// pair i of a two-channel field of the caller's: 8-byte loads where its address allows (vec)
+__device__ __forceinline__ float2 load_pair(const float* __restrict__ p, long long i, bool vec) {
+  return vec ? ((const float2*)p)[i] : make_float2(p[2 * i], p[2 * i + 1]);
+}
+static int pairs_aligned(const void* a, const void* b) { return (((uintptr_t)a | (uintptr_t)b) & 7) == 0; }
+
 // ---------------------------------------------------------------------------
 // forward
 // ---------------------------------------------------------------------------
@@ -134,7 +140,7 @@ template <int N1>
 __global__ void __launch_bounds__(NN_FWD_THREADS, 1)
     k_nn_forward(const float* __restrict__ prm, const __nv_bfloat16* __restrict__ W2t, const float* __restrict__ in,
                  float* __restrict__ out, __nv_bfloat16* __restrict__ a1_out, __nv_bfloat16* __restrict__ a2_out,
-                 long long ne, int ng) {
+                 long long ne, int ng, int vec) {
   using C = NNCfg<N1>;
   using F = FwdCfg<N1>;
   constexpr int ROWS = F::ROWS, P = C::P, NT = NN_FWD_THREADS, NW = NT / 32, LPE = N1 * N1;
@@ -165,7 +171,7 @@ __global__ void __launch_bounds__(NN_FWD_THREADS, 1)
     const int nel = (int)(ne - e0 < ng ? ne - e0 : ng), np = nel * C::NPE, nl = nel * LPE, MT = (np + 15) / 16;
     for (int i = tid; i < np; i += NT) {
       const int l = i / N1, y = l % N1, z = l / N1 % N1;
-      sIn[l / LPE * F::IS + (z + 1) * F::ZS + (y + 1) * F::YS + i % N1 + 1] = ((const float2*)in)[nb0 + i];
+      sIn[l / LPE * F::IS + (z + 1) * F::ZS + (y + 1) * F::YS + i % N1 + 1] = load_pair(in, nb0 + i, vec);
     }
     __syncthreads();
     // layer 1 (2 -> 32)
@@ -305,7 +311,16 @@ __global__ void __launch_bounds__(NN_FWD_THREADS, 1)
             acc[i][c] = keep + __shfl_xor_sync(0xffffffffu, give, h);
           }
       }
-      if (l < nl && r < N1) ((float2*)out)[nb0 + l * N1 + r] = make_float2(acc[0][0] + b30, acc[0][1] + b31);
+      if (l < nl && r < N1) {
+        const long long o = nb0 + l * N1 + r;
+        const float2 v = make_float2(acc[0][0] + b30, acc[0][1] + b31);
+        if (vec) {
+          ((float2*)out)[o] = v;
+        } else {
+          out[2 * o] = v.x;
+          out[2 * o + 1] = v.y;
+        }
+      }
     }
     if (a1_out) {
       for (int i = tid; i < np * 4; i += NT) {
@@ -445,7 +460,7 @@ template <int N1>
 __global__ void __launch_bounds__(NN_BWD_THREADS, 1)
     k_nn_backward(const float* __restrict__ prm, const __nv_bfloat16* __restrict__ W2o, const float* __restrict__ in,
                   const __nv_bfloat16* __restrict__ a1g, const __nv_bfloat16* __restrict__ a2g,
-                  const float* __restrict__ gout, float* __restrict__ part, long long ne, int ng) {
+                  const float* __restrict__ gout, float* __restrict__ part, long long ne, int ng, int vec) {
   using C = NNCfg<N1>;
   using F = FwdCfg<N1>;
   constexpr int P3 = C::P3 * C::GROUP, P = C::P, NT = NN_BWD_THREADS, NW = NT / 32, LPE = N1 * N1;
@@ -503,7 +518,7 @@ __global__ void __launch_bounds__(NN_BWD_THREADS, 1)
     const int np = (int)(ne - e0 < ng ? ne - e0 : ng) * C::NPE, MT = (np + 15) / 16;
     for (int i = tid; i < np; i += NT) {
       const int p = group_index<N1>(i);
-      const float2 x = ((const float2*)in)[nb0 + i], y = ((const float2*)gout)[nb0 + i];
+      const float2 x = load_pair(in, nb0 + i, vec), y = load_pair(gout, nb0 + i, vec);
       sG3[g3_index(i)] = y;
       split3(x.x, sIs + 8 * p);
       split3(x.y, sIs + 8 * p + 3);
@@ -797,7 +812,8 @@ static cudaError_t nn_fwd_n1(const float* prm, const __nv_bfloat16* W2t, const f
   const int ng = nn_group<N1>(ne, cap);
   const long long grid = (ne + ng - 1) / ng;
   count_launch();
-  k_nn_forward<N1><<<(unsigned)(grid < cap ? grid : cap), NN_FWD_THREADS, sm, s>>>(prm, W2t, in, out, a1, a2, ne, ng);
+  k_nn_forward<N1><<<(unsigned)(grid < cap ? grid : cap), NN_FWD_THREADS, sm, s>>>(prm, W2t, in, out, a1, a2, ne, ng,
+                                                                                      pairs_aligned(in, out));
   return cudaGetLastError();
 }
 
@@ -820,7 +836,7 @@ static cudaError_t nn_bwd_n1(const float* prm, const __nv_bfloat16* W2o, const f
                              cudaStream_t s) {
   count_launch();
   k_nn_backward<N1><<<nblk, NN_BWD_THREADS, bwd_smem<N1>(), s>>>(prm, W2o, in, a1, a2, gout, part, ne,
-                                                                                 nn_group<N1>(ne, nblk));
+                                                                    nn_group<N1>(ne, nblk), pairs_aligned(in, gout));
   return cudaGetLastError();
 }
 
