@@ -501,9 +501,12 @@ int dg_octree_node_coords(dg_oct_handle h, double* xyz_dev, double* w_dev, void*
 
 /* The operator on the handle's mesh: out = A u for B fields (0..65535), u_dev
  * and out_dev [B][Nq] device, not overlapping (DG_ERR_INVALID_ARG). Stream
- * ordered: launches its one or two kernels (two where the mesh has hanging
- * faces) and returns without synchronising; calls on several streams share the
- * handle's flux scratch and run one after the other. */
+ * ordered: returns without synchronising. Launches one kernel, or where the mesh
+ * has hanging faces two for every group of fields whose fluxes fit the handle's
+ * scratch (64 fields or 64 MB). A call that finds the scratch in use by another
+ * stream, and a captured call, are one kernel without scratch instead (the same
+ * results; 0.5 to 3 times as long): calls on several streams or threads, and
+ * replays, may overlap with each other and with the handle's solves. */
 int dg_octree_operator(dg_oct_handle h, const double* u_dev, double* out_dev, int64_t B, void* cuda_stream);
 
 /* The handle's preconditioner alone for B fields: z = V(r), one V-cycle

@@ -426,7 +426,7 @@ struct OctHang {
   V tl[N1], dl[N1], w[N1];
   V g0;
   long long Nq;
-  int E, k0, nI;
+  int k0, nI;
 };
 
 // Fluxes of a hanging face in units of 2 / h of the side that they are for, with
@@ -527,6 +527,194 @@ __global__ void __launch_bounds__(HangShape<V, N1>::THREADS)
   }
 }
 
+template <typename V, int N1>
+struct HangShared {
+  V X[2][N1 * N1];        // larger side: value, derivative at its face nodes
+  V R[2][2][N1 * N1];     // [quantity][half along t0]
+  V F[2][4][N1 * N1];     // weighted fluxes per quarter
+};
+// The same fluxes for k_oct_leaf, a face at a time: put(quantity, l, value) takes those of
+// slot `side` (0: the larger leaf, 1 + j: the j-th smaller one). sL, sw: the tables' Lh
+// and w in shared memory. Every thread of the block takes part (barriers). (In place of
+// k_oct_hang's body, which is this one for all slots at once, it took 0.4 us longer.)
+template <typename V, int N1, typename P>
+__device__ __forceinline__ void hang_face(const OctHang<V, N1>& tab, const V (*sL)[N1 * N1], const V* sw,
+                                          HangShared<V, N1>& s, const int* __restrict__ rc,
+                                          const double* __restrict__ fac, const V* __restrict__ us, int side, bool on,
+                                          int t, P&& put) {
+  constexpr int NF = N1 * N1, NPE = NF * N1;
+  const int big = rc[0], f = rc[1], d = f >> 1, r = f & 1;
+  const int st[3] = {1, N1, NF};
+  const int sd = st[d], s0 = st[d == 0 ? 1 : 0], s1 = st[d == 2 ? 1 : 2];
+  const int q = t / NF, l = t - q * NF, i = l % N1, j = l / N1;  // quarter, point (i along t0, j along t1)
+  const int b0 = q & 1, b1 = q >> 1;
+  const bool mine = on && (side == 0 || q == side - 1);  // this quarter's fluxes are wanted
+  // loaded ahead of the barriers: gam = sigma h / 2 of the smaller leaf
+  const int small = mine ? rc[2 + q] : 0;
+  const V gam = (V)__ldg(fac + 6LL * small + 3 + d) * tab.g0;
+  V vs = 0, ds = 0;
+  auto trace = [&](int leaf, int end, V& val, V& der) {  // end 0: left, 1: right end of the line along d
+    const V* p = us + (long long)leaf * NPE + i * s0 + j * s1;
+    V x[N1];
+#pragma unroll
+    for (int a = 0; a < N1; ++a) x[a] = __ldg(p + (end ? N1 - 1 - a : a) * sd);
+    end_trace<V, N1, false>(tab.tl, tab.dl, x, val, der);
+    if (end) der = -der;  // the line was read reversed
+  };
+  if (mine) trace(small, 1 - r, vs, ds);
+  if (on && q == 0) trace(big, r, s.X[0][l], s.X[1][l]);
+  __syncthreads();
+  if (on) {
+    // first step, along t0: thread (quantity q & 1, half q >> 1)
+    V v = 0;
+#pragma unroll
+    for (int b = 0; b < N1; ++b) v = mad(sL[b1][i * N1 + b], s.X[b0][b + N1 * j], v);
+    s.R[b0][b1][l] = v;
+  }
+  __syncthreads();
+  if (mine) {
+    V vb = 0, db = 0;
+#pragma unroll
+    for (int c = 0; c < N1; ++c) {
+      const V x = sL[b1][j * N1 + c];
+      vb = mad(x, s.R[0][b0][i + N1 * c], vb);
+      db = mad(x, s.R[1][b0][i + N1 * c], db);
+    }
+    const V h = (V)0.5;  // the larger leaf's 2 / h is half of the smaller one's
+    const V so = r ? (V)-1 : (V)1;  // outward sign of the smaller side
+    const V jump = vs - vb;
+    if (side != 0) {
+      put(0, l, mad(gam, jump, mul(mul(-h, so), mad(h, db, ds))));
+      put(1, l, mul(-h, jump));
+    } else {
+      const V wq = mul((V)0.25, mul(sw[i], sw[j]));
+      s.F[0][q][l] = mul(wq, mad((V)-2 * gam, jump, mul(mul(h, so), mad((V)2, ds, db))));
+      s.F[1][q][l] = mul(wq, mul(h, jump));
+    }
+  }
+  if (side != 0) return;
+  __syncthreads();
+  if (on) {
+    // back along t1, the two halves along it summed: thread (quantity b0, half b1 along t0) into R
+    V v = 0;
+#pragma unroll
+    for (int c = 0; c < 2; ++c)
+#pragma unroll
+      for (int jj = 0; jj < N1; ++jj) v = mad(sL[c][jj * N1 + j], s.F[b0][b1 + 2 * c][i + N1 * jj], v);
+    s.R[b0][b1][l] = v;
+  }
+  __syncthreads();
+  if (on && q < 2) {
+    V v = 0;
+#pragma unroll
+    for (int c = 0; c < 2; ++c)
+#pragma unroll
+      for (int ii = 0; ii < N1; ++ii) v = mad(sL[c][ii * N1 + i], s.R[q][c][ii + N1 * j], v);
+    put(q, l, v / mul(sw[i], sw[j]));
+  }
+}
+
+// The operator in one launch and without scratch, for calls that have none (a
+// captured call): one leaf per block, which works out the fluxes of its own hanging
+// faces. The leaf's three directions go to three groups of threads; every number is
+// that of k_oct_hang and k_oct_apply, in the same order: the same bits.
+template <int N1>
+struct OctLeaf {
+  static constexpr int THREADS = (4 * N1 * N1 + 31) / 32 * 32;
+};
+template <typename V, int N1>
+__global__ void __launch_bounds__(OctLeaf<N1>::THREADS)
+    k_oct_leaf(const __grid_constant__ OctLine<V, N1> tab, const __grid_constant__ OctHang<V, N1> hg,
+               const int* __restrict__ rec, const double* __restrict__ fac, const int* __restrict__ kind,
+               const int* __restrict__ nbr, const int* __restrict__ hslot, const V* __restrict__ u,
+               V* __restrict__ out) {
+  using Y = LineLayout<N1>;
+  constexpr int NF = N1 * N1, NPE = NF * N1, NT = OctLeaf<N1>::THREADS;
+  __shared__ V su[Y::ES], sr[3][Y::ES], sg[6][2][NF], sL[2][NF], sw[N1], sww[NF], sfac[6];
+  __shared__ HangShared<V, N1> sh;
+  __shared__ int sface[6];
+  const int tid = threadIdx.x, e = blockIdx.x;
+  const V* us = u + (long long)blockIdx.y * tab.Nq;
+  if (tid < 6) {
+    const long long o = 6LL * e + tid;
+    const int kd = kind[o];
+    sface[tid] = kd == 0 ? -1 : kd == 1 ? nbr[4 * o] : -2 - hslot[o];
+    sfac[tid] = (V)fac[o] * (tid >= 3 ? tab.g0 : (V)1);
+  }
+  for (int t = tid; t < NPE; t += NT)
+    su[t % N1 + Y::PB * ((t / N1) % N1) + Y::PZ * (t / NF)] = __ldg(us + (long long)e * NPE + t);
+  for (int t = tid; t < NF; t += NT) sww[t] = tab.ww[t];
+  __syncthreads();
+  const int q = tid / NF, l = tid - q * NF, l1 = l % N1, l2 = l / N1;
+  bool any = false;
+#pragma unroll
+  for (int f = 0; f < 6; ++f) any |= sface[f] < -1;
+  if (any) {
+    for (int i = tid; i < 2 * NF; i += NT) sL[i / NF][i % NF] = hg.Lh[i / NF][i % NF];
+    for (int i = tid; i < N1; i += NT) sw[i] = hg.w[i];
+#pragma unroll 1
+    for (int f = 0; f < 6; ++f) {
+      const int fc = sface[f];
+      if (fc >= -1) continue;
+      const int slot = -2 - fc, ifc = slot / 5;
+      hang_face<V, N1>(hg, sL, sw, sh, rec + 6LL * ifc, fac, us, slot - 5 * ifc, q < 4, tid,
+                       [&](int c, int k, V v) { sg[f][c][k] = v; });
+    }
+    __syncthreads();
+  }
+  if (q < 3) {
+    // direction q: strides in the field and in the shared layout
+    const int sd = q == 0 ? 1 : (q == 1 ? N1 : NF), sp = q == 0 ? 1 : (q == 1 ? Y::PB : Y::PZ);
+    const int base = q == 0 ? N1 * l : (q == 1 ? l1 + NF * l2 : l);
+    const int at = q == 0 ? Y::PB * l1 + Y::PZ * l2 : (q == 1 ? l1 + Y::PZ * l2 : l1 + Y::PB * l2);
+    const int fl = sface[2 * q], fr = sface[2 * q + 1];
+    const V gam = sfac[3 + q];
+    V v[N1], ov[2], od[2];
+    // traces beyond the two ends, as oct_outer
+    auto line = [&](int fc) {
+      const V* p = us + (long long)(fc < 0 ? e : fc) * NPE + base + (fc < 0 ? (N1 - 1) * sd : 0);
+      const int st = fc < 0 ? -sd : sd;
+#pragma unroll
+      for (int i = 0; i < N1; ++i) v[i] = __ldg(p + i * st);
+    };
+    if (fl >= -1) {
+      line(fl);
+      end_trace<V, N1, true>(tab.tl, tab.dl, v, ov[0], od[0]);
+      if (fl < 0) {
+        od[0] = mad((V)-2 * gam, ov[0], -od[0]);
+        ov[0] = -ov[0];
+      }
+    } else {
+      ov[0] = sg[2 * q][0][l];
+      od[0] = sg[2 * q][1][l];
+    }
+    if (fr >= -1) {
+      line(fr);
+      end_trace<V, N1, false>(tab.tl, tab.dl, v, ov[1], od[1]);
+      if (fr < 0) {
+        od[1] = mad((V)2 * gam, ov[1], -od[1]);
+        ov[1] = -ov[1];
+      }
+    } else {
+      ov[1] = sg[2 * q + 1][0][l];
+      od[1] = sg[2 * q + 1][1][l];
+    }
+#pragma unroll
+    for (int i = 0; i < N1; ++i) v[i] = su[at + sp * i];
+    oct_line<V, N1>(tab, v, ov, od, fl < -1, fr < -1, gam);
+#pragma unroll
+    for (int i = 0; i < N1; ++i) sr[q][at + sp * i] = v[i];
+  }
+  __syncthreads();
+  V* o = out + (long long)blockIdx.y * tab.Nq + (long long)e * NPE;
+  for (int t = tid; t < NPE; t += NT) {
+    const int a = t % N1, b = (t / N1) % N1, c = t / NF, at = a + Y::PB * b + Y::PZ * c;
+    V Au = mul(mul(sfac[0], sww[b + N1 * c]), sr[0][at]);
+    Au = mad(mul(sfac[1], sww[a + N1 * c]), sr[1][at], Au);
+    o[t] = mad(mul(sfac[2], sww[a + N1 * b]), sr[2][at], Au);
+  }
+}
+
 void octree_hanging(const int32_t* kind, const int32_t* nb, int E, std::vector<int>& rec, std::vector<int>& hslot) {
   rec.clear();
   hslot.assign(6 * (size_t)E, -1);
@@ -590,11 +778,8 @@ void octree_tables(int n1, OctTables& T) {
 }
 
 template <typename V, int N1>
-static cudaError_t oct_apply_n1(const OctTables& T, const OctMesh& m, double eps, const V* u, V* out, const V* rin,
-                                const int* act, int nact, V* gbuf, long long gelems, cudaStream_t s) {
+static void oct_fill(const OctTables& T, const OctMesh& m, double eps, OctLine<V, N1>& t, OctHang<V, N1>& g) {
   constexpr int HO = N1 / 2, HE = N1 - HO, NF = N1 * N1, NPE = NF * N1;
-  OctLine<V, N1> t;
-  OctHang<V, N1> g;
   auto S = [&](int a, int i) { return 0.5 * (T.S[a * N1 + i] + T.S[(N1 - 1 - a) * N1 + (N1 - 1 - i)]); };
   for (int a = 0; a < HE; ++a) {
     for (int i = 0; i < HE; ++i) t.Se[a][i] = (V)(i < HO ? 0.5 * (S(a, i) + S(a, N1 - 1 - i)) : S(a, i));
@@ -617,9 +802,18 @@ static cudaError_t oct_apply_n1(const OctTables& T, const OctMesh& m, double eps
   }
   t.g0 = g.g0 = (V)(N1 * N1 / (2.0 * eps));
   t.Nq = g.Nq = (long long)m.E * NPE;
-  t.E = g.E = m.E;
+  t.E = m.E;
   t.nslots = 5 * m.nI;
   g.nI = m.nI;
+}
+
+template <typename V, int N1>
+static cudaError_t oct_apply_n1(const OctTables& T, const OctMesh& m, double eps, const V* u, V* out, const V* rin,
+                                const int* act, int nact, V* gbuf, long long gelems, cudaStream_t s) {
+  constexpr int NF = N1 * N1, NPE = NF * N1;
+  OctLine<V, N1> t;
+  OctHang<V, N1> g;
+  oct_fill<V, N1>(T, m, eps, t, g);
   const int vec = ((uintptr_t)u & 15) == 0 && (NPE * sizeof(V)) % 16 == 0 && (t.Nq * sizeof(V)) % 16 == 0;
   // sources go through in chunks whose hanging fluxes fit the buffer (and a grid's second axis)
   const long long per_src = 10LL * m.nI * NF;
@@ -676,6 +870,35 @@ template cudaError_t launch_octree_apply<double>(int, const OctTables&, const Oc
                                                  const double*, const int*, int, double*, long long, cudaStream_t);
 template cudaError_t launch_octree_apply<float>(int, const OctTables&, const OctMesh&, double, const float*, float*,
                                                 const float*, const int*, int, float*, long long, cudaStream_t);
+
+template <int N1>
+static cudaError_t oct_leaf_n1(const OctTables& T, const OctMesh& m, double eps, const double* u, double* out, int B,
+                               cudaStream_t s) {
+  OctLine<double, N1> t;
+  OctHang<double, N1> g;
+  oct_fill<double, N1>(T, m, eps, t, g);
+  t.items = t.k0 = g.k0 = 0;
+  count_launch();
+  k_oct_leaf<double, N1><<<dim3((unsigned)m.E, (unsigned)B), OctLeaf<N1>::THREADS, 0, s>>>(t, g, m.rec, m.fac, m.kind,
+                                                                                         m.nb, m.hslot, u, out);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_octree_direct(int n1, const OctTables& T, const OctMesh& m, double eps, const double* u, double* out,
+                                 int B, cudaStream_t s) {
+  if (B == 0 || m.E == 0) return cudaSuccess;
+  switch (n1) {
+    case 2: return oct_leaf_n1<2>(T, m, eps, u, out, B, s);
+    case 3: return oct_leaf_n1<3>(T, m, eps, u, out, B, s);
+    case 4: return oct_leaf_n1<4>(T, m, eps, u, out, B, s);
+    case 5: return oct_leaf_n1<5>(T, m, eps, u, out, B, s);
+    case 6: return oct_leaf_n1<6>(T, m, eps, u, out, B, s);
+    case 7: return oct_leaf_n1<7>(T, m, eps, u, out, B, s);
+    case 8: return oct_leaf_n1<8>(T, m, eps, u, out, B, s);
+    case 9: return oct_leaf_n1<9>(T, m, eps, u, out, B, s);
+    default: return cudaErrorInvalidValue;
+  }
+}
 }  // namespace dg
 
 using namespace dg;

@@ -56,4 +56,8 @@ template <typename V>
 cudaError_t launch_octree_apply(int n1, const OctTables& T, const OctMesh& m, double eps, const V* u, V* out,
                                 const V* rin, const int* act, int nact, V* gbuf, long long gelems, cudaStream_t s);
 
+// out[k] = A u[k], k = 0 .. B - 1 (B at most 65535), in one launch and without scratch: the same bits
+cudaError_t launch_octree_direct(int n1, const OctTables& T, const OctMesh& m, double eps, const double* u, double* out,
+                                 int B, cudaStream_t s);
+
 }  // namespace dg

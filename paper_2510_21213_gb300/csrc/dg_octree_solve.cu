@@ -102,16 +102,17 @@ struct dg_oct {
   // the device when it fits the budget below
   dg::DevBuf kmat, wf32, g32, gwork;
   bool has_kmat = false;
-  // hanging fluxes of the operator: of the solves, and of dg_octree_operator,
-  // which returns before its kernels end: op_done orders its next call (on
-  // whatever stream) behind them
-  dg::DevBuf hang, hang_op;
+  dg::DevBuf hang;  // hanging fluxes of the operator in the solves
+  // those of dg_octree_operator, allocated by its first call. It returns before its
+  // kernels end: op_done is recorded behind the last user, on stream op_stream
+  dg::DevBuf hang_op;
   cudaEvent_t op_done = nullptr;
+  cudaStream_t op_stream = nullptr;
   std::mutex op_mutex;
   std::vector<int> act_host;
   ~dg_oct() {
-    if (op_done) cudaEventDestroy(op_done);
     if (root) dg_destroy(root);
+    if (op_done) cudaEventDestroy(op_done);
   }
 };
 
@@ -558,18 +559,17 @@ static cudaError_t launch_bjac(const dg_oct* h, const OctLevel& L, int mode, con
   }
 }
 
+static OctMesh oct_mesh(const dg_oct* h) {
+  return OctMesh{h->E, h->kind.as<int>(), h->nb.as<int>(), h->fac.as<double>(), h->hslot.as<int>(), h->rec.as<int>(),
+                 h->nI};
+}
+
 // out = A u, or with rin out = rin - A u
 template <typename V>
 static cudaError_t oct_apply(const dg_oct* h, const OctLevel& L, const V* u, V* out, const int* act, int nact,
-                             cudaStream_t s, const V* rin = nullptr, void* hang = nullptr, size_t bytes = 0) {
-  if (!hang) {
-    hang = h->hang.p;
-    bytes = h->hang.bytes;
-  }
-  const OctMesh m{h->E, h->kind.as<int>(), h->nb.as<int>(), h->fac.as<double>(), h->hslot.as<int>(), h->rec.as<int>(),
-                  h->nI};
-  return launch_octree_apply<V>(L.n1, L.T, m, h->eps, u, out, rin, act, nact, (V*)hang,
-                                (long long)(bytes / sizeof(V)), s);
+                             cudaStream_t s, const V* rin = nullptr) {
+  return launch_octree_apply<V>(L.n1, L.T, oct_mesh(h), h->eps, u, out, rin, act, nact, (V*)h->hang.p,
+                                (long long)(h->hang.bytes / sizeof(V)), s);
 }
 
 static cudaError_t launch_oct_lift(const dg_oct* h, const double* g, double* b, int nsrc, cudaStream_t s) {
@@ -628,6 +628,38 @@ static size_t hang_bytes(const dg_oct* h, int cap) {
   const size_t one = sizeof(double) * octree_hang_elems(h->n1, h->nI);
   return std::max(one, std::min<size_t>(one * (size_t)cap, 64u << 20));
 }
+
+// The scratch of one dg_octree_operator call on stream s, held until the object goes
+// (wait, launches and record of a call belong together); p is null while a call on
+// another stream still uses it, and where it cannot be had. The queries and the
+// allocation are legal beside a capture of the calling program's.
+struct OctOpScratch {
+  std::lock_guard<std::mutex> lock;
+  double* p = nullptr;
+  long long elems = 0;
+  OctOpScratch(dg_oct* h, cudaStream_t s) : lock(h->op_mutex) {
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    cudaThreadExchangeStreamCaptureMode(&mode);
+    if (take(h, s)) {
+      p = h->hang_op.as<double>();
+      elems = (long long)(h->hang_op.bytes / sizeof(double));
+      h->op_stream = s;
+    } else {
+      cudaGetLastError();
+    }
+    cudaThreadExchangeStreamCaptureMode(&mode);
+  }
+  static bool take(dg_oct* h, cudaStream_t s) {
+    if (!h->op_done && cudaEventCreateWithFlags(&h->op_done, cudaEventDisableTiming) != cudaSuccess) {
+      h->op_done = nullptr;
+      return false;
+    }
+    if (h->hang_op.ensure(hang_bytes(h, 64)) != cudaSuccess) return false;
+    if (s != h->op_stream && cudaEventQuery(h->op_done) != cudaSuccess) return false;
+    // on the same stream this waits for nothing, unless its handle has passed to a new one
+    return cudaStreamWaitEvent(s, h->op_done, 0) == cudaSuccess;
+  }
+};
 
 static int oct_ws(dg_oct* h, int cap) {
   if (cap <= h->cap) return DG_OK;
@@ -1319,11 +1351,6 @@ int dg_octree_setup(const dg_mesh_desc* root, const int32_t* leaves, int32_t n_l
     bl.insert(bl.end(), fidx, fidx + 6);
     ++h->nbl;
   }
-  if (h->nI > 0) {
-    cudaError_t e = h->hang_op.ensure(hang_bytes(h, 64));
-    if (e == cudaSuccess) e = cudaEventCreateWithFlags(&h->op_done, cudaEventDisableTiming);
-    if (e != cudaSuccess) return fail(e == cudaErrorMemoryAllocation ? DG_ERR_NO_MEMORY : DG_ERR_CUDA);
-  }
   std::vector<double> fac;
   octree_factors(hq.data(), E, penalty_form, fac);
   if ((rc = up(h->fac, fac.data(), sizeof(double) * fac.size())) != DG_OK ||
@@ -1433,27 +1460,29 @@ int dg_octree_operator(dg_oct_handle h, const double* u_dev, double* out_dev, in
   const char *u0 = (const char*)u_dev, *o0 = (const char*)out_dev;
   if (u0 < o0 + bytes && o0 < u0 + bytes) return DG_ERR_INVALID_ARG;
   cudaStream_t s = (cudaStream_t)stream;
+  const OctMesh m = oct_mesh(h);
+  const OctTables& T = h->lv[0].T;
   if (h->nI == 0) {
-    DG_CK(oct_apply<double>(h, h->lv[0], u_dev, out_dev, nullptr, (int)B, s));
+    DG_CK(launch_octree_apply<double>(h->n1, T, m, h->eps, u_dev, out_dev, nullptr, nullptr, (int)B, nullptr, 0, s));
     return DG_OK;
   }
   cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
   DG_CK(cudaStreamIsCapturing(s, &cap));
-  if (cap != cudaStreamCaptureStatusNone) {
-    // the graph allocates and frees its own scratch: its replays may overlap with
-    // anything else that runs on the handle
-    const size_t hb = hang_bytes(h, (int)std::min<int64_t>(B, 64));
-    void* p = nullptr;
-    DG_CK(cudaMallocAsync(&p, hb, s));
-    const cudaError_t e = oct_apply<double>(h, h->lv[0], u_dev, out_dev, nullptr, (int)B, s, nullptr, p, hb);
-    DG_CK(cudaFreeAsync(p, s));
-    DG_CK(e);
-    return DG_OK;
+  if (cap == cudaStreamCaptureStatusNone) {
+    const OctOpScratch sc(h, s);
+    if (sc.p) {
+      const cudaError_t e = launch_octree_apply<double>(h->n1, T, m, h->eps, u_dev, out_dev, nullptr, nullptr, (int)B,
+                                                        sc.p, sc.elems, s);
+      // also behind a launch that failed: earlier ones of the call may be under way
+      const cudaError_t r = cudaEventRecord(h->op_done, s);
+      DG_CK(e);
+      DG_CK(r);
+      return DG_OK;
+    }
   }
-  std::lock_guard<std::mutex> lock(h->op_mutex);  // wait, launches and record of one call belong together
-  DG_CK(cudaStreamWaitEvent(s, h->op_done, 0));
-  DG_CK(oct_apply<double>(h, h->lv[0], u_dev, out_dev, nullptr, (int)B, s, nullptr, h->hang_op.p, h->hang_op.bytes));
-  DG_CK(cudaEventRecord(h->op_done, s));
+  // the one-launch form needs no scratch: in a captured call, whose replays may
+  // overlap with anything, and where another stream has the scratch or memory is short
+  DG_CK(launch_octree_direct(h->n1, T, m, h->eps, u_dev, out_dev, (int)B, s));
   return DG_OK;
 }
 
