@@ -426,6 +426,21 @@ __global__ void k_gemm_splitk_reduce(GemmArgs g, int nsplit, int batch_base, int
   }
 }
 
+// a long K is split over blocks into fixed ranges (512 terms in FP32, 256 in FP64;
+// from K alone, so a batch's sums do not depend on how many batches share the call)
+template <typename T>
+static int gemm_splits(int K) {
+  constexpr int RANGE = sizeof(T) == 4 ? 512 : 256;
+  return K >= 2 * RANGE ? std::min(32, (K + RANGE - 1) / RANGE) : 1;
+}
+template <typename T>
+size_t gemm_split_bytes(long long M, long long N, int K) {
+  const int n = gemm_splits<T>(K);
+  return n > 1 ? sizeof(T) * (size_t)(n * M * N) : 0;
+}
+template size_t gemm_split_bytes<double>(long long, long long, int);
+template size_t gemm_split_bytes<float>(long long, long long, int);
+
 template <typename T>
 cudaError_t launch_gemm(const GemmArgs& g, cudaStream_t s) {
   if (g.M <= 0 || g.N <= 0 || g.nb1 * (long long)g.nb2 <= 0) return cudaSuccess;
@@ -434,12 +449,8 @@ cudaError_t launch_gemm(const GemmArgs& g, cudaStream_t s) {
   constexpr int TILE = F32 ? 64 : G64_T;
   const dim3 grid((g.N + TILE - 1) / TILE, (g.M + TILE - 1) / TILE, 1);
   if (grid.y > 65535) return cudaErrorInvalidValue;
-  // a long K is split over blocks into fixed ranges (512 terms in FP32, 256 in
-  // FP64; from K alone, so a batch's sums do not depend on how many batches
-  // share the call); batches go through in chunks that fit the workspace
-  constexpr int RANGE = F32 ? 512 : 256;
-  int nsplit = 1;
-  if (g.work && g.K >= 2 * RANGE) nsplit = std::min(32, (g.K + RANGE - 1) / RANGE);
+  // batches of a split product go through in chunks that fit the workspace
+  int nsplit = g.work ? gemm_splits<T>(g.K) : 1;
   // FP64 output larger than the workspace holds (over 500 nodes an axis): enough tiles without a split
   if (!F32 && nsplit > 1 && g.work_elems < (long long)nsplit * g.M * g.N) nsplit = 1;
   const int kc = nsplit > 1 ? ((g.K + nsplit - 1) / nsplit + 15) / 16 * 16 : g.K;

@@ -112,21 +112,27 @@ static int ensure_bc_work(dg_ctx* h, int nsrc, int NG, BcAxisTables* bct, DevBuf
   const long long N = h->Nq;
   DG_CK(flex.ensure(sizeof(T) * N * nsrc));
   long long maxface = 0;
+  // split-K partials of one source and side; as many at a time as 64 MB hold (FP64
+  // output that takes more is not split)
+  const size_t cap = 64u << 20;
+  size_t one = 0;
   for (int d = 0; d < 3; ++d) {
     const int t1 = d == 0 ? 1 : 0, t2 = d == 2 ? 1 : 2;
     maxface = std::max(maxface, (long long)bct[t1].L * bct[t2].L);
+    const size_t part = gemm_split_bytes<T>(bct[t2].L, bct[t1].L, NG * bct[t2].L);
+    if (sizeof(T) == 4 || part <= cap) one = std::max(one, part);
   }
   const size_t tb = sizeof(T) * 2 * (size_t)NG * maxface * nsrc;
   DG_CK(T1.ensure(tb));
   DG_CK(T2.ensure(tb));
-  DG_CK(h->gemm_ws.ensure(64LL << 20));  // split-K partials
+  if (one > 0) DG_CK(h->gemm_ws.ensure(std::min(cap, one * 2 * (size_t)nsrc)));
   return DG_OK;
 }
 
 static void account(dg_ctx* h) {
   long long b = 0;
   auto add = [&](const DevBuf& x) { b += (long long)x.bytes; };
-  for (auto* w : {&h->f64, &h->b64, &h->x64, &h->r64, &h->flex, &h->T1, &h->T2, &h->g, &h->part, &h->scal,
+  for (auto* w : {&h->f64, &h->b64, &h->x64, &h->r64, &h->flex, &h->T1, &h->T2, &h->g, &h->part, &h->scal, &h->gemm_ws,
                   &h->flex32, &h->T1_32, &h->T2_32, &h->g32,
                   &h->act, &h->flags, &h->pidx, &h->Wacc, &h->kpart, &h->Kdev, &h->coarse_inv, &h->d_W, &h->d_xq,
                   &h->d_axn})

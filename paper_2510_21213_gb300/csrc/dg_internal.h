@@ -210,6 +210,9 @@ cudaError_t launch_weighted_lex(const LevelOp& hop, const LevelOp* dop, const do
                                 int nsrc, cudaStream_t s);
 template <typename T>
 cudaError_t launch_gemm(const GemmArgs& g, cudaStream_t s);
+// bytes of work that one batch of a product with these sizes splits its K into (0: K is not split)
+template <typename T>
+size_t gemm_split_bytes(long long M, long long N, int K);
 cudaError_t launch_bc_direct(const LevelOp& hop, const LevelOp* dop, const double* f, const double* W,
                              const double* xq, const double* axis_nodes, int lmax, double* g, int nsrc,
                              long long gstride, long long nface, cudaStream_t s);
