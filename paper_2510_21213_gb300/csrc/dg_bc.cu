@@ -421,7 +421,7 @@ __global__ void k_gemm_splitk_reduce(GemmArgs g, int nsplit, int batch_base, int
     const int m = (int)(r / g.N), n = (int)(r - (long long)m * g.N);
     const int b1 = (int)(bz / g.nb2), b2 = (int)(bz % g.nb2);
     T* cp = (T*)g.C + b1 * g.sC1 + b2 * g.sC2 + (long long)m * g.sCm + (long long)n * g.sCn;
-    const T v = sum + car;
+    const T v = isfinite(sum) ? sum + car : sum;  // the carry of an overflow is NaN
     *cp = g.beta != 0.0 ? (T)g.alpha * v + (T)g.beta * (*cp) : (T)g.alpha * v;
   }
 }

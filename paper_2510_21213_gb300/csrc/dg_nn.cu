@@ -383,25 +383,45 @@ __device__ __forceinline__ void split3(float x, __nv_bfloat16* o) {
   o[2] = __float2bfloat16(r1 - mid);
 }
 
+// s + c <- s + c + v (TwoSum); the carry of an overflow would be NaN and is left out
+__device__ __forceinline__ void nn_two_sum(float& s, float& c, float v) {
+  const float t = s + v, b = t - s;
+  if (isfinite(t)) c += (s - (t - b)) + (v - b);
+  s = t;
+}
+
 // Adds one element's tile sums (rows g, g + 8; columns = three split parts of two
 // channels) to the running sum, compensated (TwoSum): lane c4 keeps row g + 8 (c4 >> 1), channel c4 & 1.
 __device__ __forceinline__ void join3(const float* d, int c4, float& run, float& car) {
   float x[4];
+  // lane c4's share of the quad's sums x, added up; x[c4] is this lane's
+  auto quad = [&]() {
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      x[k] += __shfl_xor_sync(0xffffffffu, x[k], 1);
+      x[k] += __shfl_xor_sync(0xffffffffu, x[k], 2);
+    }
+    return c4 == 0 ? x[0] : c4 == 1 ? x[1] : c4 == 2 ? x[2] : x[3];
+  };
 #pragma unroll
   for (int h = 0; h < 2; ++h) {
     const float p = d[2 * h] + d[2 * h + 1];
     x[2 * h] = c4 == 0 ? p : (c4 == 1 ? d[2 * h] : 0.f);
     x[2 * h + 1] = c4 == 2 ? p : (c4 == 1 ? d[2 * h + 1] : 0.f);
   }
+  float v = quad();
+  if (__any_sync(0xffffffffu, !isfinite(v))) {
+    // an overflowed activation gradient times a remainder part that is zero is
+    // NaN: what is not finite is the leading part's sum
 #pragma unroll
-  for (int k = 0; k < 4; ++k) {
-    x[k] += __shfl_xor_sync(0xffffffffu, x[k], 1);
-    x[k] += __shfl_xor_sync(0xffffffffu, x[k], 2);
+    for (int h = 0; h < 2; ++h) {
+      x[2 * h] = c4 == 0 ? d[2 * h] : 0.f;
+      x[2 * h + 1] = c4 == 1 ? d[2 * h + 1] : 0.f;
+    }
+    const float hi = quad();
+    if (!isfinite(v)) v = hi;
   }
-  const float v = c4 == 0 ? x[0] : c4 == 1 ? x[1] : c4 == 2 ? x[2] : x[3];
-  const float t = run + v, b = t - run;
-  car += (run - (t - b)) + (v - b);
-  run = t;
+  nn_two_sum(run, car, v);
 }
 
 // per-tap contraction over the nodes of the element with split columns:
