@@ -347,8 +347,8 @@ __global__ void __launch_bounds__(NN_FWD_THREADS, 1)
 // split exactly into three BF16 numbers (24 bits), so the two channels fill six
 // of the eight columns of one MMA tile and the products are those of the FP32
 // values; an element's sums are added up and joined to a compensated running sum,
-// and the blocks' partials are added in FP64 (the error against float64 sums of
-// the same operands stays below that of the FP32 chains before).
+// and so are the blocks' partials (the error against float64 sums of the same
+// operands stays below that of the FP32 chains before).
 // In SIMT form these two took 885 k products per element at two shared-memory
 // loads each, most of the kernel's time. Shared-memory activations are swizzled
 // as in the forward kernel (unswizzled rows put an ldmatrix phase on four banks),
@@ -359,11 +359,11 @@ __global__ void __launch_bounds__(NN_FWD_THREADS, 1)
 // address arithmetic and load latency, not the MMAs, set the time of the tile loops.
 // Measured (GB300, 16384 elements, p = 7): 28.8 -> 5.9 ms (7.1 with addresses worked
 // out at each load and g_a2 by nodes); cycles per element now: loads 7 k, dW3 13 k,
-// g_a2 22 k, dW2 28 k, g_a1 24 k, dW1 18 k. 2000 elements at p = 6 6.7 -> 0.84 ms.
+// g_a2 22 k, dW2 28 k, g_a1 24 k, dW1 18 k. 2000 elements at p = 6 6.7 -> 0.82 ms.
 // Elements with few nodes go through in groups (p = 1: up to 12), since one of them
-// fills neither the warps nor an MMA row tile: 4000 elements at p = 1 0.294 -> 0.134 ms
-// (one at a time 0.476), 500 at p = 4 0.587 -> 0.153 ms (0.179). What is slower: at
-// most 152 elements at p = 1 (0.054 -> 0.069 ms, staging W2).
+// fills neither the warps nor an MMA row tile: 2000 elements at p = 1 0.173 -> 0.090 ms,
+// 500 at p = 4 0.588 -> 0.130 ms. What is slower: p = 1 with at most 152 elements, by 1 to
+// 5 % of a call (49.6 -> 51.7 us at 8: staging W2).
 // ---------------------------------------------------------------------------
 constexpr int NN_BWD_THREADS = 512;
 
@@ -495,11 +495,17 @@ __global__ void __launch_bounds__(NN_BWD_THREADS, 1)
   float* sred = sW3 + 1728;                                            // [NW][32]
   float2* sG3 = (float2*)(sred + NW * 32);                             // [GROUP][P][P][.], rows as in FwdCfg
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  for (int i = tid; i < P3 * (NN_H + 8); i += NT) ((unsigned*)sA1)[i] = 0u;  // sA1, sA2, sGs, sIs
-  for (int i = tid; i < C::GROUP * F::IS; i += NT) sG3[i] = make_float2(0.f, 0.f);
+  // the borders stay zero; only the rows of the elements that this launch groups are used
+  const int rows = C::P3 * ng;
+  for (int i = tid; i < rows * NN_H / 8; i += NT) ((uint4*)sA1)[i] = ((uint4*)sA2)[i] = make_uint4(0, 0, 0, 0);
+  for (int i = tid; i < rows; i += NT) ((uint4*)sGs)[i] = ((uint4*)sIs)[i] = make_uint4(0, 0, 0, 0);
+  for (int i = tid; i < ng * F::IS; i += NT) sG3[i] = make_float2(0.f, 0.f);
   for (int i = tid; i < 1728; i += NT) sW3[i] = prm[NN_OW3 + i];
-  for (int i = tid; i < 27 * 32 * 4; i += NT)
-    *(uint4*)(sW2 + swz_w2(i >> 2, (i & 3) * 8)) = ((const uint4*)W2o)[i];
+#pragma unroll
+  for (int k = 0; k < (27 * 32 * 4 + NT - 1) / NT; ++k) {  // every load ahead of the first store
+    const int i = tid + k * NT;
+    if (i < 27 * 32 * 4) *(uint4*)(sW2 + swz_w2(i >> 2, (i & 3) * 8)) = __ldg((const uint4*)W2o + i);
+  }
   // dW2 accumulators: warp owns taps warp, warp + 16 (< 27); per tap 32 (ci) x 32 (co) = 2 x 4 mma tiles
   float accW[2][2][4][4], run1[2][2], run3[2][2], car1[2][2], car3[2][2];
 #pragma unroll
@@ -749,13 +755,32 @@ __global__ void __launch_bounds__(NN_BWD_THREADS, 1)
   }
 }
 
-__global__ void k_nn_reduce(const float* __restrict__ part, int nblk, float* __restrict__ grad) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= NN_NPARAM) return;
-  double acc = 0.0;
-#pragma unroll 16
-  for (int b = 0; b < nblk; ++b) acc += part[(long long)b * NN_NPARAM + i];
-  grad[i] = (float)acc;
+// The blocks' partials added up, compensated: NN_RSL threads take a stretch of the
+// blocks each, the stretches are joined in order. Bound by the 4 bytes per partial
+// (19 MB at 152 blocks). In FP64 the additions and conversions took 26 us there (the
+// FP64 pipe), one thread per parameter 8.9 us (too few bytes in flight).
+constexpr int NN_RSL = 8;
+__global__ void __launch_bounds__(32 * NN_RSL) k_nn_reduce(const float* __restrict__ part, int nblk,
+                                                           float* __restrict__ grad) {
+  __shared__ float sh[NN_RSL][2][32];
+  const int lane = threadIdx.x & 31, sl = threadIdx.x >> 5;
+  const int i = blockIdx.x * 32 + lane;
+  const int per = (nblk + NN_RSL - 1) / NN_RSL, b0 = sl * per, b1 = min(nblk, b0 + per);
+  float sum = 0.f, car = 0.f;
+  if (i < NN_NPARAM) {
+#pragma unroll 4
+    for (int b = b0; b < b1; ++b) nn_two_sum(sum, car, part[(long long)b * NN_NPARAM + i]);
+  }
+  sh[sl][0][lane] = sum;
+  sh[sl][1][lane] = car;
+  __syncthreads();
+  if (sl > 0 || i >= NN_NPARAM) return;
+#pragma unroll
+  for (int k = 1; k < NN_RSL; ++k) {
+    nn_two_sum(sum, car, sh[k][0][lane]);
+    car += sh[k][1][lane];
+  }
+  grad[i] = sum + car;
 }
 
 // BF16 copies of W2 in both layouts
@@ -917,7 +942,7 @@ cudaError_t nn_backward(int n1, const float* prm, const void* W2ov, const float*
   }
   if (e != cudaSuccess) return e;
   count_launch();
-  k_nn_reduce<<<(NN_NPARAM + 255) / 256, 256, 0, s>>>(part, nblk, grad);
+  k_nn_reduce<<<(NN_NPARAM + 31) / 32, 32 * NN_RSL, 0, s>>>(part, nblk, grad);
   return cudaGetLastError();
 }
 
