@@ -515,20 +515,15 @@ struct GatherCfg {
 // (d is passed in z). GE elements per block and iteration (grid-stride), one thread per node,
 // GS sources per thread (the node's position, neighbour tests and offsets shared by them).
 // All loads of the group are issued before the first sum: the contributions of one
-// source at a time left too few bytes in flight. GS = 4 in FP32 (2 is 7 % slower
-// for the smoother at p = 7, 1 17 %), 2 in FP64 (registers; 4 is 1 % slower).
+// source at a time left too few bytes in flight. At most 4 in FP32, 2 in FP64
+// (registers; 4 is 1 % slower); gather_n1 chooses.
 // Measured (GB300, FP32, d and x not touched): 16^3, p = 7, 42 sources 0.516 ->
 // 0.262 ms for 1.04 GB, 8^3, p = 6, 56 sources 66 -> 36 us.
-template <typename T>
-constexpr int gather_sources() {
-  return sizeof(T) == 4 ? 4 : 2;
-}
-template <typename T, int N1, int MODE>
+template <typename T, int N1, int MODE, int GS>
 __global__ void __launch_bounds__(GatherCfg<N1>::THREADS)
     k_schwarz_gather(const LevelOp* __restrict__ op, const T* __restrict__ zp, T* __restrict__ z, T* __restrict__ x,
                      T c1, T c2, const int* __restrict__ act, int nact) {
   constexpr int MP = N1 + 2, MP2 = MP * MP, MP3 = MP2 * MP, NPE = N1 * N1 * N1, GE = GatherCfg<N1>::GE;
-  constexpr int GS = gather_sources<T>();
   const int nx = op->n[0], ny = op->n[1], nz = op->n[2];
   const int E = op->E;
   const long long Nq = op->Nq;
@@ -634,25 +629,43 @@ __global__ void __launch_bounds__(GatherCfg<N1>::THREADS)
 }
 
 // z = M r from the patch solutions (the second kernel of the smoother)
-template <typename T, int N1>
-static cudaError_t gather_n1(const LevelOp& hop, const LevelOp* dop, const T* zp, T* z, T* x, int mode, double c1,
+template <typename T, int N1, int GS>
+static cudaError_t gather_gs(const LevelOp& hop, const LevelOp* dop, const T* zp, T* z, T* x, int mode, double c1,
                              double c2, const int* act, int nact, cudaStream_t s) {
   constexpr int GT = GatherCfg<N1>::THREADS;
   // the gather indexes one source's patch buffer with 32-bit offsets
   if ((long long)hop.E * (N1 + 2) * (N1 + 2) * (N1 + 2) >= (1LL << 31)) return cudaErrorInvalidValue;
   long long gx = (hop.E + GatherCfg<N1>::GE - 1) / GatherCfg<N1>::GE;
-  const long long ngroups = (nact + gather_sources<T>() - 1) / gather_sources<T>();
+  const long long ngroups = (nact + GS - 1) / GS;
   const long long cap = 152LL * GATHER_WAVE / ngroups + 1;
   if (gx > cap) gx = cap;
   const dim3 grid((unsigned)gx, (unsigned)ngroups);
   count_launch();
   switch (mode) {
-    case 0: k_schwarz_gather<T, N1, 0><<<grid, GT, 0, s>>>(dop, zp, z, x, (T)c1, (T)c2, act, nact); break;
-    case 1: k_schwarz_gather<T, N1, 1><<<grid, GT, 0, s>>>(dop, zp, z, x, (T)c1, (T)c2, act, nact); break;
-    case 2: k_schwarz_gather<T, N1, 2><<<grid, GT, 0, s>>>(dop, zp, z, x, (T)c1, (T)c2, act, nact); break;
-    default: k_schwarz_gather<T, N1, 3><<<grid, GT, 0, s>>>(dop, zp, z, x, (T)c1, (T)c2, act, nact); break;
+    case 0: k_schwarz_gather<T, N1, 0, GS><<<grid, GT, 0, s>>>(dop, zp, z, x, (T)c1, (T)c2, act, nact); break;
+    case 1: k_schwarz_gather<T, N1, 1, GS><<<grid, GT, 0, s>>>(dop, zp, z, x, (T)c1, (T)c2, act, nact); break;
+    case 2: k_schwarz_gather<T, N1, 2, GS><<<grid, GT, 0, s>>>(dop, zp, z, x, (T)c1, (T)c2, act, nact); break;
+    default: k_schwarz_gather<T, N1, 3, GS><<<grid, GT, 0, s>>>(dop, zp, z, x, (T)c1, (T)c2, act, nact); break;
   }
   return cudaGetLastError();
+}
+
+// As few groups as the largest size allows, all of about one size: a thread of a group
+// with fewer sources than its size repeats the loads of the last one. Smoother, FP32, us,
+// groups of 1 / 2 / 3 / 4: 16^3, p = 7, 1 source 71 / 77 / 77 / 80, 2 sources 106 / 101 /
+// 102 / 105, 5 sources 191 / 185 / 173 / 180; p = 6, 1 source 29.7 / 31.6 / 33.5 / 36.9, 3
+// sources 67 / 64 / 57 / 61, 9 sources 191 / 174 / 162 / 171.
+template <typename T, int N1>
+static cudaError_t gather_n1(const LevelOp& hop, const LevelOp* dop, const T* zp, T* z, T* x, int mode, double c1,
+                             double c2, const int* act, int nact, cudaStream_t s) {
+  constexpr int MAXGS = sizeof(T) == 4 ? 4 : 2;
+  const int groups = (nact + MAXGS - 1) / MAXGS, gs = (nact + groups - 1) / groups;
+  if constexpr (MAXGS == 4) {
+    if (gs == 4) return gather_gs<T, N1, 4>(hop, dop, zp, z, x, mode, c1, c2, act, nact, s);
+    if (gs == 3) return gather_gs<T, N1, 3>(hop, dop, zp, z, x, mode, c1, c2, act, nact, s);
+  }
+  return gs == 2 ? gather_gs<T, N1, 2>(hop, dop, zp, z, x, mode, c1, c2, act, nact, s)
+                 : gather_gs<T, N1, 1>(hop, dop, zp, z, x, mode, c1, c2, act, nact, s);
 }
 
 template <typename T>
