@@ -78,10 +78,10 @@ struct SwCfg {
   }
 };
 
-template <typename T, int N1>
+template <typename T, int N1, int EPB_ = SwCfg<T, N1>::slots(sizeof(T) == 4 ? 128 : 64)>
 struct SwShape {
   using C = SwCfg<T, N1>;
-  static constexpr int EPB = C::slots(sizeof(T) == 4 ? 128 : 64);
+  static constexpr int EPB = EPB_;
   static constexpr int THREADS = (EPB * C::TPE + 31) / 32 * 32;
   // resident threads per SM asked of ptxas (p = 6, 8^3, 56 sources: 101 us at 640, 104 at 768, 147 at 1024; two or
   // one line per thread instead of three 105 to 117)
@@ -90,15 +90,15 @@ struct SwShape {
   static constexpr size_t SMEM = sizeof(T) * ((size_t)SW_MAXCLS * 3 * C::TB + (size_t)EPB * C::SE);
 };
 
-template <typename T, int N1>
-__global__ void __launch_bounds__(SwShape<T, N1>::THREADS, SwShape<T, N1>::MINB)
+template <typename T, int N1, int EPB>
+__global__ void __launch_bounds__(SwShape<T, N1, EPB>::THREADS, SwShape<T, N1, EPB>::MINB)
     k_schwarz_patch(const __grid_constant__ SwGeom g, const unsigned char* __restrict__ blob, const T* __restrict__ r,
                     T* __restrict__ zp, const int* __restrict__ act, int nact) {
   using C = SwCfg<T, N1>;
-  using H = SwShape<T, N1>;
+  using H = SwShape<T, N1, EPB>;
   constexpr int MP = C::MP, MP2 = C::MP2, MP3 = C::MP3, NF = N1 * N1, NPE = NF * N1;
   constexpr int SJ = C::SJ, SK = C::SK, SE = C::SE, RP = C::RP, TB = C::TB, TPE = C::TPE, LPT = C::LPT;
-  constexpr int EPB = H::EPB, NT = H::THREADS;
+  constexpr int NT = H::THREADS;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   T* tabs = reinterpret_cast<T*>(smem_raw);
   T* buf = tabs + SW_MAXCLS * 3 * TB;
@@ -460,13 +460,12 @@ __global__ void __launch_bounds__(SwSmall<T, N1>::THREADS)
   });
 }
 
-template <typename T, int N1>
+template <typename T, int N1, typename H = SwShape<T, N1>>
 static cudaError_t patch_fill(const SwTables& tb, const T* r, T* zp, const int* act, int nact, cudaStream_t s) {
-  using H = SwShape<T, N1>;
   const SwGeom& g = tb.geom;
   const long long items = (long long)g.n[0] * g.n[1] * g.n[2] * nact;
   const long long groups = (items + H::EPB - 1) / H::EPB;
-  auto kern = k_schwarz_patch<T, N1>;
+  auto kern = k_schwarz_patch<T, N1, H::EPB>;
   if (H::SMEM > 48 * 1024) {
     const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)H::SMEM);
     if (e != cudaSuccess) return e;
@@ -487,10 +486,28 @@ static cudaError_t patch_fill(const SwTables& tb, const T* r, T* zp, const int* 
 // 1024 41.3 / 41.5, 4096 152 / 119; p = 6 512 54 / 68, 1024 103 / 100; p = 8 64 28.1 /
 // 29.7, 256 53.7 / 50.1; p = 1 512 4.2 / 6.6, 4096 14.6 / 14.1; FP32 p = 6 512 6.2 /
 // 7.9, 1024 9.2 / 8.0; p = 4 256 3.2 / 4.4, 1024 5.6 / 5.0; p = 2 1024 3.5 / 5.7.
+// In FP64 large blocks leave the SM that gets one more than the others alone for long: at
+// p = 7 (three patches, 320 threads) the kernel whose busiest SM has less to do, at p = 6
+// (three patches, 256 threads) blocks of one patch up to ten per SM, but not where blocks
+// of three are two for every SM. us, one patch and two lanes per line / three patches: p =
+// 7 540 68 / 99, 1050 118 / 147, 2400 256 / 275; one patch / three: p = 6 686 59 / 67, 875
+// 91 / 79, 1296 112 / 123, 1536 115 / 119, 3430 257 / 240.
 template <typename T, int N1>
 static cudaError_t patch_n1(const SwTables& tb, const T* r, T* zp, const int* act, int nact, cudaStream_t s) {
   const long long items = (long long)tb.geom.n[0] * tb.geom.n[1] * tb.geom.n[2] * nact;
-  if (items * (SwSmall<T, N1>::THREADS / 32) > 152 * (N1 < 9 ? 24 : 8)) return patch_fill<T, N1>(tb, r, zp, act, nact, s);
+  bool small = items * (SwSmall<T, N1>::THREADS / 32) <= 152 * (N1 < 9 ? 24 : 8);
+  if constexpr (sizeof(T) == 8 && N1 == 8) {
+    // the busier SM's warps, of which the small kernel's do half the work each
+    using H = SwShape<T, N1>;
+    auto busiest = [&](long long blocks, int threads) { return (blocks + 151) / 152 * threads; };
+    small |= items <= 152 * 24 && busiest(items, SwSmall<T, N1>::THREADS) / 2 <
+                                      busiest((items + H::EPB - 1) / H::EPB, H::THREADS);
+  }
+  if constexpr (sizeof(T) == 8 && N1 == 7) {
+    const bool even = items > 152 * 5 && items <= 152 * 6;  // two blocks of three on every SM
+    if (!small && items <= 152 * 10 && !even) return patch_fill<T, N1, SwShape<T, N1, 1>>(tb, r, zp, act, nact, s);
+  }
+  if (!small) return patch_fill<T, N1>(tb, r, zp, act, nact, s);
   using S = SwSmall<T, N1>;
   static_assert(S::SMEM <= 48 * 1024, "one patch and its tables");
   count_launch();
