@@ -24,18 +24,17 @@
 // per slot; in the pass along a direction a thread owns the lines of the two
 // elements that are neighbours along it, so the traces across their common face
 // stay in registers, and a brick reads 24 outer neighbours instead of the 48 of
-// eight single elements. All global reads (own elements and the outer
-// neighbours' lines, reduced to traces at once) happen before the first
-// barrier. The tables are kernel parameters: every product takes its constant
+// eight single elements. Own elements and the outer neighbours' lines (reduced to
+// traces at once) are read before the barrier ahead of the x pass, the operand of a
+// residual in the z pass. The tables are kernel parameters: every product takes its constant
 // from the constant bank, so shared memory carries only the field.
 //
 // Measured (GB300; before: one element per slot, dense blocks and tables in
 // shared memory): FP32 16^3, p = 7, 42 fields 0.720 -> 0.279 ms (2.5 TB/s of the
 // 0.70 GB in and out), 8^3, p = 6, 56 fields 0.100 -> 0.042 ms; bound by
 // shared-memory wavefronts, then by the neighbours' reads. FP64, at the rate of
-// its pipe before and after: 7.86 -> 7.25 ms and 0.955 -> 0.824 ms; at p = 3 and
-// 1, where folding saves nothing, 0.83 -> 0.86 ms and 0.089 -> 0.111 ms (16^3, 42
-// fields; 3 % and 0.4 % of an FP64 build).
+// its pipe before and after: 7.86 -> 7.01 ms and 0.954 -> 0.793 ms, p = 3 and 1 (16^3,
+// 42 fields) 0.828 -> 0.820 and 0.087 -> 0.054 ms.
 #include "dg_line.h"
 
 namespace dg {
@@ -50,6 +49,9 @@ namespace dg {
 template <typename T, int N1>
 struct ApplyTab {
   static constexpr int HO = N1 / 2, HE = N1 - HO;
+  // FP64 with few nodes: neighbours enter by their values (see line_direct)
+  static constexpr bool DIRECT = sizeof(T) == 8 && N1 <= 3;
+  static constexpr int DN = DIRECT ? N1 : 1;
   T Ke[3][HE][HE], Ko[3][HO][HO];                          // K on the even and the odd part
   T cve[3][HE], cde[3][HE], cvo[3][HO], cdo[3][HO];        // couplings (neighbour value / derivative)
   T tl[N1], dl[N1];                                        // trace and derivative at a line's left end
@@ -57,6 +59,7 @@ struct ApplyTab {
   T mm[3][N1 * N1];                                        // products of the two other axes' masses, by line
   int n[3], nb[3];                                         // elements and bricks per axis
   long long Nq, items;                                     // nodes of a source; bricks of all sources
+  T K[3][DN][DN], C[3][DN][DN], B[3][DN][DN];  // own block, coupling to the right neighbour, right boundary face
 };
 
 template <typename T, int N1>
@@ -86,7 +89,17 @@ static void fill_tab(ApplyTab<T, N1>& t, const LevelOp& op) {
     t.gam[d] = (T)(A.sigma * A.h);
     t.n[d] = op.n[d];
   }
-  if (N1 == 2) {
+  if constexpr (ApplyTab<T, N1>::DIRECT) {
+    for (int d = 0; d < 3; ++d) {
+      const AxisOp& A = op.ax[d];
+      for (int a = 0; a < N1; ++a)
+        for (int i = 0; i < N1; ++i) {
+          t.K[d][a][i] = (T)(0.5 * (A.Kd[0][a * N1 + i] + A.Kd[0][(N1 - 1 - a) * N1 + (N1 - 1 - i)]));
+          t.C[d][a][i] = (T)(A.cRv[a] * op.tl[i] + A.cRd[a] * op.dl[i]);
+          t.B[d][a][i] = (T)(A.cRd[a] * (op.dr[i] + A.sigma * A.h * op.tr[i]) - A.cRv[a] * op.tr[i]);
+        }
+    }
+  } else if (N1 == 2) {
     for (int d = 0; d < 3; ++d) {
       const AxisOp& A = op.ax[d];
       t.Ke[d][0][0] = (T)A.Kd[0][0];
@@ -104,14 +117,25 @@ static void fill_tab(ApplyTab<T, N1>& t, const LevelOp& op) {
   t.Nq = op.Nq;
 }
 
-// Launch shape. BR: elements of a brick along each axis (2 or 1).
+// Launch shape. BR: elements of a brick along each axis (2 or 1); BPB: bricks of a
+// block. FP64 at p = 2: 126 of 128 lanes at work, instead of 288 of 288 in blocks that
+// are too large for a few thousand elements.
 template <typename T, int N1, int BR>
+constexpr int apply_bpb() {
+  return sizeof(T) == 8 && N1 == 3 ? 14 : best_bpb(BR * BR * N1 * N1, sizeof(T) == 4 ? 128 : 64);
+}
+// smaller blocks for FP64 where the full ones are large (288 and 256 threads)
+template <int N1>
+constexpr int apply_few() {
+  return N1 == 6 ? 5 : N1 == 7 ? 3 : apply_bpb<double, N1, 1>();
+}
+template <typename T, int N1, int BR, int BPB_ = apply_bpb<T, N1, BR>()>
 struct ApplyCfg {
   static constexpr int NPE = N1 * N1 * N1, NF = N1 * N1;
   static constexpr int EB = BR * BR * BR;        // elements of a brick
   static constexpr int LINES = BR * BR * NF;     // threads of a brick: one (pair of) line(s) each
   static constexpr int PB = LineLayout<N1>::PB, PZ = LineLayout<N1>::PZ, ES = LineLayout<N1>::ES;
-  static constexpr int BPB = best_bpb(LINES, sizeof(T) == 4 ? 128 : 64);
+  static constexpr int BPB = BPB_;
   static constexpr int THREADS = (BPB * LINES + 31) / 32 * 32;
   static constexpr size_t SMEM = sizeof(T) * 2 * (size_t)BPB * EB * ES;
   // resident threads per SM asked of ptxas (register cap 65536 / that)
@@ -119,20 +143,75 @@ struct ApplyCfg {
   static constexpr int MINB = WANT / THREADS < 1 ? 1 : WANT / THREADS;
 };
 
+// What lies beyond the two ends of a line (pair), 0: left of the first, 1: right of the
+// last line: ov, od the traces there (value, derivative), or with DIRECT ov[end N1 + i]
+// the values of the neighbour's line (at a boundary face of the own line). The left
+// neighbour's derivative is kept along the axis in FP32 and against it in FP64, where a
+// change of sign is an operation of the pipe that bounds the kernel.
+template <typename T>
+constexpr bool left_inward() {
+  return sizeof(T) == 8;
+}
+template <typename T, int N1>
+constexpr int outer_vals() {
+  return ApplyTab<T, N1>::DIRECT ? 2 * N1 : 2;
+}
+template <typename T, int N1>
+__device__ __forceinline__ void left_end(const ApplyTab<T, N1>& tab, const T* v, T& val, T& der) {
+  if constexpr (left_inward<T>())
+    end_inward<T, N1, true>(tab.tl, tab.dl, v, val, der);
+  else
+    end_trace<T, N1, true>(tab.tl, tab.dl, v, val, der);
+}
+
+// The pass of line_op for FP64 at p = 1 and 2, bound by the FP64 pipe: the coupling
+// block of a neighbour has N1^2 entries, no more than a trace and its lifting take
+// (4 N1), and nothing is folded: 12 and 27 multiply-adds a line instead of 20 and 34
+// operations. The left neighbour's and the left boundary's blocks are the right ones'
+// mirror images. Which block an end takes is selected, not branched on: lanes at the
+// boundary would double the products of their warp. The own block comes last: its
+// error against 64-bit exact lines is then no larger than with traces.
+// Measured (GB300, 16^3, 20 fields; with traces, folded at p = 2, and before those): p =
+// 1 45 / 53 -> 27 us, p = 2 150 / 172 -> 122 us.
+template <typename T, int N1, int D>
+__device__ __forceinline__ void line_direct(const ApplyTab<T, N1>& tab, T* v, const T* ov, bool in0, bool in1) {
+  T r[N1];
+#pragma unroll
+  for (int a = 0; a < N1; ++a) {
+    const int m = N1 - 1 - a;
+    T acc = mul(in0 ? tab.C[D][m][N1 - 1] : tab.B[D][m][N1 - 1], ov[0]);
+#pragma unroll
+    for (int i = 1; i < N1; ++i)
+      acc = mad(in0 ? tab.C[D][m][N1 - 1 - i] : tab.B[D][m][N1 - 1 - i], ov[i], acc);
+#pragma unroll
+    for (int i = 0; i < N1; ++i) acc = mad(in1 ? tab.C[D][a][i] : tab.B[D][a][i], ov[N1 + i], acc);
+#pragma unroll
+    for (int i = 0; i < N1; ++i) acc = mad(tab.K[D][a][i], v[i], acc);
+    r[a] = acc;
+  }
+#pragma unroll
+  for (int a = 0; a < N1; ++a) v[a] = r[a];
+}
+
 // one pass along direction D for this thread's line (pair): on entry v[s] holds
-// the line values, ov/od the traces beyond its two ends (0: left of the first, 1:
-// right of the last line). On exit v[s] holds the unscaled result.
+// the line values, ov/od what is beyond its two ends (in0, in1: a neighbour). On exit
+// v[s] holds the unscaled result.
 template <typename T, int N1, int BR, int D>
 __device__ __forceinline__ void line_op(const ApplyTab<T, N1>& tab, T (*v)[N1], const T* ov, const T* od,
-                                        bool second) {
+                                        bool second, bool in0, bool in1) {
   constexpr int HO = N1 / 2, HE = N1 - HO;
+  if constexpr (ApplyTab<T, N1>::DIRECT) {
+    static_assert(BR == 1, "bricks are FP32's");
+    line_direct<T, N1, D>(tab, v[0], ov, in0, in1);
+    return;
+  }
   T e[BR][HE], o[BR][HO == 0 ? 1 : HO];
   T tv[BR], td[BR];  // the pair's traces on their common face
 #pragma unroll
   for (int s = 0; s < BR; ++s) {
     if (BR == 2) {
       if (s == 0)
-        end_trace<T, N1, true>(tab.tl, tab.dl, v[s], tv[s], td[s]);
+        left_end(tab, v[s], tv[s], td[s]);
       else
         end_trace<T, N1, false>(tab.tl, tab.dl, v[s], tv[s], td[s]);
     }
@@ -174,7 +253,8 @@ __device__ __forceinline__ void line_op(const ApplyTab<T, N1>& tab, T (*v)[N1], 
       v[s][1] = mad(tab.Ke[D][0][0], v1, y);
       continue;
     }
-    const T vp = nl + nr, vm = nl - nr, dm = dl - dr, dp = dl + dr;
+    constexpr bool NEG = left_inward<T>();
+    const T vp = nl + nr, vm = nl - nr, dm = NEG ? dl + dr : dl - dr, dp = NEG ? dr - dl : dl + dr;
     T O[HO == 0 ? 1 : HO];
 #pragma unroll
     for (int a = 0; a < HO; ++a) {
@@ -185,7 +265,7 @@ __device__ __forceinline__ void line_op(const ApplyTab<T, N1>& tab, T (*v)[N1], 
     }
 #pragma unroll
     for (int a = 0; a < HE; ++a) {
-      T acc = mad(tab.cde[D][a], dm, mul(tab.cve[D][a], vp));
+      T acc = mad(NEG ? -tab.cde[D][a] : tab.cde[D][a], dm, mul(tab.cve[D][a], vp));
 #pragma unroll
       for (int i = 0; i < HE; ++i) acc = mad(tab.Ke[D][a][i], e[s][i], acc);
       if (a < HO) {
@@ -198,11 +278,11 @@ __device__ __forceinline__ void line_op(const ApplyTab<T, N1>& tab, T (*v)[N1], 
   }
 }
 
-// traces beyond the ends of this thread's line (pair) along D: of the outer
-// neighbours where there are any (out0, out1), else those that the boundary
-// stands for, from the line's own values. Read reversed, the own line looks
-// like the neighbour's: value t and derivative -d at the common face. ue points
-// at the brick's first element, es is the element stride along D (elements).
+// what lies beyond the ends of this thread's line (pair) along D: the outer
+// neighbours' where there are any (out0, out1), else what the boundary stands for,
+// from the line's own values. Read reversed, the own line looks like the
+// neighbour's: value t and derivative -d at the common face. ue points at the
+// brick's first element, es is the element stride along D (elements).
 template <typename T, int N1, int BR, int D>
 __device__ __forceinline__ void outer_traces(const ApplyTab<T, N1>& tab, const T* __restrict__ ue, long long pair,
                                              int l1, int l2, long long es, bool second, bool out0, bool out1,
@@ -211,12 +291,17 @@ __device__ __forceinline__ void outer_traces(const ApplyTab<T, N1>& tab, const T
   constexpr int SD = D == 0 ? 1 : (D == 1 ? N1 : NF);
   const int base = D == 0 ? N1 * l1 + NF * l2 : (D == 1 ? l1 + NF * l2 : l1 + N1 * l2);
   const T* p = ue + pair * NPE + base;
+  if constexpr (ApplyTab<T, N1>::DIRECT) {
+    load_line<T, N1, SD>(out0 ? p - es * NPE : p, false, vec, ov);
+    load_line<T, N1, SD>(out1 ? p + es * NPE : p, false, vec, ov + N1);
+    return;
+  }
   const T gam = tab.gam[D];
   T v[N1];
   load_line<T, N1, SD>(out0 ? p - es * NPE : p, !out0, vec, v);
-  end_trace<T, N1, true>(tab.tl, tab.dl, v, ov[0], od[0]);
+  left_end(tab, v, ov[0], od[0]);
   if (!out0) {
-    od[0] = mad(-gam, ov[0], -od[0]);
+    od[0] = mad(left_inward<T>() ? gam : -gam, ov[0], -od[0]);
     ov[0] = -ov[0];
   }
   const int last = BR == 2 && second ? 1 : 0;
@@ -228,12 +313,12 @@ __device__ __forceinline__ void outer_traces(const ApplyTab<T, N1>& tab, const T
   }
 }
 
-template <typename T, int N1, int BR>
-__global__ void __launch_bounds__(ApplyCfg<T, N1, BR>::THREADS, ApplyCfg<T, N1, BR>::MINB)
+template <typename T, int N1, int BR, int BPB>
+__global__ void __launch_bounds__(ApplyCfg<T, N1, BR, BPB>::THREADS, ApplyCfg<T, N1, BR, BPB>::MINB)
     k_apply(const __grid_constant__ ApplyTab<T, N1> tab, const T* __restrict__ u, T* __restrict__ out,
             const T* __restrict__ rin, const int* __restrict__ act, int mode, int vec_i) {
-  using C = ApplyCfg<T, N1, BR>;
-  constexpr int NPE = C::NPE, NF = C::NF, EB = C::EB, BPB = C::BPB, LINES = C::LINES;
+  using C = ApplyCfg<T, N1, BR, BPB>;
+  constexpr int NPE = C::NPE, NF = C::NF, EB = C::EB, LINES = C::LINES;
   constexpr int PB = C::PB, PZ = C::PZ, ES = C::ES;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   T* su = reinterpret_cast<T*>(smem_raw);
@@ -294,7 +379,7 @@ __global__ void __launch_bounds__(ApplyCfg<T, N1, BR>::THREADS, ApplyCfg<T, N1, 
         for (int i = 0; i < N1; ++i) su[zat + 4 * s * ES + i * PZ] = v[s][i];
       }
   }
-  T ov[3][2], od[3][2];
+  T ov[3][outer_vals<T, N1>()], od[3][2];
 #define DG_OUT(d, s) ((flag & ((8 << (s)) << (2 * (d)))) != 0)
   if (have[0])
     outer_traces<T, N1, BR, 0>(tab, ue, pe[0], l1, l2, est[0], flag & 1, DG_OUT(0, 0), DG_OUT(0, 1), vec, ov[0], od[0]);
@@ -311,7 +396,7 @@ __global__ void __launch_bounds__(ApplyCfg<T, N1, BR>::THREADS, ApplyCfg<T, N1, 
     for (int s = 0; s < BR; ++s)
 #pragma unroll
       for (int i = 0; i < N1; ++i) v[s][i] = s == 0 || sec ? su[at + s * ES + i] : (T)0;
-    line_op<T, N1, BR, 0>(tab, v, ov[0], od[0], sec);
+    line_op<T, N1, BR, 0>(tab, v, ov[0], od[0], sec, DG_OUT(0, 0), DG_OUT(0, 1));
     const T sc = tab.mm[0][l];
 #pragma unroll
     for (int s = 0; s < BR; ++s)
@@ -329,7 +414,7 @@ __global__ void __launch_bounds__(ApplyCfg<T, N1, BR>::THREADS, ApplyCfg<T, N1, 
     for (int s = 0; s < BR; ++s)
 #pragma unroll
       for (int i = 0; i < N1; ++i) v[s][i] = s == 0 || sec ? su[at + 2 * s * ES + i * PB] : (T)0;
-    line_op<T, N1, BR, 1>(tab, v, ov[1], od[1], sec);
+    line_op<T, N1, BR, 1>(tab, v, ov[1], od[1], sec, DG_OUT(1, 0), DG_OUT(1, 1));
     const T sc = tab.mm[1][l];
 #pragma unroll
     for (int s = 0; s < BR; ++s)
@@ -359,7 +444,7 @@ __global__ void __launch_bounds__(ApplyCfg<T, N1, BR>::THREADS, ApplyCfg<T, N1, 
     for (int s = 0; s < BR; ++s)
 #pragma unroll
       for (int i = 0; i < N1; ++i) v[s][i] = s == 0 || sec ? su[zat + 4 * s * ES + i * PZ] : (T)0;
-    line_op<T, N1, BR, 2>(tab, v, ov[2], od[2], sec);
+    line_op<T, N1, BR, 2>(tab, v, ov[2], od[2], sec, DG_OUT(2, 0), DG_OUT(2, 1));
     const T sc = tab.mm[2][l];
 #pragma unroll
     for (int s = 0; s < BR; ++s)
@@ -367,7 +452,19 @@ __global__ void __launch_bounds__(ApplyCfg<T, N1, BR>::THREADS, ApplyCfg<T, N1, 
 #pragma unroll
         for (int i = 0; i < N1; ++i) {
           const T Au = mad(sc, v[s][i], sacc[zat + 4 * s * ES + i * PZ]);
-          out[g0 + s * est[2] * NPE + i * NF] = mode == 0 ? Au : r[s][i] - Au;
+          if constexpr (sizeof(T) == 8)
+            v[s][i] = Au;
+          else
+            out[g0 + s * est[2] * NPE + i * NF] = mode == 0 ? Au : r[s][i] - Au;
+        }
+        if constexpr (sizeof(T) == 8) {  // a branch: the FP64 pipe would pay for a select's difference
+          if (mode == 0) {
+#pragma unroll
+            for (int i = 0; i < N1; ++i) out[g0 + s * est[2] * NPE + i * NF] = v[s][i];
+          } else {
+#pragma unroll
+            for (int i = 0; i < N1; ++i) out[g0 + s * est[2] * NPE + i * NF] = r[s][i] - v[s][i];
+          }
         }
       }
   }
@@ -390,14 +487,14 @@ struct ApplySmall {
 
 template <typename T, int N1, int D>
 __device__ __forceinline__ void small_pass(const ApplyTab<T, N1>& tab, const T* su, T* res, int l1, int l2, const T* ov,
-                                           const T* od) {
+                                           const T* od, bool in0, bool in1) {
   using Y = LineLayout<N1>;
   constexpr int ST = D == 0 ? 1 : (D == 1 ? Y::PB : Y::PZ);
   const int at = D == 0 ? Y::PB * l1 + Y::PZ * l2 : (D == 1 ? l1 + Y::PZ * l2 : l1 + Y::PB * l2);
   T v[1][N1];
 #pragma unroll
   for (int i = 0; i < N1; ++i) v[0][i] = su[at + ST * i];
-  line_op<T, N1, 1, D>(tab, v, ov, od, false);
+  line_op<T, N1, 1, D>(tab, v, ov, od, false, in0, in1);
 #pragma unroll
   for (int i = 0; i < N1; ++i) res[at + ST * i] = v[0][i];
 }
@@ -417,23 +514,25 @@ __global__ void __launch_bounds__(ApplySmall<N1>::THREADS)
   for (int t = threadIdx.x; t < NPE; t += NT) su[t % N1 + Y::PB * ((t / N1) % N1) + Y::PZ * (t / NF)] = __ldg(ue + t);
   const int d = threadIdx.x / GROUP, l = threadIdx.x - d * GROUP, l1 = l % N1, l2 = l / N1;
   const bool on = l < NF, vec = vec_i != 0;
-  T ov[2], od[2];
+  T ov[outer_vals<T, N1>()], od[2];
+  const bool in0 = (d == 0 ? ex : d == 1 ? ey : ez) > 0;
+  const bool in1 = d == 0 ? ex < nx - 1 : d == 1 ? ey < ny - 1 : ez < tab.n[2] - 1;
   if (on) {
     if (d == 0)
-      outer_traces<T, N1, 1, 0>(tab, ue, 0, l1, l2, 1, false, ex > 0, ex < nx - 1, vec, ov, od);
+      outer_traces<T, N1, 1, 0>(tab, ue, 0, l1, l2, 1, false, in0, in1, vec, ov, od);
     else if (d == 1)
-      outer_traces<T, N1, 1, 1>(tab, ue, 0, l1, l2, nx, false, ey > 0, ey < ny - 1, vec, ov, od);
+      outer_traces<T, N1, 1, 1>(tab, ue, 0, l1, l2, nx, false, in0, in1, vec, ov, od);
     else
-      outer_traces<T, N1, 1, 2>(tab, ue, 0, l1, l2, (long long)nx * ny, false, ez > 0, ez < tab.n[2] - 1, vec, ov, od);
+      outer_traces<T, N1, 1, 2>(tab, ue, 0, l1, l2, (long long)nx * ny, false, in0, in1, vec, ov, od);
   }
   __syncthreads();
   if (on) {
     if (d == 0)
-      small_pass<T, N1, 0>(tab, su, sr[0], l1, l2, ov, od);
+      small_pass<T, N1, 0>(tab, su, sr[0], l1, l2, ov, od, in0, in1);
     else if (d == 1)
-      small_pass<T, N1, 1>(tab, su, sr[1], l1, l2, ov, od);
+      small_pass<T, N1, 1>(tab, su, sr[1], l1, l2, ov, od, in0, in1);
     else
-      small_pass<T, N1, 2>(tab, su, sr[2], l1, l2, ov, od);
+      small_pass<T, N1, 2>(tab, su, sr[2], l1, l2, ov, od, in0, in1);
   }
   __syncthreads();
   for (int t = threadIdx.x; t < NPE; t += NT) {
@@ -456,10 +555,10 @@ static cudaError_t apply_small(const LevelOp& hop, int mode, const T* u, T* out,
   return cudaGetLastError();
 }
 
-template <typename T, int N1, int BR>
+template <typename T, int N1, int BR, int BPB = apply_bpb<T, N1, BR>()>
 static cudaError_t apply_br(const LevelOp& hop, int mode, const T* u, T* out, const T* rin, const int* act, int nact,
                             cudaStream_t s) {
-  using C = ApplyCfg<T, N1, BR>;
+  using C = ApplyCfg<T, N1, BR, BPB>;
   ApplyTab<T, N1> tab;
   fill_tab<T, N1>(tab, hop);
   long long per = 1;
@@ -472,7 +571,7 @@ static cudaError_t apply_br(const LevelOp& hop, int mode, const T* u, T* out, co
   if (blocks > 0x7fffffffLL) return cudaErrorInvalidValue;
   // 16-byte reads of an element's values: the field and every element of it aligned
   const int vec = ((uintptr_t)u & 15) == 0 && (C::NPE * sizeof(T)) % 16 == 0 && (hop.Nq * sizeof(T)) % 16 == 0;
-  auto kern = k_apply<T, N1, BR>;
+  auto kern = k_apply<T, N1, BR, BPB>;
   if (C::SMEM > 48 * 1024) {
     const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)C::SMEM);
     if (e != cudaSuccess) return e;
@@ -483,24 +582,27 @@ static cudaError_t apply_br(const LevelOp& hop, int mode, const T* u, T* out, co
 }
 
 // Few elements: one group of threads per direction, while its warps are at most 24 per
-// SM in FP64, and 13 in FP32 or where N1^2 divides 32 (p = 1, 3: the other kernel's
-// warps are full there). Measured around the line (us, small / single elements): FP64
-// p = 4 256 elements 6.2 / 10.3, 1024 15.3 / 17.1, 4096 51 / 47; p = 6 512 23.6 / 23.9,
-// 2048 76 / 67; p = 8 256 24.8 / 31.8; p = 2 1024 9.4 / 12.4; p = 3 512 7.7 / 7.7, 2048
-// 22 / 14; p = 1 512 4.7 / 5.1, 2048 12.1 / 5.1; FP32 p = 5 315 3.7 / 4.2, 1260 6.3 /
-// 5.1; p = 4 256 2.9 / 3.3, 1024 3.9 / 3.6; p = 8 64 4.0 / 4.4, 256 5.4 / 4.5.
+// SM in FP64 (16 at p = 5, where 36 lines leave half of a group's lanes idle) and 13 in
+// FP32 and at p <= 3. Measured around the line (us, small / single elements): FP64 p = 1
+// 512 elements 3.4 / 3.6, 2048 6.8 / 3.7; p = 2 512 4.9 / 5.8, 1024 7.5 / 6.0; p = 3 512
+// 7.5 / 7.6, 2048 22 / 14; p = 4 512 9.4 / 10.0, 1024 15.1 / 16.5, 4096 51 / 45; p = 5 375
+// 15.6 / 16.0, 512 19.9 / 16.1; p = 6 512 23.5 / 23.4, 2048 75 / 65; p = 8 250 24.8 / 31.3;
+// FP32 p = 5 315 3.7 / 4.2, 1260 6.3 / 5.1; p = 4 256 2.9 / 3.3, 1024 3.9 / 3.6; p = 8 64
+// 4.0 / 4.4, 256 5.4 / 4.5.
 // Then bricks of eight elements in FP32, where reading the neighbours is what bounds
 // the kernel (single elements / bricks: p = 6 4096 elements 10.7 / 8.2 us, 512 4.1 /
 // 4.5; p = 5 2880 6.5 / 6.3, 960 4.3 / 4.9), with two blocks for every SM and, on odd
 // meshes, at least half of the elements that the bricks have room for; single
 // elements otherwise and in FP64 (bound by the FP64 pipe, to which a brick saves
-// nothing).
+// nothing), in blocks of the size that leaves the busiest SM fewer warps (small /
+// full blocks: p = 5 512 elements 16.1 / 23.1, 1372 29.1 / 42.8, 20480 362 / 342; p = 6
+// 1536 55 / 65, 2048 68 / 65).
 template <typename T, int N1>
 static cudaError_t apply_n1(const LevelOp& hop, int mode, const T* u, T* out, const T* rin, const int* act, int nact,
                             cudaStream_t s) {
   if (nact == 0) return cudaSuccess;
   const long long items = (long long)nact * hop.E;
-  constexpr int warps = sizeof(T) == 8 && 32 % (N1 * N1) != 0 ? 24 : 13;
+  constexpr int warps = sizeof(T) == 4 || N1 <= 4 ? 13 : N1 == 6 ? 16 : 24;
   if (items * (ApplySmall<N1>::THREADS / 32) <= 152 * warps)
     return apply_small<T, N1>(hop, mode, u, out, rin, act, nact, s);
   if constexpr (sizeof(T) == 4) {
@@ -508,6 +610,12 @@ static cudaError_t apply_n1(const LevelOp& hop, int mode, const T* u, T* out, co
     for (int d = 0; d < 3; ++d) br *= (hop.n[d] + 1) / 2;
     if (br / ApplyCfg<T, N1, 2>::BPB >= 2 * 152 && 8 * br <= 2 * items)
       return apply_br<T, N1, 2>(hop, mode, u, out, rin, act, nact, s);
+  } else if constexpr (apply_few<N1>() != apply_bpb<T, N1, 1>()) {
+    using F = ApplyCfg<T, N1, 1>;
+    using S = ApplyCfg<T, N1, 1, apply_few<N1>()>;
+    auto busiest = [&](long long bpb, int threads) { return ((items + bpb - 1) / bpb + 151) / 152 * (threads / 32); };
+    if (busiest(S::BPB, S::THREADS) < busiest(F::BPB, F::THREADS))
+      return apply_br<T, N1, 1, S::BPB>(hop, mode, u, out, rin, act, nact, s);
   }
   return apply_br<T, N1, 1>(hop, mode, u, out, rin, act, nact, s);
 }

@@ -41,10 +41,11 @@ struct LineLayout {
   static_assert(PZ >= PB * (N1 - 1) + N1 && ES >= (PZ + PB + 1) * (N1 - 1) + 1, "element layout overlaps");
 };
 
-// value and derivative at the left (RIGHT: right) end of a line, from the basis
-// values tl and derivatives dl at the left end (mirrored for the right one)
+// value and derivative at the left end of a line (RIGHT: at the right end, the
+// derivative into the line, that is of the reversed line), from the basis values tl
+// and derivatives dl at the left end
 template <typename T, int N1, bool RIGHT>
-__device__ __forceinline__ void end_trace(const T* tl, const T* dl, const T* v, T& val, T& der) {
+__device__ __forceinline__ void end_inward(const T* tl, const T* dl, const T* v, T& val, T& der) {
   T a = mul(tl[RIGHT ? N1 - 1 : 0], v[0]), b = mul(dl[RIGHT ? N1 - 1 : 0], v[0]);
 #pragma unroll
   for (int i = 1; i < N1; ++i) {
@@ -53,7 +54,13 @@ __device__ __forceinline__ void end_trace(const T* tl, const T* dl, const T* v, 
     b = mad(dl[k], v[i], b);
   }
   val = a;
-  der = RIGHT ? -b : b;
+  der = b;
+}
+// the same with the derivative along the axis
+template <typename T, int N1, bool RIGHT>
+__device__ __forceinline__ void end_trace(const T* tl, const T* dl, const T* v, T& val, T& der) {
+  end_inward<T, N1, RIGHT>(tl, dl, v, val, der);
+  if (RIGHT) der = -der;
 }
 
 // line of N1 values at p with stride SD, reversed where rev is set; contiguous
