@@ -621,9 +621,8 @@ static cudaError_t apply_n1(const LevelOp& hop, int mode, const T* u, T* out, co
 }
 
 template <typename T>
-cudaError_t launch_apply(const LevelOp& hop, const LevelOp* dop, int mode, const T* u, T* out, const T* rin,
-                         const int* act, int nact, cudaStream_t s) {
-  (void)dop;
+cudaError_t launch_apply(const LevelOp& hop, int mode, const T* u, T* out, const T* rin, const int* act, int nact,
+                         cudaStream_t s) {
   switch (hop.n1) {
     case 2: return apply_n1<T, 2>(hop, mode, u, out, rin, act, nact, s);
     case 3: return apply_n1<T, 3>(hop, mode, u, out, rin, act, nact, s);
@@ -664,10 +663,10 @@ cudaError_t launch_inv_diag(const LevelOp& hop, const LevelOp* dop, T* invD, cud
   return cudaGetLastError();
 }
 
-template cudaError_t launch_apply<double>(const LevelOp&, const LevelOp*, int, const double*, double*,
-                                          const double*, const int*, int, cudaStream_t);
-template cudaError_t launch_apply<float>(const LevelOp&, const LevelOp*, int, const float*, float*, const float*,
-                                         const int*, int, cudaStream_t);
+template cudaError_t launch_apply<double>(const LevelOp&, int, const double*, double*, const double*, const int*, int,
+                                          cudaStream_t);
+template cudaError_t launch_apply<float>(const LevelOp&, int, const float*, float*, const float*, const int*, int,
+                                         cudaStream_t);
 template cudaError_t launch_inv_diag<double>(const LevelOp&, const LevelOp*, double*, cudaStream_t);
 template cudaError_t launch_inv_diag<float>(const LevelOp&, const LevelOp*, float*, cudaStream_t);
 

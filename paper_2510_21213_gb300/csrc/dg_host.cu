@@ -324,7 +324,7 @@ static int pcg(dg_ctx* h, PrecWork<T>& w, const std::vector<int>& act0, const st
     }
   }
   auto phaseA = [&]() -> int {
-    DG_CK(launch_apply<T>(h->levels[0].op, h->levels[0].dop, 0, p, q, nullptr, dact, nact, s));
+    DG_CK(launch_apply<T>(h->levels[0].op, 0, p, q, nullptr, dact, nact, s));
     DG_CK(launch_dot<T>(p, q, nullptr, scal(h, S_PQ), part, Nq, dact, nact, s));
     count_launch();
     k_ratio<<<(nact + 127) / 128, 128, 0, s>>>(scal(h, S_RZ), scal(h, S_PQ), scal(h, S_AL), dact, nact, flags, 1);
@@ -358,7 +358,7 @@ static int pcg(dg_ctx* h, PrecWork<T>& w, const std::vector<int>& act0, const st
     const int lim[2] = {0, maxit};  // counter, iteration limit
     DG_CK(cudaMemcpyAsync(loop_counter(h), lim, sizeof(lim), cudaMemcpyHostToDevice, s));
     auto phaseAm = [&]() -> int {
-      DG_CK(launch_apply<T>(h->levels[0].op, h->levels[0].dop, 0, p, q, nullptr, dact, nact, s));
+      DG_CK(launch_apply<T>(h->levels[0].op, 0, p, q, nullptr, dact, nact, s));
       DG_CK(launch_dot<T>(p, q, nullptr, scal(h, S_PQ), part, Nq, dact, nact, s));
       count_launch();
       k_ratio_masked<<<(nact + 127) / 128, 128, 0, s>>>(scal(h, S_RZ), scal(h, S_PQ), scal(h, S_AL), dact, nact,
@@ -505,7 +505,7 @@ static int true_residual(dg_ctx* h, const std::vector<int>& act, const std::vect
   DG_RET(upload_act(h, act, s));
   const int* dact = h->act.as<int>();
   const int nact = (int)act.size();
-  DG_CK(launch_apply<double>(h->levels[0].op, h->levels[0].dop, 1, h->x64.as<double>(), h->r64.as<double>(),
+  DG_CK(launch_apply<double>(h->levels[0].op, 1, h->x64.as<double>(), h->r64.as<double>(),
                              h->b64.as<double>(), dact, nact, s));
   DG_CK(launch_dot<double>(h->r64.as<double>(), h->r64.as<double>(), nullptr, scal(h, S_RR), h->part.as<double>(),
                            h->Nq, dact, nact, s));
@@ -858,7 +858,7 @@ static int estimate_lambda_schwarz(dg_ctx* h, int l, double* out) {
   std::vector<double> al, be;
   const int K = (int)std::min<long long>(24, N);
   for (int k = 0; k < K; ++k) {
-    DG_CK(launch_apply<double>(L.op, L.dop, 0, p.as<double>(), q.as<double>(), nullptr, a, 1, 0));
+    DG_CK(launch_apply<double>(L.op, 0, p.as<double>(), q.as<double>(), nullptr, a, 1, 0));
     double pq = 0.0;
     DG_RET(dot(p.as<double>(), q.as<double>(), &pq));
     if (!(pq > 0.0) || !(rz > 0.0)) break;
@@ -1292,10 +1292,10 @@ int dg_apply_operator(dg_handle h, int32_t level, int32_t fp32, const void* u, v
     for (int k = 0; k < nb; ++k) a[k] = k;
     DG_RET(upload_act(h, a, s));
     if (fp32)
-      DG_CK(launch_apply<float>(L.op, L.dop, 0, (const float*)u + b0 * L.op.Nq, (float*)out + b0 * L.op.Nq, nullptr,
+      DG_CK(launch_apply<float>(L.op, 0, (const float*)u + b0 * L.op.Nq, (float*)out + b0 * L.op.Nq, nullptr,
                                 h->act.as<int>(), nb, s));
     else
-      DG_CK(launch_apply<double>(L.op, L.dop, 0, (const double*)u + b0 * L.op.Nq, (double*)out + b0 * L.op.Nq,
+      DG_CK(launch_apply<double>(L.op, 0, (const double*)u + b0 * L.op.Nq, (double*)out + b0 * L.op.Nq,
                                  nullptr, h->act.as<int>(), nb, s));
   }
   return DG_OK;

@@ -140,12 +140,11 @@ struct GemmArgs {
 // ---------------------------------------------------------------------------
 // out = A u (mode 0), out = rin - A u (mode 1), out -= A u (mode 2)
 template <typename T>
-cudaError_t launch_apply(const LevelOp& hop, const LevelOp* dop, int mode, const T* u, T* out, const T* rin,
-                         const int* act, int nact, cudaStream_t s);
+cudaError_t launch_apply(const LevelOp& hop, int mode, const T* u, T* out, const T* rin, const int* act, int nact,
+                         cudaStream_t s);
 template <typename T>
 cudaError_t launch_inv_diag(const LevelOp& hop, const LevelOp* dop, T* invD, cudaStream_t s);
 
-// invD == nullptr: the residual argument is already preconditioned
 template <typename T>
 cudaError_t launch_cheb_first(T* x, T* d, const T* r, const T* invD, double c, int set_x, long long Nq,
                               const int* act, int nact, cudaStream_t s);

@@ -292,7 +292,7 @@ static int coarse_guess(dg_ctx* h, int nsrc, const int* dact, int nact, cudaStre
     const Level& L = h->levels[l1];
     float* t = w.p.as<float>();
     float* u = w.q.as<float>();
-    DG_CK(launch_apply<float>(L.op, L.dop, 1, xl, t, bl, dact, nact, s));
+    DG_CK(launch_apply<float>(L.op, 1, xl, t, bl, dact, nact, s));
     DG_RET(mg.vcycle(l1, t, u));
     DG_CK((launch_convert<float, float>(xl, u, L.op.Nq, dact, nact, 1.0, 1, s)));
   }
@@ -346,7 +346,7 @@ static int guess_fp32(dg_ctx* h, int nsrc, const int* dact, int nact, bool use_n
   const LevelOp& F = h->levels[0].op;
   double* part = h->part.as<double>();
   DG_RET(coarse_guess(h, nsrc, dact, nact, s));
-  DG_CK(launch_apply<float>(F, h->levels[0].dop, 0, w.x.as<float>(), w.z.as<float>(), nullptr, dact, nact, s));
+  DG_CK(launch_apply<float>(F, 0, w.x.as<float>(), w.z.as<float>(), nullptr, dact, nact, s));
   DG_CK(launch_dot<float>(w.x.as<float>(), w.r.as<float>(), nullptr, scal(h, S_G1), part, Nq, dact, nact, s));
   DG_CK(launch_dot<float>(w.x.as<float>(), w.z.as<float>(), nullptr, scal(h, S_G2), part, Nq, dact, nact, s));
   count_launch();
@@ -390,7 +390,7 @@ int learned_guess(dg_ctx* h, int nsrc, const std::vector<int>& act, const std::v
   DG_RET(guess_fp32(h, nsrc, dact, nact, use_net, false, true, s));
   DG_CK((launch_convert<double, float>(x64, h->w32.q.as<float>(), Nq, dact, nact, 1.0, 0, s)));
   // energy-optimal scaling alpha = b^T x0 / x0^T A x0, residual r = b - alpha A x0 (FP64)
-  DG_CK(launch_apply<double>(h->levels[0].op, h->levels[0].dop, 0, x64, r64, nullptr, dact, nact, s));
+  DG_CK(launch_apply<double>(h->levels[0].op, 0, x64, r64, nullptr, dact, nact, s));
   DG_CK(launch_dot<double>(x64, b64, nullptr, scal(h, S_G1), part, Nq, dact, nact, s));
   DG_CK(launch_dot<double>(x64, r64, nullptr, scal(h, S_G2), part, Nq, dact, nact, s));
   count_launch();

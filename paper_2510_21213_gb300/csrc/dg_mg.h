@@ -38,7 +38,7 @@ struct MG {
     const double sig1 = theta / delta;
     const T* r0 = b;
     if (!zero_init) {
-      DG_CK(launch_apply<T>(L.op, L.dop, 1, x, res, b, act, nact, s));
+      DG_CK(launch_apply<T>(L.op, 1, x, res, b, act, nact, s));
       r0 = res;
     }
     if (sw)
@@ -50,9 +50,9 @@ struct MG {
     bool res_is_b = zero_init;  // the residual of the current x is b - A d when res_is_b
     for (int j = 2; j <= k; ++j) {
       if (res_is_b)
-        DG_CK(launch_apply<T>(L.op, L.dop, 1, d, res, b, act, nact, s));
+        DG_CK(launch_apply<T>(L.op, 1, d, res, b, act, nact, s));
       else
-        DG_CK(launch_apply<T>(L.op, L.dop, 2, d, res, nullptr, act, nact, s));
+        DG_CK(launch_apply<T>(L.op, 2, d, res, nullptr, act, nact, s));
       res_is_b = false;
       const double rho = 1.0 / (2.0 * sig1 - rho_prev);
       if (sw)
@@ -64,9 +64,9 @@ struct MG {
     }
     if (want_res) {
       if (res_is_b)
-        DG_CK(launch_apply<T>(L.op, L.dop, 1, d, res, b, act, nact, s));
+        DG_CK(launch_apply<T>(L.op, 1, d, res, b, act, nact, s));
       else
-        DG_CK(launch_apply<T>(L.op, L.dop, 2, d, res, nullptr, act, nact, s));
+        DG_CK(launch_apply<T>(L.op, 2, d, res, nullptr, act, nact, s));
     }
     return DG_OK;
   }

@@ -23,7 +23,7 @@ __global__ void k_cheb_first(T* __restrict__ x, T* __restrict__ d, const T* __re
   const long long rhs = act[blockIdx.y];
   const long long off = rhs * Nq;
   for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < Nq; i += (long long)gridDim.x * blockDim.x) {
-    const T v = invD ? c * invD[i] * r[off + i] : c * r[off + i];
+    const T v = c * invD[i] * r[off + i];
     d[off + i] = v;
     x[off + i] = set_x ? v : x[off + i] + v;
   }
@@ -34,7 +34,7 @@ __global__ void k_cheb_step(T* __restrict__ x, T* __restrict__ d, const T* __res
                             const T* __restrict__ invD, T c1, T c2, long long Nq, const int* __restrict__ act) {
   const long long off = (long long)act[blockIdx.y] * Nq;
   for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < Nq; i += (long long)gridDim.x * blockDim.x) {
-    const T v = c1 * d[off + i] + (invD ? c2 * invD[i] * res[off + i] : c2 * res[off + i]);
+    const T v = c1 * d[off + i] + c2 * invD[i] * res[off + i];
     d[off + i] = v;
     x[off + i] += v;
   }
