@@ -210,7 +210,7 @@ bool octree_faces(const dg_mesh_desc* root, const int32_t* leaves, int32_t n_lea
 // block per leaf with every face interpolated to Gauss points and back before):
 // FP32 396 -> 20 us (5 us of it the hanging faces), FP64 974 -> 255 us; the V-cycle of
 // the FP64 solve, three degrees of this operator and the leaf-block inverse, 9.8 ->
-// 4.2 ms; a mixed solve of 8 sources to 1e-10 241 -> 85 ms by this alone (43 ms with
+// 4.2 ms; a mixed solve of 8 sources to 1e-12 238 -> 84 ms by this alone (42 ms with
 // the fused leaf-block inverse and the 16-row boundary GEMM).
 // ---------------------------------------------------------------------------
 

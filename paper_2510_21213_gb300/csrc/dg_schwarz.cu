@@ -33,10 +33,9 @@
 //     by each block of a persistent grid.
 // Measured (GB300; before: all six passes through shared memory, dense
 // transforms, a division per node, tables per patch): FP64 16^3, p = 7, 42
-// sources 22.0 -> 15.6 ms, 8^3, p = 6, 56 sources 2.33 -> 1.91 ms, 4^3, p = 4, 4
-// sources 35 -> 17 us; FP32 8^3, p = 6, 56 sources 152 -> 101 us, 16^3, p = 3, 42
-// sources 273 -> 139 us, p = 1 89 -> 39 us, 6 x 10 x 8, p = 5, 21 sources 51 -> 22
-// us. FP64 runs at the rate of its pipe; FP32 issues in 55 % of the cycles with
+// sources 22.0 -> 15.6 ms, 8^3, p = 6, 56 sources 2.33 -> 1.91 ms; FP32 8^3, p = 6, 56
+// sources 150 -> 98 us, 16^3, p = 3, 42 sources 271 -> 137 us, p = 1 86 -> 37 us, 6 x 10
+// x 8, p = 5, 21 sources 49 -> 20 us (in a graph; 2 to 3 us more by single launches). FP64 runs at the rate of its pipe; FP32 issues in 55 % of the cycles with
 // a quarter of the warps resident (96 registers).
 #include "dg_fdm.h"
 #include "dg_swtc.h"
@@ -272,8 +271,9 @@ __global__ void __launch_bounds__(SwShape<T, N1, EPB>::THREADS, SwShape<T, N1, E
 // and odd parts of the nodes change hands by a shuffle. Each sum is that of
 // k_schwarz_patch, so the results are the same bits. Only the patch's own three
 // tables are staged, and the reciprocals are loaded up front.
-// Measured (GB300, FP64, inside a solve; one lane per line before): 4^3, 4 sources, p =
-// 4 14.1 -> 13.3 us, p = 2 8.9 -> 6.0.
+// Measured (GB300, FP64, 4^3, 4 sources; k_schwarz_patch with one patch per block, and
+// with the several that are used for many patches): p = 4 13.3 us (14.1, 22.4), p = 2 5.9
+// (8.9, 10.1).
 template <typename T, int N1>
 struct SwSmall {
   using C = SwCfg<T, N1>;

@@ -854,7 +854,7 @@ __global__ void k_kmat_partial(const double* __restrict__ psi, const double* __r
 // The same for N <= KSMALL: thread = one output (i, j) and one of 256 / N^2 slices
 // of a stage's nodes, so that no FMA is spent on the padding of a 32 x 32 tile
 // (10x at N = 10, 256x at N = 2); the slices are added in order at the end.
-// Measured (GB300): both kernels 4^3, p = 4, N = 2 276 -> 6 us, 8^3, p = 6, N = 10 542 -> 60 us.
+// Measured (GB300): both kernels 4^3, p = 4, N = 2 276 -> 6 us, 8^3, p = 6, N = 10 542 -> 52 us.
 __global__ void __launch_bounds__(256) k_kmat_small(const double* __restrict__ psi, const double* __restrict__ W,
                                                     const double* __restrict__ Wacc, int N, long long Nq,
                                                     double* __restrict__ part) {
