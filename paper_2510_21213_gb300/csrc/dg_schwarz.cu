@@ -35,8 +35,9 @@
 // transforms, a division per node, tables per patch): FP64 16^3, p = 7, 42
 // sources 22.0 -> 15.6 ms, 8^3, p = 6, 56 sources 2.33 -> 1.91 ms; FP32 8^3, p = 6, 56
 // sources 150 -> 98 us, 16^3, p = 3, 42 sources 271 -> 137 us, p = 1 86 -> 37 us, 6 x 10
-// x 8, p = 5, 21 sources 49 -> 20 us (in a graph; 2 to 3 us more by single launches). FP64 runs at the rate of its pipe; FP32 issues in 55 % of the cycles with
-// a quarter of the warps resident (96 registers).
+// x 8, p = 5, 21 sources 49 -> 20 us (in a graph; 2 to 3 us more by single launches).
+// FP64 runs at the rate of its pipe; FP32 issues in 55 % of the cycles with a quarter of
+// the warps resident (96 registers).
 #include "dg_fdm.h"
 #include "dg_swtc.h"
 

@@ -15,7 +15,10 @@ LO, HI, N = [-2.0, -1.0, -1.0], [2.0, 1.5, 1.0], (3, 2, 2)
 
 
 def _leaves(dgx, p):
-    leaves = dgx.dg_octree_refine(LO, HI, N, p, lambda x: np.exp(-40.0 * np.sum((x - 0.4) ** 2, axis=1)), 1e-4 if p < 4 else 1e-7, 2 if p < 7 else 1)
+    def rho(x):
+        return np.exp(-40.0 * np.sum((x - 0.4) ** 2, axis=1))
+
+    leaves = dgx.dg_octree_refine(LO, HI, N, p, rho, 1e-4 if p < 4 else 1e-7, 2 if p < 7 else 1)
     assert len(set(leaves[:, 0].tolist())) > 1
     return leaves
 
